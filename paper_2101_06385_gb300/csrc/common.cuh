@@ -16,6 +16,7 @@
 
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
+#include <stddef.h>
 #include <stdint.h>
 
 #include "../../include/sp2.h"
@@ -70,12 +71,42 @@ struct Ctl {
   double e_min, e_max;
   double trace_final;
   LayerParams next;           // parameters of the next squaring launch
-  int sigma[kMaxL + 1];       // sigma[k] = sigma_k, sigma[0] = 0
-  double iderr[kMaxL + 1];    // iderr[k] = IdErr_k
   // accelerated solve (Sec. "Accelerated Deep-NN SP2")
   int accel, pad2;
   double acc_homo, acc_lumo;  // caller's HOMO / LUMO energy estimates
   double acc_l, acc_h;        // unoccupied eigenvalues of the scaled iterate in [0, l], occupied in [h, 1]
+  // history (last: a resident solve keeps only the part before it in shared memory)
+  int sigma[kMaxL + 1];       // sigma[k] = sigma_k, sigma[0] = 0
+  double iderr[kMaxL + 1];    // iderr[k] = IdErr_k
+};
+constexpr size_t kCtlHotBytes = offsetof(Ctl, sigma);
+
+// The history a control step reads and extends: the control block's own
+// arrays, or (resident solve) the last four layers in shared memory with the
+// full record kept in the control block by one CTA.
+struct CtlHistory {
+  Ctl* c;
+  __device__ __forceinline__ int sigma(int n) const { return c->sigma[n]; }
+  __device__ __forceinline__ double iderr(int n) const { return c->iderr[n]; }
+  __device__ __forceinline__ void set(int n, int s, double e) {
+    c->sigma[n] = s;
+    c->iderr[n] = e;
+  }
+};
+struct RingHistory {
+  int* s;      // [4]
+  double* e;   // [4]
+  Ctl* record; // nullptr: this CTA keeps no record
+  __device__ __forceinline__ int sigma(int n) const { return s[n & 3]; }
+  __device__ __forceinline__ double iderr(int n) const { return e[n & 3]; }
+  __device__ __forceinline__ void set(int n, int sg, double er) {
+    s[n & 3] = sg;
+    e[n & 3] = er;
+    if (record) {
+      record->sigma[n] = sg;
+      record->iderr[n] = er;
+    }
+  }
 };
 
 // ---------------------------------------------------------------- helpers
@@ -85,75 +116,91 @@ __device__ __forceinline__ void split_fp16(float x, float lo_scale, __half& hi, 
   lo = __float2half_rn((x - __half2float(hi)) * lo_scale);
 }
 
+// Input layer Y_0 = W_0 H + B_0 - alpha_0 I (Alg. 1): off-diagonal -h inv in
+// FP32 with inv as a sum of two floats and one FMA (-h inv_hi + (-h inv_lo)
+// rounded once: the correctly rounded FP64 value except within 2^-47 of a
+// rounding boundary), the diagonal in FP64.
+struct InputScale {
+  double inv = 0.0, diag_add = 0.0;
+  float inv_hi = 0.f, inv_lo = 0.f;
+};
+__device__ __forceinline__ InputScale input_scale(double e_min, double e_max, int shift) {
+  InputScale s;
+  s.inv = 1.0 / (e_max - e_min);
+  s.diag_add = shift ? 0.0 : e_max * s.inv;
+  s.inv_hi = (float)s.inv;
+  s.inv_lo = (float)(s.inv - (double)s.inv_hi);
+  return s;
+}
+__device__ __forceinline__ float input_offdiag(float h, const InputScale& s) {
+  return fmaf(-h, s.inv_hi, -h * s.inv_lo);
+}
+__device__ __forceinline__ float input_diag(float h, const InputScale& s) {
+  return (float)(-(double)h * s.inv + s.diag_add);
+}
+
 __device__ __forceinline__ double warp_sum_d(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
 
-// Branch sigma applied to the stored iterate: sets alpha_next and the launch
-// coefficients (see the header comment).  After re-centring, the new iterate
-// is stored around alpha = 1/2: the shift difference goes into cc.
-__device__ inline void set_branch(Ctl* c, int sigma, bool final_layer) {
-  const double a = c->alpha;
-  double an, ca, cb, cc = 0.0;
+// Coefficients of the next launch as a control step chooses them: diagonal
+// update Y'_ii = ca Y_ii + cb P_ii + cc, off-diagonal ca, cb, and the shift an
+// of the iterate that the launch stores.
+struct LayerCoef {
+  double ca, cb, cc, an;
+};
+
+// Branch sigma applied to the iterate stored around alpha = a (see the header
+// comment).  After re-centring, the new iterate is stored around alpha = 1/2:
+// the shift difference goes into cc.
+__device__ inline LayerCoef branch_coef(double a, int sigma, bool recentered) {
+  LayerCoef k;
+  k.cc = 0.0;
   if (sigma > 0) {
-    an = a * a;
-    ca = 2.0 * a;
-    cb = 1.0;
+    k.an = a * a;
+    k.ca = 2.0 * a;
+    k.cb = 1.0;
   } else {
-    an = 2.0 * a - a * a;
-    ca = 2.0 - 2.0 * a;
-    cb = -1.0;
+    k.an = 2.0 * a - a * a;
+    k.ca = 2.0 - 2.0 * a;
+    k.cb = -1.0;
   }
-  if (c->recentered) {
-    cc = an - 0.5;
-    an = 0.5;
+  if (recentered) {
+    k.cc = k.an - 0.5;
+    k.an = 0.5;
   }
-  c->alpha_next = an;
-  LayerParams p;
-  p.ca = (float)ca;
-  p.cb = (float)cb;
-  p.ca_d = ca;
-  p.cb_d = cb;
-  p.cc_d = cc;
-  p.alpha_out = final_layer ? an : 0.0;
-  p.active = 1;
-  p.out_mode = final_layer ? OUT_D : OUT_Y;
-  p.rc = 0.f;
-  p.pad = 0;
-  p.rc_d = 0.0;
-  p.alpha_new = 0.0;
-  c->next = p;
+  return k;
 }
 
-// Control step of Alg. 1, run by one thread after the launch that stored a
-// new iterate (the input layer for n = 0).  trY / sqY are the FP64 sums of
-// the Y just stored.  Decides sigma_{n+1}, IdErr_{n+1} and the stop rules
-// (IdErr <= tol, IdErr <= 0, the 4.5 rule after a sign change, max_iter), or
-// moves on to the two refinement layers of Eq. 15.
 // Generalised layer S' = a S^2 + b S + c I on the stored S = alpha I + Y:
 // S' = (a alpha^2 + b alpha + c) I + (2 a alpha + b) Y + a Y^2.
-__device__ inline void set_poly(Ctl* c, double a, double b, double cp, bool final_layer) {
-  const double al = c->alpha;
-  double an = a * al * al + b * al + cp;
-  const double ca = 2.0 * a * al + b, cb = a;
-  double cc = 0.0;
-  if (c->recentered) {
-    cc = an - 0.5;
-    an = 0.5;
-  } else if (!c->shift) {
-    cc = an;
-    an = 0.0;
+__device__ inline LayerCoef poly_coef(double al, double a, double b, double cp, bool recentered, int shift) {
+  LayerCoef k;
+  k.an = a * al * al + b * al + cp;
+  k.ca = 2.0 * a * al + b;
+  k.cb = a;
+  k.cc = 0.0;
+  if (recentered) {
+    k.cc = k.an - 0.5;
+    k.an = 0.5;
+  } else if (!shift) {
+    k.cc = k.an;
+    k.an = 0.0;
   }
-  c->alpha_next = an;
+  return k;
+}
+
+__device__ inline void set_next(Ctl* c, const LayerCoef& k, float fca, float fcb, bool final_layer) {
+  c->alpha_next = k.an;
   LayerParams p;
-  p.ca = (float)ca;
-  p.cb = (float)cb;
-  p.ca_d = ca;
-  p.cb_d = cb;
-  p.cc_d = cc;
-  p.alpha_out = final_layer ? an : 0.0;
+  p.ca = fca;
+  p.cb = fcb;
+  p.ca_d = k.ca;
+  p.cb_d = k.cb;
+  p.cc_d = k.cc;
+  p.alpha_out = final_layer ? k.an : 0.0;
   p.active = 1;
   p.out_mode = final_layer ? OUT_D : OUT_Y;
   p.rc = 0.f;
@@ -188,9 +235,29 @@ __device__ inline int accel_layer(double& l, double& h, double& a, double& b, do
   return -1;
 }
 
+// Where a control step takes its coefficients from: computed when chosen
+// (here), or looked up among those that a resident solve prepared while the
+// layer's products ran.
+struct CoefNow {
+  __device__ __forceinline__ void branch(Ctl* c, int sigma, bool final_layer) const {
+    next(c, branch_coef(c->alpha, sigma, c->recentered != 0), final_layer);
+  }
+  // the accelerated layer on the bounds (l, h): the new bounds and its sign
+  __device__ __forceinline__ int accel(Ctl* c, double& l, double& h, LayerCoef& k) const {
+    double pa, pb, pc;
+    const int s = accel_layer(l, h, pa, pb, pc);
+    k = poly_coef(c->alpha, pa, pb, pc, c->recentered != 0, c->shift);
+    return s;
+  }
+  __device__ __forceinline__ void next(Ctl* c, const LayerCoef& k, bool final_layer) const {
+    set_next(c, k, (float)k.ca, (float)k.cb, final_layer);
+  }
+};
+
 // Control step of the accelerated solve: the layers follow the bounds alone;
 // IdErr is recorded for the statistics and the re-centring of the shift.
-__device__ inline void accel_control_step(Ctl* c, double trY, double sqY) {
+template <class History, class Coef>
+__device__ inline void accel_control_step(Ctl* c, double trY, double sqY, History hist, Coef coef) {
   const double N = (double)c->N;
   if (c->phase == PHASE_LOOP) {
     const int n1 = c->n + 1;
@@ -207,13 +274,13 @@ __device__ inline void accel_control_step(Ctl* c, double trY, double sqY) {
         return;
       }
     }
-    c->iderr[n1] = err;
     if (c->shift && !c->recentered && err <= kRecenterFrac * N) c->recentered = 1;
-    double l = c->acc_l, h = c->acc_h, pa, pb, pc;
-    const int s = accel_layer(l, h, pa, pb, pc);
+    double l = c->acc_l, h = c->acc_h;
+    LayerCoef lc;
+    const int s = coef.accel(c, l, h, lc);
     c->acc_l = l;
     c->acc_h = h;
-    c->sigma[n1] = s;
+    hist.set(n1, s, err);
     c->n = n1;
     const bool done = fmax(l, 1.0 - h) <= c->tol;
     const bool final_layer = done || n1 >= c->max_iter;
@@ -221,7 +288,65 @@ __device__ inline void accel_control_step(Ctl* c, double trY, double sqY) {
       c->converged_by = done ? SP2_STOP_BOUNDS : SP2_STOP_MAXITER;
       c->phase = PHASE_REFINE_B;  // the next step (after the OUT_D launch) finishes
     }
-    set_poly(c, pa, pb, pc, final_layer);
+    coef.next(c, lc, final_layer);
+  } else if (c->phase == PHASE_REFINE_B) {
+    c->trace_final = N * c->alpha + trY;
+    c->phase = PHASE_DONE;
+    c->next.active = 0;
+    if (c->status == SP2_OK && c->converged_by == SP2_STOP_MAXITER) c->status = SP2_NOT_CONVERGED;
+  }
+}
+
+// Control step of Alg. 1, run by one thread after the launch that stored a
+// new iterate (the input layer for n = 0).  trY / sqY are the FP64 sums of
+// the Y just stored.  Decides sigma_{n+1}, IdErr_{n+1} and the stop rules
+// (IdErr <= tol, IdErr <= 0, the 4.5 rule after a sign change, max_iter), or
+// moves on to the two refinement layers of Eq. 15.
+template <class History, class Coef>
+__device__ inline void control_step(Ctl* c, double trY, double sqY, History hist, Coef coef) {
+  c->trY = trY;
+  c->sqY = sqY;
+  c->alpha = c->alpha_next;
+  if (c->accel) {
+    accel_control_step(c, trY, sqY, hist, coef);
+    return;
+  }
+  const double N = (double)c->N;
+  if (c->phase == PHASE_LOOP) {
+    if (c->stop_pending) {
+      int s = (c->n >= 3) ? hist.sigma(c->n - 2) : 1;  // f_final order from sigma_{n-2}
+      s = (s >= 0) ? 1 : -1;
+      c->sigma_a = s;
+      c->phase = PHASE_REFINE_A;
+      coef.branch(c, s, false);
+      return;
+    }
+    const int n1 = c->n + 1;
+    const double a = c->alpha;
+    const double NS = N * a + trY;                      // Tr[S_n]
+    const double NX = N * a * a + 2.0 * a * trY + sqY;  // Tr[S_n^2] = ||S_n||_F^2
+    const double err = N * a * (1.0 - a) + (1.0 - 2.0 * a) * trY - sqY;  // N_S - N_X
+    const double no = (double)c->n_occ;
+    const double v = fabs(2.0 * NS - NX - no) - fabs(NX - no) - (double)hist.sigma(c->n) * c->eps;
+    const int s = (v >= 0.0) ? 1 : -1;
+    if (c->shift && !c->recentered && err <= kRecenterFrac * N) c->recentered = 1;
+    int stop = SP2_STOP_NONE;
+    if (c->tol > 0.0 && err <= c->tol)
+      stop = SP2_STOP_TOL;
+    else if (err <= 0.0)
+      stop = SP2_STOP_IDERR;
+    else if (n1 > 2 && hist.sigma(n1 - 1) != hist.sigma(n1 - 2) && err > 4.5 * hist.iderr(n1 - 2) * hist.iderr(n1 - 2))
+      stop = SP2_STOP_RULE45;
+    else if (n1 >= c->max_iter)
+      stop = SP2_STOP_MAXITER;
+    hist.set(n1, s, err);
+    c->n = n1;
+    c->stop_pending = stop;
+    if (stop) c->converged_by = stop;
+    coef.branch(c, s, false);
+  } else if (c->phase == PHASE_REFINE_A) {
+    c->phase = PHASE_REFINE_B;
+    coef.branch(c, -c->sigma_a, true);
   } else if (c->phase == PHASE_REFINE_B) {
     c->trace_final = N * c->alpha + trY;
     c->phase = PHASE_DONE;
@@ -231,56 +356,7 @@ __device__ inline void accel_control_step(Ctl* c, double trY, double sqY) {
 }
 
 __device__ inline void control_step(Ctl* c, double trY, double sqY) {
-  c->trY = trY;
-  c->sqY = sqY;
-  c->alpha = c->alpha_next;
-  if (c->accel) {
-    accel_control_step(c, trY, sqY);
-    return;
-  }
-  const double N = (double)c->N;
-  if (c->phase == PHASE_LOOP) {
-    if (c->stop_pending) {
-      int s = (c->n >= 3) ? c->sigma[c->n - 2] : 1;  // f_final order from sigma_{n-2}
-      s = (s >= 0) ? 1 : -1;
-      c->sigma_a = s;
-      c->phase = PHASE_REFINE_A;
-      set_branch(c, s, false);
-      return;
-    }
-    const int n1 = c->n + 1;
-    const double a = c->alpha;
-    const double NS = N * a + trY;                      // Tr[S_n]
-    const double NX = N * a * a + 2.0 * a * trY + sqY;  // Tr[S_n^2] = ||S_n||_F^2
-    const double err = N * a * (1.0 - a) + (1.0 - 2.0 * a) * trY - sqY;  // N_S - N_X
-    const double no = (double)c->n_occ;
-    const double v = fabs(2.0 * NS - NX - no) - fabs(NX - no) - (double)c->sigma[c->n] * c->eps;
-    const int s = (v >= 0.0) ? 1 : -1;
-    c->sigma[n1] = s;
-    c->iderr[n1] = err;
-    if (c->shift && !c->recentered && err <= kRecenterFrac * N) c->recentered = 1;
-    int stop = SP2_STOP_NONE;
-    if (c->tol > 0.0 && err <= c->tol)
-      stop = SP2_STOP_TOL;
-    else if (err <= 0.0)
-      stop = SP2_STOP_IDERR;
-    else if (n1 > 2 && c->sigma[n1 - 1] != c->sigma[n1 - 2] && err > 4.5 * c->iderr[n1 - 2] * c->iderr[n1 - 2])
-      stop = SP2_STOP_RULE45;
-    else if (n1 >= c->max_iter)
-      stop = SP2_STOP_MAXITER;
-    c->n = n1;
-    c->stop_pending = stop;
-    if (stop) c->converged_by = stop;
-    set_branch(c, s, false);
-  } else if (c->phase == PHASE_REFINE_A) {
-    c->phase = PHASE_REFINE_B;
-    set_branch(c, -c->sigma_a, true);
-  } else if (c->phase == PHASE_REFINE_B) {
-    c->trace_final = N * c->alpha + trY;
-    c->phase = PHASE_DONE;
-    c->next.active = 0;
-    if (c->status == SP2_OK && c->converged_by == SP2_STOP_MAXITER) c->status = SP2_NOT_CONVERGED;
-  }
+  control_step(c, trY, sqY, CtlHistory{c}, CoefNow{});
 }
 
 // Tile descriptor of the squaring kernels: instance b, block row I, block

@@ -14,6 +14,29 @@
 
 namespace sp2 {
 
+// Lower and upper bound over n blocks' partials, by one warp (minimum and
+// maximum do not depend on the order).  A single thread's walk over them, a
+// chain of L2 loads, was most of the kernel on small matrices (N = 1000: 38 us
+// under ncu for 125 blocks).
+__device__ __forceinline__ void fold_bounds(const double2* __restrict__ part, unsigned n, double& L, double& U,
+                                            bool& nan_seen) {
+  L = INFINITY;
+  U = -INFINITY;
+  bool bad = false;
+  for (unsigned k = threadIdx.x; k < n; k += 32) {
+    const double2 p = __ldcg(&part[k]);
+    if (isnan(p.x) || isnan(p.y)) bad = true;
+    L = fmin(L, p.x);
+    U = fmax(U, p.y);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    L = fmin(L, __shfl_xor_sync(0xffffffffu, L, o));
+    U = fmax(U, __shfl_xor_sync(0xffffffffu, U, o));
+  }
+  nan_seen = __any_sync(0xffffffffu, bad);
+}
+
 // ---------------------------------------------------------------- K1
 // One warp per row: R_i = sum_j |H_ij| - |H_ii|.  Groups of sixteen are
 // summed in FP32 as a four-level tree (relative error <= 4 x 2^-24) and
@@ -90,17 +113,12 @@ __global__ void __launch_bounds__(256) gershgorin_kernel(const float* __restrict
     s_last = (atomicAdd(ticket, 1u) == gridDim.x - 1);
   }
   __syncthreads();
-  if (!s_last || threadIdx.x != 0) return;
+  if (!s_last || threadIdx.x >= 32) return;
   __threadfence();
-  double L = INFINITY, U = -INFINITY;
-  bool nonfinite = false;
-  for (unsigned k = 0; k < gridDim.x; ++k) {
-    const double2 p = __ldcg(&partials[k]);
-    if (isnan(p.x) || isnan(p.y)) nonfinite = true;
-    L = fmin(L, p.x);
-    U = fmax(U, p.y);
-  }
-  if (isnan(L) || isnan(U)) nonfinite = true;
+  double L, U;
+  bool nonfinite;
+  fold_bounds(partials, gridDim.x, L, U, nonfinite);
+  if (threadIdx.x != 0) return;
   *ticket = 0u;
   if (bounds_out) {
     bounds_out[0] = nonfinite ? NAN : L;
@@ -195,16 +213,12 @@ __global__ void __launch_bounds__(256) gershgorin_batched_kernel(const float* co
     s_last = (atomicAdd(&tickets[b], 1u) == gridDim.x - 1);
   }
   __syncthreads();
-  if (!s_last || threadIdx.x != 0) return;
+  if (!s_last || threadIdx.x >= 32) return;
   __threadfence();
-  double L = INFINITY, U = -INFINITY;
-  bool nan_seen = false;
-  for (unsigned k = 0; k < gridDim.x; ++k) {
-    const double2 p = __ldcg(&part[k]);
-    if (isnan(p.x) || isnan(p.y)) nan_seen = true;
-    L = fmin(L, p.x);
-    U = fmax(U, p.y);
-  }
+  double L, U;
+  bool nan_seen;
+  fold_bounds(part, gridDim.x, L, U, nan_seen);
+  if (threadIdx.x != 0) return;
   tickets[b] = 0u;
   Ctl* c = ctl + b;
   c->e_min = L;
@@ -256,12 +270,7 @@ __global__ void __launch_bounds__(256) input_layer_kernel(const float* const* __
     e_min = bounds[2 * b];
     e_max = bounds[2 * b + 1];
   }
-  const double inv = 1.0 / (e_max - e_min);
-  const double diag_add = shift ? 0.0 : e_max * inv;
-  // off-diagonal y = -h inv in FP32: inv as a sum of two floats and one FMA
-  // (-h inv_hi + (-h inv_lo) rounded once), the correctly rounded FP64 value
-  // except within 2^-47 of a rounding boundary; the diagonal stays in FP64
-  const float inv_hi = (float)inv, inv_lo = (float)(inv - (double)inv_hi);
+  const InputScale in = input_scale(e_min, e_max, shift);
   double tr = 0.0, sq = 0.0;
   if (active) {
     // FP16 planes: hi (plain), or hp = 2^s hi and lo' (split); hi may be absent
@@ -294,7 +303,7 @@ __global__ void __launch_bounds__(256) input_layer_kernel(const float* const* __
               for (int u = 0; u < 4; ++u) hv[u] = (c4 + u < N) ? hrow[c4 + u] : 0.f;
             }
 #pragma unroll
-            for (int u = 0; u < 4; ++u) y[u] = (c4 + u < N) ? fmaf(-hv[u], inv_hi, -hv[u] * inv_lo) : 0.f;
+            for (int u = 0; u < 4; ++u) y[u] = (c4 + u < N) ? input_offdiag(hv[u], in) : 0.f;
             // the diagonal element (at most one per group) in FP64, once
             const int du = r - c4;
             if ((unsigned)du < 4u) {
@@ -302,7 +311,7 @@ __global__ void __launch_bounds__(256) input_layer_kernel(const float* const* __
 #pragma unroll
               for (int u = 0; u < 4; ++u)
                 if (u == du) hd = hv[u];
-              const float yd = (float)(-(double)hd * inv + diag_add);
+              const float yd = input_diag(hd, in);
               tr += (double)yd;
 #pragma unroll
               for (int u = 0; u < 4; ++u)
@@ -350,9 +359,9 @@ __global__ void __launch_bounds__(256) input_layer_kernel(const float* const* __
         if (r < N && col < N) {
           const float hv = hrow[col];
           if (r == col)
-            y = (float)(-(double)hv * inv + diag_add);
+            y = input_diag(hv, in);
           else
-            y = fmaf(-hv, inv_hi, -hv * inv_lo);
+            y = input_offdiag(hv, in);
           yrow[col] = y;
           if (r == col) tr += (double)y;
           sqf = fmaf(y, y, sqf);
@@ -408,7 +417,7 @@ __global__ void __launch_bounds__(256) input_layer_kernel(const float* const* __
   if (!active) return;
   // S_0 = alpha_0 I + Y_0; the row-norm launch that follows runs the first
   // control step (sigma_1, IdErr_1) with the exact ||Y_0||_F^2.
-  c->alpha_next = shift ? e_max * inv : 0.0;
+  c->alpha_next = shift ? e_max * in.inv : 0.0;
   c->trY_new = T;
   (void)Q;
 }
