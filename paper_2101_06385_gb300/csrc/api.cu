@@ -63,7 +63,7 @@ enum BufId {
   B_HI0, B_LO0, B_HI1, B_LO1, B_Y0, B_Y1, B_CTL, B_TILES, B_TOFF, B_TCNT, B_TPART, B_IDONE,
   B_PART, B_TICKET, B_ERR, B_DPTR, B_NS, B_HS, B_TRACES, B_PARAMS, B_BOUNDS, B_RN, B_PART2,
   B_G, B_SEG, B_GH0, B_GL0, B_GH1, B_GL1, B_DOTS, B_TDOTS, B_PARAMS2, B_NALPHA, B_HP0, B_HP1, B_RNP0, B_RNP1,
-  B_READOUT, B_RDIAG, B_SEGP, B_WAVE, B_COUNT
+  B_READOUT, B_RDIAG, B_SEGP, B_WAVE, B_PACK, B_COUNT
 };
 
 struct Buf {
@@ -713,10 +713,301 @@ sp2_status sp2_layer(const float* X, int B, int N, float a, float b, float c, fl
 
 namespace {
 
+// ---- resident solves (csrc/resident.cu) ----
+
+// Tiles of one instance on the resident kernel: the live 128 x 128 tiles of
+// the upper 256 x 256 super tiles, in units of 128.
+void resident_tiles(int N, int b, std::vector<uint32_t>* out, int* count) {
+  const int T = (N + kTcBN - 1) / kTcBN, L = (N + kResTile - 1) / kResTile;
+  int n = 0;
+  for (int I = 0; I < T; ++I)
+    for (int J = I; J < T; ++J)
+      for (int i = 2 * I; i < std::min(2 * I + 2, L); ++i)
+        for (int j = 2 * J; j < std::min(2 * J + 2, L); ++j) {
+          if (out) out->push_back(pack_tile(b, i, j, 0));
+          ++n;
+        }
+  *count = n;
+}
+
+// The resident kernel takes a solve whose largest instance has no more tiles
+// than the chip has slots (two per SM; N <= 2816 on 152 SMs): below that the
+// CTA pairs' 256 x 256 tiles cannot fill the chip (at N = 2048 there are 36
+// for 76 pairs) and every layer pays a launch.
+bool resident_fits(int Nmax) {
+  if (!tc_precision(g.precision) || !g.pair_kernel || g.snake || g.wide == 1) return false;
+  if (Nmax > 32 * kResTile) return false;
+  int n = 0;
+  resident_tiles(Nmax, 0, nullptr, &n);
+  return n <= 2 * g.num_sms;
+}
+
+// Plans the slots' tile lists: instance after instance (largest first) onto
+// the run of consecutive CTAs of one slot that is free first, by estimated
+// solve times, the first slots before the second ones.  Gangs of like size
+// then share their CTAs and take turns: while one's products run the other is
+// in its epilogue and meeting (N = 1024: 17 us of products per layer and pair
+// of tiles; unaligned, a gang also waits for its slowest CTA's other tile,
+// 28 us per layer), and a gang finds the CTAs of the one before it free
+// together.  More tiles than CTAs: the instance takes both slots.
+void resident_plan(const int* order, const int* N, const int* toff, const int* tcnt, int B, int grid, int* loff,
+                   int* list) {
+  std::vector<double> free_at((size_t)2 * grid, 0.0);
+  std::vector<int> at(B), deq(grid);
+  std::vector<int> count((size_t)2 * grid, 0);
+  for (int k = 0; k < B; ++k) {
+    const int b = order[k], t = tcnt[b];
+    const double time = 2.0 + 1.06 * ((N[b] + 63) / 64);
+    int best = 0;
+    double start = 0.0;
+    if (t > grid) {
+      best = -1;
+      for (double f : free_at) start = std::max(start, f);
+    } else {
+      bool found = false;
+      for (int c = 0; c < 2; ++c) {
+        const double* f = &free_at[(size_t)c * grid];
+        // maxima of the windows of t CTAs
+        int head = 0, tail = 0;
+        for (int x = 0; x < grid; ++x) {
+          while (tail > head && f[deq[tail - 1]] <= f[x]) --tail;
+          deq[tail++] = x;
+          if (deq[head] <= x - t) ++head;
+          if (x >= t - 1 && (!found || f[deq[head]] < start)) {
+            found = true;
+            start = f[deq[head]];
+            best = c * grid + x - t + 1;
+          }
+        }
+      }
+    }
+    at[b] = best;
+    for (int i = 0; i < t; ++i) {
+      const int sl = best < 0 ? i : best + i;
+      free_at[sl] = start + time;
+      ++count[sl];
+    }
+  }
+  loff[0] = 0;
+  for (int i = 0; i < 2 * grid; ++i) loff[i + 1] = loff[i] + count[i];
+  std::vector<int> pos(loff, loff + 2 * grid);
+  for (int k = 0; k < B; ++k) {
+    const int b = order[k];
+    for (int i = 0; i < tcnt[b]; ++i) list[pos[at[b] < 0 ? i : at[b] + i]++] = toff[b] + i;
+  }
+}
+
+// Device block of one resident call.  One copy uploads it (the zero-start
+// counters with it), and its first part is what the host reads back.
+struct ResPack {
+  size_t ctl, dots, stamps, err, back_bytes;  // read back
+  size_t H, D, tiles, toff, tcnt, ns, tickets, bytes;   // uploaded before the prologue
+  size_t loff, list, all;                             // uploaded before the resident launch
+  ResPack(int B, int nt, int grid) {
+    size_t o = 0;
+    auto take = [&](size_t n) {
+      const size_t at = o;
+      o = (o + n + 15) / 16 * 16;
+      return at;
+    };
+    ctl = take((size_t)B * sizeof(Ctl));
+    dots = take((size_t)B * 3 * sizeof(double));
+    stamps = take((size_t)B * kResStamps * sizeof(unsigned));
+    err = take(sizeof(int));
+    back_bytes = o;
+    H = take((size_t)B * sizeof(void*));
+    D = take((size_t)B * sizeof(void*));
+    tiles = take((size_t)nt * sizeof(uint32_t));
+    toff = take((size_t)B * sizeof(int));
+    tcnt = take((size_t)B * sizeof(int));
+    ns = take((size_t)B * sizeof(int));
+    tickets = take((size_t)2 * B * sizeof(unsigned));
+    bytes = o;
+    loff = take((size_t)(2 * grid + 1) * sizeof(int));
+    list = take((size_t)nt * sizeof(int));
+    all = o;
+  }
+};
+
+// B instances (largest first in the tile list) through the bounds, input-layer
+// and resident kernels, then the read-back and the statistics.  single: the
+// single-matrix entry points (their bound kernel and row-norm order).
+sp2_status resident_solve(const float* const* H, const int* N, const int* N_occ, int B, int Nmax, double tol,
+                          int max_iter, float* const* D_out, sp2_stats* stats, const double* homo, const double* lumo,
+                          bool single) {
+  const bool accel = homo != nullptr;
+  const int nlaunch = accel ? max_iter : max_iter + 2;
+  const int prec = g.precision;
+  const bool split = prec == SP2_PREC_SPLIT_FP16;
+  cudaStream_t st = g.stream;
+
+  std::vector<int> order(B);
+  for (int i = 0; i < B; ++i) order[i] = i;
+  std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return N[x] > N[y]; });
+  std::vector<uint32_t> tiles;
+  std::vector<int> toff(B), tcnt(B);
+  for (int b : order) {
+    toff[b] = (int)tiles.size();
+    resident_tiles(N[b], b, &tiles, &tcnt[b]);
+  }
+  const int nt = (int)tiles.size();
+  const int iblocks = (Nmax + 7) / 8;
+  const int ggrid = single ? (int)std::min<long long>((Nmax + 7) / 8, 4LL * g.num_sms)
+                           : (int)std::min<long long>((Nmax + 7) / 8,
+                                                      std::max((Nmax + 63) / 64, 2 * g.num_sms / B + 1));
+  const int grid = std::min(nt, g.num_sms);
+  const ResPack P(B, nt, grid);
+  void *pack, *part, *sums, *rn, *tdots;
+  CKS(ws(B_PACK, P.all, &pack));
+  CKS(ws(B_PART, (size_t)B * std::max(iblocks, ggrid) * sizeof(double2), &part));
+  CKS(ws(B_TPART, (size_t)3 * nt * sizeof(longlong2), &sums));
+  CKS(ws(B_TDOTS, (size_t)nt * sizeof(double), &tdots));
+  const long long ld_h = round_up(Nmax, 64), slot_h = ld_h * Nmax;
+  void *hi[2], *lo[2], *hp[2];
+  CKS(planes_for(split, 0, (size_t)slot_h * B * 2, &hi[0], &lo[0], &hp[0]));
+  CKS(planes_for(split, 1, (size_t)slot_h * B * 2, &hi[1], &lo[1], &hp[1]));
+  CKS(ws(B_RN, (size_t)B * Nmax * sizeof(double), &rn));
+  SqArgs carry;
+  void* rnp[2];
+  CKS(rnp_for(Nmax, B, carry, rnp));
+
+  void* h;
+  CKS(staging(P.all, &h));
+  uint8_t* hb = (uint8_t*)h;
+  memset(hb + P.dots, 0, P.back_bytes - P.dots);
+  memset(hb + P.tickets, 0, P.bytes - P.tickets);
+  Ctl* hc = (Ctl*)(hb + P.ctl);
+  for (int b = 0; b < B; ++b) {
+    init_ctl(hc + b, N[b], N_occ[b], tol, max_iter);
+    if (accel) {
+      hc[b].accel = 1;
+      hc[b].acc_homo = homo[b];
+      hc[b].acc_lumo = lumo[b];
+      hc[b].tol = tol > 0.0 ? tol : 1e-9;
+    }
+  }
+  memcpy(hb + P.H, H, B * sizeof(void*));
+  memcpy(hb + P.D, D_out, B * sizeof(void*));
+  memcpy(hb + P.tiles, tiles.data(), nt * sizeof(uint32_t));
+  memcpy(hb + P.toff, toff.data(), B * sizeof(int));
+  memcpy(hb + P.tcnt, tcnt.data(), B * sizeof(int));
+  memcpy(hb + P.ns, N, B * sizeof(int));
+  CK(cudaMemcpyAsync(pack, hb, P.bytes, cudaMemcpyHostToDevice, st));
+
+  uint8_t* dp = (uint8_t*)pack;
+  ResArgs A;
+  memset(&A, 0, sizeof(A));
+  A.H = (const float* const*)(dp + P.H);
+  A.D = (float* const*)(dp + P.D);
+  A.Ns = (const int*)(dp + P.ns);
+  A.tiles = (const uint32_t*)(dp + P.tiles);
+  A.ntiles = nt;
+  A.tile_off = (const int*)(dp + P.toff);
+  A.tile_cnt = (const int*)(dp + P.tcnt);
+  A.ctl = (Ctl*)(dp + P.ctl);
+  for (int k = 0; k < 2; ++k) {
+    A.p0[k] = (__half*)(split ? hp[k] : hi[k]);
+    A.p1[k] = (__half*)lo[k];
+    A.rnp[k] = (float*)rnp[k];
+  }
+  A.ld_h = ld_h;
+  A.slot_h = slot_h;
+  A.rn = (const double*)rn;
+  A.ld_rn = Nmax;
+  A.ld_rnp = carry.ld_rnp;
+  A.slot_rnp = carry.slot_rnp;
+  A.part = (double2*)part;
+  A.tile_dots = (double*)tdots;
+  A.dots_out = (double*)(dp + P.dots);
+  A.sums = (longlong2*)sums;
+  A.tickets = (unsigned*)(dp + P.tickets) + B;
+  unsigned* gtick = (unsigned*)(dp + P.tickets);
+  A.list_off = (const int*)(dp + P.loff);
+  A.list = (const int*)(dp + P.list);
+  A.stamps = (unsigned*)(dp + P.stamps);
+  A.lo_scale = std::ldexp(1.0f, g.lo_scale_exp);
+  A.lo_unscale = std::ldexp(1.0f, -g.lo_scale_exp);
+  A.shift = g.shift;
+  A.err = (int*)(dp + P.err);
+  A.wait_ns = g.wait_ns;
+  A.two_slots = nt > grid ? 1 : 0;
+  A.stall = (single && g.fault_stall) ? 1 : 0;
+  if (single) g.fault_stall = false;
+  ResMaps maps;
+  for (int k = 0; k < 2; ++k) {
+    CUtensorMap m[6];
+    CKS(tmaps4_for(A.p0[k], A.p1[k], Nmax, B, ld_h, slot_h, m, kTcBM));
+    maps.m[k][0] = m[0];
+    maps.m[k][1] = m[1];
+    maps.m[k][2] = m[4];
+    maps.m[k][3] = m[5];
+  }
+
+  CK(cudaEventRecord(g.ev0, st));
+  if (single) {
+    CK(launch_gershgorin(H[0], Nmax, Nmax, (long long)Nmax * Nmax, 1, (double2*)part, gtick, A.ctl, nullptr,
+                         ggrid, st, g.fault_nan ? 0 : -1));
+    g.fault_nan = false;
+  } else {
+    CK(launch_gershgorin_batched(A.H, A.Ns, A.ctl, B, (double2*)part, gtick, ggrid, st));
+  }
+  // the row norms of Y_0 in the order of the kernel that the other paths use
+  // (float4 rows: always in the batched layout, by N and D in the single one)
+  const int vec_norm = !single || ((Nmax & 3) == 0 && ((uintptr_t)D_out[0] & 15) == 0);
+  CK(launch_resident_input(A, vec_norm, Nmax, B, st));
+  // planned while the prologue runs
+  resident_plan(order.data(), N, toff.data(), tcnt.data(), B, grid, (int*)(hb + P.loff), (int*)(hb + P.list));
+  CK(cudaMemcpyAsync(dp + P.loff, hb + P.loff, P.all - P.loff, cudaMemcpyHostToDevice, st));
+  CK(cudaEventRecord(g.stage_done, st));
+  CK(cudaEventRecord(g.lev[0], st));
+  CK(launch_resident(A, maps, split, grid, st));
+  CK(cudaEventRecord(g.ev1, st));
+
+  if (!stats) return SP2_OK;
+  void* back;
+  CKS(staging(P.back_bytes, &back));
+  CK(cudaMemcpyAsync(back, pack, P.back_bytes, cudaMemcpyDeviceToHost, st));
+  CK(cudaStreamSynchronize(st));
+  const uint8_t* rb = (const uint8_t*)back;
+  float ms = 0.f, pro = 0.f;
+  CK(cudaEventElapsedTime(&ms, g.ev0, g.ev1));
+  CK(cudaEventElapsedTime(&pro, g.ev0, g.lev[0]));
+  const Ctl* cs = (const Ctl*)(rb + P.ctl);
+  const int e = *(const int*)(rb + P.err);
+  sp2_status worst = SP2_OK;
+  for (int b = 0; b < B; ++b) {
+    sp2_stats& s = stats[b];
+    fill_stats(cs[b], &s, ms, prec);
+    s.launches = nlaunch;
+    s.energy = ((const double*)(rb + P.dots))[3 * b];
+    s.prologue_ms = pro;
+    // layer times of this instance (0 past its last layer)
+    const unsigned* t = (const unsigned*)(rb + P.stamps) + (size_t)b * kResStamps;
+    for (int k = 0; k < nlaunch && t[k + 1] != 0; ++k) s.layer_ms[k] = s.square_ms[k] = (float)(t[k + 1] - t[k]) * 1e-6f;
+    sp2_status sb = status_of(cs[b], e);
+    if (accel && sb >= 0 && std::fabs(cs[b].trace_final - (double)N_occ[b]) > 0.5) {
+      if (single)
+        set_err("accelerated solve: Tr D = %.3f but N_occ = %d; the HOMO/LUMO estimates do not bracket the gap",
+                cs[b].trace_final, N_occ[b]);
+      else
+        set_err("instance %d: Tr D = %.3f but N_occ = %d; the HOMO/LUMO estimates do not bracket the gap", b,
+                cs[b].trace_final, N_occ[b]);
+      sb = SP2_ERR_BAD_ESTIMATE;
+    }
+    if (sb < 0 && worst >= 0) worst = sb;
+    if (sb == SP2_NOT_CONVERGED && worst == SP2_OK) worst = SP2_NOT_CONVERGED;
+  }
+  if (worst == SP2_OK && !single) t_err.clear();
+  return worst;
+}
+
 // The single-matrix solve; accel selects the accelerated layers (bounds from
 // the HOMO/LUMO estimates) instead of the trace rule with refinement.
 sp2_status density_matrix_impl(const float* H, int N, int N_occ, double tol, int max_iter, float* D_out,
                                sp2_stats* stats, bool accel, double homo, double lumo) {
+  if (resident_fits(N))
+    return resident_solve(&H, &N, &N_occ, 1, N, tol, max_iter, &D_out, stats, accel ? &homo : nullptr,
+                          accel ? &lumo : nullptr, true);
   const int prec = g.precision;
   const bool tc = tc_precision(prec);
   const bool split = prec == SP2_PREC_SPLIT_FP16;
@@ -1251,6 +1542,9 @@ sp2_status batched_impl(const float* const* H, const int* N, const int* N_occ, i
   const bool tc = tc_precision(prec);
   cudaStream_t st = g.stream;
   const int B = batch;
+
+  if (g.batched_sched == 0 && resident_fits(Nmax))
+    return resident_solve(H, N, N_occ, B, Nmax, tol, max_iter, D_out, stats, homo, lumo, false);
 
   // schedule: fixed (SP2_BATCHED_KERNEL=single|pairs) or tuned once per batch
   // signature by timing each candidate on the call itself (every candidate

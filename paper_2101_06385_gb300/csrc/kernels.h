@@ -143,6 +143,50 @@ size_t syrk_tc1_smem_bytes(bool split);
 cudaError_t launch_syrk_tc2(const SqArgs& a, const CUtensorMap* tmaps, bool split, int grid, cudaStream_t st);
 size_t syrk_tc2_smem_bytes(bool split);
 
+// Resident solve (csrc/resident.cu): all layers of a batch of instances in one
+// cooperative launch on 128 x 128 tiles; the tiles of one instance are
+// contiguous, starting at tile_off[b], tile_cnt[b] <= slots (two per CTA).  The
+// instances' order is the same in every slot's list.
+constexpr int kResTile = 128;
+constexpr int kResStamps = kMaxL + 2;
+constexpr long long kGangEmpty = -0x7f7f7f7f7f7f7f80ll;  // no sum of a layer
+struct ResMaps {
+  CUtensorMap m[2][4];  // per plane parity: {p0, p1} with 64 x 128 boxes, {p0, p1} with 64 x 64 boxes
+};
+struct ResArgs {
+  const float* const* H;   // [batch] inputs [n_b, n_b]
+  float* const* D;         // [batch] outputs
+  const int* Ns;           // [batch]
+  const uint32_t* tiles;   // [ntiles], rows and columns in units of 128
+  int ntiles;
+  const int* tile_off;     // [batch]
+  const int* tile_cnt;     // [batch]
+  Ctl* ctl;                // [batch]
+  __half* p0[2];           // operand planes of even / odd layers: hp (split) or hi
+  __half* p1[2];           //   lo' (split) or nullptr
+  long long ld_h, slot_h;
+  const double* rn;        // [batch][ld_rn] FP64 row norms of Y_0
+  long long ld_rn;
+  float* rnp[2];           // row-norm segment sums, as SqArgs::rnp_out
+  long long ld_rnp, slot_rnp;
+  double2* part;           // [batch][blocks] block sums of the input layer
+  longlong2* sums;         // [3][ntiles] the tiles' (tr Y', ||Y'||_F^2) of layer k at [k mod 3] in fixed point,
+                           //   kGangEmpty until published
+  double* tile_dots;       // [ntiles] Tr[D H] per tile
+  double* dots_out;        // [batch][3], entry 0: Tr[D H]
+  unsigned* tickets;       // [batch] zero: finished blocks of the input layer
+  const int* list_off;     // [2 grid + 1] slot c of CTA s processes the tiles
+  const int* list;         //   list[list_off[c grid + s]] .. in turn
+  unsigned* stamps;        // [batch][kResStamps] ns from an instance's start to the end of its k-th layer
+  float lo_scale, lo_unscale;
+  int shift, two_slots;
+  int stall;               // as SqArgs
+  int* err;
+  unsigned long long wait_ns;
+};
+cudaError_t launch_resident_input(const ResArgs& a, int vec_norm, int Nmax, int batch, cudaStream_t st);
+cudaError_t launch_resident(const ResArgs& a, const ResMaps& maps, bool split, int grid, cudaStream_t st);
+
 cudaError_t launch_syrk_simt(const SqArgs& a, int grid, cudaStream_t st);
 
 // Tensor-core squaring.  tmaps: {hi(A box), lo(A box), hi(B box), lo(B box)}

@@ -1,0 +1,1088 @@
+// Resident SP2 solve (sm_103a): every layer of many instances in one launch.
+//
+// A CTA owns one or two 128 x 128 tiles of the upper super tiles and keeps
+// each for all layers of its solve: the FP32 iterate of the tile stays in
+// tensor memory next to its accumulator, and only the FP16 operand planes go
+// through L2.  The CTAs of one instance (its gang) meet after every layer at
+// their sums in global memory and each runs the control step of Alg. 1 on the
+// same sums, so a solve costs no launch per layer and stops at its last one.
+//
+// What bounds it: for small N the chain of one layer (operand loads, K / 64
+// stages of twelve dependent MMAs at 0.47 us each, epilogue, gang meeting);
+// for many instances the tensor cores at the 128 x 128 tile's rate (1.8
+// PFLOP/s of products with every SM loading, against 2.1 of the CTA pairs'
+// 256 x 256 tiles, which leave most of the chip idle at these sizes).
+//
+// Two slots per CTA hold tiles of the same or of different instances, each
+// slot a list that the host planned.  While one slot waits for its gang or
+// runs its epilogue the other's MMAs run; the producer takes whichever slot is
+// ready.  Every list is in one order of the instances, so the earliest
+// unfinished gang has all its tiles at the front of their lists: with at most
+// one tile of an instance per slot and all CTAs resident (cooperative launch)
+// no wait is circular.  Every wait is bounded all the same.
+//
+// Tile accumulation order, epilogue arithmetic and the super-tile storage of
+// the planes (256 x 256 upper super tiles, K blocks left of the diagonal read
+// transposed) are those of the other tensor-core kernels, so D has the same
+// bits.
+//
+// CTA = 20 warps: 0 TMA producer, 1 MMA issuer (and TMEM), 2-17 epilogue
+// (one 32 x 32 chunk each), 18 and 19 control of the two slots.
+#include <cuda.h>
+#include <cuda_fp16.h>
+
+#include "common.cuh"
+#include "epilogue.cuh"
+#include "kernels.h"
+#include "tc_ptx.cuh"
+
+namespace sp2 {
+namespace res {
+
+using namespace sp2::tc;
+
+constexpr int TB = kResTile;                 // 128
+constexpr int HALF_BYTES = TB * BK * 2;      // 16 KB: one plane of one operand
+constexpr int T_BOX = 64 * 64 * 2;           // one 64 x 64 box of a transposed read
+constexpr int STAGE_SPLIT = 4 * HALF_BYTES;  // hpA loA hpB loB
+constexpr int STAGE_PLAIN = 2 * HALF_BYTES;  // hiA hiB
+constexpr int STAGES_SPLIT = 3;
+constexpr int STAGES_PLAIN = 6;
+constexpr int OPERAND_BYTES = STAGES_SPLIT * STAGE_SPLIT;
+static_assert(OPERAND_BYTES == STAGES_PLAIN * STAGE_PLAIN, "both precisions use the same shared memory");
+constexpr int EPI_WARPS = 16;               // one 32 x 32 chunk each
+constexpr int TR_BYTES = EPI_WARPS * 16 * 32 * 4;  // half a chunk per warp
+constexpr int CTL_WARP = 2 + EPI_WARPS;
+constexpr int THREADS = 32 * (CTL_WARP + 2);
+constexpr uint32_t TMEM_COLS = 512;  // two slots of an accumulator and an iterate
+constexpr uint32_t SLOT_COLS = 256, Y_COL = 128;
+constexpr uint32_t IDESC_T = (1u << 4) | ((uint32_t)(TB >> 3) << 17) | ((uint32_t)(TB >> 4) << 24);
+constexpr int WQ = 4;       // work queue entries (at most two outstanding)
+constexpr int WQ_END = 255;
+
+// The coefficients of the next launch for either branch (index bit 0: sigma <
+// 0) and either storage (bit 1: re-centred), and the accelerated layer's new
+// bounds, prepared while the layer's products run: FP64 costs 64 cycles a step
+// here and would otherwise stand in the chain of every layer.
+struct Prepared {
+  LayerCoef k[4];
+  float ca[4], cb[4];
+  double l, h;
+  int sign;
+  // the loop's decision on (tr Y, ||Y||_F^2): N alpha, N alpha^2, N alpha (1 -
+  // alpha), 2 alpha, 1 - 2 alpha, N_occ, sigma eps, the re-centring and 4.5-rule thresholds
+  int rule45;
+  double na, naa, na1, ta, oa, no, se, rc, r45;
+};
+
+struct PreparedCoef {
+  const Prepared* p;
+  __device__ __forceinline__ void put(Ctl* c, int i, bool final_layer) const {
+    set_next(c, p->k[i], p->ca[i], p->cb[i], final_layer);
+  }
+  __device__ __forceinline__ void branch(Ctl* c, int sigma, bool final_layer) const {
+    put(c, (sigma < 0 ? 1 : 0) + (c->recentered ? 2 : 0), final_layer);
+  }
+  __device__ __forceinline__ int accel(Ctl*, double& l, double& h, LayerCoef&) const {
+    l = p->l;
+    h = p->h;
+    return p->sign;
+  }
+  __device__ __forceinline__ void next(Ctl* c, const LayerCoef&, bool final_layer) const {
+    put(c, c->recentered ? 2 : 0, final_layer);
+  }
+};
+
+struct Slot {
+  int b, I, J, N;        // instance, tile row and column (128 units), size
+  int par, first;        // parity of the operand planes; first layer
+  int closed;            // no more work in this slot
+  int pad;
+  int sg[4];
+  double ie[4];
+  double hot[kCtlHotBytes / 8];  // the control block without its history
+  Prepared prep;
+};
+static_assert(kCtlHotBytes % 8 == 0, "the hot part is copied in 8-byte words");
+
+struct Shared {
+  uint64_t full[STAGES_PLAIN], empty[STAGES_PLAIN];
+  uint64_t ready[2];     // control warp -> producer: operands complete, products may start (or slot closed)
+  uint64_t coef[2];      // control warp -> epilogue: the layer's coefficients are set
+  uint64_t acc_full[2];  // MMA issuer -> epilogue
+  uint64_t epi_done[2];  // epilogue warps -> control warp
+  uint64_t wq_full[WQ];  // producer -> MMA issuer and epilogue: next slot
+  uint64_t drain, never;
+  int wq[WQ];
+  uint32_t tmem;
+  int abort;
+  long long red_t[2][EPI_WARPS], red_q[2][EPI_WARPS];  // a layer's sums per warp (fixed point)
+  double red_e[2][EPI_WARPS];                          // Tr[D H] (last layer)
+  Slot slot[2];
+};
+
+__device__ __forceinline__ Ctl* hot_ctl(Slot& s) { return reinterpret_cast<Ctl*>(s.hot); }
+
+// Loads one 128-row operand of K block k0: K-major, or the stored block left
+// of the diagonal transposed (two 64 x 64 boxes).
+__device__ __forceinline__ void load_half(uint8_t* dst, const CUtensorMap* tmK, const CUtensorMap* tmT, bool trans,
+                                          int row, int k0, int b, uint64_t* bar) {
+  if (!trans) {
+    tma_load_3d(dst, tmK, k0, row, b, bar);
+  } else {
+    tma_load_3d(dst, tmT, row, k0, b, bar);
+    tma_load_3d(dst + T_BOX, tmT, row + 64, k0, b, bar);
+  }
+}
+
+// A layer's sums tr Y' and ||Y'||_F^2 in 64-bit fixed point, exact in any
+// order: FP64 adds (64 cycles each, 19 of them a warp on the SM's one pipe)
+// would cost a layer's epilogue a microsecond, integer ones half of one
+// shuffle.  Y' has spectral norm <= 1, so a lane's FP32 sum of 32 squares is
+// at most 4 and a tile's at most 128: units of 2^-53 and 2^-50 (trace) lose
+// less than the FP64 sums did.  Anything outside (an H that is not symmetric)
+// or not a number is marked and becomes infinity or NaN in the control step.
+constexpr long long SQ_LIMIT = (1ll << 58) + (1ll << 50);  // a 32 x 32 block's 32, with rounding
+constexpr long long SQ_NAN = -1, SQ_BIG = -2;              // marks of a sum that is no number, or out of range
+constexpr double T_UNIT = 0x1p-50, Q_HI_UNIT = 0x1p-25, Q_LO_UNIT = 0x1p-53;
+
+__device__ __forceinline__ long long fix_sq(float v) {
+  // v = hi 2^-25 + lo 2^-53, both steps exact or rounded once
+  const int hi = __float2int_rz(v * 0x1p25f);
+  const int lo = __float2int_rn(fmaf(-(float)hi, 0x1p-25f, v) * 0x1p53f);
+  return ((long long)hi << 28) + (long long)lo;
+}
+
+__device__ __forceinline__ long long warp_sum_ll(long long v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// Row norm (Y^2)_rr of the layer's input: FP64 ones of the input layer, or the
+// sum of the previous layer's segment sums (at most 1 together; 2^-53 of fixed
+// point is what an FP64 sum near 1 resolves).  The segments were written by
+// other SMs during this launch: read through L2.
+__device__ __forceinline__ double row_norm(const ResArgs& a, const Slot& s, int r) {
+  if (s.first) return a.rn[(long long)s.b * a.ld_rn + r];
+  const float* p = a.rnp[s.par ^ 1] + (long long)s.b * a.slot_rnp + r;
+  const int nseg = (s.N + 31) >> 5;
+  long long acc = 0;
+  int g = 0;
+  for (; g + 16 <= nseg; g += 16) {
+    float v[16];
+#pragma unroll
+    for (int u = 0; u < 16; ++u) v[u] = __ldcg(p + (long long)(g + u) * a.ld_rnp);
+#pragma unroll
+    for (int u = 0; u < 16; ++u) acc += fix_sq(v[u]);
+  }
+  float v[16];
+#pragma unroll
+  for (int u = 0; u < 16; ++u) v[u] = g + u < nseg ? __ldcg(p + (long long)(g + u) * a.ld_rnp) : 0.f;
+#pragma unroll
+  for (int u = 0; u < 16; ++u) acc += fix_sq(v[u]);
+  return (double)acc * Q_LO_UNIT;
+}
+
+// Turns the warp's 32 x 32 chunk from one row per lane (v) to four consecutive
+// columns of eight rows (p: register 4 i + e = row 4 i + lane / 8, column
+// 4 (lane mod 8) + e), sixteen rows at a time through the warp's 2 KB.
+template <class Sink>
+__device__ __forceinline__ void turn(float* trb, const uint32_t (&v)[32], int lane, Sink sink) {
+  const int r4 = lane >> 3, c4 = lane & 7;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    if ((lane >> 4) == h) {
+#pragma unroll
+      for (int m = 0; m < 8; ++m)
+        *epi::tr_at(trb, lane & 15, m) = make_float4(__uint_as_float(v[4 * m]), __uint_as_float(v[4 * m + 1]),
+                                                     __uint_as_float(v[4 * m + 2]), __uint_as_float(v[4 * m + 3]));
+    }
+    __syncwarp();
+#pragma unroll
+    for (int i = 4 * h; i < 4 * h + 4; ++i) sink(i, *epi::tr_at(trb, 4 * (i - 4 * h) + r4, c4));
+    __syncwarp();
+  }
+}
+
+// One layer of the warp's 32 x 32 chunk of a slot's tile (the lane layouts and
+// arithmetic of epi::tile).  False: the accumulator wait failed.
+template <bool SPLIT>
+__device__ __forceinline__ bool epilogue(const ResArgs& a, Shared& sh, int c, uint32_t acc_phase, uint32_t tmem_base,
+                                         int ew, int q, int lane, float* trb, unsigned long long lim) {
+  const Slot& s = sh.slot[c];
+  const Ctl* ct = reinterpret_cast<const Ctl*>(s.hot);
+  const int b = s.b, N = s.N, first = s.first;
+  const int hc = ew >> 2;
+  const int R0 = s.I * TB + q * 32;
+  const int nrows = min(32, N - R0);
+  const int c0 = s.J * TB + hc * 32;
+  const bool mirror = (s.I >> 1) != (s.J >> 1);
+  const float unscale = SPLIT ? a.lo_unscale * a.lo_unscale : 1.f;
+  const float lo_scale = a.lo_scale;
+  const int r4 = lane >> 3, c4 = lane & 7;
+  const int ce = c0 + 4 * c4;
+  const int rdiag = R0 + 4 * c4 + r4;
+  // the one diagonal element a lane holds (chunk c0 == R0 of a diagonal tile,
+  // a warp-uniform condition): row = column = rdiag, register 4 c4 + r4
+  const bool dchunk = !mirror && c0 == R0;
+  const bool dlane = dchunk && rdiag < N;
+  const int id = 4 * c4 + r4;
+  const bool live = nrows > 0 && c0 < ((N + 63) & ~63);
+  const uint32_t tacc = tmem_base + c * SLOT_COLS + ((uint32_t)(q * 32) << 16) + hc * 32;
+  const uint32_t ty = tacc + Y_COL;
+  const float* H = a.H[b];
+
+  // old values and the diagonal's row norm before the accumulator wait
+  float y[32];
+  double rn_l = 0.0;
+  if (live) {
+    if (dlane) rn_l = row_norm(a, s, rdiag);
+    if (first) {
+      const InputScale in = input_scale(ct->e_min, ct->e_max, a.shift);
+      const bool vec_h = (N & 3) == 0 && (reinterpret_cast<uintptr_t>(H) & 15) == 0;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const bool rok = 4 * i + r4 < nrows;
+        const float4 o = rok ? epi::ld4(H + (long long)(R0 + 4 * i + r4) * N + ce, ce, N, vec_h)
+                             : make_float4(0.f, 0.f, 0.f, 0.f);
+        y[4 * i] = o.x;
+        y[4 * i + 1] = o.y;
+        y[4 * i + 2] = o.z;
+        y[4 * i + 3] = o.w;
+      }
+      float hd = 0.f;
+      if (dchunk) {
+#pragma unroll
+        for (int k = 0; k < 32; ++k)
+          if (k == id) hd = y[k];
+      }
+#pragma unroll
+      for (int k = 0; k < 32; ++k) y[k] = input_offdiag(y[k], in);
+      if (dchunk) {
+        const float yd0 = input_diag(hd, in);
+#pragma unroll
+        for (int k = 0; k < 32; ++k)
+          if (k == id) y[k] = yd0;
+      }
+    } else {
+      uint32_t w[32];
+      __syncwarp();
+      tmem_ld32(ty, w);
+      tmem_ld_wait();
+#pragma unroll
+      for (int k = 0; k < 32; ++k) y[k] = __uint_as_float(w[k]);
+    }
+  }
+  // the previous layer's control step runs under this layer's products
+  if (!__all_sync(0xffffffffu, mbar_wait(&sh.coef[c], acc_phase, &sh.abort, lim))) return false;
+  const LayerParams p = ct->next;
+  const bool outD = (p.out_mode == OUT_D);
+  // the diagonal needs no product: its square comes from the row norms
+  long long tr = 0, sq = 0;
+  float ydf = 0.f, ydo = 0.f;
+  if (dchunk) {
+    float yold_d = 0.f;
+#pragma unroll
+    for (int k = 0; k < 32; ++k)
+      if (k == id) yold_d = y[k];
+    if (dlane) {
+      const double yd = p.ca_d * (double)yold_d + p.cb_d * rn_l + p.cc_d;
+      tr = __double2ll_rn(yd * 0x1p50);
+      ydf = (float)yd;
+      ydo = outD ? (float)(yd + p.alpha_out) : ydf;
+    }
+    tr = warp_sum_ll(tr);
+  }
+  if (!__all_sync(0xffffffffu, mbar_wait(&sh.acc_full[c], acc_phase, &sh.abort, lim))) return false;
+  tc_fence_after();
+
+  double dtr = 0.0;
+  if (live) {
+    const bool full = nrows == 32 && c0 + 32 <= N;
+    {
+      uint32_t v[32];
+      __syncwarp();
+      tmem_ld32(tacc, v);
+      tmem_ld_wait();
+      const float cbu = p.cb * unscale;
+      turn(trb, v, lane, [&](int i, const float4& pv) {
+        y[4 * i] = fmaf(p.ca, y[4 * i], cbu * pv.x);
+        y[4 * i + 1] = fmaf(p.ca, y[4 * i + 1], cbu * pv.y);
+        y[4 * i + 2] = fmaf(p.ca, y[4 * i + 2], cbu * pv.z);
+        y[4 * i + 3] = fmaf(p.ca, y[4 * i + 3], cbu * pv.w);
+      });
+    }
+    if (!full) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+          if (!(4 * i + r4 < nrows && ce + e < N)) y[4 * i + e] = 0.f;
+    }
+    if (dchunk) {
+#pragma unroll
+      for (int k = 0; k < 32; ++k)
+        if (dlane && k == id) y[k] = ydf;
+    }
+    // sums of squares: per row over the 32 columns, per column over the 32
+    // rows (the mirror's rows), and the lane's share of ||Y'||_F^2
+    float rs[8], cs[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      rs[i] = 0.f;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        rs[i] = fmaf(y[4 * i + e], y[4 * i + e], rs[i]);
+        cs[e] = fmaf(y[4 * i + e], y[4 * i + e], cs[e]);
+      }
+    }
+    const float sql = ((rs[0] + rs[1]) + (rs[2] + rs[3])) + ((rs[4] + rs[5]) + (rs[6] + rs[7]));
+    const bool nan = __any_sync(0xffffffffu, isnan(sql)), big = __any_sync(0xffffffffu, !(sql < 16.f));
+    if (!outD) {
+      // operand planes of Y' (Eq. 12) first: they are what the gang waits for
+      __half* p0 = a.p0[s.par ^ 1] + (long long)b * a.slot_h + (long long)(R0 + r4) * a.ld_h + ce;
+      __half* p1 = SPLIT ? a.p1[s.par ^ 1] + (long long)b * a.slot_h + (long long)(R0 + r4) * a.ld_h + ce : nullptr;
+      const __half2 s2 = __float2half2_rn(lo_scale);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        uint32_t pa[2], pl[2];
+#pragma unroll
+        for (int e2 = 0; e2 < 2; ++e2) {
+          // hp = 2^s fp16(x) and lo' = fp16(2^s x - hp): both differences are exact
+          const float x0 = y[4 * i + 2 * e2], x1 = y[4 * i + 2 * e2 + 1];
+          __half2 p2 = __floats2half2_rn(x0, x1);
+          if (SPLIT) {
+            p2 = __hmul2(p2, s2);
+            const float2 pf = __half22float2(p2);
+            const __half2 l2 = __floats2half2_rn(fmaf(x0, lo_scale, -pf.x), fmaf(x1, lo_scale, -pf.y));
+            pl[e2] = *reinterpret_cast<const uint32_t*>(&l2);
+          }
+          pa[e2] = *reinterpret_cast<const uint32_t*>(&p2);
+        }
+        if (4 * i + r4 < nrows) {
+          *reinterpret_cast<uint2*>(p0) = make_uint2(pa[0], pa[1]);
+          if (SPLIT) *reinterpret_cast<uint2*>(p1) = make_uint2(pl[0], pl[1]);
+        }
+        p0 += 4 * a.ld_h;
+        if (SPLIT) p1 += 4 * a.ld_h;
+      }
+      // row norms of the next layer
+      float* rnp = a.rnp[s.par] + (long long)b * a.slot_rnp;
+      const float rsum = epi::lane_sums<8, 0>(rs);
+      if (rdiag < N && c0 < N) rnp[(long long)(c0 >> 5) * a.ld_rnp + rdiag] = rsum;
+      if (mirror) {
+        const float csum = epi::lane_sums<4, 3>(cs);
+        const int cm = c0 + 4 * c4 + r4;
+        if (cm < N) rnp[(long long)(R0 >> 5) * a.ld_rnp + cm] = csum;
+      }
+      uint32_t w[32];
+#pragma unroll
+      for (int k = 0; k < 32; ++k) w[k] = __float_as_uint(y[k]);
+      __syncwarp();
+      tmem_st32(ty, w);
+    }
+    sq = warp_sum_ll(fix_sq(sql));
+    if (nan || big || sq > SQ_LIMIT) sq = nan ? SQ_NAN : SQ_BIG;
+    if (!outD) fence_proxy_async();  // the planes are read by the TMA units next
+    if (outD) {
+      if (dchunk) {
+#pragma unroll
+        for (int k = 0; k < 32; ++k)
+          if (dlane && k == id) y[k] = ydo;
+      }
+      float* D = a.D[b];
+      const bool vec_n =
+          (N & 3) == 0 && ((reinterpret_cast<uintptr_t>(D) | reinterpret_cast<uintptr_t>(H)) & 15) == 0;
+      float eo = 0.f;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        if (4 * i + r4 < nrows) {
+          const long long o = (long long)(R0 + 4 * i + r4) * N + ce;
+          const float4 hv = epi::ld4(H + o, ce, N, vec_n);
+          epi::st4(D + o, make_float4(y[4 * i], y[4 * i + 1], y[4 * i + 2], y[4 * i + 3]), ce, N, vec_n);
+          eo = fmaf(y[4 * i], hv.x, eo);
+          eo = fmaf(y[4 * i + 1], hv.y, eo);
+          eo = fmaf(y[4 * i + 2], hv.z, eo);
+          eo = fmaf(y[4 * i + 3], hv.w, eo);
+        }
+      }
+      dtr = warp_sum_d((double)eo);
+      if (mirror) {
+        dtr *= 2.0;
+        // back to lane = row, sixteen rows at a time: the mirror column is
+        // contiguous across lanes
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+#pragma unroll
+          for (int i = 4 * h; i < 4 * h + 4; ++i)
+            *epi::tr_at(trb, 4 * (i - 4 * h) + r4, c4) = make_float4(y[4 * i], y[4 * i + 1], y[4 * i + 2], y[4 * i + 3]);
+          __syncwarp();
+          if ((lane >> 4) == h && lane < nrows) {
+#pragma unroll
+            for (int m = 0; m < 8; ++m) {
+              const float4 o = *epi::tr_at(trb, lane & 15, m);
+              const float ov[4] = {o.x, o.y, o.z, o.w};
+#pragma unroll
+              for (int e = 0; e < 4; ++e)
+                if (c0 + 4 * m + e < N) D[(long long)(c0 + 4 * m + e) * N + R0 + lane] = ov[e];
+            }
+          }
+          __syncwarp();
+        }
+      }
+    }
+  }
+  tmem_st_wait();
+  tc_fence_before();
+  __syncwarp();
+  if (lane == 0) {
+    sh.red_t[c][ew] = tr;
+    sh.red_q[c][ew] = sq;
+    if (outD) sh.red_e[c][ew] = dtr;
+    mbar_arrive(&sh.epi_done[c]);
+  }
+  return true;
+}
+
+// Sum over the sixteen epilogue warps (lanes 0-15 hold their values).
+__device__ __forceinline__ long long sum16(long long v) {
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// The warp's worst mark (0: every lane's sum is a number).
+__device__ __forceinline__ long long worst_mark(long long v) {
+  const bool nan = __any_sync(0xffffffffu, v == SQ_NAN), big = __any_sync(0xffffffffu, v == SQ_BIG);
+  return nan ? SQ_NAN : big ? SQ_BIG : 0;
+}
+
+// A tile's sums of one layer as its gang sees them: the slot holds GANG_EMPTY
+// until the tile has published them, both words at once.
+__device__ __forceinline__ longlong2 ld_sums(const longlong2* p) {
+  longlong2 v;
+  asm volatile("ld.relaxed.gpu.global.v2.s64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_sums(longlong2* p, long long x, long long y) {
+  asm volatile("st.relaxed.gpu.global.v2.s64 [%0], {%1, %2};" ::"l"(p), "l"(x), "l"(y) : "memory");
+}
+
+// Waits for the sums of all cnt tiles of the gang (slots p[0 .. cnt)) and adds
+// them: T, and Q as 2^28 q_hi + q_lo; the next layer's products are released
+// (ready) before the sums are added.  False: abort or time-out.
+__device__ __forceinline__ bool meet(const ResArgs& a, Shared& sh, const longlong2* p, int cnt, int lane,
+                                     uint64_t* ready, long long& T, long long& q_hi, long long& q_lo, long long& bad,
+                                     unsigned long long idle) {
+  T = q_hi = q_lo = 0;
+  bad = 0;
+  const uint64_t w0 = globaltimer();
+  for (int i0 = 0; i0 < cnt; i0 += 128) {
+    longlong2 v[4];
+    bool have[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int i = i0 + 32 * u + lane;
+      have[u] = i >= cnt;
+      if (!have[u]) v[u] = ld_sums(p + i);
+    }
+    for (int spin = 0;; ++spin) {
+      bool all = true;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        if (have[u]) continue;
+        if (v[u].x != kGangEmpty && v[u].y != kGangEmpty) {
+          have[u] = true;
+          T += v[u].x;
+          q_hi += v[u].y >> 28;
+          q_lo += v[u].y & ((1ll << 28) - 1);
+          if (v[u].y < 0) bad = bad == SQ_NAN ? bad : v[u].y;
+        } else {
+          all = false;
+          v[u] = ld_sums(p + i0 + 32 * u + lane);
+        }
+      }
+      if (__all_sync(0xffffffffu, all)) break;
+      if ((spin & 31) == 31) {
+        const bool stop = *(volatile int*)&sh.abort || *(volatile int*)a.err != 0 || globaltimer() - w0 > idle;
+        if (__any_sync(0xffffffffu, stop)) return false;
+      }
+    }
+  }
+  __threadfence();  // the gang's planes and row norms, with its sums
+  __syncwarp();
+  if (lane == 0 && ready) mbar_arrive(ready);
+  T = warp_sum_ll(T);
+  q_hi = warp_sum_ll(q_hi);
+  q_lo = warp_sum_ll(q_lo);
+  bad = worst_mark(bad);
+  return true;
+}
+
+// What the next control step can be given beforehand: the candidates (lanes
+// 0-3) and the constants of the loop's decision (lane 4).
+__device__ __forceinline__ void prepare(Slot& s, int lane) {
+  if (lane == 4) {
+    const Ctl* c = hot_ctl(s);
+    const double a = c->alpha_next, N = (double)c->N;
+    const RingHistory hist{s.sg, s.ie, nullptr};
+    const int n1 = c->n + 1;
+    s.prep.na = N * a;
+    s.prep.naa = N * a * a;
+    s.prep.na1 = N * a * (1.0 - a);
+    s.prep.ta = 2.0 * a;
+    s.prep.oa = 1.0 - 2.0 * a;
+    s.prep.no = (double)c->n_occ;
+    s.prep.se = (double)hist.sigma(c->n) * c->eps;
+    s.prep.rc = kRecenterFrac * N;
+    s.prep.rule45 = n1 > 2 && hist.sigma(n1 - 1) != hist.sigma(n1 - 2);
+    s.prep.r45 = n1 > 2 ? 4.5 * hist.iderr(n1 - 2) * hist.iderr(n1 - 2) : 0.0;
+  }
+  if (lane < 4) {
+    const Ctl* c = hot_ctl(s);
+    const bool rec = (lane & 2) != 0;
+    LayerCoef k;
+    if (c->accel) {
+      double l = c->acc_l, h = c->acc_h, pa, pb, pc;
+      const int sg = accel_layer(l, h, pa, pb, pc);
+      k = poly_coef(c->alpha_next, pa, pb, pc, rec, c->shift);
+      if (lane == 0) {
+        s.prep.l = l;
+        s.prep.h = h;
+        s.prep.sign = sg;
+      }
+    } else {
+      k = branch_coef(c->alpha_next, (lane & 1) ? -1 : 1, rec);
+    }
+    s.prep.k[lane] = k;
+    s.prep.ca[lane] = (float)k.ca;
+    s.prep.cb[lane] = (float)k.cb;
+  }
+  __syncwarp();
+}
+
+// The control step of the resident solve: control_step's decision of the loop
+// with everything that does not depend on the sums taken from Prepared and the
+// comparisons side by side (a chain of seven FP64 operations instead of some
+// twenty); the other phases as they are.
+__device__ __forceinline__ void resident_step(Slot& s, double trY, double sqY, RingHistory hist) {
+  Ctl* c = hot_ctl(s);
+  const Prepared& p = s.prep;
+  if (c->phase != PHASE_LOOP || c->stop_pending || c->accel) {
+    control_step(c, trY, sqY, hist, PreparedCoef{&p});
+    return;
+  }
+  const int n1 = c->n + 1, max_iter = c->max_iter, rule45 = p.rule45;
+  const double tol = c->tol, no = p.no;
+  const double NX = fma(p.ta, trY, p.naa) + sqY;             // Tr[S_n^2] = ||S_n||_F^2
+  const double NS2 = fma(2.0, trY, 2.0 * p.na - no);         // 2 Tr[S_n] - N_occ
+  const double err = fma(p.oa, trY, p.na1) - sqY;            // N_S - N_X
+  const double v = fabs(NS2 - NX) - fabs(NX - no) - p.se;
+  const bool center = err <= p.rc, low = err <= tol, zero = err <= 0.0, r45 = err > p.r45;
+  const int sg = (v >= 0.0) ? 1 : -1;
+  const int recentered = (c->recentered || (c->shift && center)) ? 1 : 0;
+  int stop = SP2_STOP_NONE;
+  if (tol > 0.0 && low)
+    stop = SP2_STOP_TOL;
+  else if (zero)
+    stop = SP2_STOP_IDERR;
+  else if (rule45 && r45)
+    stop = SP2_STOP_RULE45;
+  else if (n1 >= max_iter)
+    stop = SP2_STOP_MAXITER;
+  c->trY = trY;
+  c->sqY = sqY;
+  c->alpha = c->alpha_next;
+  c->recentered = recentered;
+  c->n = n1;
+  c->stop_pending = stop;
+  if (stop) c->converged_by = stop;
+  PreparedCoef{&p}.branch(c, sg, false);
+  hist.set(n1, sg, err);
+}
+
+// Control of one slot: takes the tiles of its list and drives their layers.
+__device__ __forceinline__ void control(const ResArgs& a, Shared& sh, int c, int lane, unsigned long long idle) {
+  Slot& s = sh.slot[c];
+  Ctl* hot = hot_ctl(s);
+  const int sl = c * (int)gridDim.x + (int)blockIdx.x;
+  uint32_t done_phase = 0;
+  bool ok = true;
+  for (int li = a.list_off[sl]; ok && li < a.list_off[sl + 1]; ++li) {
+    const int t = a.list[li];
+    int b, I, J, h;
+    unpack_tile(a.tiles[t], b, I, J, h);
+    const Ctl* gc = a.ctl + b;
+    // the control block as the input layer's control step left it
+    const double* src = reinterpret_cast<const double*>(gc);
+    for (int i = lane; i < (int)(kCtlHotBytes / 8); i += 32) s.hot[i] = __ldcg(src + i);
+    __syncwarp();
+    const int n0 = hot->n;
+    if (lane < 4) {
+      const int n = n0 - lane;
+      if (n >= 0) {
+        s.sg[n & 3] = gc->sigma[n];
+        s.ie[n & 3] = gc->iderr[n];
+      }
+    }
+    const int cnt = a.tile_cnt[b], off = a.tile_off[b];
+    const bool leader = t == off;
+    const bool twice = (I >> 1) != (J >> 1);  // the mirror's squares
+    bool act = hot->next.active != 0;
+    unsigned* st = a.stamps + (long long)b * kResStamps;
+    uint64_t t0 = 0;
+    if (act && leader && lane == 0) t0 = globaltimer();
+    if (lane == 0) {
+      s.b = b;
+      s.I = I;
+      s.J = J;
+      s.N = hot->N;
+      s.par = 0;
+      s.first = 1;
+      s.closed = 0;
+      if (act) {
+        mbar_arrive(&sh.ready[c]);
+        mbar_arrive(&sh.coef[c]);
+      }
+    }
+    __syncwarp();
+    for (int k = 0; act; ++k) {
+      prepare(s, lane);
+      if (!__all_sync(0xffffffffu, mbar_wait(&sh.epi_done[c], done_phase, &sh.abort, idle))) {
+        ok = false;
+        break;
+      }
+      done_phase ^= 1u;
+      // after the launch that writes D the solve is over; any other layer has
+      // a next one, whose products need this one's planes but not its sums
+      const bool outD = hot->next.out_mode == OUT_D;
+      if (lane == 0 && !outD) {
+        s.par ^= 1;
+        s.first = 0;
+        if (cnt == 1) mbar_arrive(&sh.ready[c]);
+      }
+      const long long rq = lane < EPI_WARPS ? sh.red_q[c][lane] : 0;
+      long long bad = worst_mark(rq);
+      long long T = sum16(lane < EPI_WARPS ? sh.red_t[c][lane] : 0);
+      long long Q = sum16(rq) << (twice ? 1 : 0);
+      double E = 0.0;
+      if (outD) E = warp_sum_d(lane < EPI_WARPS ? sh.red_e[c][lane] : 0.0);
+      long long q_hi = Q >> 28, q_lo = Q & ((1ll << 28) - 1);
+      if (cnt > 1) {
+        if (lane == 0) {
+          if (outD) a.tile_dots[t] = E;
+          __threadfence();  // the CTA's planes and row norms before its sums
+          st_sums(a.sums + (long long)(k % 3) * a.ntiles + t, T, bad ? bad : Q);
+        }
+        if (!meet(a, sh, a.sums + (long long)(k % 3) * a.ntiles + off, cnt, lane, outD ? nullptr : &sh.ready[c], T,
+                  q_hi, q_lo, bad, idle)) {
+          ok = false;
+          break;
+        }
+        // every tile has read the sums of the layer before: its slot is free for the layer after next
+        if (lane == 0) st_sums(a.sums + (long long)((k + 2) % 3) * a.ntiles + t, kGangEmpty, kGangEmpty);
+        if (outD && leader) {
+          E = 0.0;
+          for (int i = lane; i < cnt; i += 32) E += __ldcg(&a.tile_dots[off + i]);
+          E = warp_sum_d(E);
+        }
+      }
+      if (lane == 0) {
+        const double off = __longlong_as_double(bad == SQ_NAN ? 0x7ff8000000000000ll : 0x7ff0000000000000ll);
+        const double trY = bad == SQ_NAN ? off : (double)T * T_UNIT;
+        const double sqY = bad ? off : (double)q_hi * Q_HI_UNIT + (double)q_lo * Q_LO_UNIT;
+        resident_step(s, trY, sqY, RingHistory{s.sg, s.ie, leader ? a.ctl + b : nullptr});
+        if (!outD) mbar_arrive(&sh.coef[c]);
+        if (leader) {
+          if (outD) a.dots_out[3 * b] = E;
+          if (k + 1 < kResStamps) st[k + 1] = (unsigned)(globaltimer() - t0);
+        }
+      }
+      __syncwarp();
+      act = hot->next.active != 0;
+      if (!act && leader) {
+        // the final state for the host; the history was recorded layer by layer
+        double* dst = reinterpret_cast<double*>(a.ctl + b);
+        for (int i = lane; i < (int)(kCtlHotBytes / 8); i += 32) dst[i] = s.hot[i];
+      }
+    }
+    __syncwarp();
+  }
+  if (!ok && lane == 0) {
+    atomicExch(a.err, (int)SP2_ERR_DEVICE_TIMEOUT);
+    *(volatile int*)&sh.abort = 1;
+  }
+  if (lane == 0) {
+    s.closed = 1;
+    mbar_arrive(&sh.ready[c]);
+  }
+}
+
+template <bool SPLIT>
+__global__ void __launch_bounds__(THREADS, 1) resident_kernel(const __grid_constant__ ResMaps maps, const ResArgs a) {
+  constexpr int STAGES = SPLIT ? STAGES_SPLIT : STAGES_PLAIN;
+  constexpr int STAGE_BYTES = SPLIT ? STAGE_SPLIT : STAGE_PLAIN;
+  constexpr int PLANES = SPLIT ? 2 : 1;
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  uint8_t* smem = smem_raw;
+  float* trbuf = reinterpret_cast<float*>(smem + OPERAND_BYTES);
+  Shared& sh = *reinterpret_cast<Shared*>(smem + OPERAND_BYTES + TR_BYTES);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (smem_u32(smem_raw) & 1023u) {  // the swizzled operand tiles need it; the same for every CTA
+    if (threadIdx.x == 0) atomicExch(a.err, (int)SP2_ERR_UNSUPPORTED);
+    return;
+  }
+
+  if (threadIdx.x == 0) {
+    sh.abort = 0;
+    for (int k = 0; k < STAGES; ++k) {
+      mbar_init(&sh.full[k], 1);
+      mbar_init(&sh.empty[k], 1);
+    }
+    for (int k = 0; k < 2; ++k) {
+      mbar_init(&sh.ready[k], 1);
+      mbar_init(&sh.coef[k], 1);
+      mbar_init(&sh.acc_full[k], 1);
+      mbar_init(&sh.epi_done[k], EPI_WARPS);
+    }
+    for (int k = 0; k < WQ; ++k) mbar_init(&sh.wq_full[k], 1);
+    mbar_init(&sh.drain, 1);
+    mbar_init(&sh.never, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  if (warp == 1) {
+    tmem_alloc(&sh.tmem, TMEM_COLS);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = sh.tmem;
+  volatile int* abort_flag = &sh.abort;
+  const unsigned long long lim = a.wait_ns ? a.wait_ns : kTimeoutNs;
+  // waits for work (a gang still forming) last as long as other solves do
+  const unsigned long long idle = lim > kTimeoutNs ? lim : kTimeoutNs;
+
+  if (warp == 0) {
+    // ------------------------------------------------------------ producer
+    if (lane == 0) {
+      uint32_t rphase = 0;  // bit c: phase of ready[c]
+      bool open0 = true, open1 = a.two_slots != 0, ok = true;
+      int last = 1, stage = 0;
+      uint32_t phase = 0, seq = 0;
+      uint32_t armed[STAGES];
+#pragma unroll
+      for (int k = 0; k < STAGES; ++k) armed[k] = 0;
+      for (int k = 0; k < 8; ++k)
+        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&maps.m[k >> 2][k & 3])) : "memory");
+      while (ok && (open0 || open1)) {
+        int c = -1;
+        const uint64_t w0 = globaltimer();
+        for (int spin = 0; c < 0; ++spin) {
+          const int o = last ^ 1;
+          if ((o ? open1 : open0) && mbar_test(&sh.ready[o], (rphase >> o) & 1u))
+            c = o;
+          else if ((last ? open1 : open0) && mbar_test(&sh.ready[last], (rphase >> last) & 1u))
+            c = last;
+          else if ((spin & 63) == 63 && (*abort_flag || globaltimer() - w0 > idle))
+            break;
+        }
+        if (c < 0) {
+          ok = false;
+          break;
+        }
+        rphase ^= 1u << c;
+        last = c;
+        const volatile Slot& s = sh.slot[c];
+        if (s.closed) {
+          (c ? open1 : open0) = false;
+          continue;
+        }
+        const int b = s.b, I = s.I, J = s.J, N = s.N, par = s.par;
+        // (the planes' writers have fenced them against the async proxy)
+        sh.wq[seq % WQ] = c;
+        mbar_arrive(&sh.wq_full[seq % WQ]);
+        ++seq;
+        const CUtensorMap* m = maps.m[par];
+        const bool same = I == J;  // diagonal tile: one operand serves as both
+        const int rowA = I * TB, rowB = J * TB, nk = (N + BK - 1) / BK;
+        for (int kb = 0; kb < nk; ++kb) {
+          if (!mbar_wait(&sh.empty[stage], phase ^ 1u, abort_flag, lim)) {
+            ok = false;
+            break;
+          }
+          uint8_t* dst = smem + stage * STAGE_BYTES;
+          mbar_expect_tx(&sh.full[stage], (same ? 1 : 2) * PLANES * HALF_BYTES);
+          ++armed[stage];
+          const int k0 = kb * BK, ks = k0 / BN;  // super column of this K block
+          const bool ta = ks < (I >> 1), tb = ks < (J >> 1);
+          load_half(dst, &m[0], &m[2], ta, rowA, k0, b, &sh.full[stage]);
+          if (SPLIT) load_half(dst + HALF_BYTES, &m[1], &m[3], ta, rowA, k0, b, &sh.full[stage]);
+          if (!same) {
+            load_half(dst + PLANES * HALF_BYTES, &m[0], &m[2], tb, rowB, k0, b, &sh.full[stage]);
+            if (SPLIT) load_half(dst + 3 * HALF_BYTES, &m[1], &m[3], tb, rowB, k0, b, &sh.full[stage]);
+          }
+          if (++stage == STAGES) {
+            stage = 0;
+            phase ^= 1u;
+          }
+        }
+      }
+      sh.wq[seq % WQ] = WQ_END;
+      mbar_arrive(&sh.wq_full[seq % WQ]);
+      if (!ok || *abort_flag) {
+        atomicExch(a.err, (int)SP2_ERR_DEVICE_TIMEOUT);
+        *abort_flag = 1;
+        for (int k = 0; k < STAGES; ++k) {  // copies in flight land before the CTA leaves
+          if (armed[k] == 0) continue;
+          const uint64_t t0 = globaltimer();
+          while (!mbar_test(&sh.full[k], (armed[k] - 1u) & 1u) && globaltimer() - t0 < lim) {
+          }
+        }
+      }
+    }
+  } else if (warp == 1) {
+    // ------------------------------------------------------------ MMA issuer
+    if (lane == 0) {
+      int stage = 0;
+      uint32_t phase = 0;
+      bool ok = true, issued = false;
+      if (a.stall && !mbar_wait(&sh.never, 0, abort_flag, lim)) ok = false;
+      for (uint32_t seq = 0; ok; ++seq) {
+        if (!mbar_wait(&sh.wq_full[seq % WQ], (seq / WQ) & 1u, abort_flag, idle)) {
+          ok = false;
+          break;
+        }
+        const int c = *(volatile int*)&sh.wq[seq % WQ];
+        if (c == WQ_END) break;
+        const volatile Slot& s = sh.slot[c];
+        const int I = s.I, J = s.J, nk = (s.N + BK - 1) / BK;
+        const bool same = I == J;
+        tc_fence_after();
+        const uint32_t d = tmem_base + c * SLOT_COLS;
+        for (int kb = 0; kb < nk; ++kb) {
+          if (!mbar_wait(&sh.full[stage], phase, abort_flag, lim)) {
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+          const uint32_t st = smem_u32(smem + stage * STAGE_BYTES);
+          const uint32_t sb = same ? st : st + PLANES * HALF_BYTES;
+          const int ks = kb * BK / BN;
+          const bool ta = ks < (I >> 1), tb = ks < (J >> 1);
+          const uint32_t idesc = IDESC_T | (ta ? IDESC_A_MN : 0u) | (tb ? IDESC_B_MN : 0u);
+#pragma unroll
+          for (int u = 0; u < BK / UMMA_K; ++u) {
+            const uint32_t oa = ta ? u * 2048u : u * UMMA_K * 2u, ob = tb ? u * 2048u : u * UMMA_K * 2u;
+            const uint64_t a0 = ta ? make_desc_mn128(st + oa) : make_desc_sw128(st + oa);
+            const uint64_t b0 = tb ? make_desc_mn128(sb + ob) : make_desc_sw128(sb + ob);
+            mma_f16_id(d, a0, b0, idesc, (kb > 0 || u > 0) ? 1u : 0u);  // hp hp (plain: hi hi)
+            if (SPLIT) {
+              const uint32_t la = st + HALF_BYTES + oa, lb = sb + HALF_BYTES + ob;
+              const uint64_t a1 = ta ? make_desc_mn128(la) : make_desc_sw128(la);
+              const uint64_t b1 = tb ? make_desc_mn128(lb) : make_desc_sw128(lb);
+              mma_f16_id(d, a1, b0, idesc, 1u);  // lo' hp
+              mma_f16_id(d, a0, b1, idesc, 1u);  // hp lo'
+            }
+          }
+          mma_commit(&sh.empty[stage]);
+          issued = true;
+          if (++stage == STAGES) {
+            stage = 0;
+            phase ^= 1u;
+          }
+        }
+        if (ok) mma_commit(&sh.acc_full[c]);
+      }
+      if (!ok || *abort_flag) {
+        atomicExch(a.err, (int)SP2_ERR_DEVICE_TIMEOUT);
+        *abort_flag = 1;
+      }
+      if (issued) {
+        mma_commit(&sh.drain);
+        const uint64_t t0 = globaltimer();
+        while (!mbar_test(&sh.drain, 0) && globaltimer() - t0 < lim) {
+        }
+      }
+    }
+  } else if (warp >= CTL_WARP) {
+    const int c = warp - CTL_WARP;
+    if (c == 0 || a.two_slots) control(a, sh, c, lane, idle);
+  } else {
+    // ------------------------------------------------------------ epilogue
+    const int ew = warp - 2, q = warp & 3;
+    uint32_t aphase = 0;  // bit c: phase of acc_full[c]
+    for (uint32_t seq = 0;; ++seq) {
+      if (!__all_sync(0xffffffffu, mbar_wait(&sh.wq_full[seq % WQ], (seq / WQ) & 1u, abort_flag, idle))) break;
+      const int c = *(volatile int*)&sh.wq[seq % WQ];
+      if (c == WQ_END) break;
+      if (!epilogue<SPLIT>(a, sh, c, (aphase >> c) & 1u, tmem_base, ew, q, lane, trbuf + ew * (16 * 32), lim)) {
+        if (lane == 0) atomicExch(a.err, (int)SP2_ERR_DEVICE_TIMEOUT);
+        *abort_flag = 1;
+        break;
+      }
+      aphase ^= 1u << c;
+    }
+  }
+
+  __syncwarp();
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if (warp == 1) {
+    __syncwarp();
+    tmem_dealloc(tmem_base, TMEM_COLS);
+  }
+}
+
+}  // namespace res
+
+// ---------------------------------------------------------------- input layer
+// The resident solve's input layer: one warp per row of H forms Y_0 (kept by
+// nobody: the first layer's epilogue forms its tile of it again from H), writes
+// its operand planes from the row's super tile on, up to the padded row length
+// (the only part the operand loads read), and sums the row's squares in FP64
+// in the order of rownorm_kernel (vec_norm: its float4 form).  The last block
+// of an instance adds the traces and runs the first control step.  HBM-bound:
+// H read once, half the planes written.
+__global__ void __launch_bounds__(256) resident_input_kernel(const ResArgs a, int vec_norm) {
+  const int b = blockIdx.y;
+  const int N = a.Ns[b];
+  const int nb = (N + 7) / 8;
+  if ((int)blockIdx.x >= nb) return;
+  Ctl* c = a.ctl + b;
+  if (c->phase == PHASE_ERROR) return;
+  const InputScale in = input_scale(c->e_min, c->e_max, a.shift);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int r = blockIdx.x * 8 + warp;
+  double acc = 0.0, tr = 0.0;
+  if (r < N) {
+    const float* row = a.H[b] + (long long)r * N;
+    __half* p0 = a.p0[0] + (long long)b * a.slot_h + (long long)r * a.ld_h;
+    __half* p1 = a.p1[0] ? a.p1[0] + (long long)b * a.slot_h + (long long)r * a.ld_h : nullptr;
+    const int cs = r & ~(kTcBN - 1), kpad = (N + 63) & ~63;
+    const bool vec_h = (N & 3) == 0 && (reinterpret_cast<uintptr_t>(a.H[b]) & 15) == 0;
+    // the diagonal once per row: FP64 per element, even predicated off, would
+    // bound the pass (1.97 ms against 0.33 for the bounds' pass over the same
+    // 512 matrices)
+    const float yd = input_diag(row[r], in);
+    tr = lane == 0 ? (double)yd : 0.0;
+    auto y0 = [&](float h, int col) { return col == r ? yd : input_offdiag(h, in); };
+    // FP16 planes of four columns; plain FP16 keeps hi alone
+    auto put = [&](int col, const float (&y)[4]) {
+      uint32_t pa[2], pl[2];
+      const __half2 s2 = __float2half2_rn(a.lo_scale);
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const __half2 h2 = __floats2half2_rn(y[2 * e], y[2 * e + 1]);
+        const float2 hf = __half22float2(h2);
+        const __half2 l2 = __floats2half2_rn((y[2 * e] - hf.x) * a.lo_scale, (y[2 * e + 1] - hf.y) * a.lo_scale);
+        const __half2 p2 = p1 ? __hmul2(h2, s2) : h2;
+        pa[e] = *reinterpret_cast<const uint32_t*>(&p2);
+        pl[e] = *reinterpret_cast<const uint32_t*>(&l2);
+      }
+      *reinterpret_cast<uint2*>(p0 + col) = make_uint2(pa[0], pa[1]);
+      if (p1) *reinterpret_cast<uint2*>(p1 + col) = make_uint2(pl[0], pl[1]);
+    };
+    const int n4 = N >> 2;
+    for (int j0 = 0; j0 < (kpad >> 2); j0 += 32 * 8) {
+      float f = 0.f;
+      float4 hv[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int col = (j0 + u * 32 + lane) * 4;
+        hv[u] = col < N ? epi::ld4(row + col, col, N, vec_h) : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int j = j0 + u * 32 + lane, col = 4 * j;
+        if (col < kpad) {
+          float y[4] = {hv[u].x, hv[u].y, hv[u].z, hv[u].w};
+#pragma unroll
+          for (int e = 0; e < 4; ++e) y[e] = col + e < N ? y0(y[e], col + e) : 0.f;
+          if (j < n4) {
+            f = fmaf(y[0], y[0], f);
+            f = fmaf(y[1], y[1], f);
+            f = fmaf(y[2], y[2], f);
+            f = fmaf(y[3], y[3], f);
+          }
+          if (col >= cs) put(col, y);
+        }
+      }
+      if (vec_norm && j0 < n4) acc += (double)f;
+    }
+    // columns past the last float4, or every column in FP64 (rownorm_kernel's two tails)
+    for (int j = (vec_norm ? n4 << 2 : 0) + lane; j < N; j += 32) {
+      const double yv = (double)y0(row[j], j);
+      acc += yv * yv;
+    }
+    acc = warp_sum_d(acc);
+    if (lane == 0) const_cast<double*>(a.rn)[(long long)b * a.ld_rn + r] = acc;
+  }
+  __shared__ double s_q[8], s_t[8];
+  __shared__ bool s_last;
+  if (lane == 0) {
+    s_q[warp] = acc;
+    s_t[warp] = tr;
+  }
+  __syncthreads();
+  // the gang's slots of the resident launch
+  const int cnt = a.tile_cnt[b], off = a.tile_off[b];
+  for (int i = blockIdx.x * 256 + threadIdx.x; i < 3 * cnt; i += nb * 256)
+    a.sums[(long long)(i / cnt) * a.ntiles + off + i % cnt] = make_longlong2(kGangEmpty, kGangEmpty);
+  double2* part = a.part + (long long)b * gridDim.x;
+  if (threadIdx.x == 0) {
+    double q = 0.0, t = 0.0;
+    for (int w = 0; w < 8; ++w) {
+      q += s_q[w];
+      t += s_t[w];
+    }
+    part[blockIdx.x] = make_double2(t, q);
+    __threadfence();
+    s_last = atomicAdd(&a.tickets[b], 1u) == (unsigned)nb - 1u;
+  }
+  __syncthreads();
+  if (!s_last || warp != 0) return;
+  __threadfence();
+  double T = 0.0, Q = 0.0;
+  for (int k = lane; k < nb; k += 32) {
+    const double2 p = __ldcg(&part[k]);
+    T += p.x;
+    Q += p.y;
+  }
+  T = warp_sum_d(T);
+  Q = warp_sum_d(Q);
+  if (lane == 0) {
+    c->alpha_next = a.shift ? c->e_max * (1.0 / (c->e_max - c->e_min)) : 0.0;
+    control_step(c, T, Q);
+  }
+}
+
+cudaError_t launch_resident_input(const ResArgs& a, int vec_norm, int Nmax, int batch, cudaStream_t st) {
+  resident_input_kernel<<<dim3((Nmax + 7) / 8, batch), 256, 0, st>>>(a, vec_norm);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_resident(const ResArgs& a, const ResMaps& maps, bool split, int grid, cudaStream_t st) {
+  constexpr int smem = res::OPERAND_BYTES + res::TR_BYTES + (int)sizeof(res::Shared);
+  static_assert(smem <= 227 * 1024, "shared memory");
+  cudaError_t e = split ? cudaFuncSetAttribute(res::resident_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)
+                        : cudaFuncSetAttribute(res::resident_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid, 1, 1);
+  cfg.blockDim = dim3(res::THREADS, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeCooperative;  // the gangs wait on one another
+  attr[0].val.cooperative = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return split ? cudaLaunchKernelEx(&cfg, res::resident_kernel<true>, maps, a)
+               : cudaLaunchKernelEx(&cfg, res::resident_kernel<false>, maps, a);
+}
+
+}  // namespace sp2

@@ -1,0 +1,89 @@
+"""The resident solve (all layers of a batch in one launch on 128 x 128 tiles)
+against the launch-per-layer kernels it takes over from: the same bits, at the
+edges of its tiles and of its range."""
+import os
+
+import numpy as np
+import pytest
+
+import oracle as o
+import sp2_inputs as si
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def _with_env(name, value, fn):
+    import paper_2101_06385_gb300 as sp2
+
+    os.environ[name] = value
+    sp2.finalize()
+    sp2.init(0)
+    try:
+        return fn(sp2)
+    finally:
+        del os.environ[name]
+        sp2.finalize()
+        sp2.init(0)
+
+
+@pytest.fixture(scope="module")
+def sp2():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2101_06385_gb300 as m
+
+    m.init(0)
+    return m
+
+
+# one tile, its edge, a lone last row and column of tiles, the lower tile of a
+# diagonal super tile, odd rows, more tiles than CTAs, the largest size
+@pytest.mark.parametrize("N", [1, 31, 128, 129, 257, 385, 1021, 2053, 2816])
+@pytest.mark.parametrize("mode", ["split", "fp16", "accelerated"])
+def test_single_solve_same_bits(sp2, N, mode):
+    n_occ = max(1, N // 3)
+    h = si.gapped_hamiltonian(N, n_occ, (-1.0, -0.1), (0.1, 1.0), seed=300 + N, device="cuda" if N > 1000 else "cpu")
+    H = torch.from_numpy(h.h32()).cuda()
+
+    def solve(m):
+        if mode == "accelerated":
+            return m.density_matrix_accelerated(H, n_occ, -0.1, 0.1, precision="split")
+        return m.density_matrix(H, n_occ, precision=mode)
+
+    D, st = solve(sp2)
+    D1, s1 = _with_env("SP2_SQUARE_KERNEL", "single", solve)
+    assert torch.equal(D, D1)
+    assert st.sigmas == s1.sigmas and st.converged_by == s1.converged_by
+    # times of the layers it ran, none after them
+    ran = st.iterations + (0 if mode == "accelerated" else 2)
+    assert all(t > 0 for t in st.layer_ms[:ran]) and not any(st.layer_ms[ran:])
+
+
+# an instance on both slots of every CTA among small ones, and more instances
+# than slots (each slot works through a list)
+@pytest.mark.parametrize("sizes", [[2500, 64, 700, 1, 300], [1000, 96] * 20 + [130] * 300 + [7, 513]])
+def test_batch_same_bits(sp2, sizes):
+    kinds = {N: si.gapped_hamiltonian(N, N // 2, (-1.0, -0.05), (0.05, 1.0), seed=400 + N) for N in set(sizes)}
+    Hs = [torch.from_numpy(kinds[N].h32()).cuda() for N in sizes]
+    n_occ = [N // 2 for N in sizes]
+    Ds, st = sp2.density_matrix_batched(Hs, n_occ)
+    Dp, sp = _with_env("SP2_BATCHED_KERNEL", "pairs", lambda m: m.density_matrix_batched(Hs, n_occ))
+    for a, b in zip(Ds, Dp):
+        assert torch.equal(a, b)
+    assert [s.sigmas for s in st] == [s.sigmas for s in sp]
+    m = o.error_metrics(Ds[0].cpu().numpy().astype(np.float64), o.density_matrix_closed_form(kinds[sizes[0]].Q, n_occ[0]),
+                        n_occ[0])
+    assert m["max_abs"] <= 5e-5 and m["trace_err"] <= 1e-4, m
+
+
+def test_input_that_is_not_symmetric_stops_alike(sp2):
+    """Symmetry is assumed, not checked: an iterate that leaves the range of the
+    layer's fixed-point sums stops the solve as it does on the other kernels."""
+    N = 300
+    H = torch.zeros(N, N, device="cuda")
+    H += torch.diag(torch.linspace(-1, 1, N, device="cuda"))
+    H[: N // 2, N // 2:] = 5.0  # the rows' bounds hold for H, not for its upper triangle mirrored
+    D, st = sp2.density_matrix(H, N // 2)
+    D1, s1 = _with_env("SP2_SQUARE_KERNEL", "single", lambda m: m.density_matrix(H, N // 2))
+    assert st.status == s1.status and st.converged_by == s1.converged_by
