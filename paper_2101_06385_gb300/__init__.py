@@ -259,12 +259,13 @@ def _stats_many(st, B: int) -> List[Stats]:
     lmax = max(col["launches"]) if B else 0
     sig = a["sigma"][:, :nmax].tolist()
     ide = a["iderr"][:, :nmax].tolist()
-    # per-launch times are shared by the instances of one call: convert once
+    # times past an instance's last layer are zero: convert the columns in use
+    # and, where both records agree, once
     la, sa = a["layer_ms"][:, :lmax], a["square_ms"][:, :lmax]
-    if B and (la == la[0]).all() and (sa == sa[0]).all():
-        lms, sms = [la[0].tolist()] * B, [sa[0].tolist()] * B
-    else:
-        lms, sms = la.tolist(), sa.tolist()
+    used = int(np.flatnonzero(la.any(0) | sa.any(0)).max(initial=-1)) + 1
+    rest = [0.0] * (lmax - used)
+    lms = [row + rest for row in la[:, :used].tolist()]
+    sms = [list(row) for row in lms] if (la == sa).all() else [row + rest for row in sa[:, :used].tolist()]
     out = []
     for i in range(B):
         n, nl, c = col["iterations"][i], col["launches"][i], col["converged_by"][i]
