@@ -390,6 +390,15 @@ sp2_status status_of(const Ctl& c, int dev_err) {
   return SP2_OK;
 }
 
+// The accelerated solves' check of the caller's estimates (instance >= 0: of a batch).
+sp2_status check_estimate(const Ctl& c, sp2_status s, int N_occ, int instance) {
+  if (s < 0 || std::fabs(c.trace_final - (double)N_occ) <= 0.5) return s;
+  char who[32] = "accelerated solve";
+  if (instance >= 0) snprintf(who, sizeof who, "instance %d", instance);
+  set_err("%s: Tr D = %.3f but N_occ = %d; the HOMO/LUMO estimates do not bracket the gap", who, c.trace_final, N_occ);
+  return SP2_ERR_BAD_ESTIMATE;
+}
+
 }  // namespace
 
 extern "C" {
@@ -985,20 +994,119 @@ sp2_status resident_solve(const float* const* H, const int* N, const int* N_occ,
     const unsigned* t = (const unsigned*)(rb + P.stamps) + (size_t)b * kResStamps;
     for (int k = 0; k < nlaunch && t[k + 1] != 0; ++k) s.layer_ms[k] = s.square_ms[k] = (float)(t[k + 1] - t[k]) * 1e-6f;
     sp2_status sb = status_of(cs[b], e);
-    if (accel && sb >= 0 && std::fabs(cs[b].trace_final - (double)N_occ[b]) > 0.5) {
-      if (single)
-        set_err("accelerated solve: Tr D = %.3f but N_occ = %d; the HOMO/LUMO estimates do not bracket the gap",
-                cs[b].trace_final, N_occ[b]);
-      else
-        set_err("instance %d: Tr D = %.3f but N_occ = %d; the HOMO/LUMO estimates do not bracket the gap", b,
-                cs[b].trace_final, N_occ[b]);
-      sb = SP2_ERR_BAD_ESTIMATE;
-    }
+    if (accel) sb = check_estimate(cs[b], sb, N_occ[b], single ? -1 : b);
     if (sb < 0 && worst >= 0) worst = sb;
     if (sb == SP2_NOT_CONVERGED && worst == SP2_OK) worst = SP2_NOT_CONVERGED;
   }
   if (worst == SP2_OK && !single) t_err.clear();
   return worst;
+}
+
+// Upper tiles of side ts of an N x N matrix.
+long long upper_tiles(int N, int ts) {
+  const long long T = (N + ts - 1) / ts;
+  return T * (T + 1) / 2;
+}
+
+// Tile side of the resident FP32 solve, or 0 for the launch-per-layer kernels:
+// by the measured cost of the busiest CTA, about 30 cycles per k and tile of
+// side 32, 70 of side 64, against 240 of a wave of 128 x 128 tiles.
+int fp32_tile(int N) {
+  if (g.precision != SP2_PREC_FP32 || !g.pair_kernel || N > 2048) return 0;
+  const long long c32 = 30 * ((upper_tiles(N, 32) + g.num_sms - 1) / g.num_sms);
+  const long long c64 = 70 * ((upper_tiles(N, 64) + g.num_sms - 1) / g.num_sms);
+  return std::min(c32, c64) > 240 ? 0 : c32 <= c64 ? 32 : 64;
+}
+
+// The single FP32 solve on the resident kernel (csrc/resident_fp32.cu).
+sp2_status fp32_solve(const float* H, int N, int N_occ, double tol, int max_iter, float* D_out, sp2_stats* stats,
+                      bool accel, double homo, double lumo, int tile) {
+  cudaStream_t st = g.stream;
+  const int T = (N + tile - 1) / tile, nt = (int)upper_tiles(N, tile), grid = std::min(nt, g.num_sms);
+  const int nlaunch = accel ? max_iter : max_iter + 2;
+  const int ggrid = (int)std::min<long long>((N + 7) / 8, 4LL * g.num_sms);
+  const int igrid = (int)std::min<long long>(N, 8LL * g.num_sms);
+  const int rgrid = (int)std::min<long long>((N + 7) / 8, 2LL * g.num_sms);
+  // one upload: control block, stamps, error word (read back), then pointers,
+  // size, tickets and the tiles
+  const size_t o_st = sizeof(Ctl), o_err = o_st + (kResStamps + 2) / 2 * 8, o_ptr = o_err + 16,
+               o_tiles = o_ptr + 64, bytes = o_tiles + (size_t)nt * sizeof(uint32_t);
+  static_assert(sizeof(Ctl) % 8 == 0, "the offsets after it keep 8-byte alignment");
+  const size_t sums_bytes = (size_t)6 * grid * sizeof(longlong2);
+  void *pack, *part, *rn, *sums, *Y[2];
+  CKS(ws(B_PACK, bytes, &pack));
+  CKS(ws(B_TPART, sums_bytes, &sums));
+  CKS(ws(B_PART, std::max(std::max(ggrid, igrid), rgrid) * sizeof(double2), &part));
+  CKS(ws(B_RN, (size_t)N * sizeof(double), &rn));
+  const long long ld_y = round_up(N, 4), slot_y = ld_y * N;
+  CKS(ws(B_Y0, (size_t)slot_y * 4, &Y[0]));
+  CKS(ws(B_Y1, (size_t)slot_y * 4, &Y[1]));
+  void* h;
+  CKS(staging(bytes, &h));
+  uint8_t* hb = (uint8_t*)h;
+  memset(hb, 0, o_tiles);
+  Ctl* hc = (Ctl*)hb;
+  init_ctl(hc, N, N_occ, tol, max_iter);
+  if (accel) {
+    hc->accel = 1;
+    hc->acc_homo = homo;
+    hc->acc_lumo = lumo;
+    hc->tol = tol > 0.0 ? tol : 1e-9;
+  }
+  memcpy(hb + o_ptr, &H, sizeof(void*));
+  memcpy(hb + o_ptr + 8, &N, sizeof(int));
+  uint32_t* ht = (uint32_t*)(hb + o_tiles);
+  for (int I = 0; I < T; ++I)
+    for (int J = I; J < T; ++J) *ht++ = pack_tile(0, I, J, 0);
+  uint8_t* dp = (uint8_t*)pack;
+  CK(cudaMemcpyAsync(dp, hb, bytes, cudaMemcpyHostToDevice, st));
+  CK(cudaEventRecord(g.stage_done, st));
+  CK(cudaMemsetAsync(sums, kGangEmptyByte, sums_bytes, st));
+  Res32Args A;
+  memset(&A, 0, sizeof(A));
+  A.Y[0] = (float*)Y[0];
+  A.Y[1] = (float*)Y[1];
+  A.ld_y = ld_y;
+  A.N = N;
+  A.D = D_out;
+  A.tiles = (const uint32_t*)(dp + o_tiles);
+  A.ntiles = nt;
+  A.ctl = (Ctl*)dp;
+  A.rn = (double*)rn;
+  A.sums = (longlong2*)sums;
+  A.stamps = (unsigned*)(dp + o_st);
+  A.err = (int*)(dp + o_err);
+  A.wait_ns = g.wait_ns;
+  const float* const* hp = (const float* const*)(dp + o_ptr);
+  const int* np = (const int*)(dp + o_ptr + 8);
+  unsigned* tick = (unsigned*)(dp + o_ptr + 16);
+  CK(cudaEventRecord(g.ev0, st));
+  CK(launch_gershgorin(H, N, N, (long long)N * N, 1, (double2*)part, tick, A.ctl, nullptr, ggrid, st,
+                       g.fault_nan ? 0 : -1));
+  g.fault_nan = false;
+  CK(launch_input_layer(hp, np, N, A.Y[0], ld_y, slot_y, nullptr, nullptr, nullptr, 0, 0, N, N, 0.f, A.ctl, nullptr,
+                        (double2*)part, tick, g.shift, 1, 1, igrid, st));
+  CK(launch_rownorm(A.Y[0], ld_y, slot_y, np, 1, N, A.rn, N, A.ctl, (double2*)part, tick, rgrid, st));
+  CK(cudaEventRecord(g.lev[0], st));
+  CK(launch_resident_fp32(A, tile, grid, st));
+  CK(cudaEventRecord(g.ev1, st));
+  if (!stats) return SP2_OK;
+  void* back;
+  CKS(staging(o_ptr, &back));
+  CK(cudaMemcpyAsync(back, dp, o_ptr, cudaMemcpyDeviceToHost, st));
+  CK(cudaStreamSynchronize(st));
+  float ms = 0.f, pro = 0.f;
+  CK(cudaEventElapsedTime(&ms, g.ev0, g.ev1));
+  CK(cudaEventElapsedTime(&pro, g.ev0, g.lev[0]));
+  const Ctl& c = *(const Ctl*)back;
+  fill_stats(c, stats, ms, SP2_PREC_FP32);
+  stats->launches = nlaunch;
+  stats->prologue_ms = pro;
+  const unsigned* t = (const unsigned*)((const uint8_t*)back + o_st);
+  for (int k = 0; k < nlaunch && t[k + 1] != 0; ++k)
+    stats->layer_ms[k] = stats->square_ms[k] = (float)(t[k + 1] - t[k]) * 1e-6f;
+  const sp2_status rs = status_of(c, *(const int*)((const uint8_t*)back + o_err));
+  return accel ? check_estimate(c, rs, N_occ, -1) : rs;
 }
 
 // The single-matrix solve; accel selects the accelerated layers (bounds from
@@ -1008,6 +1116,8 @@ sp2_status density_matrix_impl(const float* H, int N, int N_occ, double tol, int
   if (resident_fits(N))
     return resident_solve(&H, &N, &N_occ, 1, N, tol, max_iter, &D_out, stats, accel ? &homo : nullptr,
                           accel ? &lumo : nullptr, true);
+  if (const int tile = fp32_tile(N))
+    return fp32_solve(H, N, N_occ, tol, max_iter, D_out, stats, accel, homo, lumo, tile);
   const int prec = g.precision;
   const bool tc = tc_precision(prec);
   const bool split = prec == SP2_PREC_SPLIT_FP16;
@@ -1218,12 +1328,7 @@ sp2_status density_matrix_impl(const float* H, int N, int N_occ, double tol, int
     stats->square_ms[k] = sm;
   }
   const sp2_status rs = status_of(c, e);
-  if (accel && rs >= 0 && std::fabs(c.trace_final - (double)N_occ) > 0.5) {
-    set_err("accelerated solve: Tr D = %.3f but N_occ = %d; the HOMO/LUMO estimates do not bracket the gap",
-            c.trace_final, N_occ);
-    return SP2_ERR_BAD_ESTIMATE;
-  }
-  return rs;
+  return accel ? check_estimate(c, rs, N_occ, -1) : rs;
 }
 
 }  // namespace
@@ -1610,11 +1715,7 @@ sp2_status batched_impl(const float* const* H, const int* N, const int* N_occ, i
       stats[b].square_ms[k] = sms[k];
     }
     sp2_status sb = status_of(cs[b], e);
-    if (accel && sb >= 0 && std::fabs(cs[b].trace_final - (double)N_occ[b]) > 0.5) {
-      set_err("instance %d: Tr D = %.3f but N_occ = %d; the HOMO/LUMO estimates do not bracket the gap", b,
-              cs[b].trace_final, N_occ[b]);
-      sb = SP2_ERR_BAD_ESTIMATE;
-    }
+    if (accel) sb = check_estimate(cs[b], sb, N_occ[b], b);
     if (sb < 0 && worst >= 0) worst = sb;
     if (sb == SP2_NOT_CONVERGED && worst == SP2_OK) worst = SP2_NOT_CONVERGED;
   }

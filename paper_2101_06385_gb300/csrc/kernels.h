@@ -149,7 +149,8 @@ size_t syrk_tc2_smem_bytes(bool split);
 // instances' order is the same in every slot's list.
 constexpr int kResTile = 128;
 constexpr int kResStamps = kMaxL + 2;
-constexpr long long kGangEmpty = -0x7f7f7f7f7f7f7f80ll;  // no sum of a layer
+constexpr long long kGangEmpty = -0x7f7f7f7f7f7f7f80ll;  // no sum of a layer: every byte kGangEmptyByte
+constexpr int kGangEmptyByte = 0x80;
 struct ResMaps {
   CUtensorMap m[2][4];  // per plane parity: {p0, p1} with 64 x 128 boxes, {p0, p1} with 64 x 64 boxes
 };
@@ -170,8 +171,8 @@ struct ResArgs {
   float* rnp[2];           // row-norm segment sums, as SqArgs::rnp_out
   long long ld_rnp, slot_rnp;
   double2* part;           // [batch][blocks] block sums of the input layer
-  longlong2* sums;         // [3][ntiles] the tiles' (tr Y', ||Y'||_F^2) of layer k at [k mod 3] in fixed point,
-                           //   kGangEmpty until published
+  longlong2* sums;         // [3][ntiles] meeting rows of successive layers: the tiles' (tr Y', ||Y'||_F^2) in
+                           //   fixed point, kGangEmpty until published
   double* tile_dots;       // [ntiles] Tr[D H] per tile
   double* dots_out;        // [batch][3], entry 0: Tr[D H]
   unsigned* tickets;       // [batch] zero: finished blocks of the input layer
@@ -186,6 +187,24 @@ struct ResArgs {
 };
 cudaError_t launch_resident_input(const ResArgs& a, int vec_norm, int Nmax, int batch, cudaStream_t st);
 cudaError_t launch_resident(const ResArgs& a, const ResMaps& maps, bool split, int grid, cudaStream_t st);
+
+// Resident FP32 solve (csrc/resident_fp32.cu): one instance, all layers in one
+// cooperative launch; Y_0, its row norms and the first control step are there.
+struct Res32Args {
+  float* Y[2];             // iterates of even / odd layers, leading dimension ld_y (a multiple of 4)
+  long long ld_y;
+  int N;
+  float* D;
+  const uint32_t* tiles;   // [ntiles] upper tiles in units of the tile side
+  int ntiles;
+  Ctl* ctl;
+  double* rn;              // [N] row norms of the layer's input
+  longlong2* sums;         // [2][3][grid] kGangEmpty: meeting rows of the traces, of the square norms
+  unsigned* stamps;        // as ResArgs
+  int* err;
+  unsigned long long wait_ns;
+};
+cudaError_t launch_resident_fp32(const Res32Args& a, int tile, int grid, cudaStream_t st);
 
 cudaError_t launch_syrk_simt(const SqArgs& a, int grid, cudaStream_t st);
 

@@ -404,14 +404,12 @@ __global__ void __launch_bounds__(256) input_layer_kernel(const float* const* __
     s_last = (atomicAdd(&tickets[b], 1u) == gridDim.x - 1);
   }
   __syncthreads();
-  if (!s_last || threadIdx.x != 0) return;
+  if (!s_last || threadIdx.x >= 32) return;
   __threadfence();
-  double T = 0.0, Q = 0.0;
-  for (unsigned k = 0; k < gridDim.x; ++k) {
-    const double2 p = __ldcg(&part[k]);
-    T += p.x;
-    Q += p.y;
-  }
+  double T = 0.0;
+  for (unsigned k = threadIdx.x; k < gridDim.x; k += 32) T += __ldcg(&part[k]).x;
+  T = warp_sum_d(T);
+  if (threadIdx.x != 0) return;
   tickets[b] = 0u;
   Ctl* c = ctl + b;
   if (!active) return;
@@ -419,7 +417,6 @@ __global__ void __launch_bounds__(256) input_layer_kernel(const float* const* __
   // control step (sigma_1, IdErr_1) with the exact ||Y_0||_F^2.
   c->alpha_next = shift ? e_max * in.inv : 0.0;
   c->trY_new = T;
-  (void)Q;
 }
 
 // ---------------------------------------------------------------- row norms
@@ -485,10 +482,12 @@ __global__ void __launch_bounds__(256) rownorm_kernel(const float* __restrict__ 
     s_last = (atomicAdd(&tickets[b], 1u) == gridDim.x - 1);
   }
   __syncthreads();
-  if (!s_last || threadIdx.x != 0) return;
+  if (!s_last || threadIdx.x >= 32) return;
   __threadfence();
   double Q = 0.0;
-  for (unsigned k = 0; k < gridDim.x; ++k) Q += __ldcg(&part[k]).x;
+  for (unsigned k = threadIdx.x; k < gridDim.x; k += 32) Q += __ldcg(&part[k]).x;
+  Q = warp_sum_d(Q);
+  if (threadIdx.x != 0) return;
   tickets[b] = 0u;
   Ctl* c = ctl + b;
   control_step(c, c->trY_new, Q);

@@ -34,6 +34,7 @@
 #include "common.cuh"
 #include "epilogue.cuh"
 #include "kernels.h"
+#include "resident.cuh"
 #include "tc_ptx.cuh"
 
 namespace sp2 {
@@ -60,50 +61,13 @@ constexpr uint32_t IDESC_T = (1u << 4) | ((uint32_t)(TB >> 3) << 17) | ((uint32_
 constexpr int WQ = 4;       // work queue entries (at most two outstanding)
 constexpr int WQ_END = 255;
 
-// The coefficients of the next launch for either branch (index bit 0: sigma <
-// 0) and either storage (bit 1: re-centred), and the accelerated layer's new
-// bounds, prepared while the layer's products run: FP64 costs 64 cycles a step
-// here and would otherwise stand in the chain of every layer.
-struct Prepared {
-  LayerCoef k[4];
-  float ca[4], cb[4];
-  double l, h;
-  int sign;
-  // the loop's decision on (tr Y, ||Y||_F^2): N alpha, N alpha^2, N alpha (1 -
-  // alpha), 2 alpha, 1 - 2 alpha, N_occ, sigma eps, the re-centring and 4.5-rule thresholds
-  int rule45;
-  double na, naa, na1, ta, oa, no, se, rc, r45;
-};
-
-struct PreparedCoef {
-  const Prepared* p;
-  __device__ __forceinline__ void put(Ctl* c, int i, bool final_layer) const {
-    set_next(c, p->k[i], p->ca[i], p->cb[i], final_layer);
-  }
-  __device__ __forceinline__ void branch(Ctl* c, int sigma, bool final_layer) const {
-    put(c, (sigma < 0 ? 1 : 0) + (c->recentered ? 2 : 0), final_layer);
-  }
-  __device__ __forceinline__ int accel(Ctl*, double& l, double& h, LayerCoef&) const {
-    l = p->l;
-    h = p->h;
-    return p->sign;
-  }
-  __device__ __forceinline__ void next(Ctl* c, const LayerCoef&, bool final_layer) const {
-    put(c, c->recentered ? 2 : 0, final_layer);
-  }
-};
-
 struct Slot {
   int b, I, J, N;        // instance, tile row and column (128 units), size
   int par, first;        // parity of the operand planes; first layer
   int closed;            // no more work in this slot
   int pad;
-  int sg[4];
-  double ie[4];
-  double hot[kCtlHotBytes / 8];  // the control block without its history
-  Prepared prep;
+  SolveState st;
 };
-static_assert(kCtlHotBytes % 8 == 0, "the hot part is copied in 8-byte words");
 
 struct Shared {
   uint64_t full[STAGES_PLAIN], empty[STAGES_PLAIN];
@@ -120,8 +84,6 @@ struct Shared {
   double red_e[2][EPI_WARPS];                          // Tr[D H] (last layer)
   Slot slot[2];
 };
-
-__device__ __forceinline__ Ctl* hot_ctl(Slot& s) { return reinterpret_cast<Ctl*>(s.hot); }
 
 // Loads one 128-row operand of K block k0: K-major, or the stored block left
 // of the diagonal transposed (two 64 x 64 boxes).
@@ -151,12 +113,6 @@ __device__ __forceinline__ long long fix_sq(float v) {
   const int hi = __float2int_rz(v * 0x1p25f);
   const int lo = __float2int_rn(fmaf(-(float)hi, 0x1p-25f, v) * 0x1p53f);
   return ((long long)hi << 28) + (long long)lo;
-}
-
-__device__ __forceinline__ long long warp_sum_ll(long long v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
 }
 
 // Row norm (Y^2)_rr of the layer's input: FP64 ones of the input layer, or the
@@ -211,7 +167,7 @@ template <bool SPLIT>
 __device__ __forceinline__ bool epilogue(const ResArgs& a, Shared& sh, int c, uint32_t acc_phase, uint32_t tmem_base,
                                          int ew, int q, int lane, float* trb, unsigned long long lim) {
   const Slot& s = sh.slot[c];
-  const Ctl* ct = reinterpret_cast<const Ctl*>(s.hot);
+  const Ctl* ct = s.st.ctl();
   const int b = s.b, N = s.N, first = s.first;
   const int hc = ew >> 2;
   const int R0 = s.I * TB + q * 32;
@@ -445,28 +401,10 @@ __device__ __forceinline__ bool epilogue(const ResArgs& a, Shared& sh, int c, ui
   return true;
 }
 
-// Sum over the sixteen epilogue warps (lanes 0-15 hold their values).
-__device__ __forceinline__ long long sum16(long long v) {
-#pragma unroll
-  for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
 // The warp's worst mark (0: every lane's sum is a number).
 __device__ __forceinline__ long long worst_mark(long long v) {
   const bool nan = __any_sync(0xffffffffu, v == SQ_NAN), big = __any_sync(0xffffffffu, v == SQ_BIG);
   return nan ? SQ_NAN : big ? SQ_BIG : 0;
-}
-
-// A tile's sums of one layer as its gang sees them: the slot holds GANG_EMPTY
-// until the tile has published them, both words at once.
-__device__ __forceinline__ longlong2 ld_sums(const longlong2* p) {
-  longlong2 v;
-  asm volatile("ld.relaxed.gpu.global.v2.s64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ void st_sums(longlong2* p, long long x, long long y) {
-  asm volatile("st.relaxed.gpu.global.v2.s64 [%0], {%1, %2};" ::"l"(p), "l"(x), "l"(y) : "memory");
 }
 
 // Waits for the sums of all cnt tiles of the gang (slots p[0 .. cnt)) and adds
@@ -477,41 +415,13 @@ __device__ __forceinline__ bool meet(const ResArgs& a, Shared& sh, const longlon
                                      unsigned long long idle) {
   T = q_hi = q_lo = 0;
   bad = 0;
-  const uint64_t w0 = globaltimer();
-  for (int i0 = 0; i0 < cnt; i0 += 128) {
-    longlong2 v[4];
-    bool have[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int i = i0 + 32 * u + lane;
-      have[u] = i >= cnt;
-      if (!have[u]) v[u] = ld_sums(p + i);
-    }
-    for (int spin = 0;; ++spin) {
-      bool all = true;
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        if (have[u]) continue;
-        if (v[u].x != kGangEmpty && v[u].y != kGangEmpty) {
-          have[u] = true;
-          T += v[u].x;
-          q_hi += v[u].y >> 28;
-          q_lo += v[u].y & ((1ll << 28) - 1);
-          if (v[u].y < 0) bad = bad == SQ_NAN ? bad : v[u].y;
-        } else {
-          all = false;
-          v[u] = ld_sums(p + i0 + 32 * u + lane);
-        }
-      }
-      if (__all_sync(0xffffffffu, all)) break;
-      if ((spin & 31) == 31) {
-        const bool stop = *(volatile int*)&sh.abort || *(volatile int*)a.err != 0 || globaltimer() - w0 > idle;
-        if (__any_sync(0xffffffffu, stop)) return false;
-      }
-    }
-  }
-  __threadfence();  // the gang's planes and row norms, with its sums
-  __syncwarp();
+  if (!gather(p, cnt, lane, a.err, &sh.abort, idle, [&](const longlong2& v) {
+        T += v.x;
+        q_hi += v.y >> 28;
+        q_lo += v.y & ((1ll << 28) - 1);
+        if (v.y < 0) bad = bad == SQ_NAN ? bad : v.y;
+      }))
+    return false;
   if (lane == 0 && ready) mbar_arrive(ready);
   T = warp_sum_ll(T);
   q_hi = warp_sum_ll(q_hi);
@@ -520,92 +430,10 @@ __device__ __forceinline__ bool meet(const ResArgs& a, Shared& sh, const longlon
   return true;
 }
 
-// What the next control step can be given beforehand: the candidates (lanes
-// 0-3) and the constants of the loop's decision (lane 4).
-__device__ __forceinline__ void prepare(Slot& s, int lane) {
-  if (lane == 4) {
-    const Ctl* c = hot_ctl(s);
-    const double a = c->alpha_next, N = (double)c->N;
-    const RingHistory hist{s.sg, s.ie, nullptr};
-    const int n1 = c->n + 1;
-    s.prep.na = N * a;
-    s.prep.naa = N * a * a;
-    s.prep.na1 = N * a * (1.0 - a);
-    s.prep.ta = 2.0 * a;
-    s.prep.oa = 1.0 - 2.0 * a;
-    s.prep.no = (double)c->n_occ;
-    s.prep.se = (double)hist.sigma(c->n) * c->eps;
-    s.prep.rc = kRecenterFrac * N;
-    s.prep.rule45 = n1 > 2 && hist.sigma(n1 - 1) != hist.sigma(n1 - 2);
-    s.prep.r45 = n1 > 2 ? 4.5 * hist.iderr(n1 - 2) * hist.iderr(n1 - 2) : 0.0;
-  }
-  if (lane < 4) {
-    const Ctl* c = hot_ctl(s);
-    const bool rec = (lane & 2) != 0;
-    LayerCoef k;
-    if (c->accel) {
-      double l = c->acc_l, h = c->acc_h, pa, pb, pc;
-      const int sg = accel_layer(l, h, pa, pb, pc);
-      k = poly_coef(c->alpha_next, pa, pb, pc, rec, c->shift);
-      if (lane == 0) {
-        s.prep.l = l;
-        s.prep.h = h;
-        s.prep.sign = sg;
-      }
-    } else {
-      k = branch_coef(c->alpha_next, (lane & 1) ? -1 : 1, rec);
-    }
-    s.prep.k[lane] = k;
-    s.prep.ca[lane] = (float)k.ca;
-    s.prep.cb[lane] = (float)k.cb;
-  }
-  __syncwarp();
-}
-
-// The control step of the resident solve: control_step's decision of the loop
-// with everything that does not depend on the sums taken from Prepared and the
-// comparisons side by side (a chain of seven FP64 operations instead of some
-// twenty); the other phases as they are.
-__device__ __forceinline__ void resident_step(Slot& s, double trY, double sqY, RingHistory hist) {
-  Ctl* c = hot_ctl(s);
-  const Prepared& p = s.prep;
-  if (c->phase != PHASE_LOOP || c->stop_pending || c->accel) {
-    control_step(c, trY, sqY, hist, PreparedCoef{&p});
-    return;
-  }
-  const int n1 = c->n + 1, max_iter = c->max_iter, rule45 = p.rule45;
-  const double tol = c->tol, no = p.no;
-  const double NX = fma(p.ta, trY, p.naa) + sqY;             // Tr[S_n^2] = ||S_n||_F^2
-  const double NS2 = fma(2.0, trY, 2.0 * p.na - no);         // 2 Tr[S_n] - N_occ
-  const double err = fma(p.oa, trY, p.na1) - sqY;            // N_S - N_X
-  const double v = fabs(NS2 - NX) - fabs(NX - no) - p.se;
-  const bool center = err <= p.rc, low = err <= tol, zero = err <= 0.0, r45 = err > p.r45;
-  const int sg = (v >= 0.0) ? 1 : -1;
-  const int recentered = (c->recentered || (c->shift && center)) ? 1 : 0;
-  int stop = SP2_STOP_NONE;
-  if (tol > 0.0 && low)
-    stop = SP2_STOP_TOL;
-  else if (zero)
-    stop = SP2_STOP_IDERR;
-  else if (rule45 && r45)
-    stop = SP2_STOP_RULE45;
-  else if (n1 >= max_iter)
-    stop = SP2_STOP_MAXITER;
-  c->trY = trY;
-  c->sqY = sqY;
-  c->alpha = c->alpha_next;
-  c->recentered = recentered;
-  c->n = n1;
-  c->stop_pending = stop;
-  if (stop) c->converged_by = stop;
-  PreparedCoef{&p}.branch(c, sg, false);
-  hist.set(n1, sg, err);
-}
-
 // Control of one slot: takes the tiles of its list and drives their layers.
 __device__ __forceinline__ void control(const ResArgs& a, Shared& sh, int c, int lane, unsigned long long idle) {
   Slot& s = sh.slot[c];
-  Ctl* hot = hot_ctl(s);
+  Ctl* hot = s.st.ctl();
   const int sl = c * (int)gridDim.x + (int)blockIdx.x;
   uint32_t done_phase = 0;
   bool ok = true;
@@ -614,18 +442,7 @@ __device__ __forceinline__ void control(const ResArgs& a, Shared& sh, int c, int
     int b, I, J, h;
     unpack_tile(a.tiles[t], b, I, J, h);
     const Ctl* gc = a.ctl + b;
-    // the control block as the input layer's control step left it
-    const double* src = reinterpret_cast<const double*>(gc);
-    for (int i = lane; i < (int)(kCtlHotBytes / 8); i += 32) s.hot[i] = __ldcg(src + i);
-    __syncwarp();
-    const int n0 = hot->n;
-    if (lane < 4) {
-      const int n = n0 - lane;
-      if (n >= 0) {
-        s.sg[n & 3] = gc->sigma[n];
-        s.ie[n & 3] = gc->iderr[n];
-      }
-    }
+    s.st.load(gc, lane);  // as the input layer's control step left it
     const int cnt = a.tile_cnt[b], off = a.tile_off[b];
     const bool leader = t == off;
     const bool twice = (I >> 1) != (J >> 1);  // the mirror's squares
@@ -648,7 +465,7 @@ __device__ __forceinline__ void control(const ResArgs& a, Shared& sh, int c, int
     }
     __syncwarp();
     for (int k = 0; act; ++k) {
-      prepare(s, lane);
+      prepare(s.st, lane);
       if (!__all_sync(0xffffffffu, mbar_wait(&sh.epi_done[c], done_phase, &sh.abort, idle))) {
         ok = false;
         break;
@@ -664,24 +481,22 @@ __device__ __forceinline__ void control(const ResArgs& a, Shared& sh, int c, int
       }
       const long long rq = lane < EPI_WARPS ? sh.red_q[c][lane] : 0;
       long long bad = worst_mark(rq);
-      long long T = sum16(lane < EPI_WARPS ? sh.red_t[c][lane] : 0);
-      long long Q = sum16(rq) << (twice ? 1 : 0);
+      long long T = warp_sum_ll(lane < EPI_WARPS ? sh.red_t[c][lane] : 0);
+      long long Q = warp_sum_ll(rq) << (twice ? 1 : 0);
       double E = 0.0;
       if (outD) E = warp_sum_d(lane < EPI_WARPS ? sh.red_e[c][lane] : 0.0);
       long long q_hi = Q >> 28, q_lo = Q & ((1ll << 28) - 1);
       if (cnt > 1) {
         if (lane == 0) {
           if (outD) a.tile_dots[t] = E;
-          __threadfence();  // the CTA's planes and row norms before its sums
-          st_sums(a.sums + (long long)(k % 3) * a.ntiles + t, T, bad ? bad : Q);
+          publish(a.sums, a.ntiles, k, t, T, bad ? bad : Q);
         }
         if (!meet(a, sh, a.sums + (long long)(k % 3) * a.ntiles + off, cnt, lane, outD ? nullptr : &sh.ready[c], T,
                   q_hi, q_lo, bad, idle)) {
           ok = false;
           break;
         }
-        // every tile has read the sums of the layer before: its slot is free for the layer after next
-        if (lane == 0) st_sums(a.sums + (long long)((k + 2) % 3) * a.ntiles + t, kGangEmpty, kGangEmpty);
+        if (lane == 0) empty_slot(a.sums, a.ntiles, k, t);
         if (outD && leader) {
           E = 0.0;
           for (int i = lane; i < cnt; i += 32) E += __ldcg(&a.tile_dots[off + i]);
@@ -692,7 +507,7 @@ __device__ __forceinline__ void control(const ResArgs& a, Shared& sh, int c, int
         const double off = __longlong_as_double(bad == SQ_NAN ? 0x7ff8000000000000ll : 0x7ff0000000000000ll);
         const double trY = bad == SQ_NAN ? off : (double)T * T_UNIT;
         const double sqY = bad ? off : (double)q_hi * Q_HI_UNIT + (double)q_lo * Q_LO_UNIT;
-        resident_step(s, trY, sqY, RingHistory{s.sg, s.ie, leader ? a.ctl + b : nullptr});
+        resident_step(s.st, trY, sqY, leader ? a.ctl + b : nullptr);
         if (!outD) mbar_arrive(&sh.coef[c]);
         if (leader) {
           if (outD) a.dots_out[3 * b] = E;
@@ -702,9 +517,7 @@ __device__ __forceinline__ void control(const ResArgs& a, Shared& sh, int c, int
       __syncwarp();
       act = hot->next.active != 0;
       if (!act && leader) {
-        // the final state for the host; the history was recorded layer by layer
-        double* dst = reinterpret_cast<double*>(a.ctl + b);
-        for (int i = lane; i < (int)(kCtlHotBytes / 8); i += 32) dst[i] = s.hot[i];
+        s.st.store(a.ctl + b, lane);
       }
     }
     __syncwarp();

@@ -1,0 +1,232 @@
+// What the resident solves share (csrc/resident.cu on the tensor cores,
+// csrc/resident_fp32.cu): the solve's state in shared memory, its control step
+// with everything prepared that can be, and the meeting of a gang.
+#pragma once
+
+#include "common.cuh"
+#include "kernels.h"
+#include "tc_ptx.cuh"
+
+namespace sp2 {
+namespace res {
+
+// The coefficients of the next launch for either branch (index bit 0: sigma <
+// 0) and either storage (bit 1: re-centred), and the accelerated layer's new
+// bounds, prepared while the layer's products run: FP64 costs 64 cycles a step
+// here and would otherwise stand in the chain of every layer.
+struct Prepared {
+  LayerCoef k[4];
+  float ca[4], cb[4];
+  double l, h;
+  int sign;
+  // the loop's decision on (tr Y, ||Y||_F^2): N alpha, N alpha^2, N alpha (1 -
+  // alpha), 2 alpha, 1 - 2 alpha, N_occ, sigma eps, the re-centring and 4.5-rule thresholds
+  int rule45;
+  double na, naa, na1, ta, oa, no, se, rc, r45;
+};
+
+struct PreparedCoef {
+  const Prepared* p;
+  __device__ __forceinline__ void put(Ctl* c, int i, bool final_layer) const {
+    set_next(c, p->k[i], p->ca[i], p->cb[i], final_layer);
+  }
+  __device__ __forceinline__ void branch(Ctl* c, int sigma, bool final_layer) const {
+    put(c, (sigma < 0 ? 1 : 0) + (c->recentered ? 2 : 0), final_layer);
+  }
+  __device__ __forceinline__ int accel(Ctl*, double& l, double& h, LayerCoef&) const {
+    l = p->l;
+    h = p->h;
+    return p->sign;
+  }
+  __device__ __forceinline__ void next(Ctl* c, const LayerCoef&, bool final_layer) const {
+    put(c, c->recentered ? 2 : 0, final_layer);
+  }
+};
+
+// A solve's control block without its history, the history's last four layers
+// and the prepared step, in shared memory.
+struct SolveState {
+  int sg[4];
+  double ie[4];
+  double hot[kCtlHotBytes / 8];
+  Prepared prep;
+  __device__ __forceinline__ Ctl* ctl() { return reinterpret_cast<Ctl*>(hot); }
+  __device__ __forceinline__ const Ctl* ctl() const { return reinterpret_cast<const Ctl*>(hot); }
+  // by one warp
+  __device__ __forceinline__ void load(const Ctl* gc, int lane) {
+    const double* src = reinterpret_cast<const double*>(gc);
+    for (int i = lane; i < (int)(kCtlHotBytes / 8); i += 32) hot[i] = __ldcg(src + i);
+    __syncwarp();
+    const int n = ctl()->n - lane;
+    if (lane < 4 && n >= 0) {
+      sg[n & 3] = gc->sigma[n];
+      ie[n & 3] = gc->iderr[n];
+    }
+    __syncwarp();
+  }
+  // the final state for the host (the history was recorded layer by layer)
+  __device__ __forceinline__ void store(Ctl* gc, int lane) const {
+    double* dst = reinterpret_cast<double*>(gc);
+    for (int i = lane; i < (int)(kCtlHotBytes / 8); i += 32) dst[i] = hot[i];
+  }
+};
+static_assert(kCtlHotBytes % 8 == 0, "the hot part is copied in 8-byte words");
+
+// What the next control step can be given beforehand: the candidates (lanes
+// 0-3) and the constants of the loop's decision (lane 4).
+__device__ __forceinline__ void prepare(SolveState& s, int lane) {
+  if (lane == 4) {
+    const Ctl* c = s.ctl();
+    const double a = c->alpha_next, N = (double)c->N;
+    const RingHistory hist{s.sg, s.ie, nullptr};
+    const int n1 = c->n + 1;
+    s.prep.na = N * a;
+    s.prep.naa = N * a * a;
+    s.prep.na1 = N * a * (1.0 - a);
+    s.prep.ta = 2.0 * a;
+    s.prep.oa = 1.0 - 2.0 * a;
+    s.prep.no = (double)c->n_occ;
+    s.prep.se = (double)hist.sigma(c->n) * c->eps;
+    s.prep.rc = kRecenterFrac * N;
+    s.prep.rule45 = n1 > 2 && hist.sigma(n1 - 1) != hist.sigma(n1 - 2);
+    s.prep.r45 = n1 > 2 ? 4.5 * hist.iderr(n1 - 2) * hist.iderr(n1 - 2) : 0.0;
+  }
+  if (lane < 4) {
+    const Ctl* c = s.ctl();
+    const bool rec = (lane & 2) != 0;
+    LayerCoef k;
+    if (c->accel) {
+      double l = c->acc_l, h = c->acc_h, pa, pb, pc;
+      const int sg = accel_layer(l, h, pa, pb, pc);
+      k = poly_coef(c->alpha_next, pa, pb, pc, rec, c->shift);
+      if (lane == 0) {
+        s.prep.l = l;
+        s.prep.h = h;
+        s.prep.sign = sg;
+      }
+    } else {
+      k = branch_coef(c->alpha_next, (lane & 1) ? -1 : 1, rec);
+    }
+    s.prep.k[lane] = k;
+    s.prep.ca[lane] = (float)k.ca;
+    s.prep.cb[lane] = (float)k.cb;
+  }
+  __syncwarp();
+}
+
+// The control step of the resident solve: control_step's decision of the loop
+// with everything that does not depend on the sums taken from Prepared and the
+// comparisons side by side (a chain of seven FP64 operations instead of some
+// twenty); the other phases as they are.
+__device__ __forceinline__ void resident_step(SolveState& s, double trY, double sqY, Ctl* record) {
+  Ctl* c = s.ctl();
+  RingHistory hist{s.sg, s.ie, record};
+  const Prepared& p = s.prep;
+  if (c->phase != PHASE_LOOP || c->stop_pending || c->accel) {
+    control_step(c, trY, sqY, hist, PreparedCoef{&p});
+    return;
+  }
+  const int n1 = c->n + 1, max_iter = c->max_iter, rule45 = p.rule45;
+  const double tol = c->tol, no = p.no;
+  const double NX = fma(p.ta, trY, p.naa) + sqY;             // Tr[S_n^2] = ||S_n||_F^2
+  const double NS2 = fma(2.0, trY, 2.0 * p.na - no);         // 2 Tr[S_n] - N_occ
+  const double err = fma(p.oa, trY, p.na1) - sqY;            // N_S - N_X
+  const double v = fabs(NS2 - NX) - fabs(NX - no) - p.se;
+  const bool center = err <= p.rc, low = err <= tol, zero = err <= 0.0, r45 = err > p.r45;
+  const int sg = (v >= 0.0) ? 1 : -1;
+  const int recentered = (c->recentered || (c->shift && center)) ? 1 : 0;
+  int stop = SP2_STOP_NONE;
+  if (tol > 0.0 && low)
+    stop = SP2_STOP_TOL;
+  else if (zero)
+    stop = SP2_STOP_IDERR;
+  else if (rule45 && r45)
+    stop = SP2_STOP_RULE45;
+  else if (n1 >= max_iter)
+    stop = SP2_STOP_MAXITER;
+  c->trY = trY;
+  c->sqY = sqY;
+  c->alpha = c->alpha_next;
+  c->recentered = recentered;
+  c->n = n1;
+  c->stop_pending = stop;
+  if (stop) c->converged_by = stop;
+  PreparedCoef{&p}.branch(c, sg, false);
+  hist.set(n1, sg, err);
+}
+
+__device__ __forceinline__ long long warp_sum_ll(long long v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// The meeting of a gang after a layer: each member publishes two words in its
+// slot of the gang's row and waits until every slot of the row is written.
+// Three rows serve successive layers: once a member has met for layer k, every
+// member has read the row of layer k - 1, so it empties its slot there, which
+// the row of layer k + 2 reuses.  (A row per reader, written by all, measured
+// 2 % faster at 144 members and 3 % slower on 512 small gangs.)
+__device__ __forceinline__ longlong2 ld_sums(const longlong2* p) {
+  longlong2 v;
+  asm volatile("ld.relaxed.gpu.global.v2.s64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_sums(longlong2* p, long long x, long long y) {
+  asm volatile("st.relaxed.gpu.global.v2.s64 [%0], {%1, %2};" ::"l"(p), "l"(x), "l"(y) : "memory");
+}
+
+// Member `me` publishes (x, y) in layer k's row of rows[3][stride], with
+// everything the CTA has written before (lane 0 of one warp).
+__device__ __forceinline__ void publish(longlong2* rows, long long stride, int k, int me, long long x, long long y) {
+  __threadfence();
+  st_sums(rows + (k % 3) * stride + me, x, y);
+}
+// after the meeting of layer k
+__device__ __forceinline__ void empty_slot(longlong2* rows, long long stride, int k, int me) {
+  st_sums(rows + ((k + 2) % 3) * stride + me, kGangEmpty, kGangEmpty);
+}
+
+// Waits until every slot p[0 .. cnt) is written and hands each to add (one
+// warp; lane l takes slots l, l + 32, ...).  False: abort or time-out.
+template <class Add>
+__device__ __forceinline__ bool gather(const longlong2* p, int cnt, int lane, const int* err,
+                                       const volatile int* abort_flag, unsigned long long limit, Add add) {
+  const uint64_t w0 = sp2::tc::globaltimer();
+  for (int i0 = 0; i0 < cnt; i0 += 128) {
+    longlong2 v[4];
+    bool have[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int i = i0 + 32 * u + lane;
+      have[u] = i >= cnt;
+      if (!have[u]) v[u] = ld_sums(p + i);
+    }
+    for (int spin = 0;; ++spin) {
+      bool all = true;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        if (have[u]) continue;
+        if (v[u].x != kGangEmpty && v[u].y != kGangEmpty) {
+          have[u] = true;
+          add(v[u]);
+        } else {
+          all = false;
+          v[u] = ld_sums(p + i0 + 32 * u + lane);
+        }
+      }
+      if (__all_sync(0xffffffffu, all)) break;
+      if ((spin & 31) == 31) {
+        const bool stop =
+            *abort_flag || *(const volatile int*)err != 0 || sp2::tc::globaltimer() - w0 > limit;
+        if (__any_sync(0xffffffffu, stop)) return false;
+      }
+    }
+  }
+  __threadfence();  // what the gang wrote before its sums
+  __syncwarp();
+  return true;
+}
+
+}  // namespace res
+}  // namespace sp2
