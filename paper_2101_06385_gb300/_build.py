@@ -15,8 +15,8 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libsp2.so")
-SOURCES = ["api.cu", "prep.cu", "syrk_simt.cu", "syrk_tc.cu", "syrk_tc1.cu", "syrk_tc2.cu", "resident.cu", "resident_fp32.cu", "noalloc.cu"]
-HEADERS = ["common.cuh", "kernels.h", "tile_finish.cuh", "tc_ptx.cuh", "epilogue.cuh", "resident.cuh"]
+SOURCES = ["api.cu", "prep.cu", "syrk_simt.cu", "syrk_tc.cu", "syrk_tc1.cu", "syrk_tc2.cu", "resident.cu", "resident_fp32.cu", "resident_net.cu", "noalloc.cu"]
+HEADERS = ["common.cuh", "kernels.h", "tile_finish.cuh", "tc_ptx.cuh", "epilogue.cuh", "resident.cuh", "resident_tc.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ARCH + ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",
                 "-Xcompiler", "-Wno-deprecated-declarations"]

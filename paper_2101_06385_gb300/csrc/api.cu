@@ -63,7 +63,7 @@ enum BufId {
   B_HI0, B_LO0, B_HI1, B_LO1, B_Y0, B_Y1, B_CTL, B_TILES, B_TOFF, B_TCNT, B_TPART, B_IDONE,
   B_PART, B_TICKET, B_ERR, B_DPTR, B_NS, B_HS, B_TRACES, B_PARAMS, B_BOUNDS, B_RN, B_PART2,
   B_G, B_SEG, B_GH0, B_GL0, B_GH1, B_GL1, B_DOTS, B_TDOTS, B_PARAMS2, B_NALPHA, B_HP0, B_HP1, B_RNP0, B_RNP1,
-  B_READOUT, B_RDIAG, B_SEGP, B_WAVE, B_PACK, B_COUNT
+  B_READOUT, B_RDIAG, B_SEGP, B_WAVE, B_PACK, B_PLANES0, B_PLANES1, B_COUNT
 };
 
 struct Buf {
@@ -1833,6 +1833,311 @@ sp2_status network_prologue(const float* H, int B, int N, int L, const float* co
 }
 }  // namespace
 
+namespace {
+
+// The resident network kernel takes matrices up to n_many in any number and
+// larger ones while the batch's tiles fit the slots.  The launches' CTA pairs
+// cannot fill the chip with few matrices and pay for the padding of small ones
+// (forward, 8 layers: two of N = 2048 502 against 641 us, 300 of 256 1.02
+// against 1.22 ms; backward 1.27 against 1.48 and 2.3 against 2.9 ms); on many
+// large ones their 256 x 256 tiles are faster (32 of 2048: 6.3 against 5.9 and
+// 17.2 against 14.4 ms).  n_many: 1024 forward (30 of them 1.23 against 1.32
+// ms), 512 backward (30 of 1024 3.1 against 2.9 ms).
+bool net_fits(int B, int N, int n_many) {
+  if (!resident_fits(N)) return false;
+  int n = 0;
+  resident_tiles(N, 0, nullptr, &n);
+  return N <= n_many || (long long)n * B <= 2 * g.num_sms;
+}
+
+// A run of the resident network kernel (csrc/resident_net.cu) over B matrices
+// of size N: the plan of its tiles, the pool of plane pairs, the operations.
+// The host fills ops, params and the FP64 tables, then go() uploads and runs.
+struct NetRun {
+  int B, N, per = 0, nt = 0, grid = 0, pool = 0;
+  NetArgs A;
+  NetMaps maps;
+  std::vector<NetOp> ops;
+  std::vector<LayerParams> params;
+  std::vector<double> table;      // FP64 values the operations point into (by index until go())
+  uint8_t* pack = nullptr;        // [ops][params][table][lists][tiles][err]
+  size_t o_params = 0, o_table = 0, o_loff = 0, o_list = 0, o_tiles = 0, o_err = 0, bytes = 0;
+
+  sp2_status init(int B_, int N_, int pool_, bool split, const Ctl* ctl, int nops, size_t nparams, size_t ntable) {
+    B = B_;
+    N = N_;
+    pool = pool_;
+    memset(&A, 0, sizeof(A));
+    resident_tiles(N, 0, nullptr, &per);
+    nt = per * B;
+    grid = std::min(nt, g.num_sms);
+    const long long ld_h = round_up(N, 64), slot_h = ld_h * N;
+    void *p0, *p1 = nullptr, *sums;
+    CKS(ws(B_PLANES0, (size_t)slot_h * B * pool * 2, &p0));
+    if (split) CKS(ws(B_PLANES1, (size_t)slot_h * B * pool * 2, &p1));
+    CKS(ws(B_TPART, (size_t)3 * nt * sizeof(longlong2), &sums));
+    SqArgs carry;
+    void* rnp[2];
+    CKS(rnp_for(N, B, carry, rnp));
+    size_t o = 0;
+    auto take = [&](size_t n) {
+      const size_t at = o;
+      o = (o + n + 15) / 16 * 16;
+      return at;
+    };
+    take(nops * sizeof(NetOp));
+    o_params = take(nparams * sizeof(LayerParams));
+    o_table = take(ntable * sizeof(double));
+    o_loff = take((size_t)(2 * grid + 1) * sizeof(int));
+    o_list = take((size_t)nt * sizeof(int));
+    o_tiles = take((size_t)nt * sizeof(uint32_t));
+    o_err = take(sizeof(int));
+    bytes = o;
+    void* pk;
+    CKS(ws(B_PACK, bytes, &pk));
+    pack = (uint8_t*)pk;
+    A.N = N;
+    A.batch = B;
+    A.per = per;
+    A.ntiles = nt;
+    A.ops = (const NetOp*)pack;
+    A.lp = (const LayerParams*)(pack + o_params);
+    A.ctl = ctl;
+    A.p0 = (__half*)p0;
+    A.p1 = (__half*)p1;
+    A.ld_h = ld_h;
+    A.slot_h = slot_h;
+    A.rnp[0] = (float*)rnp[0];
+    A.rnp[1] = (float*)rnp[1];
+    A.ld_rnp = carry.ld_rnp;
+    A.slot_rnp = carry.slot_rnp;
+    A.tiles = (const uint32_t*)(pack + o_tiles);
+    A.list_off = (const int*)(pack + o_loff);
+    A.list = (const int*)(pack + o_list);
+    A.sums = (longlong2*)sums;
+    A.lo_scale = std::ldexp(1.0f, g.lo_scale_exp);
+    A.lo_unscale = std::ldexp(1.0f, -g.lo_scale_exp);
+    A.shift = g.shift;
+    A.two_slots = nt > grid ? 1 : 0;
+    A.err = (int*)(pack + o_err);
+    A.wait_ns = g.wait_ns;
+    CUtensorMap m[6];
+    CKS(tmaps4_for(p0, p1, N, B * pool, ld_h, slot_h, m, kTcBM));
+    maps.m[0] = m[0];
+    maps.m[1] = m[1];
+    maps.m[2] = m[4];
+    maps.m[3] = m[5];
+    return SP2_OK;
+  }
+  const double* dev(size_t table_index) const { return (const double*)(pack + o_table) + table_index; }
+
+  // the records, in one upload
+  sp2_status upload() {
+    A.nops = (int)ops.size();
+    void* h;
+    CKS(staging(bytes, &h));
+    uint8_t* hb = (uint8_t*)h;
+    memcpy(hb, ops.data(), ops.size() * sizeof(NetOp));
+    memcpy(hb + o_params, params.data(), params.size() * sizeof(LayerParams));
+    memcpy(hb + o_table, table.data(), table.size() * sizeof(double));
+    std::vector<int> order(B), Ns(B, N), toff(B), tcnt(B, per);
+    std::vector<uint32_t> tiles;
+    for (int b = 0; b < B; ++b) {
+      order[b] = b;
+      toff[b] = b * per;
+      int n;
+      resident_tiles(N, b, &tiles, &n);
+    }
+    resident_plan(order.data(), Ns.data(), toff.data(), tcnt.data(), B, grid, (int*)(hb + o_loff), (int*)(hb + o_list));
+    memcpy(hb + o_tiles, tiles.data(), nt * sizeof(uint32_t));
+    *(int*)(hb + o_err) = 0;
+    CK(cudaMemcpyAsync(pack, hb, bytes, cudaMemcpyHostToDevice, g.stream));
+    CK(cudaEventRecord(g.stage_done, g.stream));
+    CK(cudaMemsetAsync(A.sums, kGangEmptyByte, (size_t)3 * nt * sizeof(longlong2), g.stream));
+    return SP2_OK;
+  }
+  // inputs of one kind into the plane pairs from pool entry `entry` on
+  NetInput input(int from, const float* in, int entry) const {
+    NetInput x;
+    memset(&x, 0, sizeof(x));
+    x.N = N;
+    x.batch = B;
+    x.from = from;
+    x.shift = g.shift;
+    x.in = in;
+    x.ctl = A.ctl;
+    x.p0 = A.p0 + (long long)entry * B * A.slot_h;
+    x.p1 = A.p1 ? A.p1 + (long long)entry * B * A.slot_h : nullptr;
+    x.ld_h = A.ld_h;
+    x.slot_h = A.slot_h;
+    x.lo_scale = A.lo_scale;
+    return x;
+  }
+};
+
+NetOp net_square(int y, int out, int layer, int rnp) {
+  NetOp o;
+  memset(&o, 0, sizeof(o));
+  o.y = y;
+  o.out = out;
+  o.layer = layer;
+  o.rnp = rnp;
+  return o;
+}
+
+// The network's forward pass on the resident kernel (net_fits).
+sp2_status net_forward_resident(const float* H, int B, int N, int L, const NetPlan& plan, const Ctl* ctl, int ckpt_every,
+                                float* X_out, float* ckpt) {
+  const bool split = g.precision == SP2_PREC_SPLIT_FP16;
+  const size_t mats = (size_t)B * N * N;
+  NetRun R;
+  void* rn;
+  CKS(ws(B_RN, (size_t)B * N * sizeof(double), &rn));
+  CKS(R.init(B, N, 2, split, ctl, L, plan.params.size(), plan.alpha.size()));
+  R.params = plan.params;
+  R.table = plan.alpha;
+  for (int n = 0; n < L; ++n) {
+    const bool last = n == L - 1, kept = ckpt && (n + 1) % ckpt_every == 0;
+    NetOp o = net_square(n & 1, last ? -1 : (n & 1) ^ 1, n, n & 1);
+    o.from = n == 0 ? NET_INPUT : NET_TMEM;
+    o.in = H;
+    o.rn = n == 0 ? (const double*)rn : nullptr;
+    o.tmem = last ? 0 : 1;
+    float* slot = kept ? ckpt + (size_t)((n + 1) / ckpt_every) * mats : nullptr;
+    if (last) {
+      o.full = X_out;
+      o.exact = 1;
+      o.full2 = slot;
+    } else if (kept) {
+      o.full = slot;
+      o.full_add = R.dev((size_t)(n + 1) * B);
+    }
+    R.ops.push_back(o);
+  }
+  CKS(R.upload());
+  NetInput x = R.input(NET_INPUT, H, 0);
+  x.vec_norm = (N & 3) == 0 && ((uintptr_t)X_out & 15) == 0;
+  x.rn = (double*)rn;
+  x.x0 = ckpt;
+  x.alpha0 = R.dev(0);
+  CK(launch_net_input(x, B, g.stream));
+  CK(launch_resident_net(R.A, R.maps, split, R.grid, g.stream));
+  return SP2_OK;
+}
+
+// The network's adjoint on the resident kernel: per checkpoint segment, from
+// the last one, the recomputation of its iterates and the adjoint layers.
+// dots: host [L][B][3].
+sp2_status net_backward_resident(int B, int N, int L, const NetPlan& plan, const std::vector<LayerParams>& bp,
+                                 const Ctl* ctl, int ce, const float* ckpt, const float* G_out, float* G_in,
+                                 const double** dots_host) {
+  const bool split = g.precision == SP2_PREC_SPLIT_FP16;
+  cudaStream_t st = g.stream;
+  const size_t mats = (size_t)B * N * N;
+  const int nseg = (L + ce - 1) / ce;
+  // pool: the segments' first iterates, the others of a segment, G twice
+  const int p_rec = nseg, p_g = nseg + std::min(ce, L) - 1;
+  NetRun R;
+  void *rn, *keep, *tdots, *dots;
+  CKS(ws(B_RN, (size_t)nseg * B * N * sizeof(double), &rn));
+  CKS(R.init(B, N, p_g + 2, split, ctl, 2 * L, 2 * plan.params.size(), plan.alpha.size()));
+  const size_t tile_store = (size_t)R.nt * kResTile * kResTile;
+  CKS(ws(B_SEG, tile_store * 4 * std::max(1, std::min(ce, L) - 1), &keep));
+  CKS(ws(B_TDOTS, (size_t)L * R.nt * 3 * sizeof(double), &tdots));
+  CKS(ws(B_DOTS, (size_t)L * B * 3 * sizeof(double) + 16, &dots));
+  R.A.tile_dots = (double*)tdots;
+  R.params = plan.params;
+  R.params.insert(R.params.end(), bp.begin(), bp.end());
+  R.table.resize(plan.alpha.size());
+  for (size_t i = 0; i < R.table.size(); ++i) R.table[i] = -plan.alpha[i];
+  auto store = [&](int k) { return (float*)keep + tile_store * (size_t)(k - 1); };  // iterate n0 + k, k >= 1
+  int gcur = 0;
+  bool first = true;
+  for (int s = nseg - 1; s >= 0; --s) {
+    const int n0 = s * ce, n1 = std::min(n0 + ce, L);
+    auto planes = [&](int k) { return k == 0 ? s : p_rec + k - 1; };
+    const float* X0 = ckpt + (size_t)s * mats;
+    for (int n = n0; n + 1 < n1; ++n) {
+      const int k = n - n0;
+      NetOp o = net_square(planes(k), planes(k + 1), n, k & 1);
+      if (k == 0) {
+        o.from = NET_X;
+        o.in = X0;
+        o.add = R.dev((size_t)n0 * B);
+        o.rn = (const double*)rn + (size_t)s * B * N;
+      } else {
+        o.from = NET_KEPT;
+        o.in = store(k);
+      }
+      o.keep = store(k + 1);
+      R.ops.push_back(o);
+    }
+    for (int n = n1 - 1; n >= n0; --n) {
+      const int k = n - n0;
+      NetOp o = net_square(planes(k), n == 0 ? -1 : p_g + (gcur ^ 1), L + n, 0);
+      o.kind = 1;
+      o.g = p_g + gcur;
+      o.dot = n;
+      o.from = first ? NET_FULL : NET_TMEM;
+      o.in = G_out;
+      o.tmem = n == 0 ? 0 : 1;
+      if (k == 0) {
+        o.aux_x = X0;
+        o.aux_add = R.dev((size_t)n0 * B);
+      } else {
+        o.aux = store(k);
+      }
+      if (n == 0) o.full = G_in;
+      R.ops.push_back(o);
+      first = false;
+      gcur ^= 1;
+    }
+  }
+  CKS(R.upload());
+  NetInput x = R.input(NET_X, ckpt, 0);
+  x.add = R.dev(0);
+  x.add_stride = (long long)ce * B;
+  x.vec_norm = (N & 3) == 0;
+  x.rn = (double*)rn;
+  CK(launch_net_input(x, nseg * B, st));
+  CK(launch_net_input(R.input(NET_FULL, G_out, p_g), B, st));
+  CK(launch_resident_net(R.A, R.maps, split, R.grid, st));
+  CK(launch_net_dots((const double*)tdots, R.nt, R.per, L, B, (double*)dots, st));
+  void* hd;
+  const size_t db = (size_t)L * B * 3 * sizeof(double);
+  CKS(staging(db + 16, &hd));
+  CK(cudaMemcpyAsync(hd, dots, db, cudaMemcpyDeviceToHost, st));
+  CK(cudaMemcpyAsync((char*)hd + db, R.A.err, sizeof(int), cudaMemcpyDeviceToHost, st));
+  CK(cudaStreamSynchronize(st));
+  if (*(const int*)((char*)hd + db)) {
+    set_err("a bounded device wait timed out");
+    return SP2_ERR_DEVICE_TIMEOUT;
+  }
+  *dots_host = (const double*)hd;
+  return SP2_OK;
+}
+
+// dcoef from the dot products [L][B][3] (tr G, <G, Y_n>, <Y_n G + G Y_n, Y_n>):
+// dL/da_n = <G, X_n^2> = alpha^2 tr G + 2 alpha <G, Y_n> + <Y_n G + G Y_n, Y_n> / 2
+// dL/db_n = <G, X_n>   = alpha tr G + <G, Y_n>;   dL/dc_n = tr G
+void coef_gradient(const double* dd, const NetPlan& plan, int L, int B, double* dcoef) {
+  for (int n = 0; n < L; ++n) {
+    double da = 0.0, db = 0.0, dc = 0.0;
+    for (int b = 0; b < B; ++b) {
+      const double al = plan.alpha[(size_t)n * B + b];
+      const double* v = dd + ((size_t)n * B + b) * 3;
+      da += al * al * v[0] + 2.0 * al * v[1] + 0.5 * v[2];
+      db += al * v[0] + v[1];
+      dc += v[0];
+    }
+    dcoef[3 * n] = da;
+    dcoef[3 * n + 1] = db;
+    dcoef[3 * n + 2] = dc;
+  }
+}
+
+}  // namespace
+
 sp2_status sp2_network_forward(const float* H, int B, int N, int L, const float* coef, int ckpt_every, float* X_out,
                                float* ckpt, double* bounds) {
   t_err.clear();
@@ -1857,6 +2162,8 @@ sp2_status sp2_network_forward(const float* H, int B, int N, int L, const float*
   if (bounds)
     CK(cudaMemcpy2DAsync(bounds, 2 * sizeof(double), (char*)ctl + offsetof(Ctl, e_min), sizeof(Ctl),
                          2 * sizeof(double), B, cudaMemcpyDeviceToDevice, st));
+  if (net_fits(B, N, 1024))
+    return net_forward_resident(H, B, N, L, plan, (const Ctl*)ctl, ckpt_every, X_out, ckpt);
   int ntiles = 0;
   // tensor-core layers on CTA pairs (super-tile pairs sharing B) unless
   // single CTAs are selected, as for the single solve
@@ -1995,12 +2302,14 @@ sp2_status sp2_network_backward(const float* H, int B, int N, int L, const float
   cudaStream_t st = g.stream;
   const long long slot = (long long)N * N;
   const int ce = ckpt_every;
-  void* G;
-  CKS(ws(B_G, (size_t)B * slot * 4, &G));
+  // (the planes of all segments' first iterates, as large as the checkpoints, within 32 GiB)
+  const bool resident = net_fits(B, N, 512) && (double)((L + ce - 1) / ce + ce + 1) * B * round_up(N, 64) * N * 4.0 < 0x1p35;
+  void* G = nullptr;
+  if (!resident) CKS(ws(B_G, (size_t)B * slot * 4, &G));
   bool ok = false;
   NetPlan plan;
   void *ctl, *ns, *hs, *dptr;
-  CKS(network_prologue(H, B, N, L, coef, &ok, plan, &ctl, &ns, &hs, &dptr, (float*)G));
+  CKS(network_prologue(H, B, N, L, coef, &ok, plan, &ctl, &ns, &hs, &dptr, G ? (float*)G : const_cast<float*>(G_out)));
 
   // backward coefficients: G_n = (2 a_n alpha_n + b_n) G + a_n (Y_n G + G Y_n)
   std::vector<LayerParams> bp((size_t)L * B);
@@ -2023,6 +2332,12 @@ sp2_status sp2_network_backward(const float* H, int B, int N, int L, const float
       plan.params[(size_t)n * B + b].out_mode = OUT_Y;
       plan.params[(size_t)n * B + b].alpha_out = 0.0;
     }
+  if (resident) {
+    const double* dd = nullptr;
+    CKS(net_backward_resident(B, N, L, plan, bp, (const Ctl*)ctl, ce, ckpt, G_out, G_in, &dd));
+    coef_gradient(dd, plan, L, B, dcoef);
+    return SP2_OK;
+  }
   // CTA pairs (M = 256 MMAs) unless the single-CTA kernel was selected; the
   // pair kernel keeps the operand planes as upper super tiles
   const bool pairs = g.pair_kernel;
@@ -2194,21 +2509,7 @@ sp2_status sp2_network_backward(const float* H, int B, int N, int L, const float
     set_err("a bounded device wait timed out");
     return SP2_ERR_DEVICE_TIMEOUT;
   }
-  // dL/da_n = <G, X_n^2> = alpha^2 tr G + 2 alpha <G, Y_n> + <Y_n G + G Y_n, Y_n> / 2
-  // dL/db_n = <G, X_n>   = alpha tr G + <G, Y_n>;   dL/dc_n = tr G
-  for (int n = 0; n < L; ++n) {
-    double da = 0.0, db = 0.0, dc = 0.0;
-    for (int b = 0; b < B; ++b) {
-      const double al = plan.alpha[(size_t)n * B + b];
-      const double* v = dd + ((size_t)n * B + b) * 3;
-      da += al * al * v[0] + 2.0 * al * v[1] + 0.5 * v[2];
-      db += al * v[0] + v[1];
-      dc += v[0];
-    }
-    dcoef[3 * n] = da;
-    dcoef[3 * n + 1] = db;
-    dcoef[3 * n + 2] = dc;
-  }
+  coef_gradient(dd, plan, L, B, dcoef);
   return SP2_OK;
 }
 
@@ -2331,6 +2632,38 @@ sp2_status sp2_fermi_expansion(const float* H, int B, int N, int L, const double
     }
   }
 
+  if (net_fits(B, N, 1024)) {
+    NetRun run;
+    void *rn, *R;
+    CKS(ws(B_RN, (size_t)B * N * sizeof(double), &rn));
+    CKS(run.init(B, N, 2, split, (const Ctl*)ctl, L, params.size(), d0.size()));
+    CKS(ws(B_READOUT, (size_t)run.nt * kResTile * kResTile * sizeof(float), &R));
+    run.params = params;
+    run.table = d0;
+    run.A.shift = 1;
+    run.A.R = (float*)R;
+    run.A.r_scale = (float)(-c[0]);
+    run.A.r_add = run.dev(0);
+    for (int n = 0; n < L; ++n) {
+      const bool last = n == L - 1;
+      NetOp o = net_square(n & 1, last ? -1 : (n & 1) ^ 1, n, n & 1);
+      o.from = n == 0 ? NET_INPUT : NET_TMEM;
+      o.in = H;
+      o.rn = n == 0 ? (const double*)rn : nullptr;
+      o.tmem = last ? 0 : 1;
+      o.readout = n == 0 ? 2 : 1;
+      o.full = last ? D_out : nullptr;
+      run.ops.push_back(o);
+    }
+    CKS(run.upload());
+    NetInput x = run.input(NET_INPUT, H, 0);
+    x.shift = 1;
+    x.vec_norm = (N & 3) == 0 && ((uintptr_t)D_out & 15) == 0;
+    x.rn = (double*)rn;
+    CK(launch_net_input(x, B, st));
+    CK(launch_resident_net(run.A, run.maps, split, run.grid, st));
+    return SP2_OK;
+  }
   int ntiles = 0;
   CKS(upload_tiles(N, B, 2, &ntiles));
   void *prm, *dd, *R, *rn;

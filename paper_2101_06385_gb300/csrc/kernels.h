@@ -188,6 +188,76 @@ struct ResArgs {
 cudaError_t launch_resident_input(const ResArgs& a, int vec_norm, int Nmax, int batch, cudaStream_t st);
 cudaError_t launch_resident(const ResArgs& a, const ResMaps& maps, bool split, int grid, cudaStream_t st);
 
+// Resident network layers (csrc/resident_net.cu).  One operation of every
+// tile; planes are pool entries of [pool][batch] plane pairs.
+enum NetFrom : int { NET_TMEM = 0, NET_INPUT = 1, NET_X = 2, NET_FULL = 3, NET_KEPT = 4 };
+struct NetOp {
+  int kind;                // 0: P = Y Y, 1: P = Y G + G Y (with dot products)
+  int y, g;                // pool entries of the planes of Y and G
+  int out;                 // pool entry written, or -1
+  int layer;               // coefficients lp[layer][batch]
+  int dot;                 // kind 1: layer of the dot products
+  int from;                // the old value: tensor memory, the input layer of `in`, a matrix `in` with add[b] on
+                           //   its diagonal, `in` as it is ([batch][N][N]), or `in` a tile-private store
+  int tmem;                // 1: the new value stays in tensor memory
+  int rnp;                 // segment sums: written at this parity, read at the other (or rn)
+  int exact;               // full's diagonal from the unrounded FP64 one plus the coefficients' alpha_out
+  int readout;             // 1: R += rc X', D = I - R into full; 2: R starts here as r_scale Y + r_add[b] I
+  const float* in;
+  const double* add;
+  const double* rn;        // [batch][N] FP64 row norms of the input, or nullptr
+  float* keep;             // tile-private store of the new value, or nullptr
+  const float* aux;        // kind 1: tile-private store of Y, or nullptr: the matrix aux_x with aux_add[b] on its diagonal
+  const float* aux_x;
+  const double* aux_add;
+  float* full;             // whole result matrices [batch][N][N], or nullptr
+  float* full2;            // a second copy
+  const double* full_add;  // [batch] added to full's diagonal, or nullptr
+};
+struct NetMaps {
+  CUtensorMap m[4];        // {p0, p1} with 64 x 128 boxes, {p0, p1} with 64 x 64 boxes; pool x batch slots
+};
+struct NetArgs {
+  int N, batch, nops, per, ntiles;  // per: tiles of a matrix
+  const NetOp* ops;
+  const LayerParams* lp;   // [layers][batch]
+  const Ctl* ctl;          // [batch] bounds (NET_INPUT)
+  __half* p0;
+  __half* p1;              // nullptr: plain FP16
+  long long ld_h, slot_h;
+  float* rnp[2];
+  long long ld_rnp, slot_rnp;
+  float* R;                // tile-private readout
+  float r_scale;
+  const double* r_add;     // [batch]
+  double* tile_dots;       // [layers][ntiles][3]
+  const uint32_t* tiles;
+  const int* list_off;     // as ResArgs
+  const int* list;
+  longlong2* sums;         // [3][ntiles] kGangEmpty: meeting rows
+  float lo_scale, lo_unscale;
+  int shift, two_slots;
+  int* err;
+  unsigned long long wait_ns;
+};
+struct NetInput {
+  int N, batch, from, shift, vec_norm;
+  const float* in;         // [count][N][N], matrix m of batch index m mod batch
+  const double* add;       // NET_X: add[m / batch * add_stride + m mod batch] on the diagonal
+  long long add_stride;
+  const Ctl* ctl;
+  __half* p0;              // plane pair m
+  __half* p1;
+  long long ld_h, slot_h;
+  double* rn;              // [count][N], or nullptr
+  float* x0;               // [count][N][N] Y_0 + alpha0 I, or nullptr
+  const double* alpha0;
+  float lo_scale;
+};
+cudaError_t launch_net_input(const NetInput& x, int count, cudaStream_t st);
+cudaError_t launch_net_dots(const double* tile_dots, int ntiles, int per, int L, int B, double* out, cudaStream_t st);
+cudaError_t launch_resident_net(const NetArgs& a, const NetMaps& maps, bool split, int grid, cudaStream_t st);
+
 // Resident FP32 solve (csrc/resident_fp32.cu): one instance, all layers in one
 // cooperative launch; Y_0, its row norms and the first control step are there.
 struct Res32Args {

@@ -35,31 +35,13 @@
 #include "epilogue.cuh"
 #include "kernels.h"
 #include "resident.cuh"
+#include "resident_tc.cuh"
 #include "tc_ptx.cuh"
 
 namespace sp2 {
 namespace res {
 
 using namespace sp2::tc;
-
-constexpr int TB = kResTile;                 // 128
-constexpr int HALF_BYTES = TB * BK * 2;      // 16 KB: one plane of one operand
-constexpr int T_BOX = 64 * 64 * 2;           // one 64 x 64 box of a transposed read
-constexpr int STAGE_SPLIT = 4 * HALF_BYTES;  // hpA loA hpB loB
-constexpr int STAGE_PLAIN = 2 * HALF_BYTES;  // hiA hiB
-constexpr int STAGES_SPLIT = 3;
-constexpr int STAGES_PLAIN = 6;
-constexpr int OPERAND_BYTES = STAGES_SPLIT * STAGE_SPLIT;
-static_assert(OPERAND_BYTES == STAGES_PLAIN * STAGE_PLAIN, "both precisions use the same shared memory");
-constexpr int EPI_WARPS = 16;               // one 32 x 32 chunk each
-constexpr int TR_BYTES = EPI_WARPS * 16 * 32 * 4;  // half a chunk per warp
-constexpr int CTL_WARP = 2 + EPI_WARPS;
-constexpr int THREADS = 32 * (CTL_WARP + 2);
-constexpr uint32_t TMEM_COLS = 512;  // two slots of an accumulator and an iterate
-constexpr uint32_t SLOT_COLS = 256, Y_COL = 128;
-constexpr uint32_t IDESC_T = (1u << 4) | ((uint32_t)(TB >> 3) << 17) | ((uint32_t)(TB >> 4) << 24);
-constexpr int WQ = 4;       // work queue entries (at most two outstanding)
-constexpr int WQ_END = 255;
 
 struct Slot {
   int b, I, J, N;        // instance, tile row and column (128 units), size
@@ -84,18 +66,6 @@ struct Shared {
   double red_e[2][EPI_WARPS];                          // Tr[D H] (last layer)
   Slot slot[2];
 };
-
-// Loads one 128-row operand of K block k0: K-major, or the stored block left
-// of the diagonal transposed (two 64 x 64 boxes).
-__device__ __forceinline__ void load_half(uint8_t* dst, const CUtensorMap* tmK, const CUtensorMap* tmT, bool trans,
-                                          int row, int k0, int b, uint64_t* bar) {
-  if (!trans) {
-    tma_load_3d(dst, tmK, k0, row, b, bar);
-  } else {
-    tma_load_3d(dst, tmT, row, k0, b, bar);
-    tma_load_3d(dst + T_BOX, tmT, row + 64, k0, b, bar);
-  }
-}
 
 // A layer's sums tr Y' and ||Y'||_F^2 in 64-bit fixed point, exact in any
 // order: FP64 adds (64 cycles each, 19 of them a warp on the SM's one pipe)
@@ -138,27 +108,6 @@ __device__ __forceinline__ double row_norm(const ResArgs& a, const Slot& s, int 
 #pragma unroll
   for (int u = 0; u < 16; ++u) acc += fix_sq(v[u]);
   return (double)acc * Q_LO_UNIT;
-}
-
-// Turns the warp's 32 x 32 chunk from one row per lane (v) to four consecutive
-// columns of eight rows (p: register 4 i + e = row 4 i + lane / 8, column
-// 4 (lane mod 8) + e), sixteen rows at a time through the warp's 2 KB.
-template <class Sink>
-__device__ __forceinline__ void turn(float* trb, const uint32_t (&v)[32], int lane, Sink sink) {
-  const int r4 = lane >> 3, c4 = lane & 7;
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    if ((lane >> 4) == h) {
-#pragma unroll
-      for (int m = 0; m < 8; ++m)
-        *epi::tr_at(trb, lane & 15, m) = make_float4(__uint_as_float(v[4 * m]), __uint_as_float(v[4 * m + 1]),
-                                                     __uint_as_float(v[4 * m + 2]), __uint_as_float(v[4 * m + 3]));
-    }
-    __syncwarp();
-#pragma unroll
-    for (int i = 4 * h; i < 4 * h + 4; ++i) sink(i, *epi::tr_at(trb, 4 * (i - 4 * h) + r4, c4));
-    __syncwarp();
-  }
 }
 
 // One layer of the warp's 32 x 32 chunk of a slot's tile (the lane layouts and
@@ -297,32 +246,8 @@ __device__ __forceinline__ bool epilogue(const ResArgs& a, Shared& sh, int c, ui
     const bool nan = __any_sync(0xffffffffu, isnan(sql)), big = __any_sync(0xffffffffu, !(sql < 16.f));
     if (!outD) {
       // operand planes of Y' (Eq. 12) first: they are what the gang waits for
-      __half* p0 = a.p0[s.par ^ 1] + (long long)b * a.slot_h + (long long)(R0 + r4) * a.ld_h + ce;
-      __half* p1 = SPLIT ? a.p1[s.par ^ 1] + (long long)b * a.slot_h + (long long)(R0 + r4) * a.ld_h + ce : nullptr;
-      const __half2 s2 = __float2half2_rn(lo_scale);
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        uint32_t pa[2], pl[2];
-#pragma unroll
-        for (int e2 = 0; e2 < 2; ++e2) {
-          // hp = 2^s fp16(x) and lo' = fp16(2^s x - hp): both differences are exact
-          const float x0 = y[4 * i + 2 * e2], x1 = y[4 * i + 2 * e2 + 1];
-          __half2 p2 = __floats2half2_rn(x0, x1);
-          if (SPLIT) {
-            p2 = __hmul2(p2, s2);
-            const float2 pf = __half22float2(p2);
-            const __half2 l2 = __floats2half2_rn(fmaf(x0, lo_scale, -pf.x), fmaf(x1, lo_scale, -pf.y));
-            pl[e2] = *reinterpret_cast<const uint32_t*>(&l2);
-          }
-          pa[e2] = *reinterpret_cast<const uint32_t*>(&p2);
-        }
-        if (4 * i + r4 < nrows) {
-          *reinterpret_cast<uint2*>(p0) = make_uint2(pa[0], pa[1]);
-          if (SPLIT) *reinterpret_cast<uint2*>(p1) = make_uint2(pl[0], pl[1]);
-        }
-        p0 += 4 * a.ld_h;
-        if (SPLIT) p1 += 4 * a.ld_h;
-      }
+      const long long po = (long long)b * a.slot_h + (long long)(R0 + r4) * a.ld_h + ce;
+      store_planes<SPLIT>(y, a.p0[s.par ^ 1] + po, SPLIT ? a.p1[s.par ^ 1] + po : nullptr, a.ld_h, nrows - r4, lo_scale);
       // row norms of the next layer
       float* rnp = a.rnp[s.par] + (long long)b * a.slot_rnp;
       const float rsum = epi::lane_sums<8, 0>(rs);
@@ -775,7 +700,7 @@ __global__ void __launch_bounds__(256) resident_input_kernel(const ResArgs a, in
     const float* row = a.H[b] + (long long)r * N;
     __half* p0 = a.p0[0] + (long long)b * a.slot_h + (long long)r * a.ld_h;
     __half* p1 = a.p1[0] ? a.p1[0] + (long long)b * a.slot_h + (long long)r * a.ld_h : nullptr;
-    const int cs = r & ~(kTcBN - 1), kpad = (N + 63) & ~63;
+    const int cs = r & ~(kTcBN - 1);
     const bool vec_h = (N & 3) == 0 && (reinterpret_cast<uintptr_t>(a.H[b]) & 15) == 0;
     // the diagonal once per row: FP64 per element, even predicated off, would
     // bound the pass (1.97 ms against 0.33 for the bounds' pass over the same
@@ -783,54 +708,7 @@ __global__ void __launch_bounds__(256) resident_input_kernel(const ResArgs a, in
     const float yd = input_diag(row[r], in);
     tr = lane == 0 ? (double)yd : 0.0;
     auto y0 = [&](float h, int col) { return col == r ? yd : input_offdiag(h, in); };
-    // FP16 planes of four columns; plain FP16 keeps hi alone
-    auto put = [&](int col, const float (&y)[4]) {
-      uint32_t pa[2], pl[2];
-      const __half2 s2 = __float2half2_rn(a.lo_scale);
-#pragma unroll
-      for (int e = 0; e < 2; ++e) {
-        const __half2 h2 = __floats2half2_rn(y[2 * e], y[2 * e + 1]);
-        const float2 hf = __half22float2(h2);
-        const __half2 l2 = __floats2half2_rn((y[2 * e] - hf.x) * a.lo_scale, (y[2 * e + 1] - hf.y) * a.lo_scale);
-        const __half2 p2 = p1 ? __hmul2(h2, s2) : h2;
-        pa[e] = *reinterpret_cast<const uint32_t*>(&p2);
-        pl[e] = *reinterpret_cast<const uint32_t*>(&l2);
-      }
-      *reinterpret_cast<uint2*>(p0 + col) = make_uint2(pa[0], pa[1]);
-      if (p1) *reinterpret_cast<uint2*>(p1 + col) = make_uint2(pl[0], pl[1]);
-    };
-    const int n4 = N >> 2;
-    for (int j0 = 0; j0 < (kpad >> 2); j0 += 32 * 8) {
-      float f = 0.f;
-      float4 hv[8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int col = (j0 + u * 32 + lane) * 4;
-        hv[u] = col < N ? epi::ld4(row + col, col, N, vec_h) : make_float4(0.f, 0.f, 0.f, 0.f);
-      }
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int j = j0 + u * 32 + lane, col = 4 * j;
-        if (col < kpad) {
-          float y[4] = {hv[u].x, hv[u].y, hv[u].z, hv[u].w};
-#pragma unroll
-          for (int e = 0; e < 4; ++e) y[e] = col + e < N ? y0(y[e], col + e) : 0.f;
-          if (j < n4) {
-            f = fmaf(y[0], y[0], f);
-            f = fmaf(y[1], y[1], f);
-            f = fmaf(y[2], y[2], f);
-            f = fmaf(y[3], y[3], f);
-          }
-          if (col >= cs) put(col, y);
-        }
-      }
-      if (vec_norm && j0 < n4) acc += (double)f;
-    }
-    // columns past the last float4, or every column in FP64 (rownorm_kernel's two tails)
-    for (int j = (vec_norm ? n4 << 2 : 0) + lane; j < N; j += 32) {
-      const double yv = (double)y0(row[j], j);
-      acc += yv * yv;
-    }
+    acc = res::plane_row(row, N, vec_h, vec_norm, y0, cs, p0, p1, a.lo_scale, lane, [](int, const float (&)[4]) {});
     acc = warp_sum_d(acc);
     if (lane == 0) const_cast<double*>(a.rn)[(long long)b * a.ld_rn + r] = acc;
   }

@@ -131,3 +131,45 @@ def test_input_that_is_not_symmetric_stops_alike(sp2):
     D, st = sp2.density_matrix(H, N // 2)
     D1, s1 = _with_env("SP2_SQUARE_KERNEL", "single", lambda m: m.density_matrix(H, N // 2))
     assert st.status == s1.status and st.converged_by == s1.converged_by
+
+
+# one matrix a CTA, gangs, more matrices than slots; segments of one layer, of
+# several, longer than the network; sizes off every boundary
+@pytest.mark.parametrize("B,N,L,ce", [(8, 128, 7, 3), (1, 1, 3, 1), (3, 257, 5, 2), (5, 100, 6, 1), (2, 1000, 4, 4),
+                                      (400, 40, 3, 2), (1, 2053, 3, 2)])
+@pytest.mark.parametrize("precision", ["split", "fp16"])
+def test_network_same_bits(sp2, B, N, L, ce, precision):
+    g = torch.Generator(device="cuda").manual_seed(N + B)
+    H = torch.randn(B, N, N, generator=g, device="cuda")
+    H = ((H + H.mT) / (2 * N**0.5)).contiguous() + torch.diag(torch.linspace(-1, 1, N, device="cuda"))
+    G = torch.randn(B, N, N, generator=g, device="cuda") / N
+    G = (G + G.mT).contiguous()
+    coef = torch.rand(L, 3, generator=torch.Generator().manual_seed(L)) - torch.tensor([0.5, 0.0, 0.5])
+
+    def run(m):
+        m.set_precision(precision)
+        X, ck, bounds = m.network_forward(H, coef, ce)
+        dcoef, G0 = m.network_backward(H, coef, ce, ck, G)
+        m.set_precision("split")
+        return X, ck, bounds, G0, dcoef
+
+    got, want = run(sp2), _with_env("SP2_SQUARE_KERNEL", "single", run)
+    for a, b in zip(got[:4], want[:4]):
+        assert torch.equal(a, b)
+    # FP64 sums of the same FP32 parts in another order
+    assert torch.allclose(got[4], want[4], rtol=1e-12, atol=1e-12 * float(want[4].abs().max()))
+
+
+@pytest.mark.parametrize("B,N", [(1, 1), (3, 130), (2, 1000), (200, 64), (1, 2053)])
+@pytest.mark.parametrize("window", [None, (-4.0, 4.0)])
+def test_expansion_same_values(sp2, B, N, window):
+    g = torch.Generator(device="cuda").manual_seed(N + B)
+    H = torch.randn(B, N, N, generator=g, device="cuda")
+    H = ((H + H.mT) / (2 * N**0.5)).contiguous() + torch.diag(torch.linspace(-1, 1, N, device="cuda"))
+    theta = [(0.4, 0.9, -0.1), (-1.0, 2.0, 0.0), (1.0, 0.0, 0.05), (-0.7, 1.5, 0.1)]
+    c = [0.1, -0.05, 0.2, 0.3, 0.5]
+    D, bounds = sp2.fermi_expansion(H, theta, c, window)
+    D1, b1 = _with_env("SP2_SQUARE_KERNEL", "single", lambda m: m.fermi_expansion(H, theta, c, window))
+    # the diagonal's FP64 row norms add in another order: one rounding to FP32 at most
+    assert torch.equal(bounds, b1)
+    assert float((D - D1).abs().max()) <= 2**-23 * float(D1.abs().max())
