@@ -1852,30 +1852,39 @@ bool net_fits(int B, int N, int n_many) {
 
 // A run of the resident network kernel (csrc/resident_net.cu) over B matrices
 // of size N: the plan of its tiles, the pool of plane pairs, the operations.
-// The host fills ops, params and the FP64 tables, then go() uploads and runs.
+// One upload, the bounds, the coefficients (planned on the device), the inputs,
+// the layers: nothing waits for the GPU but the check of the bounds, at the end.
 struct NetRun {
-  int B, N, per = 0, nt = 0, grid = 0, pool = 0;
+  int B, N, L, per = 0, nt = 0, grid = 0, pool = 0, ngrid = 0;
   NetArgs A;
   NetMaps maps;
+  NetPlanArgs plan;
   std::vector<NetOp> ops;
-  std::vector<LayerParams> params;
-  std::vector<double> table;      // FP64 values the operations point into (by index until go())
-  uint8_t* pack = nullptr;        // [ops][params][table][lists][tiles][err]
-  size_t o_params = 0, o_table = 0, o_loff = 0, o_list = 0, o_tiles = 0, o_err = 0, bytes = 0;
+  std::vector<double> coef;
+  uint8_t* pack = nullptr;  // uploaded: [ops][ctl][H][N][tickets][coef][lists][tiles][err]; then [params][table][status]
+  size_t o_ctl = 0, o_hs = 0, o_ns = 0, o_tick = 0, o_coef = 0, o_loff = 0, o_list = 0, o_tiles = 0, o_err = 0, up = 0;
+  size_t o_params = 0, o_table = 0, o_status = 0, bytes = 0;
+  double2* part = nullptr;
 
-  sp2_status init(int B_, int N_, int pool_, bool split, const Ctl* ctl, int nops, size_t nparams, size_t ntable) {
+  // nops operations, coef set, ntable FP64 values
+  sp2_status init(int B_, int N_, int L_, int pool_, bool split, int nops, size_t nparams, size_t ntable) {
     B = B_;
     N = N_;
+    L = L_;
     pool = pool_;
     memset(&A, 0, sizeof(A));
+    memset(&plan, 0, sizeof(plan));
     resident_tiles(N, 0, nullptr, &per);
     nt = per * B;
     grid = std::min(nt, g.num_sms);
+    ngrid = (int)std::min<long long>((N + 7) / 8, std::max((N + 63) / 64, 2 * g.num_sms / B + 1));
     const long long ld_h = round_up(N, 64), slot_h = ld_h * N;
-    void *p0, *p1 = nullptr, *sums;
+    void *p0, *p1 = nullptr, *sums, *prt;
     CKS(ws(B_PLANES0, (size_t)slot_h * B * pool * 2, &p0));
     if (split) CKS(ws(B_PLANES1, (size_t)slot_h * B * pool * 2, &p1));
     CKS(ws(B_TPART, (size_t)3 * nt * sizeof(longlong2), &sums));
+    CKS(ws(B_PART, (size_t)B * ngrid * sizeof(double2), &prt));
+    part = (double2*)prt;
     SqArgs carry;
     void* rnp[2];
     CKS(rnp_for(N, B, carry, rnp));
@@ -1886,12 +1895,19 @@ struct NetRun {
       return at;
     };
     take(nops * sizeof(NetOp));
-    o_params = take(nparams * sizeof(LayerParams));
-    o_table = take(ntable * sizeof(double));
+    o_ctl = take((size_t)B * sizeof(Ctl));
+    o_hs = take((size_t)B * sizeof(void*));
+    o_ns = take((size_t)B * sizeof(int));
+    o_tick = take((size_t)B * sizeof(unsigned));
+    o_coef = take(coef.size() * sizeof(double));
     o_loff = take((size_t)(2 * grid + 1) * sizeof(int));
     o_list = take((size_t)nt * sizeof(int));
     o_tiles = take((size_t)nt * sizeof(uint32_t));
     o_err = take(sizeof(int));
+    up = o;
+    o_params = take(nparams * sizeof(LayerParams));
+    o_table = take(ntable * sizeof(double));
+    o_status = take((size_t)B * sizeof(int));
     bytes = o;
     void* pk;
     CKS(ws(B_PACK, bytes, &pk));
@@ -1902,7 +1918,7 @@ struct NetRun {
     A.ntiles = nt;
     A.ops = (const NetOp*)pack;
     A.lp = (const LayerParams*)(pack + o_params);
-    A.ctl = ctl;
+    A.ctl = (const Ctl*)(pack + o_ctl);
     A.p0 = (__half*)p0;
     A.p1 = (__half*)p1;
     A.ld_h = ld_h;
@@ -1921,6 +1937,14 @@ struct NetRun {
     A.two_slots = nt > grid ? 1 : 0;
     A.err = (int*)(pack + o_err);
     A.wait_ns = g.wait_ns;
+    plan.batch = B;
+    plan.L = L;
+    plan.shift = g.shift;
+    plan.coef = (const double*)(pack + o_coef);
+    plan.ctl = A.ctl;
+    plan.lp = (LayerParams*)(pack + o_params);
+    plan.table = (double*)(pack + o_table);
+    plan.status = (int*)(pack + o_status);
     CUtensorMap m[6];
     CKS(tmaps4_for(p0, p1, N, B * pool, ld_h, slot_h, m, kTcBM));
     maps.m[0] = m[0];
@@ -1931,15 +1955,28 @@ struct NetRun {
   }
   const double* dev(size_t table_index) const { return (const double*)(pack + o_table) + table_index; }
 
-  // the records, in one upload
-  sp2_status upload() {
+  // The records in one upload, the bounds (of H, or the given window) and the
+  // plan; `back` receives the statuses after them (check()).
+  sp2_status start(const float* H, const double* window, int** back) {
+    cudaStream_t st = g.stream;
     A.nops = (int)ops.size();
     void* h;
-    CKS(staging(bytes, &h));
+    CKS(staging(up + (size_t)B * sizeof(int), &h));
     uint8_t* hb = (uint8_t*)h;
     memcpy(hb, ops.data(), ops.size() * sizeof(NetOp));
-    memcpy(hb + o_params, params.data(), params.size() * sizeof(LayerParams));
-    memcpy(hb + o_table, table.data(), table.size() * sizeof(double));
+    Ctl* hc = (Ctl*)(hb + o_ctl);
+    const float** hh = (const float**)(hb + o_hs);
+    for (int b = 0; b < B; ++b) {
+      init_ctl(hc + b, N, N / 2, 0.0, 1);
+      if (window) {
+        hc[b].e_min = window[0];
+        hc[b].e_max = window[1];
+      }
+      hh[b] = H + (size_t)b * N * N;
+      ((int*)(hb + o_ns))[b] = N;
+      ((unsigned*)(hb + o_tick))[b] = 0u;
+    }
+    memcpy(hb + o_coef, coef.data(), coef.size() * sizeof(double));
     std::vector<int> order(B), Ns(B, N), toff(B), tcnt(B, per);
     std::vector<uint32_t> tiles;
     for (int b = 0; b < B; ++b) {
@@ -1951,10 +1988,33 @@ struct NetRun {
     resident_plan(order.data(), Ns.data(), toff.data(), tcnt.data(), B, grid, (int*)(hb + o_loff), (int*)(hb + o_list));
     memcpy(hb + o_tiles, tiles.data(), nt * sizeof(uint32_t));
     *(int*)(hb + o_err) = 0;
-    CK(cudaMemcpyAsync(pack, hb, bytes, cudaMemcpyHostToDevice, g.stream));
-    CK(cudaEventRecord(g.stage_done, g.stream));
-    CK(cudaMemsetAsync(A.sums, kGangEmptyByte, (size_t)3 * nt * sizeof(longlong2), g.stream));
+    CK(cudaMemcpyAsync(pack, hb, up, cudaMemcpyHostToDevice, st));
+    if (!window)
+      CK(launch_gershgorin_batched((const float* const*)(pack + o_hs), (const int*)(pack + o_ns), (Ctl*)(pack + o_ctl),
+                                   B, part, (unsigned*)(pack + o_tick), ngrid, st));
+    CK(launch_net_plan(plan, st));
+    if (back) {
+      *back = (int*)(hb + up);
+      CK(cudaMemcpyAsync(*back, pack + o_status, (size_t)B * sizeof(int), cudaMemcpyDeviceToHost, st));
+    }
+    CK(cudaEventRecord(g.stage_done, st));  // also: the statuses are on the host
+    CK(cudaMemsetAsync(A.sums, kGangEmptyByte, (size_t)3 * nt * sizeof(longlong2), st));
     return SP2_OK;
+  }
+  // the statuses of the bounds, once they are on the host
+  sp2_status check(const int* status) const {
+    for (int b = 0; b < B; ++b) {
+      if (status[b] < 0) {
+        set_err("instance %d: %s", b,
+                status[b] == SP2_ERR_NONFINITE ? "non-finite spectral bounds" : "degenerate spectrum");
+        return (sp2_status)status[b];
+      }
+    }
+    return SP2_OK;
+  }
+  sp2_status wait_and_check(const int* back) const {
+    CK(cudaEventSynchronize(g.stage_done));
+    return check(back);
   }
   // inputs of one kind into the plane pairs from pool entry `entry` on
   NetInput input(int from, const float* in, int entry) const {
@@ -1963,7 +2023,7 @@ struct NetRun {
     x.N = N;
     x.batch = B;
     x.from = from;
-    x.shift = g.shift;
+    x.shift = A.shift;
     x.in = in;
     x.ctl = A.ctl;
     x.p0 = A.p0 + (long long)entry * B * A.slot_h;
@@ -1986,16 +2046,16 @@ NetOp net_square(int y, int out, int layer, int rnp) {
 }
 
 // The network's forward pass on the resident kernel (net_fits).
-sp2_status net_forward_resident(const float* H, int B, int N, int L, const NetPlan& plan, const Ctl* ctl, int ckpt_every,
-                                float* X_out, float* ckpt) {
+sp2_status net_forward_resident(const float* H, int B, int N, int L, const float* coef, int ckpt_every, float* X_out,
+                                float* ckpt, double* bounds) {
   const bool split = g.precision == SP2_PREC_SPLIT_FP16;
   const size_t mats = (size_t)B * N * N;
   NetRun R;
   void* rn;
   CKS(ws(B_RN, (size_t)B * N * sizeof(double), &rn));
-  CKS(R.init(B, N, 2, split, ctl, L, plan.params.size(), plan.alpha.size()));
-  R.params = plan.params;
-  R.table = plan.alpha;
+  R.coef.assign(coef, coef + 3 * L);
+  CKS(R.init(B, N, L, 2, split, L, (size_t)L * B, (size_t)(L + 1) * B));
+  R.plan.bounds = bounds;
   for (int n = 0; n < L; ++n) {
     const bool last = n == L - 1, kept = ckpt && (n + 1) % ckpt_every == 0;
     NetOp o = net_square(n & 1, last ? -1 : (n & 1) ^ 1, n, n & 1);
@@ -2014,7 +2074,8 @@ sp2_status net_forward_resident(const float* H, int B, int N, int L, const NetPl
     }
     R.ops.push_back(o);
   }
-  CKS(R.upload());
+  int* back = nullptr;
+  CKS(R.start(H, nullptr, &back));
   NetInput x = R.input(NET_INPUT, H, 0);
   x.vec_norm = (N & 3) == 0 && ((uintptr_t)X_out & 15) == 0;
   x.rn = (double*)rn;
@@ -2022,34 +2083,33 @@ sp2_status net_forward_resident(const float* H, int B, int N, int L, const NetPl
   x.alpha0 = R.dev(0);
   CK(launch_net_input(x, B, g.stream));
   CK(launch_resident_net(R.A, R.maps, split, R.grid, g.stream));
-  return SP2_OK;
+  return R.wait_and_check(back);
 }
+
+void coef_gradient(const double* dd, const double* alpha, int L, int B, double* dcoef);
 
 // The network's adjoint on the resident kernel: per checkpoint segment, from
 // the last one, the recomputation of its iterates and the adjoint layers.
-// dots: host [L][B][3].
-sp2_status net_backward_resident(int B, int N, int L, const NetPlan& plan, const std::vector<LayerParams>& bp,
-                                 const Ctl* ctl, int ce, const float* ckpt, const float* G_out, float* G_in,
-                                 const double** dots_host) {
+sp2_status net_backward_resident(const float* H, int B, int N, int L, const float* coef, int ce, const float* ckpt,
+                                 const float* G_out, double* dcoef, float* G_in) {
   const bool split = g.precision == SP2_PREC_SPLIT_FP16;
   cudaStream_t st = g.stream;
-  const size_t mats = (size_t)B * N * N;
+  const size_t mats = (size_t)B * N * N, nalpha = (size_t)(L + 1) * B;
   const int nseg = (L + ce - 1) / ce;
   // pool: the segments' first iterates, the others of a segment, G twice
   const int p_rec = nseg, p_g = nseg + std::min(ce, L) - 1;
   NetRun R;
   void *rn, *keep, *tdots, *dots;
   CKS(ws(B_RN, (size_t)nseg * B * N * sizeof(double), &rn));
-  CKS(R.init(B, N, p_g + 2, split, ctl, 2 * L, 2 * plan.params.size(), plan.alpha.size()));
+  R.coef.assign(coef, coef + 3 * L);
+  CKS(R.init(B, N, L, p_g + 2, split, 2 * L, (size_t)2 * L * B, 2 * nalpha));
+  R.plan.backward = 1;
   const size_t tile_store = (size_t)R.nt * kResTile * kResTile;
   CKS(ws(B_SEG, tile_store * 4 * std::max(1, std::min(ce, L) - 1), &keep));
   CKS(ws(B_TDOTS, (size_t)L * R.nt * 3 * sizeof(double), &tdots));
   CKS(ws(B_DOTS, (size_t)L * B * 3 * sizeof(double) + 16, &dots));
   R.A.tile_dots = (double*)tdots;
-  R.params = plan.params;
-  R.params.insert(R.params.end(), bp.begin(), bp.end());
-  R.table.resize(plan.alpha.size());
-  for (size_t i = 0; i < R.table.size(); ++i) R.table[i] = -plan.alpha[i];
+  auto minus_alpha = [&](int n) { return R.dev(nalpha + (size_t)n * B); };
   auto store = [&](int k) { return (float*)keep + tile_store * (size_t)(k - 1); };  // iterate n0 + k, k >= 1
   int gcur = 0;
   bool first = true;
@@ -2063,7 +2123,7 @@ sp2_status net_backward_resident(int B, int N, int L, const NetPlan& plan, const
       if (k == 0) {
         o.from = NET_X;
         o.in = X0;
-        o.add = R.dev((size_t)n0 * B);
+        o.add = minus_alpha(n0);
         o.rn = (const double*)rn + (size_t)s * B * N;
       } else {
         o.from = NET_KEPT;
@@ -2083,7 +2143,7 @@ sp2_status net_backward_resident(int B, int N, int L, const NetPlan& plan, const
       o.tmem = n == 0 ? 0 : 1;
       if (k == 0) {
         o.aux_x = X0;
-        o.aux_add = R.dev((size_t)n0 * B);
+        o.aux_add = minus_alpha(n0);
       } else {
         o.aux = store(k);
       }
@@ -2093,9 +2153,9 @@ sp2_status net_backward_resident(int B, int N, int L, const NetPlan& plan, const
       gcur ^= 1;
     }
   }
-  CKS(R.upload());
+  CKS(R.start(H, nullptr, nullptr));
   NetInput x = R.input(NET_X, ckpt, 0);
-  x.add = R.dev(0);
+  x.add = minus_alpha(0);
   x.add_stride = (long long)ce * B;
   x.vec_norm = (N & 3) == 0;
   x.rn = (double*)rn;
@@ -2103,28 +2163,33 @@ sp2_status net_backward_resident(int B, int N, int L, const NetPlan& plan, const
   CK(launch_net_input(R.input(NET_FULL, G_out, p_g), B, st));
   CK(launch_resident_net(R.A, R.maps, split, R.grid, st));
   CK(launch_net_dots((const double*)tdots, R.nt, R.per, L, B, (double*)dots, st));
+  // dot products, shifts, statuses, error word
+  const size_t db = (size_t)L * B * 3 * sizeof(double), ab = nalpha * sizeof(double), sb = (size_t)B * sizeof(int);
   void* hd;
-  const size_t db = (size_t)L * B * 3 * sizeof(double);
-  CKS(staging(db + 16, &hd));
-  CK(cudaMemcpyAsync(hd, dots, db, cudaMemcpyDeviceToHost, st));
-  CK(cudaMemcpyAsync((char*)hd + db, R.A.err, sizeof(int), cudaMemcpyDeviceToHost, st));
+  CKS(staging(db + ab + sb + 16, &hd));
+  char* hp = (char*)hd;
+  CK(cudaMemcpyAsync(hp, dots, db, cudaMemcpyDeviceToHost, st));
+  CK(cudaMemcpyAsync(hp + db, R.plan.table, ab, cudaMemcpyDeviceToHost, st));
+  CK(cudaMemcpyAsync(hp + db + ab, R.plan.status, sb, cudaMemcpyDeviceToHost, st));
+  CK(cudaMemcpyAsync(hp + db + ab + sb, R.A.err, sizeof(int), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
-  if (*(const int*)((char*)hd + db)) {
+  CKS(R.check((const int*)(hp + db + ab)));
+  if (*(const int*)(hp + db + ab + sb)) {
     set_err("a bounded device wait timed out");
     return SP2_ERR_DEVICE_TIMEOUT;
   }
-  *dots_host = (const double*)hd;
+  coef_gradient((const double*)hp, (const double*)(hp + db), L, B, dcoef);
   return SP2_OK;
 }
 
 // dcoef from the dot products [L][B][3] (tr G, <G, Y_n>, <Y_n G + G Y_n, Y_n>):
 // dL/da_n = <G, X_n^2> = alpha^2 tr G + 2 alpha <G, Y_n> + <Y_n G + G Y_n, Y_n> / 2
 // dL/db_n = <G, X_n>   = alpha tr G + <G, Y_n>;   dL/dc_n = tr G
-void coef_gradient(const double* dd, const NetPlan& plan, int L, int B, double* dcoef) {
+void coef_gradient(const double* dd, const double* alpha, int L, int B, double* dcoef) {
   for (int n = 0; n < L; ++n) {
     double da = 0.0, db = 0.0, dc = 0.0;
     for (int b = 0; b < B; ++b) {
-      const double al = plan.alpha[(size_t)n * B + b];
+      const double al = alpha[(size_t)n * B + b];
       const double* v = dd + ((size_t)n * B + b) * 3;
       da += al * al * v[0] + 2.0 * al * v[1] + 0.5 * v[2];
       db += al * v[0] + v[1];
@@ -2152,6 +2217,7 @@ sp2_status sp2_network_forward(const float* H, int B, int N, int L, const float*
       set_err("sp2_network_forward: non-finite coefficient");
       return SP2_ERR_INVALID_ARG;
     }
+  if (net_fits(B, N, 1024)) return net_forward_resident(H, B, N, L, coef, ckpt_every, X_out, ckpt, bounds);
   const bool tc = tc_precision(g.precision);
   const bool split = g.precision == SP2_PREC_SPLIT_FP16;
   cudaStream_t st = g.stream;
@@ -2162,8 +2228,6 @@ sp2_status sp2_network_forward(const float* H, int B, int N, int L, const float*
   if (bounds)
     CK(cudaMemcpy2DAsync(bounds, 2 * sizeof(double), (char*)ctl + offsetof(Ctl, e_min), sizeof(Ctl),
                          2 * sizeof(double), B, cudaMemcpyDeviceToDevice, st));
-  if (net_fits(B, N, 1024))
-    return net_forward_resident(H, B, N, L, plan, (const Ctl*)ctl, ckpt_every, X_out, ckpt);
   int ntiles = 0;
   // tensor-core layers on CTA pairs (super-tile pairs sharing B) unless
   // single CTAs are selected, as for the single solve
@@ -2303,13 +2367,14 @@ sp2_status sp2_network_backward(const float* H, int B, int N, int L, const float
   const long long slot = (long long)N * N;
   const int ce = ckpt_every;
   // (the planes of all segments' first iterates, as large as the checkpoints, within 32 GiB)
-  const bool resident = net_fits(B, N, 512) && (double)((L + ce - 1) / ce + ce + 1) * B * round_up(N, 64) * N * 4.0 < 0x1p35;
-  void* G = nullptr;
-  if (!resident) CKS(ws(B_G, (size_t)B * slot * 4, &G));
+  if (net_fits(B, N, 512) && (double)((L + ce - 1) / ce + ce + 1) * B * round_up(N, 64) * N * 4.0 < 0x1p35)
+    return net_backward_resident(H, B, N, L, coef, ce, ckpt, G_out, dcoef, G_in);
+  void* G;
+  CKS(ws(B_G, (size_t)B * slot * 4, &G));
   bool ok = false;
   NetPlan plan;
   void *ctl, *ns, *hs, *dptr;
-  CKS(network_prologue(H, B, N, L, coef, &ok, plan, &ctl, &ns, &hs, &dptr, G ? (float*)G : const_cast<float*>(G_out)));
+  CKS(network_prologue(H, B, N, L, coef, &ok, plan, &ctl, &ns, &hs, &dptr, (float*)G));
 
   // backward coefficients: G_n = (2 a_n alpha_n + b_n) G + a_n (Y_n G + G Y_n)
   std::vector<LayerParams> bp((size_t)L * B);
@@ -2332,12 +2397,6 @@ sp2_status sp2_network_backward(const float* H, int B, int N, int L, const float
       plan.params[(size_t)n * B + b].out_mode = OUT_Y;
       plan.params[(size_t)n * B + b].alpha_out = 0.0;
     }
-  if (resident) {
-    const double* dd = nullptr;
-    CKS(net_backward_resident(B, N, L, plan, bp, (const Ctl*)ctl, ce, ckpt, G_out, G_in, &dd));
-    coef_gradient(dd, plan, L, B, dcoef);
-    return SP2_OK;
-  }
   // CTA pairs (M = 256 MMAs) unless the single-CTA kernel was selected; the
   // pair kernel keeps the operand planes as upper super tiles
   const bool pairs = g.pair_kernel;
@@ -2509,7 +2568,7 @@ sp2_status sp2_network_backward(const float* H, int B, int N, int L, const float
     set_err("a bounded device wait timed out");
     return SP2_ERR_DEVICE_TIMEOUT;
   }
-  coef_gradient(dd, plan, L, B, dcoef);
+  coef_gradient(dd, plan.alpha.data(), L, B, dcoef);
   return SP2_OK;
 }
 
@@ -2539,6 +2598,42 @@ sp2_status sp2_fermi_expansion(const float* H, int B, int N, int L, const double
   const bool split = g.precision == SP2_PREC_SPLIT_FP16;
   cudaStream_t st = g.stream;
   const long long slot = (long long)N * N;
+
+  if (net_fits(B, N, 1024)) {
+    NetRun run;
+    void *rn, *R;
+    CKS(ws(B_RN, (size_t)B * N * sizeof(double), &rn));
+    run.coef.assign(theta, theta + 3 * L);
+    run.coef.insert(run.coef.end(), c, c + L + 1);
+    CKS(run.init(B, N, L, 2, split, L, (size_t)L * B, B));
+    CKS(ws(B_READOUT, (size_t)run.nt * kResTile * kResTile * sizeof(float), &R));
+    run.plan.expansion = 1;
+    run.plan.bounds = bounds;
+    run.A.shift = 1;
+    run.A.R = (float*)R;
+    run.A.r_scale = (float)(-c[0]);
+    run.A.r_add = run.dev(0);
+    for (int n = 0; n < L; ++n) {
+      const bool last = n == L - 1;
+      NetOp o = net_square(n & 1, last ? -1 : (n & 1) ^ 1, n, n & 1);
+      o.from = n == 0 ? NET_INPUT : NET_TMEM;
+      o.in = H;
+      o.rn = n == 0 ? (const double*)rn : nullptr;
+      o.tmem = last ? 0 : 1;
+      o.readout = n == 0 ? 2 : 1;
+      o.full = last ? D_out : nullptr;
+      run.ops.push_back(o);
+    }
+    const double window[2] = {e_lo, e_hi};
+    int* back = nullptr;
+    CKS(run.start(H, fixed ? window : nullptr, fixed ? nullptr : &back));
+    NetInput x = run.input(NET_INPUT, H, 0);
+    x.vec_norm = (N & 3) == 0 && ((uintptr_t)D_out & 15) == 0;
+    x.rn = (double*)rn;
+    CK(launch_net_input(x, B, st));
+    CK(launch_resident_net(run.A, run.maps, split, run.grid, st));
+    return fixed ? SP2_OK : run.wait_and_check(back);
+  }
 
   // per-instance records; fixed bounds go straight into the control blocks
   void *ctl, *ns, *hs, *dptr;
@@ -2632,38 +2727,6 @@ sp2_status sp2_fermi_expansion(const float* H, int B, int N, int L, const double
     }
   }
 
-  if (net_fits(B, N, 1024)) {
-    NetRun run;
-    void *rn, *R;
-    CKS(ws(B_RN, (size_t)B * N * sizeof(double), &rn));
-    CKS(run.init(B, N, 2, split, (const Ctl*)ctl, L, params.size(), d0.size()));
-    CKS(ws(B_READOUT, (size_t)run.nt * kResTile * kResTile * sizeof(float), &R));
-    run.params = params;
-    run.table = d0;
-    run.A.shift = 1;
-    run.A.R = (float*)R;
-    run.A.r_scale = (float)(-c[0]);
-    run.A.r_add = run.dev(0);
-    for (int n = 0; n < L; ++n) {
-      const bool last = n == L - 1;
-      NetOp o = net_square(n & 1, last ? -1 : (n & 1) ^ 1, n, n & 1);
-      o.from = n == 0 ? NET_INPUT : NET_TMEM;
-      o.in = H;
-      o.rn = n == 0 ? (const double*)rn : nullptr;
-      o.tmem = last ? 0 : 1;
-      o.readout = n == 0 ? 2 : 1;
-      o.full = last ? D_out : nullptr;
-      run.ops.push_back(o);
-    }
-    CKS(run.upload());
-    NetInput x = run.input(NET_INPUT, H, 0);
-    x.shift = 1;
-    x.vec_norm = (N & 3) == 0 && ((uintptr_t)D_out & 15) == 0;
-    x.rn = (double*)rn;
-    CK(launch_net_input(x, B, st));
-    CK(launch_resident_net(run.A, run.maps, split, run.grid, st));
-    return SP2_OK;
-  }
   int ntiles = 0;
   CKS(upload_tiles(N, B, 2, &ntiles));
   void *prm, *dd, *R, *rn;

@@ -254,6 +254,20 @@ struct NetInput {
   const double* alpha0;
   float lo_scale;
 };
+// The layers' coefficients and FP64 shifts from the bounds in ctl, on the device.
+struct NetPlanArgs {
+  int batch, L, shift;
+  int expansion;           // 1: finite-temperature expansion (coef: theta [L][3], then c [L + 1]), table = readout's
+                           //   identity part [batch]; 0: network (coef [L][3]), table = alpha_n [L + 1][batch]
+  int backward;            // network: also the adjoint's coefficients at lp[L + n], and table + (L + 1) batch = -alpha_n
+  const double* coef;
+  const Ctl* ctl;
+  LayerParams* lp;
+  double* table;
+  int* status;             // [batch] sp2_status of the bounds
+  double* bounds;          // [batch][2] caller's copy, or nullptr
+};
+cudaError_t launch_net_plan(const NetPlanArgs& a, cudaStream_t st);
 cudaError_t launch_net_input(const NetInput& x, int count, cudaStream_t st);
 cudaError_t launch_net_dots(const double* tile_dots, int ntiles, int per, int L, int B, double* out, cudaStream_t st);
 cudaError_t launch_resident_net(const NetArgs& a, const NetMaps& maps, bool split, int grid, cudaStream_t st);

@@ -105,12 +105,23 @@ __device__ __forceinline__ double row_norm(const NetArgs& a, const NetOp& o, int
   return from_fixed(acc, e);
 }
 
-// Sum over the warp's lanes of one FP32 value each.
-__device__ __forceinline__ double lanes_sum(float v) {
-  const int e = __reduce_max_sync(0xffffffffu, (__float_as_int(v) >> 23) & 255);
-  if (e == 0) return 0.0;  // zeros (and denormals)
-  if (!fixed_ok(e)) return warp_sum_d((double)v);
-  return from_fixed(warp_sum_ll(to_fixed(v, e)), e);
+// Sums over the warp's lanes of one FP32 value each, two side by side.
+__device__ __forceinline__ void lanes_sum(float u, float v, double& su, double& sv) {
+  const int eu = __reduce_max_sync(0xffffffffu, (__float_as_int(u) >> 23) & 255);
+  const int ev = __reduce_max_sync(0xffffffffu, (__float_as_int(v) >> 23) & 255);
+  if (fixed_ok(eu) && fixed_ok(ev)) {
+    long long a = to_fixed(u, eu), b = to_fixed(v, ev);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      a += __shfl_xor_sync(0xffffffffu, a, o);
+      b += __shfl_xor_sync(0xffffffffu, b, o);
+    }
+    su = from_fixed(a, eu);
+    sv = from_fixed(b, ev);
+  } else {
+    su = eu ? warp_sum_d((double)u) : 0.0;  // (exponent 0: zeros, and denormals)
+    sv = ev ? warp_sum_d((double)v) : 0.0;
+  }
 }
 
 // The lane's four columns of its eight rows of a matrix of the batch.
@@ -274,6 +285,11 @@ __device__ __forceinline__ bool epilogue(const NetArgs& a, Shared& sh, int c, ui
       if (dlane) dtr = yold_d;
     }
   }
+  float4 x4[4];  // kind 1: Y's rows of a half
+  if (live && adj) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) x4[i] = aux4(i);
+  }
   if (!__all_sync(0xffffffffu, mbar_wait(&sh.acc_full[c], acc_phase, &sh.abort, lim))) return false;
   tc_fence_after();
 
@@ -282,12 +298,11 @@ __device__ __forceinline__ bool epilogue(const NetArgs& a, Shared& sh, int c, ui
     const float cbu = p.cb * unscale;
     float p_d = 0.f;
     {
-      float4 x4[4];  // kind 1: Y's rows of a half
       const float ca = p.ca;
       turn_tmem(trb, tacc, lane, [&](int h) {
-        if (adj) {
+        if (adj && h == 1) {
 #pragma unroll
-          for (int i = 0; i < 4; ++i) x4[i] = aux4(4 * h + i);
+          for (int i = 0; i < 4; ++i) x4[i] = aux4(4 + i);
         }
       }, [&](int i, const float4& pv) {
         if (adj) {
@@ -450,17 +465,19 @@ __device__ __forceinline__ bool epilogue(const NetArgs& a, Shared& sh, int c, ui
         }
       }
     }
-    if (o.out >= 0) fence_proxy_async();  // the planes are read by the TMA units next
   }
-  tmem_st_wait();
-  tc_fence_before();
   double s0 = 0.0, s1 = 0.0, s2 = 0.0;
   if (adj) {
     const double twice = mirror ? 2.0 : 1.0;
-    if (dchunk) s0 = lanes_sum(dtr);
-    s1 = lanes_sum(gy) * twice;
-    s2 = lanes_sum(py) * twice;
+    lanes_sum(gy, py, s1, s2);
+    s1 *= twice;
+    s2 *= twice;
+    double none;
+    if (dchunk) lanes_sum(dtr, 0.f, s0, none);
   }
+  if (live && o.out >= 0) fence_proxy_async();  // the planes are read by the TMA units next
+  tmem_st_wait();
+  tc_fence_before();
   __syncwarp();
   if (lane == 0) {
     if (adj) {
@@ -819,6 +836,68 @@ __global__ void __launch_bounds__(256) net_input_kernel(const NetInput x) {
   }
 }
 
+// One thread per matrix walks through its layers: X_n = alpha_n I + Y_n with
+// alpha_0 = e_max / (e_max - e_min) (0 without the shift) and alpha_{n+1} = a
+// alpha^2 + b alpha + c, Y' = (2 a alpha + b) Y + a Y^2.  On the device so that
+// no call waits for the bounds before it can enqueue its layers.
+__global__ void net_plan_kernel(const NetPlanArgs a) {
+  const int b = blockIdx.x * blockDim.x + threadIdx.x, B = a.batch, L = a.L;
+  if (b >= B) return;
+  const Ctl& c = a.ctl[b];
+  const double lo = c.e_min, hi = c.e_max;
+  a.status[b] = c.status < 0 ? c.status : 0;
+  if (a.bounds) {
+    a.bounds[2 * b] = lo;
+    a.bounds[2 * b + 1] = hi;
+  }
+  LayerParams p;
+  memset(&p, 0, sizeof(p));
+  p.active = 1;
+  if (a.expansion) {
+    // S_0 = alpha_0 I + Y_0, Y_0 = -H/w; X_0 = I - S_0 = (1 - alpha_0) I - Y_0
+    const double* rc = a.coef + 3 * L;
+    double al = 1.0 - hi / (hi - lo);
+    a.table[b] = rc[0] * al;  // R_0 = c_0 X_0
+    for (int n = 0; n < L; ++n) {
+      const double t = a.coef[3 * n], u = a.coef[3 * n + 1], v = a.coef[3 * n + 2];
+      const double an = t * al * al + u * al + v;
+      p.ca_d = (n == 0 ? -1.0 : 1.0) * (2.0 * t * al + u);
+      p.cb_d = t;
+      p.ca = (float)p.ca_d;
+      p.cb = (float)p.cb_d;
+      p.rc_d = rc[n + 1];
+      p.rc = (float)rc[n + 1];
+      p.alpha_new = an;
+      a.lp[(long long)n * B + b] = p;
+      al = an;
+    }
+    return;
+  }
+  double al = a.shift ? hi / (hi - lo) : 0.0;
+  double* minus = a.table + (long long)(L + 1) * B;
+  for (int n = 0; n <= L; ++n) {
+    a.table[(long long)n * B + b] = al;
+    if (a.backward) minus[(long long)n * B + b] = -al;
+    if (n == L) break;
+    const double ca = a.coef[3 * n], cb = a.coef[3 * n + 1], cc = a.coef[3 * n + 2];
+    p.ca_d = 2.0 * ca * al + cb;
+    p.cb_d = ca;
+    p.ca = (float)p.ca_d;
+    p.cb = (float)p.cb_d;
+    if (a.backward) {
+      // G_n = (2 a_n alpha_n + b_n) G + a_n (Y_n G + G Y_n)
+      p.cc_d = 0.0;
+      a.lp[(long long)(L + n) * B + b] = p;
+    }
+    const double an = a.shift ? ca * al * al + cb * al + cc : 0.0;
+    p.cc_d = a.shift ? 0.0 : cc;
+    p.alpha_out = n == L - 1 ? an : 0.0;
+    a.lp[(long long)n * B + b] = p;
+    p.alpha_out = 0.0;
+    al = an;
+  }
+}
+
 // Dot products of a layer and matrix: the tiles' in their order, by one warp.
 __global__ void net_dots_kernel(const double* __restrict__ tile_dots, int ntiles, int per, double* __restrict__ out) {
   const int n = blockIdx.x, b = blockIdx.y, lane = threadIdx.x;
@@ -841,6 +920,11 @@ __global__ void net_dots_kernel(const double* __restrict__ tile_dots, int ntiles
 }
 
 }  // namespace net
+
+cudaError_t launch_net_plan(const NetPlanArgs& a, cudaStream_t st) {
+  net::net_plan_kernel<<<(a.batch + 31) / 32, 32, 0, st>>>(a);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_net_input(const NetInput& x, int count, cudaStream_t st) {
   net::net_input_kernel<<<dim3(count, (x.N + 7) / 8), 256, 0, st>>>(x);
