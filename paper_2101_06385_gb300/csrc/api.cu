@@ -869,7 +869,7 @@ sp2_status resident_solve(const float* const* H, const int* N, const int* N_occ,
   void *pack, *part, *sums, *rn, *tdots;
   CKS(ws(B_PACK, P.all, &pack));
   CKS(ws(B_PART, (size_t)B * std::max(iblocks, ggrid) * sizeof(double2), &part));
-  CKS(ws(B_TPART, (size_t)3 * nt * sizeof(longlong2), &sums));
+  CKS(ws(B_TPART, (size_t)B * kMeetRows * sizeof(long long), &sums));
   CKS(ws(B_TDOTS, (size_t)nt * sizeof(double), &tdots));
   const long long ld_h = round_up(Nmax, 64), slot_h = ld_h * Nmax;
   void *hi[2], *lo[2], *hp[2];
@@ -928,7 +928,7 @@ sp2_status resident_solve(const float* const* H, const int* N, const int* N_occ,
   A.part = (double2*)part;
   A.tile_dots = (double*)tdots;
   A.dots_out = (double*)(dp + P.dots);
-  A.sums = (longlong2*)sums;
+  A.sums = (long long*)sums;
   A.tickets = (unsigned*)(dp + P.tickets) + B;
   unsigned* gtick = (unsigned*)(dp + P.tickets);
   A.list_off = (const int*)(dp + P.loff);
@@ -1028,14 +1028,12 @@ sp2_status fp32_solve(const float* H, int N, int N_occ, double tol, int max_iter
   const int igrid = (int)std::min<long long>(N, 8LL * g.num_sms);
   const int rgrid = (int)std::min<long long>((N + 7) / 8, 2LL * g.num_sms);
   // one upload: control block, stamps, error word (read back), then pointers,
-  // size, tickets and the tiles
+  // size, tickets, the meeting rows and the tiles
   const size_t o_st = sizeof(Ctl), o_err = o_st + (kResStamps + 2) / 2 * 8, o_ptr = o_err + 16,
-               o_tiles = o_ptr + 64, bytes = o_tiles + (size_t)nt * sizeof(uint32_t);
+               o_sums = o_ptr + 64, o_tiles = o_sums + 2 * kMeetRows * sizeof(long long), bytes = o_tiles + (size_t)nt * sizeof(uint32_t);
   static_assert(sizeof(Ctl) % 8 == 0, "the offsets after it keep 8-byte alignment");
-  const size_t sums_bytes = (size_t)6 * grid * sizeof(longlong2);
-  void *pack, *part, *rn, *sums, *Y[2];
+  void *pack, *part, *rn, *Y[2];
   CKS(ws(B_PACK, bytes, &pack));
-  CKS(ws(B_TPART, sums_bytes, &sums));
   CKS(ws(B_PART, std::max(std::max(ggrid, igrid), rgrid) * sizeof(double2), &part));
   CKS(ws(B_RN, (size_t)N * sizeof(double), &rn));
   const long long ld_y = round_up(N, 4), slot_y = ld_y * N;
@@ -1061,7 +1059,6 @@ sp2_status fp32_solve(const float* H, int N, int N_occ, double tol, int max_iter
   uint8_t* dp = (uint8_t*)pack;
   CK(cudaMemcpyAsync(dp, hb, bytes, cudaMemcpyHostToDevice, st));
   CK(cudaEventRecord(g.stage_done, st));
-  CK(cudaMemsetAsync(sums, kGangEmptyByte, sums_bytes, st));
   Res32Args A;
   memset(&A, 0, sizeof(A));
   A.Y[0] = (float*)Y[0];
@@ -1073,7 +1070,7 @@ sp2_status fp32_solve(const float* H, int N, int N_occ, double tol, int max_iter
   A.ntiles = nt;
   A.ctl = (Ctl*)dp;
   A.rn = (double*)rn;
-  A.sums = (longlong2*)sums;
+  A.sums = (long long*)(dp + o_sums);
   A.stamps = (unsigned*)(dp + o_st);
   A.err = (int*)(dp + o_err);
   A.wait_ns = g.wait_ns;
@@ -1882,7 +1879,7 @@ struct NetRun {
     void *p0, *p1 = nullptr, *sums, *prt;
     CKS(ws(B_PLANES0, (size_t)slot_h * B * pool * 2, &p0));
     if (split) CKS(ws(B_PLANES1, (size_t)slot_h * B * pool * 2, &p1));
-    CKS(ws(B_TPART, (size_t)3 * nt * sizeof(longlong2), &sums));
+    CKS(ws(B_TPART, (size_t)B * kMeetRows * sizeof(long long), &sums));
     CKS(ws(B_PART, (size_t)B * ngrid * sizeof(double2), &prt));
     part = (double2*)prt;
     SqArgs carry;
@@ -1930,7 +1927,7 @@ struct NetRun {
     A.tiles = (const uint32_t*)(pack + o_tiles);
     A.list_off = (const int*)(pack + o_loff);
     A.list = (const int*)(pack + o_list);
-    A.sums = (longlong2*)sums;
+    A.sums = (long long*)sums;
     A.lo_scale = std::ldexp(1.0f, g.lo_scale_exp);
     A.lo_unscale = std::ldexp(1.0f, -g.lo_scale_exp);
     A.shift = g.shift;
@@ -1998,7 +1995,7 @@ struct NetRun {
       CK(cudaMemcpyAsync(*back, pack + o_status, (size_t)B * sizeof(int), cudaMemcpyDeviceToHost, st));
     }
     CK(cudaEventRecord(g.stage_done, st));  // also: the statuses are on the host
-    CK(cudaMemsetAsync(A.sums, kGangEmptyByte, (size_t)3 * nt * sizeof(longlong2), st));
+    CK(cudaMemsetAsync(A.sums, 0, (size_t)B * kMeetRows * sizeof(long long), st));
     return SP2_OK;
   }
   // the statuses of the bounds, once they are on the host

@@ -149,8 +149,7 @@ size_t syrk_tc2_smem_bytes(bool split);
 // instances' order is the same in every slot's list.
 constexpr int kResTile = 128;
 constexpr int kResStamps = kMaxL + 2;
-constexpr long long kGangEmpty = -0x7f7f7f7f7f7f7f80ll;  // no sum of a layer: every byte kGangEmptyByte
-constexpr int kGangEmptyByte = 0x80;
+constexpr int kMeetRows = 96;  // words of a gang's meeting rows
 struct ResMaps {
   CUtensorMap m[2][4];  // per plane parity: {p0, p1} with 64 x 128 boxes, {p0, p1} with 64 x 64 boxes
 };
@@ -171,8 +170,7 @@ struct ResArgs {
   float* rnp[2];           // row-norm segment sums, as SqArgs::rnp_out
   long long ld_rnp, slot_rnp;
   double2* part;           // [batch][blocks] block sums of the input layer
-  longlong2* sums;         // [3][ntiles] meeting rows of successive layers: the tiles' (tr Y', ||Y'||_F^2) in
-                           //   fixed point, kGangEmpty until published
+  long long* sums;         // [batch][kMeetRows] meeting rows (csrc/resident.cuh), zero
   double* tile_dots;       // [ntiles] Tr[D H] per tile
   double* dots_out;        // [batch][3], entry 0: Tr[D H]
   unsigned* tickets;       // [batch] zero: finished blocks of the input layer
@@ -234,7 +232,7 @@ struct NetArgs {
   const uint32_t* tiles;
   const int* list_off;     // as ResArgs
   const int* list;
-  longlong2* sums;         // [3][ntiles] kGangEmpty: meeting rows
+  long long* sums;         // [batch][kMeetRows] meeting rows, zero
   float lo_scale, lo_unscale;
   int shift, two_slots;
   int* err;
@@ -283,7 +281,7 @@ struct Res32Args {
   int ntiles;
   Ctl* ctl;
   double* rn;              // [N] row norms of the layer's input
-  longlong2* sums;         // [2][3][grid] kGangEmpty: meeting rows of the traces, of the square norms
+  long long* sums;         // [2][kMeetRows] meeting rows of the traces and of the square norms, zero
   unsigned* stamps;        // as ResArgs
   int* err;
   unsigned long long wait_ns;

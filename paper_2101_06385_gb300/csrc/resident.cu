@@ -75,8 +75,7 @@ struct Shared {
 // less than the FP64 sums did.  Anything outside (an H that is not symmetric)
 // or not a number is marked and becomes infinity or NaN in the control step.
 constexpr long long SQ_LIMIT = (1ll << 58) + (1ll << 50);  // a 32 x 32 block's 32, with rounding
-constexpr long long SQ_NAN = -1, SQ_BIG = -2;              // marks of a sum that is no number, or out of range
-constexpr double T_UNIT = 0x1p-50, Q_HI_UNIT = 0x1p-25, Q_LO_UNIT = 0x1p-53;
+constexpr long long WARP_NAN = -1, WARP_BIG = -2;          // marks of a warp's sum that is no number, or out of range
 
 __device__ __forceinline__ long long fix_sq(float v) {
   // v = hi 2^-25 + lo 2^-53, both steps exact or rounded once
@@ -264,7 +263,7 @@ __device__ __forceinline__ bool epilogue(const ResArgs& a, Shared& sh, int c, ui
       tmem_st32(ty, w);
     }
     sq = warp_sum_ll(fix_sq(sql));
-    if (nan || big || sq > SQ_LIMIT) sq = nan ? SQ_NAN : SQ_BIG;
+    if (nan || big || sq > SQ_LIMIT) sq = nan ? WARP_NAN : WARP_BIG;
     if (!outD) fence_proxy_async();  // the planes are read by the TMA units next
     if (outD) {
       if (dchunk) {
@@ -326,35 +325,6 @@ __device__ __forceinline__ bool epilogue(const ResArgs& a, Shared& sh, int c, ui
   return true;
 }
 
-// The warp's worst mark (0: every lane's sum is a number).
-__device__ __forceinline__ long long worst_mark(long long v) {
-  const bool nan = __any_sync(0xffffffffu, v == SQ_NAN), big = __any_sync(0xffffffffu, v == SQ_BIG);
-  return nan ? SQ_NAN : big ? SQ_BIG : 0;
-}
-
-// Waits for the sums of all cnt tiles of the gang (slots p[0 .. cnt)) and adds
-// them: T, and Q as 2^28 q_hi + q_lo; the next layer's products are released
-// (ready) before the sums are added.  False: abort or time-out.
-__device__ __forceinline__ bool meet(const ResArgs& a, Shared& sh, const longlong2* p, int cnt, int lane,
-                                     uint64_t* ready, long long& T, long long& q_hi, long long& q_lo, long long& bad,
-                                     unsigned long long idle) {
-  T = q_hi = q_lo = 0;
-  bad = 0;
-  if (!gather(p, cnt, lane, a.err, &sh.abort, idle, [&](const longlong2& v) {
-        T += v.x;
-        q_hi += v.y >> 28;
-        q_lo += v.y & ((1ll << 28) - 1);
-        if (v.y < 0) bad = bad == SQ_NAN ? bad : v.y;
-      }))
-    return false;
-  if (lane == 0 && ready) mbar_arrive(ready);
-  T = warp_sum_ll(T);
-  q_hi = warp_sum_ll(q_hi);
-  q_lo = warp_sum_ll(q_lo);
-  bad = worst_mark(bad);
-  return true;
-}
-
 // Control of one slot: takes the tiles of its list and drives their layers.
 __device__ __forceinline__ void control(const ResArgs& a, Shared& sh, int c, int lane, unsigned long long idle) {
   Slot& s = sh.slot[c];
@@ -370,6 +340,7 @@ __device__ __forceinline__ void control(const ResArgs& a, Shared& sh, int c, int
     s.st.load(gc, lane);  // as the input layer's control step left it
     const int cnt = a.tile_cnt[b], off = a.tile_off[b];
     const bool leader = t == off;
+    long long* rows = a.sums + (long long)b * kMeetRows;
     const bool twice = (I >> 1) != (J >> 1);  // the mirror's squares
     bool act = hot->next.active != 0;
     unsigned* st = a.stamps + (long long)b * kResStamps;
@@ -404,24 +375,27 @@ __device__ __forceinline__ void control(const ResArgs& a, Shared& sh, int c, int
         s.first = 0;
         if (cnt == 1) mbar_arrive(&sh.ready[c]);
       }
-      const long long rq = lane < EPI_WARPS ? sh.red_q[c][lane] : 0;
-      long long bad = worst_mark(rq);
-      long long T = warp_sum_ll(lane < EPI_WARPS ? sh.red_t[c][lane] : 0);
-      long long Q = warp_sum_ll(rq) << (twice ? 1 : 0);
+      // the tile's sums: squares that are no number, or out of range, are marked
+      long long rq = lane < EPI_WARPS ? sh.red_q[c][lane] : 0;
+      const long long mark = __any_sync(0xffffffffu, rq == WARP_NAN) ? SQ_NAN
+                             : __any_sync(0xffffffffu, rq == WARP_BIG) ? SQ_BIG : 0;
+      rq = warp_sum_ll(rq) << (twice ? 1 : 0);
+      GangSums G{warp_sum_ll(lane < EPI_WARPS ? sh.red_t[c][lane] : 0), mark ? mark : rq >> 28,
+                 mark ? 0 : rq & ((1ll << 28) - 1)};
       double E = 0.0;
       if (outD) E = warp_sum_d(lane < EPI_WARPS ? sh.red_e[c][lane] : 0.0);
-      long long q_hi = Q >> 28, q_lo = Q & ((1ll << 28) - 1);
       if (cnt > 1) {
         if (lane == 0) {
           if (outD) a.tile_dots[t] = E;
-          publish(a.sums, a.ntiles, k, t, T, bad ? bad : Q);
+          meet_join(rows, k, t - off, G);
         }
-        if (!meet(a, sh, a.sums + (long long)(k % 3) * a.ntiles + off, cnt, lane, outD ? nullptr : &sh.ready[c], T,
-                  q_hi, q_lo, bad, idle)) {
+        if (!meet_wait(rows, k, cnt, lane, a.err, &sh.abort, idle)) {
           ok = false;
           break;
         }
-        if (lane == 0) empty_slot(a.sums, a.ntiles, k, t);
+        if (lane == 0 && !outD) mbar_arrive(&sh.ready[c]);
+        G = meet_sums(rows, k, lane);
+        if (leader) meet_empty(rows, k, lane);
         if (outD && leader) {
           E = 0.0;
           for (int i = lane; i < cnt; i += 32) E += __ldcg(&a.tile_dots[off + i]);
@@ -429,9 +403,8 @@ __device__ __forceinline__ void control(const ResArgs& a, Shared& sh, int c, int
         }
       }
       if (lane == 0) {
-        const double off = __longlong_as_double(bad == SQ_NAN ? 0x7ff8000000000000ll : 0x7ff0000000000000ll);
-        const double trY = bad == SQ_NAN ? off : (double)T * T_UNIT;
-        const double sqY = bad ? off : (double)q_hi * Q_HI_UNIT + (double)q_lo * Q_LO_UNIT;
+        double trY, sqY;
+        to_double(G, trY, sqY);
         resident_step(s.st, trY, sqY, leader ? a.ctl + b : nullptr);
         if (!outD) mbar_arrive(&sh.coef[c]);
         if (leader) {
@@ -719,10 +692,8 @@ __global__ void __launch_bounds__(256) resident_input_kernel(const ResArgs a, in
     s_t[warp] = tr;
   }
   __syncthreads();
-  // the gang's slots of the resident launch
-  const int cnt = a.tile_cnt[b], off = a.tile_off[b];
-  for (int i = blockIdx.x * 256 + threadIdx.x; i < 3 * cnt; i += nb * 256)
-    a.sums[(long long)(i / cnt) * a.ntiles + off + i % cnt] = make_longlong2(kGangEmpty, kGangEmpty);
+  // the gang's meeting rows of the resident launch
+  if (blockIdx.x == 0 && threadIdx.x < kMeetRows) a.sums[(long long)b * kMeetRows + threadIdx.x] = 0;
   double2* part = a.part + (long long)b * gridDim.x;
   if (threadIdx.x == 0) {
     double q = 0.0, t = 0.0;

@@ -161,72 +161,97 @@ __device__ __forceinline__ long long warp_sum_ll(long long v) {
   return v;
 }
 
-// The meeting of a gang after a layer: each member publishes two words in its
-// slot of the gang's row and waits until every slot of the row is written.
-// Three rows serve successive layers: once a member has met for layer k, every
-// member has read the row of layer k - 1, so it empties its slot there, which
-// the row of layer k + 2 reuses.  (A row per reader, written by all, measured
-// 2 % faster at 144 members and 3 % slower on 512 small gangs.)
-__device__ __forceinline__ longlong2 ld_sums(const longlong2* p) {
-  longlong2 v;
-  asm volatile("ld.relaxed.gpu.global.v2.s64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "l"(p) : "memory");
+// A layer's sums over a gang in 64-bit fixed point, exact in any order: tr Y' in
+// units of 2^-50, ||Y'||_F^2 as q_hi 2^-25 + q_lo 2^-53 (q_lo of each member in
+// [0, 2^28)).  A member whose squares are no number, or out of range, adds
+// SQ_NAN or SQ_BIG to q_hi, far above any sum (N 2^25) and each other.
+struct GangSums {
+  long long t, q_hi, q_lo;
+};
+constexpr long long SQ_NAN = 1ll << 52, SQ_BIG = 1ll << 42;
+constexpr double T_UNIT = 0x1p-50, Q_HI_UNIT = 0x1p-25, Q_LO_UNIT = 0x1p-53;
+
+__device__ __forceinline__ void to_double(const GangSums& s, double& trY, double& sqY) {
+  const bool nan = s.q_hi >= SQ_NAN / 2, big = s.q_hi >= SQ_BIG / 2;
+  const double off = __longlong_as_double(nan ? 0x7ff8000000000000ll : 0x7ff0000000000000ll);
+  trY = nan ? off : (double)s.t * T_UNIT;
+  sqY = big ? off : (double)s.q_hi * Q_HI_UNIT + (double)s.q_lo * Q_LO_UNIT;
+}
+
+// The meeting of a gang after a layer.  Members add their sums and then their
+// count into one of eight sectors of the layer's row; a member waits until the
+// counts make up the gang.  Three rows serve successive layers: once a member
+// has met for layer k every member is done with the row of layer k - 1, so the
+// leader empties it then, for layer k + 2.  With a slot per member that everyone
+// polled, 144 readers (N = 2048) of 144 slots took 4 us from the last write to
+// the last read; so met, a solve takes, by calls of the public entry: N = 2048
+// single FP16 873 -> 795 us, N = 1000 748 -> 712 us, FP32 N = 512 622 -> 480 us.
+constexpr int MEET_GROUPS = 8, MEET_WORDS = 4;  // a sector: t, q_hi, count and q_lo, unused
+static_assert(3 * MEET_GROUPS * MEET_WORDS == kMeetRows, "three rows");
+constexpr int MEET_SHIFT = 40;                  // the count above q_lo (304 x 2^28 < 2^37)
+
+__device__ __forceinline__ long long* meet_row(long long* rows, int k) {
+  return rows + (k % 3) * (MEET_GROUPS * MEET_WORDS);
+}
+
+__device__ __forceinline__ void red_add(long long* p, long long v) {
+  asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+__device__ __forceinline__ long long ld_word(const long long* p) {
+  long long v;
+  asm volatile("ld.relaxed.gpu.global.s64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
   return v;
 }
-__device__ __forceinline__ void st_sums(longlong2* p, long long x, long long y) {
-  asm volatile("st.relaxed.gpu.global.v2.s64 [%0], {%1, %2};" ::"l"(p), "l"(x), "l"(y) : "memory");
-}
 
-// Member `me` publishes (x, y) in layer k's row of rows[3][stride], with
-// everything the CTA has written before (lane 0 of one warp).
-__device__ __forceinline__ void publish(longlong2* rows, long long stride, int k, int me, long long x, long long y) {
+// Member `me` joins layer k's meeting with its sums and everything the CTA has
+// written before (one thread); sums: whether there are any.
+__device__ __forceinline__ void meet_join(long long* rows, int k, int me, const GangSums& s, bool sums = true) {
+  long long* p = meet_row(rows, k) + (me % MEET_GROUPS) * MEET_WORDS;
+  if (sums) {
+    red_add(p, s.t);
+    red_add(p + 1, s.q_hi);
+  }
   __threadfence();
-  st_sums(rows + (k % 3) * stride + me, x, y);
-}
-// after the meeting of layer k
-__device__ __forceinline__ void empty_slot(longlong2* rows, long long stride, int k, int me) {
-  st_sums(rows + ((k + 2) % 3) * stride + me, kGangEmpty, kGangEmpty);
+  red_add(p + 2, (1ll << MEET_SHIFT) + s.q_lo);
 }
 
-// Waits until every slot p[0 .. cnt) is written and hands each to add (one
-// warp; lane l takes slots l, l + 32, ...).  False: abort or time-out.
-template <class Add>
-__device__ __forceinline__ bool gather(const longlong2* p, int cnt, int lane, const int* err,
-                                       const volatile int* abort_flag, unsigned long long limit, Add add) {
+// Waits (one warp) until all cnt members have joined.  False: abort or time-out.
+__device__ __forceinline__ bool meet_wait(long long* rows, int k, int cnt, int lane, const int* err,
+                                          const volatile int* abort_flag, unsigned long long limit) {
+  const long long* p = meet_row(rows, k) + (lane % MEET_GROUPS) * MEET_WORDS + 2;
   const uint64_t w0 = sp2::tc::globaltimer();
-  for (int i0 = 0; i0 < cnt; i0 += 128) {
-    longlong2 v[4];
-    bool have[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int i = i0 + 32 * u + lane;
-      have[u] = i >= cnt;
-      if (!have[u]) v[u] = ld_sums(p + i);
-    }
-    for (int spin = 0;; ++spin) {
-      bool all = true;
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        if (have[u]) continue;
-        if (v[u].x != kGangEmpty && v[u].y != kGangEmpty) {
-          have[u] = true;
-          add(v[u]);
-        } else {
-          all = false;
-          v[u] = ld_sums(p + i0 + 32 * u + lane);
-        }
-      }
-      if (__all_sync(0xffffffffu, all)) break;
-      if ((spin & 31) == 31) {
-        const bool stop =
-            *abort_flag || *(const volatile int*)err != 0 || sp2::tc::globaltimer() - w0 > limit;
-        if (__any_sync(0xffffffffu, stop)) return false;
-      }
+  for (int spin = 0;; ++spin) {
+    const int have = lane < MEET_GROUPS ? (int)(ld_word(p) >> MEET_SHIFT) : 0;
+    if ((int)__reduce_add_sync(0xffffffffu, have) >= cnt) break;
+    if ((spin & 31) == 31) {
+      const bool stop = *abort_flag || *(const volatile int*)err != 0 || sp2::tc::globaltimer() - w0 > limit;
+      if (__any_sync(0xffffffffu, stop)) return false;
     }
   }
-  __threadfence();  // what the gang wrote before its sums
+  __threadfence();  // what the gang wrote before it joined
   __syncwarp();
   return true;
 }
+
+// The sums of a meeting that is complete (one warp, in every lane).
+__device__ __forceinline__ GangSums meet_sums(long long* rows, int k, int lane) {
+  const long long* p = meet_row(rows, k) + (lane % MEET_GROUPS) * MEET_WORDS;
+  GangSums s{ld_word(p), ld_word(p + 1), ld_word(p + 2) & ((1ll << MEET_SHIFT) - 1)};
+#pragma unroll
+  for (int o = MEET_GROUPS / 2; o > 0; o >>= 1) {
+    s.t += __shfl_xor_sync(0xffffffffu, s.t, o);
+    s.q_hi += __shfl_xor_sync(0xffffffffu, s.q_hi, o);
+    s.q_lo += __shfl_xor_sync(0xffffffffu, s.q_lo, o);
+  }
+  return s;
+}
+
+// After the meeting of layer k, by the leader's warp.
+__device__ __forceinline__ void meet_empty(long long* rows, int k, int lane) {
+  __stcg(meet_row(rows, k + 2) + lane, 0ll);
+  __syncwarp();
+}
+static_assert(MEET_GROUPS * MEET_WORDS == 32, "one word a lane");
 
 }  // namespace res
 }  // namespace sp2

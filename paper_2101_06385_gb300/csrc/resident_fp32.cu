@@ -102,6 +102,14 @@ __device__ __forceinline__ double row_norms(const float* Y, long long ld, int N,
   return blk;
 }
 
+// A CTA's sum of row norms for the meeting (they are at most 1 each).
+__device__ __forceinline__ GangSums to_fixed(double q) {
+  if (isnan(q)) return GangSums{0, SQ_NAN, 0};
+  if (!(q < 0x1p15)) return GangSums{0, SQ_BIG, 0};
+  const long long hi = __double2ll_rd(q * 0x1p25);
+  return GangSums{0, hi, min((1ll << 28) - 1, __double2ll_rn((q * 0x1p25 - (double)hi) * 0x1p28))};
+}
+
 // The control warp: meetings and control steps, layer after layer.  False: abort.
 template <int TS>
 __device__ __forceinline__ bool control(const Res32Args& a, Shared<TS>& sh, int lane, unsigned long long lim) {
@@ -121,31 +129,27 @@ __device__ __forceinline__ bool control(const Res32Args& a, Shared<TS>& sh, int 
     const uint32_t ph = k & 1;
     if (!__all_sync(0xffffffffu, mbar_wait(&sh.tiles_done, ph, &sh.abort, lim))) return false;
     const bool outD = hot->next.out_mode == OUT_D;
-    long long T = warp_sum_ll(lane < FW ? sh.red_t[lane] : 0);
-    if (lane == 0) publish(a.sums, G, k, me, T, 0);
-    T = 0;
-    if (!gather(a.sums + (k % 3) * G, G, lane, a.err, ab, lim, [&](const longlong2& v) { T += v.x; })) return false;
-    if (lane == 0) {
-      if (!outD) mbar_arrive(&sh.gate);
-      empty_slot(a.sums, G, k, me);
-    }
-    T = warp_sum_ll(T);
-    double Q = 0.0;
+    const long long T = warp_sum_ll(lane < FW ? sh.red_t[lane] : 0);
+    if (lane == 0) meet_join(a.sums, k, me, GangSums{T, 0, 0});
+    if (!meet_wait(a.sums, k, G, lane, a.err, ab, lim)) return false;
+    if (lane == 0 && !outD) mbar_arrive(&sh.gate);
+    GangSums S = meet_sums(a.sums, k, lane);
+    if (me == 0) meet_empty(a.sums, k, lane);
     if (!outD) {
       if (!__all_sync(0xffffffffu, mbar_wait(&sh.rn_done, ph, &sh.abort, lim))) return false;
-      if (lane < RN_WARPS) Q = sh.red_q[lane];
-      Q = warp_sum_d(Q);
-      longlong2* norms = a.sums + 3 * G;
-      if (lane == 0) publish(norms, G, k, me, __double_as_longlong(Q), 0);
-      Q = 0.0;
-      if (!gather(norms + (k % 3) * G, G, lane, a.err, ab, lim,
-                  [&](const longlong2& v) { Q += __longlong_as_double(v.x); }))
-        return false;
-      if (lane == 0) empty_slot(norms, G, k, me);
-      Q = warp_sum_d(Q);
+      const double Q = warp_sum_d(lane < RN_WARPS ? sh.red_q[lane] : 0.0);
+      long long* norms = a.sums + kMeetRows;
+      if (lane == 0) meet_join(norms, k, me, to_fixed(Q));
+      if (!meet_wait(norms, k, G, lane, a.err, ab, lim)) return false;
+      const GangSums q = meet_sums(norms, k, lane);
+      if (me == 0) meet_empty(norms, k, lane);
+      S.q_hi = q.q_hi;
+      S.q_lo = q.q_lo;
     }
     if (lane == 0) {
-      resident_step(sh.st, (double)T * 0x1p-50, Q, me == 0 ? a.ctl : nullptr);
+      double trY, sqY;
+      to_double(S, trY, sqY);
+      resident_step(sh.st, trY, sqY, me == 0 ? a.ctl : nullptr);
       if (!outD) mbar_arrive(&sh.coef);
       if (me == 0 && k + 1 < kResStamps) a.stamps[k + 1] = (unsigned)(globaltimer() - t0);
     }

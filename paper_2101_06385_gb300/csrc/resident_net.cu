@@ -501,6 +501,7 @@ __device__ __forceinline__ void control(const NetArgs& a, Shared& sh, int c, int
     int b, I, J, h;
     unpack_tile(a.tiles[t], b, I, J, h);
     const int off = t - t % cnt;  // every matrix has the same number of tiles
+    long long* rows = a.sums + (long long)b * kMeetRows;
     // lane l holds word l of the next operation and of its coefficients
     constexpr int OW = sizeof(NetOp) / 8, PW = sizeof(LayerParams) / 8;
     static_assert(OW <= 32 && PW <= 32, "one word a lane");
@@ -542,13 +543,12 @@ __device__ __forceinline__ void control(const NetArgs& a, Shared& sh, int c, int
       }
       __syncwarp();
       if (k + 1 < a.nops && cnt > 1) {
-        if (lane == 0) publish(a.sums, a.ntiles, k, t, 1, 1);
-        if (!gather(a.sums + (long long)(k % 3) * a.ntiles + off, cnt, lane, a.err, &sh.abort, idle,
-                    [](const longlong2&) {})) {
+        if (lane == 0) meet_join(rows, k, t - off, GangSums{0, 0, 0}, false);
+        if (!meet_wait(rows, k, cnt, lane, a.err, &sh.abort, idle)) {
           ok = false;
           break;
         }
-        if (lane == 0) empty_slot(a.sums, a.ntiles, k, t);
+        if (t == off) meet_empty(rows, k, lane);
       }
       if (k + 1 < a.nops) begin();
       if (kind != 0) {  // under the next operation's products
