@@ -63,7 +63,7 @@ enum BufId {
   B_HI0, B_LO0, B_HI1, B_LO1, B_Y0, B_Y1, B_CTL, B_TILES, B_TOFF, B_TCNT, B_TPART, B_IDONE,
   B_PART, B_TICKET, B_ERR, B_DPTR, B_NS, B_HS, B_TRACES, B_PARAMS, B_BOUNDS, B_RN, B_PART2,
   B_G, B_SEG, B_GH0, B_GL0, B_GH1, B_GL1, B_DOTS, B_TDOTS, B_PARAMS2, B_NALPHA, B_HP0, B_HP1, B_RNP0, B_RNP1,
-  B_READOUT, B_RDIAG, B_SEGP, B_WAVE, B_PACK, B_PLANES0, B_PLANES1, B_COUNT
+  B_READOUT, B_RDIAG, B_SEGP, B_WAVE, B_PACK, B_PLANES0, B_PLANES1, B_OPS, B_COUNT
 };
 
 struct Buf {
@@ -221,7 +221,7 @@ sp2_status upload_tiles(int N, int B, int kind, int* ntiles_out) {
   CKS(ws(B_TILES, nt * sizeof(uint32_t), &dt));
   CKS(ws(B_TOFF, B * sizeof(int), &doff));
   CKS(ws(B_TCNT, B * sizeof(int), &dcnt));
-  CKS(ws(B_TPART, nt * sizeof(double2), &dpart));
+  CKS(ws(B_TPART, 2 * nt * sizeof(double2), &dpart));  // two halves: lists of layers
   CKS(ws(B_IDONE, B * sizeof(unsigned), &ddone, true));
   if (!(g.tiles_key_N == N && g.tiles_key_B == B && g.tiles_key_kind == kind)) {
     size_t bytes = nt * sizeof(uint32_t) + 2 * B * sizeof(int);
@@ -268,21 +268,19 @@ bool make_tmap_f16(CUtensorMap* out, const void* base, int cols, int rows, int b
 
 namespace {
 
-// Tensor maps {p0(A box), p1(A box), p0(B box), p1(B box)} for the
-// single-accumulator squaring kernels: p0 = hp = 2^s hi and p1 = lo' for the
-// split product, p0 = hi (p1 unused, null) for plain FP16.  For the CTA-pair
-// kernel (box_b = kTcBM) m holds six maps: also {p0, p1} with 64 x 64 boxes,
-// its transposed reads of the K blocks left of the diagonal.
+// Tensor maps of a plane pair: p0 = hp = 2^s hi and p1 = lo' for the split
+// product, p0 = hi (p1 unused, null) for plain FP16.  {p0, p1} with boxes of 64
+// columns x 128 rows, then {p0, p1} with 64 x rows2: the 256 B rows of the
+// single-CTA kernel, or (kTransBox) the transposed reads of the K blocks left of
+// the diagonal by the kernels that keep upper tiles.
+constexpr int kTransBox = 64;
 sp2_status tmaps4_for(const void* p0, const void* p1, int N, int B, long long ld_h, long long slot_h, CUtensorMap* m,
-                      int box_b = kTcBN) {
+                      int rows2 = kTcBN) {
   const void* p1_ = p1 ? p1 : p0;
-  bool ok = make_tmap_f16(&m[0], p0, N, N, B, ld_h, slot_h, 64, kTcBM) &&
-            make_tmap_f16(&m[1], p1_, N, N, B, ld_h, slot_h, 64, kTcBM) &&
-            make_tmap_f16(&m[2], p0, N, N, B, ld_h, slot_h, 64, box_b) &&
-            make_tmap_f16(&m[3], p1_, N, N, B, ld_h, slot_h, 64, box_b);
-  if (ok && box_b == kTcBM)
-    ok = make_tmap_f16(&m[4], p0, N, N, B, ld_h, slot_h, 64, 64) &&
-         make_tmap_f16(&m[5], p1_, N, N, B, ld_h, slot_h, 64, 64);
+  const bool ok = make_tmap_f16(&m[0], p0, N, N, B, ld_h, slot_h, 64, kTcBM) &&
+                  make_tmap_f16(&m[1], p1_, N, N, B, ld_h, slot_h, 64, kTcBM) &&
+                  make_tmap_f16(&m[2], p0, N, N, B, ld_h, slot_h, 64, rows2) &&
+                  make_tmap_f16(&m[3], p1_, N, N, B, ld_h, slot_h, 64, rows2);
   if (!ok) {
     set_err("cuTensorMapEncodeTiled failed (N=%d, ld=%lld)", N, ld_h);
     return SP2_ERR_CUDA;
@@ -335,6 +333,87 @@ sp2_status wave_counters(int ntiles, int grid, int nkt, int nlaunch, unsigned** 
   CKS(ws(B_WAVE, *per * (size_t)nlaunch * sizeof(unsigned), &wv, true));
   *wave = (unsigned*)wv;
   return SP2_OK;
+}
+
+// A pool of operand plane pairs, [entries][B] matrices of size N, for the
+// CTA-pair kernel.
+struct PlanePool {
+  __half *p0 = nullptr, *p1 = nullptr;
+  long long ld_h = 0, slot_h = 0, entry = 0;
+  CUtensorMap m[4];
+  sp2_status init(bool split, int entries, int N, int B) {
+    ld_h = round_up(N, 64);
+    slot_h = ld_h * N;
+    entry = slot_h * B;
+    void *a, *b = nullptr;
+    CKS(ws(split ? B_HP0 : B_HI0, (size_t)entry * entries * 2, &a));
+    if (split) CKS(ws(B_LO0, (size_t)entry * entries * 2, &b));
+    p0 = (__half*)a;
+    p1 = (__half*)b;
+    return tmaps4_for(p0, p1, N, B * entries, ld_h, slot_h, m, kTransBox);
+  }
+  __half* p0_of(int k) const { return p0 + entry * k; }
+  __half* p1_of(int k) const { return p1 ? p1 + entry * k : nullptr; }
+};
+
+// Lists of layers for the CTA-pair kernel (one launch each), their flags and
+// records in one device buffer, uploaded with one copy.
+struct PairLists {
+  std::vector<LayerOp> ops;
+  std::vector<int> first;  // first layer of each list
+  int B = 1;
+  uint8_t* dev = nullptr;
+  size_t o_rec = 0, o_stamps = 0, o_ops = 0, bytes = 0;
+
+  void begin() { first.push_back((int)ops.size()); }
+  // device buffer for the lists as they are; records of control steps for one list
+  sp2_status alloc(int B_, bool ctl) {
+    B = B_;
+    o_rec = round_up(2 * sizeof(unsigned) * B * first.size(), 64);
+    o_stamps = o_rec + (ctl ? (ops.size() + 1) * sizeof(LayerParams) : 0);
+    o_ops = o_stamps + (ctl ? (ops.size() + 1) * sizeof(unsigned long long) : 0);
+    bytes = o_ops + ops.size() * sizeof(LayerOp);
+    void* p;
+    CKS(ws(B_OPS, bytes, &p));
+    dev = (uint8_t*)p;
+    return SP2_OK;
+  }
+  void fill(void* host) const {
+    memset(host, 0, o_ops);
+    memcpy((uint8_t*)host + o_ops, ops.data(), ops.size() * sizeof(LayerOp));
+  }
+  // grouped: all layers of a group of instances before the next group, the
+  // smallest groups of at least 1.9 units per pair (an instance's next layer
+  // then never waits for its last), so that a group's planes and iterates stay
+  // in the 129 MB L2 from layer to layer
+  PairList list(int i, bool ctl, bool grouped, int per) const {
+    PairList l;
+    memset(&l, 0, sizeof(l));
+    l.ops = (const LayerOp*)(dev + o_ops) + first[i];
+    l.nops = (i + 1 < (int)first.size() ? first[i + 1] : (int)ops.size()) - first[i];
+    l.batch = B;
+    l.per = per;
+    if (grouped) {
+      const int need = (int)std::ceil(1.9 * (g.num_sms / 2) / per);
+      l.groups = std::max(1, B / std::max(1, need));
+    }
+    l.done = (unsigned*)dev + (size_t)2 * B * i;
+    l.step = l.done + B;
+    if (ctl) {
+      l.rec = (LayerParams*)(dev + o_rec);
+      l.stamps = (unsigned long long*)(dev + o_stamps);
+    }
+    return l;
+  }
+};
+
+// One layer, as SqArgs describes it.
+PairList one_layer(int B) {
+  PairList l;
+  memset(&l, 0, sizeof(l));
+  l.nops = 1;
+  l.batch = B;
+  return l;
 }
 
 void init_ctl(Ctl* c, int N, int n_occ, double tol, int max_iter) {
@@ -944,12 +1023,7 @@ sp2_status resident_solve(const float* const* H, const int* N, const int* N_occ,
   if (single) g.fault_stall = false;
   ResMaps maps;
   for (int k = 0; k < 2; ++k) {
-    CUtensorMap m[6];
-    CKS(tmaps4_for(A.p0[k], A.p1[k], Nmax, B, ld_h, slot_h, m, kTcBM));
-    maps.m[k][0] = m[0];
-    maps.m[k][1] = m[1];
-    maps.m[k][2] = m[4];
-    maps.m[k][3] = m[5];
+    CKS(tmaps4_for(A.p0[k], A.p1[k], Nmax, B, ld_h, slot_h, maps.m[k], kTransBox));
   }
 
   CK(cudaEventRecord(g.ev0, st));
@@ -1151,12 +1225,43 @@ sp2_status density_matrix_impl(const float* H, int N, int N_occ, double tol, int
   CKS(ws(B_RN, (size_t)N * sizeof(double), &rn));
   // Tr[D H] from the launch that writes D: per-tile partials, then the sum
   void *tdots, *dots;
-  CKS(ws(B_TDOTS, (size_t)ntiles * 3 * sizeof(double), &tdots));
+  CKS(ws(B_TDOTS, (size_t)ntiles * 2 * 3 * sizeof(double), &tdots));
   CKS(ws(B_DOTS, 3 * sizeof(double), &dots, true));
+  const bool pairs = tc && g.pair_kernel;
+  // launches enqueued (CTA pairs: layers of the list): the loop's layers plus the
+  // two of Eq. 15 (the accelerated solve has no refinement layers)
+  const int nlaunch = accel ? max_iter : max_iter + 2;
+  SqArgs A;
+  memset(&A, 0, sizeof(A));
+  PlanePool pool;
+  PairLists lists;
+  void* rnp[2];
+  if (tc) CKS(rnp_for(N, 1, A, rnp));
+  if (pairs) {
+    CKS(pool.init(split, 2, N, 1));
+    lists.begin();
+    for (int k = 0; k < nlaunch; ++k) {
+      LayerOp o;
+      memset(&o, 0, sizeof(o));
+      o.y = k & 1;
+      o.g = -1;
+      o.tri_y = 1;  // between layers only the upper triangle of Y' is kept
+      o.Yin = o.Yout = D_out;
+      o.p0_out = pool.p0_of((k & 1) ^ 1);
+      o.p1_out = pool.p1_of((k & 1) ^ 1);
+      o.rn = (const double*)rn;
+      o.rnp_out = (float*)rnp[k & 1];
+      o.rnp_in = k ? (const float*)rnp[(k - 1) & 1] : nullptr;
+      o.dots_out = (double*)dots;
+      lists.ops.push_back(o);
+    }
+    CKS(lists.alloc(1, true));
+  }
 
   // small per-call records through pinned staging
   void* h;
-  CKS(staging(sizeof(Ctl) + 64, &h));
+  const size_t rec_bytes = round_up(sizeof(Ctl) + 64, 64);
+  CKS(staging(rec_bytes + lists.bytes, &h));
   Ctl* hc = (Ctl*)h;
   init_ctl(hc, N, N_occ, tol, max_iter);
   if (accel) {
@@ -1165,9 +1270,6 @@ sp2_status density_matrix_impl(const float* H, int N, int N_occ, double tol, int
     hc->acc_lumo = lumo;
     hc->tol = tol > 0.0 ? tol : 1e-9;
   }
-  // launches enqueued: the loop's layers plus the two of Eq. 15 (the
-  // accelerated solve has no refinement layers)
-  const int nlaunch = accel ? max_iter : max_iter + 2;
   int* hn = (int*)(hc + 1);
   hn[0] = N;
   const float** hh = (const float**)(hn + 2);
@@ -1178,10 +1280,12 @@ sp2_status density_matrix_impl(const float* H, int N, int N_occ, double tol, int
   CK(cudaMemcpyAsync(ns, hn, sizeof(int), cudaMemcpyHostToDevice, st));
   CK(cudaMemcpyAsync(hs, hh, sizeof(float*), cudaMemcpyHostToDevice, st));
   CK(cudaMemcpyAsync(dptr, hd, sizeof(float*), cudaMemcpyHostToDevice, st));
+  if (pairs) {
+    lists.fill((uint8_t*)h + rec_bytes);
+    CK(cudaMemcpyAsync(lists.dev, (uint8_t*)h + rec_bytes, lists.bytes, cudaMemcpyHostToDevice, st));
+  }
   CK(cudaEventRecord(g.stage_done, st));
 
-  SqArgs A;
-  memset(&A, 0, sizeof(A));
   A.wait_ns = g.wait_ns;
   A.Dptr = (float* const*)dptr;
   A.Ns = (const int*)ns;
@@ -1212,9 +1316,17 @@ sp2_status density_matrix_impl(const float* H, int N, int N_occ, double tol, int
 
   if (tc) {
     const long long ld_h = round_up(N, 64), slot_h = ld_h * N;
-    void *hi[2], *lo[2], *hp[2];
-    CKS(planes_for(split, 0, (size_t)slot_h * 2, &hi[0], &lo[0], &hp[0]));
-    CKS(planes_for(split, 1, (size_t)slot_h * 2, &hi[1], &lo[1], &hp[1]));
+    void *hi[2] = {}, *lo[2] = {}, *hp[2] = {};
+    CUtensorMap m[2][4];
+    if (pairs) {
+      (split ? hp[0] : hi[0]) = pool.p0;
+      lo[0] = pool.p1;
+    } else {
+      for (int k = 0; k < 2; ++k) {
+        CKS(planes_for(split, k, (size_t)slot_h * 2, &hi[k], &lo[k], &hp[k]));
+        CKS(tmaps4_for(split ? hp[k] : hi[k], lo[k], N, 1, ld_h, slot_h, m[k]));
+      }
+    }
     // K2: Y_0 into D_out, split into buffer 0
     // Buffers hold N rows of ld_h columns; the tensor maps declare N x N, so
     // TMA zero-fills every element outside the matrix.
@@ -1224,55 +1336,51 @@ sp2_status density_matrix_impl(const float* H, int N, int N_occ, double tol, int
     // FP64 row norms of Y_0 and the first control step (sigma_1, IdErr_1)
     CK(launch_rownorm(D_out, N, (long long)N * N, (const int*)ns, 1, N, (double*)rn, N, (Ctl*)ctl, (double2*)part,
                       (unsigned*)tick, rgrid, st));
-    CUtensorMap m[2][6];  // four maps, six for the CTA-pair kernel
-    const int boxb = g.pair_kernel ? kTcBM : kTcBN;
-    CKS(tmaps4_for(split ? hp[0] : hi[0], lo[0], N, 1, ld_h, slot_h, m[0], boxb));
-    CKS(tmaps4_for(split ? hp[1] : hi[1], lo[1], N, 1, ld_h, slot_h, m[1], boxb));
     A.Yin = D_out;
     A.Yout = D_out;
     A.ld_y = N;
     A.slot_y = (long long)N * N;
     A.ld_h = ld_h;
     A.slot_h = slot_h;
-    const int grid = std::min(ntiles, g.num_sms) & (g.pair_kernel ? ~1 : ~0);
-    // one launch per layer: the epilogue leaves the row norms of Y' for the
-    // next launch and the last tile runs the control step
-    void* rnp[2];
-    CKS(rnp_for(N, 1, A, rnp));
+    // the epilogue leaves the row norms of Y' for the next layer and the last
+    // tile runs the control step
     A.fused_ctl = 1;
-    A.tri_y = 1;  // between launches only the upper triangle of Y' is kept
-    A.tri_planes = g.pair_kernel ? 1 : 0;  // and of the planes, where the kernel reads them so
-    // epoch counters of the soft pair synchronisation, one zeroed slice per launch
-    unsigned* wave = nullptr;
-    size_t wave_per_launch = 0;
-    A.wide = wide ? 1 : 0;
-    if (g.pair_kernel && g.wave_sync > 0) {
-      const int ncl = grid / 2, nsuper = ntiles / 2;
-      // units of work per pair: super tiles, or wide units of two
-      const long long stages = (long long)((nsuper + ncl - 1) / ncl) * ((N + 63) / 64);
-      wave_per_launch = (size_t)(stages / g.wave_sync + 2);
-      void* wv;
-      CKS(ws(B_WAVE, wave_per_launch * nlaunch * sizeof(unsigned), &wv, true));
-      wave = (unsigned*)wv;
-      A.sync_stages = g.wave_sync;
-      A.snake = g.snake;
-    }
+    A.tri_y = 1;  // between layers only the upper triangle of Y' is kept
     CK(cudaEventRecord(g.lev[0], st));
-    for (int k = 0; k < nlaunch; ++k) {
-      A.wave_ctr = wave ? wave + (size_t)k * wave_per_launch : nullptr;
-      const int cur = k & 1;
-      A.hi_out = (__half*)hi[cur ^ 1];
-      A.lo_out = (__half*)lo[cur ^ 1];
-      A.hp_out = (__half*)hp[cur ^ 1];
-      rnp_step(A, rnp, k);
-      A.stall = (k == 0 && g.fault_stall) ? 1 : 0;
+    if (pairs) {
+      // All layers in one launch.  With a launch each (N = 4096: 145 us a layer),
+      // the 58 launches after convergence took 8.9 us apiece and every layer its
+      // launch, fill and control step.
+      PairList l = lists.list(0, true, false, 0);
+      A.tri_planes = 1;
+      A.wide = wide ? 1 : 0;
+      A.stall = g.fault_stall ? 1 : 0;
       g.fault_stall = false;
-      if (g.pair_kernel)
-        CK(launch_syrk_tc2(A, m[cur], split, grid, st));
-      else
+      const int grid = std::min(wide ? ntiles / 2 : ntiles, g.num_sms) & ~1;  // every pair has a unit
+      // epoch counters of the soft pair synchronisation, one zeroed slice per
+      // layer (per pair: super tiles, or wide units of two)
+      unsigned* wave = nullptr;
+      size_t per = 0;
+      CKS(wave_counters(ntiles, grid, (N + 63) / 64, nlaunch, &wave, &per));
+      A.wave_ctr = wave;
+      l.wave_per = (int)per;
+      A.sync_stages = g.wave_sync;
+      A.snake = wave ? g.snake : 0;
+      CK(launch_syrk_tc2(A, l, false, pool.m, split, grid, st));
+    } else {
+      const int grid = std::min(ntiles, g.num_sms);
+      for (int k = 0; k < nlaunch; ++k) {
+        const int cur = k & 1;
+        A.hi_out = (__half*)hi[cur ^ 1];
+        A.lo_out = (__half*)lo[cur ^ 1];
+        A.hp_out = (__half*)hp[cur ^ 1];
+        rnp_step(A, rnp, k);
+        A.stall = (k == 0 && g.fault_stall) ? 1 : 0;
+        g.fault_stall = false;
         CK(launch_syrk_tc1(A, m[cur], split, grid, st));
-      CK(cudaEventRecord(g.lsq[k], st));
-      CK(cudaEventRecord(g.lev[k + 1], st));
+        CK(cudaEventRecord(g.lsq[k], st));
+        CK(cudaEventRecord(g.lev[k + 1], st));
+      }
     }
   } else {
     const long long ld_y = round_up(N, 4), slot_y = ld_y * N;
@@ -1302,10 +1410,13 @@ sp2_status density_matrix_impl(const float* H, int N, int N_occ, double tol, int
 
   if (!stats) return SP2_OK;
   void* hb;
-  CKS(staging(sizeof(Ctl) + 64, &hb));
+  const size_t stamp_bytes = pairs ? (nlaunch + 1) * sizeof(unsigned long long) : 0;
+  CKS(staging(rec_bytes + stamp_bytes, &hb));
   CK(cudaMemcpyAsync(hb, ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, st));
   CK(cudaMemcpyAsync((char*)hb + sizeof(Ctl), err, sizeof(int), cudaMemcpyDeviceToHost, st));
   CK(cudaMemcpyAsync((char*)hb + sizeof(Ctl) + 16, dots, sizeof(double), cudaMemcpyDeviceToHost, st));
+  if (pairs)
+    CK(cudaMemcpyAsync((char*)hb + rec_bytes, lists.dev + lists.o_stamps, stamp_bytes, cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
   float ms = 0.f;
   CK(cudaEventElapsedTime(&ms, g.ev0, g.ev1));
@@ -1317,10 +1428,15 @@ sp2_status density_matrix_impl(const float* H, int N, int N_occ, double tol, int
   float pm = 0.f;
   CK(cudaEventElapsedTime(&pm, g.ev0, g.lev[0]));
   stats->prologue_ms = pm;
+  const unsigned long long* t = (const unsigned long long*)((const char*)hb + rec_bytes);
   for (int k = 0; k < nlaunch; ++k) {
     float lm = 0.f, sm = 0.f;
-    CK(cudaEventElapsedTime(&lm, g.lev[k], g.lev[k + 1]));
-    CK(cudaEventElapsedTime(&sm, g.lev[k], g.lsq[k]));
+    if (pairs) {
+      if (t[k + 1]) lm = sm = (float)(t[k + 1] - t[k]) * 1e-6f;  // 0 past the last layer
+    } else {
+      CK(cudaEventElapsedTime(&lm, g.lev[k], g.lev[k + 1]));
+      CK(cudaEventElapsedTime(&sm, g.lev[k], g.lsq[k]));
+    }
     stats->layer_ms[k] = lm;
     stats->square_ms[k] = sm;
   }
@@ -1484,14 +1600,13 @@ sp2_status batched_once(const float* const* H, const int* N, const int* N_occ, i
   void* Y[2] = {nullptr, nullptr};
   void *hi[2] = {nullptr, nullptr}, *lo[2] = {nullptr, nullptr}, *hp[2] = {nullptr, nullptr};
   void* rnp[2] = {nullptr, nullptr};
-  CUtensorMap m[2][6];  // four maps, six for the CTA-pair kernel
+  CUtensorMap m[2][4];
   CKS(ws(B_Y0, (size_t)slot_y * B * 4, &Y[0]));
   if (tc) {
     CKS(planes_for(split, 0, (size_t)slot_h * B * 2, &hi[0], &lo[0], &hp[0]));
     CKS(planes_for(split, 1, (size_t)slot_h * B * 2, &hi[1], &lo[1], &hp[1]));
-    const int boxb = pairs ? kTcBM : kTcBN;
-    CKS(tmaps4_for(split ? hp[0] : hi[0], lo[0], Nmax, B, ld_h, slot_h, m[0], boxb));
-    CKS(tmaps4_for(split ? hp[1] : hi[1], lo[1], Nmax, B, ld_h, slot_h, m[1], boxb));
+    for (int k = 0; k < 2; ++k)
+      CKS(tmaps4_for(split ? hp[k] : hi[k], lo[k], Nmax, B, ld_h, slot_h, m[k], pairs ? kTransBox : kTcBN));
     CKS(rnp_for(Nmax, B, A, rnp));
     A.Yin = (float*)Y[0];
     A.Yout = (float*)Y[0];
@@ -1535,7 +1650,7 @@ sp2_status batched_once(const float* const* H, const int* N, const int* N_occ, i
         A.hp_out = (__half*)hp[cur ^ 1];
         rnp_step(A, rnp, k);
         if (pairs)
-          CK(launch_syrk_tc2(A, m[cur], split, grid, st));
+          CK(launch_syrk_tc2(A, one_layer(B), false, m[cur], split, grid, st));
         else
           CK(launch_syrk_tc1(A, m[cur], split, grid, st));
         CK(cudaEventRecordWithFlags(g.lsq[k], st, evf));
@@ -1942,13 +2057,7 @@ struct NetRun {
     plan.lp = (LayerParams*)(pack + o_params);
     plan.table = (double*)(pack + o_table);
     plan.status = (int*)(pack + o_status);
-    CUtensorMap m[6];
-    CKS(tmaps4_for(p0, p1, N, B * pool, ld_h, slot_h, m, kTcBM));
-    maps.m[0] = m[0];
-    maps.m[1] = m[1];
-    maps.m[2] = m[4];
-    maps.m[3] = m[5];
-    return SP2_OK;
+    return tmaps4_for(p0, p1, N, B * pool, ld_h, slot_h, maps.m, kTransBox);
   }
   const double* dev(size_t table_index) const { return (const double*)(pack + o_table) + table_index; }
 
@@ -2238,18 +2347,54 @@ sp2_status sp2_network_forward(const float* H, int B, int N, int L, const float*
   CKS(ws(B_PART, (size_t)B * igrid * sizeof(double2), &part));
   CKS(ws(B_TICKET, std::max(64, B) * sizeof(unsigned), &tick, true));
   CKS(ws(B_ERR, sizeof(int), &err, true));
+  auto ckpt_slot = [&](int k) { return ckpt + (size_t)k * B * N * N; };
+  SqArgs A;
+  memset(&A, 0, sizeof(A));
+  void* rnp[2] = {nullptr, nullptr};
+  if (tc) CKS(rnp_for(N, B, A, rnp));
+  PlanePool pool;
+  PairLists lists;
+  if (pairs) {
+    CKS(pool.init(split, 2, N, B));
+    lists.begin();
+    for (int n = 0; n < L; ++n) {
+      LayerOp o;
+      memset(&o, 0, sizeof(o));
+      o.y = n & 1;
+      o.g = -1;
+      // only the upper super tiles of Y' are stored; a checkpoint is written
+      // whole beside them
+      o.tri_y = 1;
+      o.Yin = o.Yout = X_out;
+      o.p0_out = pool.p0_of((n & 1) ^ 1);
+      o.p1_out = pool.p1_of((n & 1) ^ 1);
+      o.rn = (const double*)rn;
+      o.rnp_out = (float*)rnp[n & 1];
+      o.rnp_in = n ? (const float*)rnp[(n - 1) & 1] : nullptr;
+      o.lp = (const LayerParams*)params + (size_t)n * B;
+      if (ckpt && (n + 1) % ckpt_every == 0 && n < L - 1) {
+        o.X = ckpt_slot((n + 1) / ckpt_every);
+        o.x_add = (const double*)alpha + (size_t)(n + 1) * B;
+      }
+      lists.ops.push_back(o);
+    }
+    CKS(lists.alloc(B, false));
+  }
   void* h;
-  CKS(staging(plan.params.size() * sizeof(LayerParams) + plan.alpha.size() * sizeof(double), &h));
+  const size_t plan_bytes = plan.params.size() * sizeof(LayerParams) + plan.alpha.size() * sizeof(double);
+  CKS(staging(plan_bytes + lists.bytes, &h));
   memcpy(h, plan.params.data(), plan.params.size() * sizeof(LayerParams));
   memcpy((char*)h + plan.params.size() * sizeof(LayerParams), plan.alpha.data(), plan.alpha.size() * sizeof(double));
   CK(cudaMemcpyAsync(params, h, plan.params.size() * sizeof(LayerParams), cudaMemcpyHostToDevice, st));
   CK(cudaMemcpyAsync(alpha, (char*)h + plan.params.size() * sizeof(LayerParams), plan.alpha.size() * sizeof(double),
                      cudaMemcpyHostToDevice, st));
+  if (pairs) {
+    lists.fill((uint8_t*)h + plan_bytes);
+    CK(cudaMemcpyAsync(lists.dev, (uint8_t*)h + plan_bytes, lists.bytes, cudaMemcpyHostToDevice, st));
+  }
   CK(cudaEventRecord(g.stage_done, st));
 
   const long long slot = (long long)N * N;
-  SqArgs A;
-  memset(&A, 0, sizeof(A));
   A.wait_ns = g.wait_ns;
   A.Dptr = (float* const*)dptr;
   A.Ns = (const int*)ns;
@@ -2271,20 +2416,23 @@ sp2_status sp2_network_forward(const float* H, int B, int N, int L, const float*
   A.slot_y = slot;
   const int mgrid = (int)std::min<long long>(N, std::max(1, 4 * g.num_sms / B + 1));
   const int rgrid = (int)std::min<long long>((N + 7) / 8, std::max(1, 2 * g.num_sms / B + 1));
-  auto ckpt_slot = [&](int k) { return ckpt + (size_t)k * B * slot; };
 
   void* Y[2] = {X_out, nullptr};
   void *hi[2] = {nullptr, nullptr}, *lo[2] = {nullptr, nullptr}, *hp[2] = {nullptr, nullptr};
   long long ld_h = 0, slot_h = 0;
-  CUtensorMap m[2][6];  // four maps, six for the CTA-pair kernel
+  CUtensorMap m[2][4];
   if (tc) {
     ld_h = round_up(N, 64);
     slot_h = ld_h * N;
-    CKS(planes_for(split, 0, (size_t)slot_h * B * 2, &hi[0], &lo[0], &hp[0]));
-    CKS(planes_for(split, 1, (size_t)slot_h * B * 2, &hi[1], &lo[1], &hp[1]));
-    const int boxb = pairs ? kTcBM : kTcBN;
-    CKS(tmaps4_for(split ? hp[0] : hi[0], lo[0], N, B, ld_h, slot_h, m[0], boxb));
-    CKS(tmaps4_for(split ? hp[1] : hi[1], lo[1], N, B, ld_h, slot_h, m[1], boxb));
+    if (pairs) {
+      (split ? hp[0] : hi[0]) = pool.p0;
+      lo[0] = pool.p1;
+    } else {
+      for (int k = 0; k < 2; ++k) {
+        CKS(planes_for(split, k, (size_t)slot_h * B * 2, &hi[k], &lo[k], &hp[k]));
+        CKS(tmaps4_for(split ? hp[k] : hi[k], lo[k], N, B, ld_h, slot_h, m[k]));
+      }
+    }
     A.ld_h = ld_h;
     A.slot_h = slot_h;
   } else {
@@ -2300,8 +2448,17 @@ sp2_status sp2_network_forward(const float* H, int B, int N, int L, const float*
                         g.shift, 0, B, igrid, st));
   if (ckpt)
     CK(launch_materialize((float*)Y[0], N, slot, N, B, (const double*)alpha, ckpt_slot(0), N, slot, mgrid, st));
-  void* rnp[2] = {nullptr, nullptr};
-  if (tc) CKS(rnp_for(N, B, A, rnp));
+  if (pairs) {
+    // every layer in one launch (with one each, and the checkpoints copied by
+    // passes of their own, 64 x 2048 x 20 layers took 27 ms)
+    CK(launch_rownorm(X_out, N, slot, (const int*)ns, B, N, (double*)rn, N, nullptr, nullptr, nullptr, rgrid, st));
+    A.tri_planes = 1;
+    CK(launch_syrk_tc2(A, lists.list(0, false, true, ntiles / 2 / B), false, pool.m, split,
+                       std::min(ntiles, g.num_sms) & ~1, st));
+    if (ckpt && L % ckpt_every == 0)
+      CK(cudaMemcpyAsync(ckpt_slot(L / ckpt_every), X_out, (size_t)B * slot * 4, cudaMemcpyDeviceToDevice, st));
+    return SP2_OK;
+  }
   for (int n = 0; n < L; ++n) {
     const int cur = n & 1;
     float* Yc = (float*)Y[tc ? 0 : cur];
@@ -2313,20 +2470,14 @@ sp2_status sp2_network_forward(const float* H, int B, int N, int L, const float*
       A.Yin = X_out;
       A.Yout = X_out;
       // Only the upper super tiles of Y' are stored unless whole rows are read
-      // after this launch (a checkpoint; the last layer writes X_L whole
-      // anyway); the CTA-pair kernel reads its operands from the upper super
-      // tiles of the planes alone, so their mirror is never stored.
+      // after this launch (a checkpoint; the last layer writes X_L whole anyway)
       const bool to_ckpt = ckpt && (n + 1) % ckpt_every == 0;
       A.tri_y = to_ckpt ? 0 : 1;
-      A.tri_planes = pairs ? 1 : 0;
       A.hi_out = (__half*)hi[cur ^ 1];
       A.lo_out = (__half*)lo[cur ^ 1];
       A.hp_out = (__half*)hp[cur ^ 1];
       rnp_step(A, rnp, n);
-      if (pairs)
-        CK(launch_syrk_tc2(A, m[cur], split, std::min(ntiles, g.num_sms) & ~1, st));
-      else
-        CK(launch_syrk_tc1(A, m[cur], split, std::min(ntiles, g.num_sms), st));
+      CK(launch_syrk_tc1(A, m[cur], split, std::min(ntiles, g.num_sms), st));
     } else {
       A.Yin = Yc;
       A.Yout = (float*)Y[cur ^ 1];
@@ -2397,12 +2548,10 @@ sp2_status sp2_network_backward(const float* H, int B, int N, int L, const float
   // CTA pairs (M = 256 MMAs) unless the single-CTA kernel was selected; the
   // pair kernel keeps the operand planes as upper super tiles
   const bool pairs = g.pair_kernel;
-  const int nmap = pairs ? 6 : 4;
-  const int boxb = pairs ? kTcBM : kTcBN;
   int ntiles = 0;
   CKS(upload_tiles(N, B, pairs ? 2 : 1, &ntiles));
   const long long ld_h = round_up(N, 64), slot_h = ld_h * N;
-  void *params, *params2, *nal, *rn, *err, *seg, *segp, *gh[2], *gl[2] = {nullptr, nullptr}, *dots, *tdots;
+  void *params, *params2, *nal, *rn, *err, *seg, *segp = nullptr, *gh[2] = {}, *gl[2] = {}, *dots, *tdots;
   CKS(ws(B_PARAMS, plan.params.size() * sizeof(LayerParams), &params));
   CKS(ws(B_PARAMS2, bp.size() * sizeof(LayerParams), &params2));
   CKS(ws(B_NALPHA, nalpha.size() * sizeof(double), &nal));
@@ -2410,44 +2559,105 @@ sp2_status sp2_network_backward(const float* H, int B, int N, int L, const float
   CKS(ws(B_ERR, sizeof(int), &err, true));
   CKS(ws(B_SEG, (size_t)ce * B * slot * 4, &seg));
   // operand planes of the ce iterates of a segment, kept from the
-  // recomputation for the adjoint layers: p0 = hp (split) or hi (plain) and
-  // p1 = lo' (split only)
+  // recomputation for the adjoint layers, and of G (twice): p0 = hp (split) or
+  // hi (plain) and p1 = lo' (split only)
   const int nplanes = split ? 2 : 1;
   const size_t plane_bytes = (size_t)slot_h * B * 2;
-  CKS(ws(B_SEGP, plane_bytes * nplanes * ce, &segp));
-  CKS(ws(B_GH0, plane_bytes, &gh[0]));
-  CKS(ws(B_GH1, plane_bytes, &gh[1]));
-  if (split) {
-    CKS(ws(B_GL0, plane_bytes, &gl[0]));
-    CKS(ws(B_GL1, plane_bytes, &gl[1]));
+  PlanePool pool;  // CTA pairs: entries 0 .. ce - 1, G in ce and ce + 1
+  if (pairs) {
+    CKS(pool.init(split, ce + 2, N, B));
+  } else {
+    CKS(ws(B_SEGP, plane_bytes * nplanes * ce, &segp));
+    CKS(ws(B_GH0, plane_bytes, &gh[0]));
+    CKS(ws(B_GH1, plane_bytes, &gh[1]));
+    if (split) {
+      CKS(ws(B_GL0, plane_bytes, &gl[0]));
+      CKS(ws(B_GL1, plane_bytes, &gl[1]));
+    }
   }
   CKS(ws(B_DOTS, (size_t)L * B * 3 * sizeof(double), &dots, true));
-  CKS(ws(B_TDOTS, (size_t)ntiles * 3 * sizeof(double), &tdots));
+  CKS(ws(B_TDOTS, (size_t)ntiles * 2 * 3 * sizeof(double), &tdots));
+  SqArgs A;
+  memset(&A, 0, sizeof(A));
+  void* rnp[2];
+  CKS(rnp_for(N, B, A, rnp));  // the row-norm carry of the recomputation
+  auto segY = [&](int i) { return (float*)seg + (size_t)i * B * slot; };
+  // planes of Y_{n0 + k} and of G
+  auto segp0 = [&](int k) {
+    return pairs ? pool.p0_of(k) : (__half*)((char*)segp + plane_bytes * nplanes * k);
+  };
+  auto segp1 = [&](int k) {
+    return pairs ? pool.p1_of(k) : split ? (__half*)((char*)segp + plane_bytes * (nplanes * k + 1)) : nullptr;
+  };
+  auto g0 = [&](int k) { return pairs ? pool.p0_of(ce + k) : (__half*)gh[k]; };
+  auto g1 = [&](int k) { return pairs ? pool.p1_of(ce + k) : (__half*)gl[k]; };
+  const int nseg_layers = (L + ce - 1) / ce;
+  PairLists lists;
+  if (pairs) {
+    int gp = 0;
+    for (int sgi = nseg_layers - 1; sgi >= 0; --sgi) {
+      const int n0 = sgi * ce, n1 = std::min(n0 + ce, L);
+      lists.begin();
+      for (int n = n0; n + 1 < n1; ++n) {
+        // the recomputed iterates are read only on upper super tiles
+        const int k = n - n0;
+        LayerOp o;
+        memset(&o, 0, sizeof(o));
+        o.y = k;
+        o.g = -1;
+        o.tri_y = 1;
+        o.Yin = segY(k);
+        o.Yout = segY(k + 1);
+        o.p0_out = pool.p0_of(k + 1);
+        o.p1_out = pool.p1_of(k + 1);
+        o.rn = (const double*)rn;
+        o.rnp_out = (float*)rnp[k & 1];
+        o.rnp_in = k ? (const float*)rnp[(k - 1) & 1] : nullptr;
+        o.lp = (const LayerParams*)params + (size_t)n * B;
+        lists.ops.push_back(o);
+      }
+      for (int n = n1 - 1; n >= n0; --n, gp ^= 1) {
+        LayerOp o;
+        memset(&o, 0, sizeof(o));
+        o.y = n - n0;
+        o.g = ce + gp;
+        // G is read on upper super tiles only, except after the last adjoint
+        // layer (dL/dX_0 is returned whole)
+        o.tri_y = n == 0 ? 0 : 1;
+        o.Yin = o.Yout = (float*)G;
+        o.aux = segY(n - n0);
+        o.p0_out = pool.p0_of(ce + (gp ^ 1));
+        o.p1_out = pool.p1_of(ce + (gp ^ 1));
+        o.lp = (const LayerParams*)params2 + (size_t)n * B;
+        o.dots_out = (double*)dots + (size_t)n * B * 3;
+        lists.ops.push_back(o);
+      }
+    }
+    CKS(lists.alloc(B, false));
+  }
   void* h;
   const size_t pb = plan.params.size() * sizeof(LayerParams), bb2 = bp.size() * sizeof(LayerParams),
                ab = nalpha.size() * sizeof(double);
-  CKS(staging(pb + bb2 + ab, &h));
+  CKS(staging(pb + bb2 + ab + lists.bytes, &h));
   memcpy(h, plan.params.data(), pb);
   memcpy((char*)h + pb, bp.data(), bb2);
   memcpy((char*)h + pb + bb2, nalpha.data(), ab);
   CK(cudaMemcpyAsync(params, h, pb, cudaMemcpyHostToDevice, st));
   CK(cudaMemcpyAsync(params2, (char*)h + pb, bb2, cudaMemcpyHostToDevice, st));
   CK(cudaMemcpyAsync(nal, (char*)h + pb + bb2, ab, cudaMemcpyHostToDevice, st));
+  if (pairs) {
+    lists.fill((char*)h + pb + bb2 + ab);
+    CK(cudaMemcpyAsync(lists.dev, (char*)h + pb + bb2 + ab, lists.bytes, cudaMemcpyHostToDevice, st));
+  }
   CK(cudaEventRecord(g.stage_done, st));
 
-  // operand planes: Y_n and G as hp = 2^s hi and lo' (split) or hi (plain);
-  // the planes of Y_{n0 + k} are segp0(k) / segp1(k), those of G live in gh
-  // (hp or hi) and gl (lo')
-  auto segp0 = [&](int k) { return (__half*)((char*)segp + plane_bytes * nplanes * k); };
-  auto segp1 = [&](int k) { return split ? (__half*)((char*)segp + plane_bytes * (nplanes * k + 1)) : nullptr; };
-  std::vector<CUtensorMap> mY((size_t)ce * 6);
-  for (int k = 0; k < ce; ++k) CKS(tmaps4_for(segp0(k), segp1(k), N, B, ld_h, slot_h, &mY[(size_t)k * 6], boxb));
-  CUtensorMap mG4[2][6];
-  CKS(tmaps4_for(gh[0], gl[0], N, B, ld_h, slot_h, mG4[0], boxb));
-  CKS(tmaps4_for(gh[1], gl[1], N, B, ld_h, slot_h, mG4[1], boxb));
+  std::vector<CUtensorMap> mY(pairs ? 0 : (size_t)ce * 4);
+  CUtensorMap mG4[2][4];
+  if (!pairs) {
+    for (int k = 0; k < ce; ++k) CKS(tmaps4_for(segp0(k), segp1(k), N, B, ld_h, slot_h, &mY[(size_t)k * 4]));
+    for (int k = 0; k < 2; ++k) CKS(tmaps4_for(gh[k], gl[k], N, B, ld_h, slot_h, mG4[k]));
+  }
   const float ls = std::ldexp(1.0f, g.lo_scale_exp);
-  SqArgs A;
-  memset(&A, 0, sizeof(A));
   A.wait_ns = g.wait_ns;
   A.Dptr = (float* const*)dptr;
   A.Ns = (const int*)ns;
@@ -2469,16 +2679,12 @@ sp2_status sp2_network_backward(const float* H, int B, int N, int L, const float
   const int mgrid = (int)std::min<long long>(N, std::max(1, 4 * g.num_sms / B + 1));
   const int rgrid = (int)std::min<long long>((N + 7) / 8, std::max(1, 2 * g.num_sms / B + 1));
   const int tgrid = std::min(ntiles, g.num_sms) & (pairs ? ~1 : ~0);
-  auto segY = [&](int i) { return (float*)seg + (size_t)i * B * slot; };
-  void* rnp[2];
-  SqArgs R0 = A;  // row-norm carry of the recomputation (rnp_for sets its strides)
-  CKS(rnp_for(N, B, R0, rnp));
+  const SqArgs& R0 = A;
 
   CK(cudaMemcpyAsync(G, G_out, (size_t)B * slot * 4, cudaMemcpyDeviceToDevice, st));
-  CK(launch_split_pad((float*)G, N, slot, N, B, ls, split ? nullptr : (__half*)gh[0], (__half*)gl[0],
-                      split ? (__half*)gh[0] : nullptr, ld_h, slot_h, sgrid, st));
+  CK(launch_split_pad((float*)G, N, slot, N, B, ls, split ? nullptr : g0(0), g1(0), split ? g0(0) : nullptr, ld_h,
+                      slot_h, sgrid, st));
   int cur = 0;
-  const int nseg_layers = (L + ce - 1) / ce;
 
   for (int sgi = nseg_layers - 1; sgi >= 0; --sgi) {
     const int n0 = sgi * ce, n1 = std::min(n0 + ce, L);
@@ -2491,6 +2697,17 @@ sp2_status sp2_network_backward(const float* H, int B, int N, int L, const float
                         ld_h, slot_h, sgrid, st));
     if (n1 - n0 > 1)
       CK(launch_rownorm(segY(0), N, slot, (const int*)ns, B, N, (double*)rn, N, nullptr, nullptr, nullptr, rgrid, st));
+    if (pairs) {
+      // the segment's recomputation and adjoint layers in one launch
+      SqArgs P = A;
+      P.tri_planes = 1;
+      P.tile_dots = (double*)tdots;
+      P.rn = (const double*)rn;
+      P.ld_rn = N;
+      CK(launch_syrk_tc2(P, lists.list(nseg_layers - 1 - sgi, false, true, ntiles / 2 / B), true, pool.m, split, tgrid,
+                         st));
+      continue;
+    }
     for (int n = n0; n + 1 < n1; ++n) {
       const int k = n - n0;
       SqArgs F = R0;
@@ -2507,30 +2724,15 @@ sp2_status sp2_network_backward(const float* H, int B, int N, int L, const float
       // the recomputed iterates are read only on upper super tiles (the next
       // layer's old values, the adjoint epilogue's aux)
       F.tri_y = 1;
-      F.tri_planes = pairs ? 1 : 0;
-      if (pairs)
-        CK(launch_syrk_tc2(F, &mY[(size_t)k * 6], split, tgrid, st));
-      else
-        CK(launch_syrk_tc1(F, &mY[(size_t)k * 6], split, tgrid, st));
+      CK(launch_syrk_tc1(F, &mY[(size_t)k * 4], split, tgrid, st));
     }
     for (int n = n1 - 1; n >= n0; --n) {
       const int k = n - n0;
       float* Yn = segY(k);
-      const CUtensorMap* mYk = &mY[(size_t)k * 6];
+      const CUtensorMap* mYk = &mY[(size_t)k * 4];
       const CUtensorMap* mGk = mG4[cur];
-      // segment 1: Y_n rows x G rows (Y G), segment 2: G rows x Y_n rows (G Y);
-      // the pair kernel takes per segment {A, A lo, B, B lo, A transposed,
-      // A lo transposed} and reads B's transposed blocks through the other
-      // segment's A maps
-      CUtensorMap m8[12];
-      if (pairs) {
-        const CUtensorMap t[12] = {mYk[0], mYk[1], mGk[2], mGk[3], mYk[4], mYk[5],
-                                   mGk[0], mGk[1], mYk[2], mYk[3], mGk[4], mGk[5]};
-        for (int i = 0; i < 12; ++i) m8[i] = t[i];
-      } else {
-        const CUtensorMap t[8] = {mYk[0], mYk[1], mGk[2], mGk[3], mGk[0], mGk[1], mYk[2], mYk[3]};
-        for (int i = 0; i < 8; ++i) m8[i] = t[i];
-      }
+      // segment 1: Y_n rows x G rows (Y G), segment 2: G rows x Y_n rows (G Y)
+      const CUtensorMap m8[8] = {mYk[0], mYk[1], mGk[2], mGk[3], mGk[0], mGk[1], mYk[2], mYk[3]};
       SqArgs Bk = A;
       Bk.Yin = (float*)G;
       Bk.Yout = (float*)G;
@@ -2546,11 +2748,7 @@ sp2_status sp2_network_backward(const float* H, int B, int N, int L, const float
       // G is read on upper super tiles only, except after the last adjoint
       // layer (dL/dX_0 is returned whole)
       Bk.tri_y = n == 0 ? 0 : 1;
-      Bk.tri_planes = pairs ? 1 : 0;
-      if (pairs)
-        CK(launch_syrk_tc2(Bk, m8, split, tgrid, st));
-      else
-        CK(launch_syrk_tc1(Bk, m8, split, tgrid, st));
+      CK(launch_syrk_tc1(Bk, m8, split, tgrid, st));
       cur ^= 1;
     }
   }
@@ -2731,9 +2929,36 @@ sp2_status sp2_fermi_expansion(const float* H, int B, int N, int L, const double
   CKS(ws(B_RDIAG, (size_t)B * sizeof(double), &dd));
   CKS(ws(B_READOUT, (size_t)B * slot * sizeof(float), &R));
   CKS(ws(B_RN, (size_t)B * N * sizeof(double), &rn));
+  SqArgs A;
+  memset(&A, 0, sizeof(A));
+  void* rnp[2];
+  CKS(rnp_for(N, B, A, rnp));
+  PlanePool pool;
+  CKS(pool.init(split, 2, N, B));
+  PairLists lists;
+  lists.begin();
+  for (int n = 0; n < L; ++n) {
+    LayerOp o;
+    memset(&o, 0, sizeof(o));
+    o.y = n & 1;
+    o.g = -1;
+    o.tri_y = 1;  // between layers only the upper triangle of Y' is kept
+    o.Yin = o.Yout = D_out;
+    o.p0_out = pool.p0_of((n & 1) ^ 1);
+    o.p1_out = pool.p1_of((n & 1) ^ 1);
+    o.rn = (const double*)rn;
+    o.rnp_out = (float*)rnp[n & 1];
+    o.rnp_in = n ? (const float*)rnp[(n - 1) & 1] : nullptr;
+    o.lp = (const LayerParams*)prm + (size_t)n * B;
+    lists.ops.push_back(o);
+  }
+  CKS(lists.alloc(B, false));
   {
     void* h;
-    CKS(staging(params.size() * sizeof(LayerParams) + (size_t)B * sizeof(double), &h));
+    const size_t plan_bytes = params.size() * sizeof(LayerParams) + (size_t)B * sizeof(double);
+    CKS(staging(plan_bytes + lists.bytes, &h));
+    lists.fill((char*)h + plan_bytes);
+    CK(cudaMemcpyAsync(lists.dev, (char*)h + plan_bytes, lists.bytes, cudaMemcpyHostToDevice, st));
     memcpy(h, params.data(), params.size() * sizeof(LayerParams));
     memcpy((char*)h + params.size() * sizeof(LayerParams), d0.data(), (size_t)B * sizeof(double));
     CK(cudaMemcpyAsync(prm, h, params.size() * sizeof(LayerParams), cudaMemcpyHostToDevice, st));
@@ -2742,15 +2967,6 @@ sp2_status sp2_fermi_expansion(const float* H, int B, int N, int L, const double
     CK(cudaEventRecord(g.stage_done, st));
   }
   const long long ld_h = round_up(N, 64), slot_h = ld_h * N;
-  void *hi[2], *lo[2], *hp[2];
-  CKS(planes_for(split, 0, (size_t)slot_h * B * 2, &hi[0], &lo[0], &hp[0]));
-  CKS(planes_for(split, 1, (size_t)slot_h * B * 2, &hi[1], &lo[1], &hp[1]));
-  CUtensorMap m[2][6];  // four maps, six for the CTA-pair kernel
-  CKS(tmaps4_for(split ? hp[0] : hi[0], lo[0], N, B, ld_h, slot_h, m[0], kTcBM));
-  CKS(tmaps4_for(split ? hp[1] : hi[1], lo[1], N, B, ld_h, slot_h, m[1], kTcBM));
-
-  SqArgs A;
-  memset(&A, 0, sizeof(A));
   A.wait_ns = g.wait_ns;
   A.Dptr = (float* const*)dptr;
   A.Ns = (const int*)ns;
@@ -2773,35 +2989,16 @@ sp2_status sp2_fermi_expansion(const float* H, int B, int N, int L, const double
   A.ld_h = ld_h;
   A.slot_h = slot_h;
   A.R = (float*)R;
-  A.tri_y = 1;       // between launches only the upper triangle of Y' is kept
-  A.tri_planes = 1;  // and of the planes (the CTA-pair kernel)
-  void* rnp[2];
-  CKS(rnp_for(N, B, A, rnp));
+  A.tri_planes = 1;  // upper super tiles only
 
   // S_0 (shifted form) into D_out and its planes, R_0 = c_0 X_0, row norms of Y_0
-  CK(launch_input_layer((const float* const*)hs, (const int*)ns, N, D_out, N, slot, (__half*)hi[0], (__half*)lo[0],
-                        (__half*)hp[0], ld_h, slot_h, N, (int)ld_h, A.lo_scale, (Ctl*)ctl, nullptr, (double2*)part,
-                        (unsigned*)tick, 1, 0, B, igrid, st));
+  CK(launch_input_layer((const float* const*)hs, (const int*)ns, N, D_out, N, slot, split ? nullptr : pool.p0,
+                        pool.p1, split ? pool.p0 : nullptr, ld_h, slot_h, N, (int)ld_h, A.lo_scale, (Ctl*)ctl,
+                        nullptr, (double2*)part, (unsigned*)tick, 1, 0, B, igrid, st));
   CK(launch_readout_init(D_out, N, slot, N, B, (float)(-c[0]), (const double*)dd, (float*)R, igrid, st));
   CK(launch_rownorm(D_out, N, slot, (const int*)ns, B, N, (double*)rn, N, nullptr, nullptr, nullptr, rgrid, st));
-  const int grid = std::min(ntiles, g.num_sms) & ~1;
-  // the pairs keep their K progress loosely in step, as in the single solve
-  // (measured: 15.1-15.2 -> 14.7-14.8 ms at B = 64, N = 2048, 11 layers; the
-  // network's layers gain nothing from it and its adjoint loses 1.5 %)
-  unsigned* wave = nullptr;
-  size_t wave_per = 0;
-  CKS(wave_counters(ntiles, grid, (N + 63) / 64, L, &wave, &wave_per));
-  A.sync_stages = wave ? g.wave_sync : 0;
-  for (int n = 0; n < L; ++n) {
-    const int cur = n & 1;
-    A.wave_ctr = wave ? wave + (size_t)n * wave_per : nullptr;
-    A.lp = (const LayerParams*)prm + (size_t)n * B;
-    A.hi_out = (__half*)hi[cur ^ 1];
-    A.lo_out = (__half*)lo[cur ^ 1];
-    A.hp_out = (__half*)hp[cur ^ 1];
-    rnp_step(A, rnp, n);
-    CK(launch_syrk_tc2(A, m[cur], split, grid, st));
-  }
+  CK(launch_syrk_tc2(A, lists.list(0, false, true, ntiles / 2 / B), false, pool.m, split,
+                     std::min(ntiles, g.num_sms) & ~1, st));
   return SP2_OK;
 }
 

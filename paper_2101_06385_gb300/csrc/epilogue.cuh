@@ -76,12 +76,33 @@ __device__ __forceinline__ uint32_t pack_h2(__half a, __half b) {
   return (uint32_t)__half_as_ushort(a) | ((uint32_t)__half_as_ushort(b) << 16);
 }
 
+// The layer of a launch of one layer.
+__device__ __forceinline__ LayerOp layer_of(const SqArgs& a, bool split) {
+  LayerOp o;
+  o.y = 0;
+  o.g = -1;
+  o.tri_y = a.tri_y;
+  o.Yin = a.Yin;
+  o.Yout = a.Yout;
+  o.aux = a.aux;
+  o.p0_out = split ? a.hp_out : a.hi_out;
+  o.p1_out = a.lo_out;
+  o.rn = a.rn;
+  o.rnp_in = a.rnp_in;
+  o.rnp_out = a.rnp_out;
+  o.lp = a.lp;
+  o.dots_out = a.dots_out;
+  o.X = nullptr;
+  o.x_add = nullptr;
+  return o;
+}
+
 // (Y^2)_rr = sum_k Y_rk^2 of the input iterate: from the FP64 row norms, or
 // summed in FP64 from the FP32 segment sums the previous launch left (eight
 // accumulators over interleaved segments, combined in a fixed order).
-__device__ __forceinline__ double row_norm(const SqArgs& a, int b, int N, int r) {
-  if (!a.rnp_in) return a.rn ? a.rn[(long long)b * a.ld_rn + r] : 0.0;
-  const float* p = a.rnp_in + (long long)b * a.slot_rnp + r;
+__device__ __forceinline__ double row_norm(const SqArgs& a, const LayerOp& o, int b, int N, int r) {
+  if (!o.rnp_in) return o.rn ? o.rn[(long long)b * a.ld_rn + r] : 0.0;
+  const float* p = o.rnp_in + (long long)b * a.slot_rnp + r;
   const int nseg = (N + 31) >> 5;
   double acc[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
   int s = 0;
@@ -159,14 +180,14 @@ __device__ __forceinline__ float lane_sums(float (&s)[N_]) {
   return s[0];
 }
 
-// Tile t with accumulator use `it` (buffer it & 1).  Returns 0 when the
-// tile's instance is inactive (nothing issued for it), 1 when done, -1 when
-// the accumulator wait failed.
-// ADJ (adjoint mode, a.aux set): the tile also accumulates, over its part
+// Tile t of layer o with coefficients p and accumulator use `it` (buffer it &
+// 1).  False when the accumulator wait failed.
+// ADJ (adjoint mode, o.aux set): the tile also accumulates, over its part
 // of the full symmetric matrices, tr Yin, <Yin, aux> and <P, aux> on the
 // old values, summed per instance into a.dots_out.
 // RO (readout mode, a.R set): R += rc X' on the upper tiles, D = I - R in
 // the launch that writes D (finite-temperature expansion).
+// KEEP: o.X may be set.
 // PAIR (CTA-pair kernels): the accumulator was written by the pair's MMA
 // issuer in the even CTA, and the release of a buffer is an arrive on that
 // CTA's barrier, empty_cl + 8 x buffer (a shared::cluster address).
@@ -179,15 +200,14 @@ __device__ __forceinline__ float lane_sums(float (&s)[N_]) {
 // aux then covers four whole 128-byte row segments.  Stores of the mirror
 // block go back through the buffer to the row-per-lane layout, where they
 // are contiguous too.
-template <bool SPLIT, bool ADJ = false, bool RO = false, bool PAIR = false>
-__device__ __forceinline__ int tile(const SqArgs& a, int t, uint32_t it, uint32_t tmem_base, uint64_t* tmem_full,
-                                    uint64_t* tmem_empty, volatile int* abort_flag, Shared& sh, int ew, int q,
-                                    int lane, float* trb, uint32_t empty_cl = 0u) {
+template <bool SPLIT, bool ADJ = false, bool RO = false, bool PAIR = false, bool KEEP = false>
+__device__ __forceinline__ bool tile(const SqArgs& a, const LayerOp& o, const LayerParams& p, int t, uint32_t it,
+                                     uint32_t tmem_base, uint64_t* tmem_full, uint64_t* tmem_empty,
+                                     volatile int* abort_flag, Shared& sh, int ew, int q, int lane, float* trb,
+                                     uint32_t empty_cl = 0u) {
   using namespace sp2::tc;
   int b, I, J, h;
   unpack_tile(a.tiles[t], b, I, J, h);
-  const LayerParams p = load_params(a, b);
-  if (!p.active) return 0;
   const int N = a.Ns[b];
   const int hc = ew >> 2;
   const int R0 = I * BN + h * BM + q * 32;  // first of the warp's 32 rows
@@ -197,8 +217,8 @@ __device__ __forceinline__ int tile(const SqArgs& a, int t, uint32_t it, uint32_
   // split: the accumulator holds 2^(2s) P (both operand planes scaled by 2^s)
   const float unscale = SPLIT ? a.lo_unscale * a.lo_unscale : 1.f;
   const float lo_scale = a.lo_scale;
-  float* Y = a.Yout + (long long)b * a.slot_y;
-  const float* Yold = a.Yin + (long long)b * a.slot_y;
+  float* Y = o.Yout + (long long)b * a.slot_y;
+  const float* Yold = o.Yin + (long long)b * a.slot_y;
   const long long ld = a.ld_y;
   const int cbase = J * BN + hc * 128;      // first column of the warp's half
   const int r4 = lane >> 3, c4 = lane & 7;
@@ -209,7 +229,7 @@ __device__ __forceinline__ int tile(const SqArgs& a, int t, uint32_t it, uint32_
   double rn_l = 0.0;
   const int rdiag = R0 + 4 * c4 + r4;
   const bool dwarp = !mirror && (unsigned)(R0 - cbase) < 128u;  // the warp's columns hold its diagonal
-  if (dwarp && rdiag < N) rn_l = row_norm(a, b, N, rdiag);
+  if (dwarp && rdiag < N) rn_l = row_norm(a, o, b, N, rdiag);
   if (lane < nrows) {
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
@@ -225,25 +245,25 @@ __device__ __forceinline__ int tile(const SqArgs& a, int t, uint32_t it, uint32_
   if (!got) {
     if (lane == 0) atomicExch(a.err, (int)SP2_ERR_DEVICE_TIMEOUT);
     *abort_flag = 1;
-    return -1;
+    return false;
   }
   tc_fence_after();
 
-  float* rnp = a.rnp_out ? a.rnp_out + (long long)b * a.slot_rnp : nullptr;
-  __half* ho = a.hi_out ? a.hi_out + (long long)b * a.slot_h : nullptr;
-  __half* lo_ = a.lo_out ? a.lo_out + (long long)b * a.slot_h : nullptr;
-  __half* hp_ = a.hp_out ? a.hp_out + (long long)b * a.slot_h : nullptr;
-  // the plane scaled like the accumulator's operands: hp for split, hi for plain
-  __half* const pa_out = SPLIT ? hp_ : ho;
+  float* rnp = o.rnp_out ? o.rnp_out + (long long)b * a.slot_rnp : nullptr;
+  // the plane scaled like the accumulator's operands (hp for split, hi for plain) and lo'
+  __half* const pa_out = o.p0_out ? o.p0_out + (long long)b * a.slot_h : nullptr;
+  __half* const lo_ = o.p1_out ? o.p1_out + (long long)b * a.slot_h : nullptr;
   const long long ldh = a.ld_h;
   float* D = outD ? a.Dptr[b] : nullptr;
   // 16-byte accesses where every row start of the matrix is 16-byte aligned:
   // Y, Y_old (and R, aux) with leading dimension ld; D and H with N
   const float* Rb0 = RO ? a.R + (long long)b * a.slot_y : nullptr;
-  const float* Xb0 = ADJ ? a.aux + (long long)b * a.slot_y : nullptr;
+  const float* Xb0 = ADJ ? o.aux + (long long)b * a.slot_y : nullptr;
+  float* const X = (KEEP && o.X) ? o.X + (long long)b * a.slot_y : nullptr;
   const bool vec_y = (ld & 3) == 0 &&
                      ((reinterpret_cast<uintptr_t>(Y) | reinterpret_cast<uintptr_t>(Yold) |
-                       reinterpret_cast<uintptr_t>(Rb0) | reinterpret_cast<uintptr_t>(Xb0)) & 15) == 0;
+                       reinterpret_cast<uintptr_t>(Rb0) | reinterpret_cast<uintptr_t>(Xb0) | reinterpret_cast<uintptr_t>(X)) &
+                      15) == 0;
   const float* Hb0 = (outD && !ADJ && a.Hobs) ? a.Hobs[b] : nullptr;
   const bool vec_n = (N & 3) == 0 &&
                      ((reinterpret_cast<uintptr_t>(D) | reinterpret_cast<uintptr_t>(Hb0)) & 15) == 0;
@@ -257,7 +277,7 @@ __device__ __forceinline__ int tile(const SqArgs& a, int t, uint32_t it, uint32_
   const int kpad = (N + 63) & ~63;
   const bool rows_live = nrows > 0;
   // mirror blocks stored in this launch (off-diagonal tiles only)
-  const bool mir_y = mirror && (outD || !a.tri_y);
+  const bool mir_y = mirror && (outD || !o.tri_y || X);
   const bool mir_p = mirror && !outD && !a.tri_planes && (pa_out || lo_);
 
 #pragma unroll 1
@@ -284,12 +304,12 @@ __device__ __forceinline__ int tile(const SqArgs& a, int t, uint32_t it, uint32_
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       const bool rok = 4 * i + r4 < nrows;
-      const float4 o = rok ? ld4(Yold + (long long)(R0 + 4 * i + r4) * ld + ce, ce, N, vec_y)
+      const float4 v = rok ? ld4(Yold + (long long)(R0 + 4 * i + r4) * ld + ce, ce, N, vec_y)
                            : make_float4(0.f, 0.f, 0.f, 0.f);
-      y[4 * i] = o.x;
-      y[4 * i + 1] = o.y;
-      y[4 * i + 2] = o.z;
-      y[4 * i + 3] = o.w;
+      y[4 * i] = v.x;
+      y[4 * i + 1] = v.y;
+      y[4 * i + 2] = v.z;
+      y[4 * i + 3] = v.w;
     }
     {
       uint32_t v[32];
@@ -332,7 +352,7 @@ __device__ __forceinline__ int tile(const SqArgs& a, int t, uint32_t it, uint32_
           float x[4] = {0.f, 0.f, 0.f, 0.f};
           if (4 * i + r4 < nrows) {
             const float4 xv =
-                ld4(a.aux + (long long)b * a.slot_y + (long long)(R0 + 4 * i + r4) * ld + ce, ce, N, vec_y);
+                ld4(Xb0 + (long long)(R0 + 4 * i + r4) * ld + ce, ce, N, vec_y);
             x[0] = xv.x;
             x[1] = xv.y;
             x[2] = xv.z;
@@ -367,7 +387,7 @@ __device__ __forceinline__ int tile(const SqArgs& a, int t, uint32_t it, uint32_
     double yd = 0.0;
     if (dchunk) {
       if (dlane) {
-        const double pd = (a.rn || a.rnp_in) ? rn_l : (double)p_d;
+        const double pd = (o.rn || o.rnp_in) ? rn_l : (double)p_d;
         yd = p.ca_d * (double)yold_d + p.cb_d * pd + p.cc_d;
         tr += yd;
         ydo = outD ? (float)(yd + p.alpha_out) : (float)yd;
@@ -476,6 +496,18 @@ __device__ __forceinline__ int tile(const SqArgs& a, int t, uint32_t it, uint32_
         if (4 * i + r4 < nrows)
           st4(Y + (long long)(R0 + 4 * i + r4) * ld + ce, make_float4(y[4 * i], y[4 * i + 1], y[4 * i + 2], y[4 * i + 3]),
               ce, N, vec_y);
+      if (X) {
+        // X' = Y' + x_add I (the diagonal in FP64)
+        const float xd = dlane ? (float)((double)(float)yd + o.x_add[b]) : 0.f;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          float v[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) v[e] = dlane && 4 * i + e == id ? xd : y[4 * i + e];
+          if (4 * i + r4 < nrows)
+            st4(X + (long long)(R0 + 4 * i + r4) * ld + ce, make_float4(v[0], v[1], v[2], v[3]), ce, N, vec_y);
+        }
+      }
     }
     // FP16 planes of Y' (Eq. 12): the row segments, four halves per plane and
     // lane (columns up to the padded row length carry zeros)
@@ -512,11 +544,11 @@ __device__ __forceinline__ int tile(const SqArgs& a, int t, uint32_t it, uint32_
       __syncwarp();
 #pragma unroll
       for (int m = 0; m < 8; ++m) {
-        const float4 o = *tr_at(trb, lane, m);
-        y[4 * m] = o.x;
-        y[4 * m + 1] = o.y;
-        y[4 * m + 2] = o.z;
-        y[4 * m + 3] = o.w;
+        const float4 v = *tr_at(trb, lane, m);
+        y[4 * m] = v.x;
+        y[4 * m + 1] = v.y;
+        y[4 * m + 2] = v.z;
+        y[4 * m + 3] = v.w;
       }
       __syncwarp();
       if (lane < nrows) {
@@ -529,7 +561,7 @@ __device__ __forceinline__ int tile(const SqArgs& a, int t, uint32_t it, uint32_
               if (outD)
                 D[(long long)c * N + r] = y[k];
               else
-                Y[(long long)c * ld + r] = y[k];
+                (X ? X : Y)[(long long)c * ld + r] = y[k];
             }
             if (mir_p) {
               __half hh, ll;
@@ -557,6 +589,7 @@ __device__ __forceinline__ int tile(const SqArgs& a, int t, uint32_t it, uint32_
     dgy = warp_sum_d(dgy);
     dpy = warp_sum_d(dpy);
   }
+  __syncwarp();  // the warp's stores come before lane 0's arrival
   const int slot = (int)(it & (SLOTS - 1));
   unsigned last = 0;
   if (lane == 0) {
@@ -600,15 +633,16 @@ __device__ __forceinline__ int tile(const SqArgs& a, int t, uint32_t it, uint32_
       atomicExch(a.err, (int)SP2_ERR_DEVICE_TIMEOUT);
     }
   }
-  return 1;
+  return true;
 }
 
 // The finisher warp's work for one active tile: waits for the tile's entry
-// (the it-th of the CTA), writes its per-tile sums and runs
-// finish_tile_warp (the instance's control step after its last tile).
-// False on an abort.
-__device__ __forceinline__ bool finish_entry(const SqArgs& a, uint32_t it, Shared& sh, volatile int* abort_flag,
-                                             int lane, unsigned long long lim) {
+// (the it-th of the CTA), writes its per-tile dots to tile_dots and hands its
+// sums to finish(entry).  False on an abort.
+template <class Finish>
+__device__ __forceinline__ bool finish_entry(const SqArgs& a, double* tile_dots, uint32_t it, Shared& sh,
+                                             volatile int* abort_flag, int lane, unsigned long long lim,
+                                             Finish finish) {
   using namespace sp2::tc;
   const uint32_t e = it % FQ;
   if (!__all_sync(0xffffffffu, mbar_wait(&sh.fin_full[e], (it / FQ) & 1u, abort_flag, lim))) {
@@ -618,13 +652,13 @@ __device__ __forceinline__ bool finish_entry(const SqArgs& a, uint32_t it, Share
   }
   const FinEntry f = sh.fq[e];
   if (lane == 0 && f.dots) {
-    a.tile_dots[3 * (long long)f.t + 0] = f.d0;
-    a.tile_dots[3 * (long long)f.t + 1] = f.d1;
-    a.tile_dots[3 * (long long)f.t + 2] = f.d2;
+    tile_dots[3 * (long long)f.t + 0] = f.d0;
+    tile_dots[3 * (long long)f.t + 1] = f.d1;
+    tile_dots[3 * (long long)f.t + 2] = f.d2;
   }
   __syncwarp();
   if (lane == 0) mbar_arrive(&sh.fin_empty[e]);
-  finish_tile_warp(a, f.t, f.b, f.T, f.Q, f.out_mode);
+  finish(f);
   return true;
 }
 
@@ -640,28 +674,11 @@ __device__ __forceinline__ void finisher(const SqArgs& a, int first, int stride,
     int b, I, J, h;
     unpack_tile(a.tiles[t], b, I, J, h);
     if (!load_params(a, b).active) continue;
-    if (!finish_entry(a, it, sh, abort_flag, lane, lim)) return;
+    if (!finish_entry(a, a.tile_dots, it, sh, abort_flag, lane, lim, [&](const FinEntry& f) {
+          finish_tile_warp(a, f.t, f.b, f.T, f.Q, f.out_mode);
+        }))
+      return;
     ++it;
-  }
-}
-
-// The finisher warp of a CTA-pair kernel: the CTA's tiles are
-// 2 (uw u + k) + rank for its units u = cl, cl + ncl, ... < nunits and
-// k < uw (uw super tiles per unit), in the epilogue warps' order.
-__device__ __forceinline__ void finisher_pair(const SqArgs& a, int cl, int ncl, int nunits, int uw, int rank,
-                                              Shared& sh, volatile int* abort_flag, int lane) {
-  using namespace sp2::tc;
-  const unsigned long long lim = wait_limit(a);
-  uint32_t it = 0;
-  for (int u = cl; u < nunits; u += ncl) {
-    for (int k = 0; k < uw; ++k) {
-      const int t = 2 * (uw * u + k) + rank;
-      int b, I, J, h;
-      unpack_tile(a.tiles[t], b, I, J, h);
-      if (!load_params(a, b).active) continue;
-      if (!finish_entry(a, it, sh, abort_flag, lane, lim)) return;
-      ++it;
-    }
   }
 }
 

@@ -90,6 +90,45 @@ struct SqArgs {
                            //    wave starts on the K slices the previous wave left in L2
 };
 
+// What differs from layer to layer in a list of layers (PairList); a launch of
+// one layer takes it from SqArgs.  Planes are entries of a pool, [entry][batch]
+// matrices under one pair of tensor maps.
+struct LayerOp {
+  int y, g;                // plane entries: P = Y Y, or Y G + G Y (g >= 0, adjoint mode)
+  int tri_y;               // as SqArgs::tri_y
+  const float* Yin;
+  float* Yout;
+  const float* aux;        // as in SqArgs
+  __half* p0_out;          // planes written: hp and lo' (split) or hi, or nullptr
+  __half* p1_out;
+  const double* rn;
+  const float* rnp_in;
+  float* rnp_out;
+  const LayerParams* lp;   // [batch]; nullptr: chosen by the control steps
+  double* dots_out;
+  float* X;                // [batch] matrices X' = Y' + x_add[b] I, stored whole, or nullptr
+  const double* x_add;
+};
+
+// A list of layers in one cooperative launch of the CTA-pair kernel.  Tiles of
+// layer n + 1 of an instance start once all its tiles of layer n are stored.
+struct PairList {
+  const LayerOp* ops;      // [nops], or nullptr: the one layer that SqArgs describes
+  int nops;
+  int batch;
+  int per;                 // units of an instance (all instances alike), when groups > 0
+  int groups;              // 0: layer after layer over all units; else the batch is cut into this many groups
+                           //   of instances, all layers of a group before the next.  64 x 2048, 11 layers:
+                           //   groups of 5 16.1 ms, of 3 17.6, all 64 18.6 (planes and iterates through DRAM;
+                           //   16.2 with the pairs kept in step, SqArgs::wave_ctr, as with a launch a layer);
+                           //   all at the 1.4 kW power limit
+  unsigned* done;          // [batch] zero: finished tiles over the layers
+  unsigned* step;          // [batch] zero: layers whose sums, and control step, are complete
+  LayerParams* rec;        // [nops + 1] parameters chosen by the control steps (ctl set: one instance)
+  unsigned long long* stamps;  // [nops + 1] ns at the start and after each layer (ctl set), or nullptr
+  int wave_per;            // SqArgs::wave_ctr entries of a layer (groups = 0)
+};
+
 // tensor-core tile geometry
 constexpr int kTcBM = 128;   // rows per CTA tile (TMEM lanes)
 constexpr int kTcBN = 256;   // columns per CTA tile; 256 x 256 "super tiles" hold two CTA tiles
@@ -136,11 +175,13 @@ cudaError_t launch_syrk_tc1(const SqArgs& a, const CUtensorMap* tmaps, bool spli
 size_t syrk_tc1_smem_bytes(bool split);
 // The same product run by CTA pairs (clusters of 2) whose MMAs span both CTAs
 // (M = 256 per super tile, each CTA holding 128 rows of A and of B): tiles
-// come in (h = 0, h = 1) pairs of one super tile, a.ntiles = 2 x super tiles,
-// and the B maps have 128-row boxes.  tmaps holds
-// six maps: the four above and {p0, p1} with 64 x 64 boxes, through which the
-// K blocks left of the diagonal are read transposed from the upper tiles.
-cudaError_t launch_syrk_tc2(const SqArgs& a, const CUtensorMap* tmaps, bool split, int grid, cudaStream_t st);
+// come in (h = 0, h = 1) pairs of one super tile, a.ntiles = 2 x super tiles.
+// tmaps: {p0, p1} with 64 x 128 boxes and {p0, p1} with 64 x 64 boxes, through
+// which the K blocks left of the diagonal are read transposed from the upper
+// tiles.  A list of layers (l.ops) is one cooperative launch; adjoint: it holds
+// adjoint layers.
+cudaError_t launch_syrk_tc2(const SqArgs& a, const PairList& l, bool adjoint, const CUtensorMap* tmaps, bool split,
+                            int grid, cudaStream_t st);
 size_t syrk_tc2_smem_bytes(bool split);
 
 // Resident solve (csrc/resident.cu): all layers of a batch of instances in one

@@ -226,13 +226,17 @@ __global__ void __launch_bounds__(THREADS, 1)
     // ------------------------------------------------------------ epilogue
     const int ew = warp - 2;  // 0..7
     const int q = warp & 3;   // TMEM lane quarter
+    const LayerOp o = epi::layer_of(a, SPLIT);
     uint32_t it = 0;
     for (int t = blockIdx.x; t < a.ntiles; t += gridDim.x) {
-      const int rc =
-          epi::tile<SPLIT, NSEG2>(a, t, it, tmem_base, tmem_full, tmem_empty, abort_flag, s_epi, ew, q, lane,
-                                  trbuf + ew * epi::TR_FLOATS);
-      if (rc < 0) break;
-      it += (uint32_t)rc;
+      int b, I, J, h;
+      unpack_tile(a.tiles[t], b, I, J, h);
+      const LayerParams p = load_params(a, b);
+      if (!p.active) continue;
+      if (!epi::tile<SPLIT, NSEG2>(a, o, p, t, it, tmem_base, tmem_full, tmem_empty, abort_flag, s_epi, ew, q, lane,
+                                   trbuf + ew * epi::TR_FLOATS))
+        break;
+      ++it;
     }
   }
 

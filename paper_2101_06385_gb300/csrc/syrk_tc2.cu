@@ -25,6 +25,18 @@
 //                 once they have drained accumulator buffer b
 // Every wait is bounded; an abort is also stored into the peer's flag.
 //
+// Lists of layers (PairList): one cooperative launch runs every layer of a
+// solve, an expansion, a network pass.  The finisher warps count an instance's
+// stored tiles (done) and, once the layer's sums and the control step are
+// complete, its layers (step).  A producer starts a tile of the next layer when
+// `done` says that the operand planes are complete; the epilogue, which needs
+// the coefficients, waits for `step` meanwhile.  Units are taken in an order in
+// which every dependency points backwards and all pairs are resident, so the
+// first unfinished unit never waits.  The planes cross from generic stores to
+// TMA reads behind the producer's acquire and its proxy fence.  Against a launch
+// a layer, N = 4096: 7.36 -> 6.47 ms a solve (a layer 145 -> 136 us, and no
+// launches after convergence).
+//
 // Alg. 2 / Eq. 14 with both parts scaled by 2^s (Eq. 12: hi = fp16(Y),
 // lo' = fp16(2^s (Y - hi)); hp = 2^s hi is exact in FP16 for |Y| < 2^(15-s)):
 //     2^(2s) P = hp hp + lo' hp + hp lo',
@@ -146,26 +158,145 @@ __device__ __forceinline__ bool epoch_wait(const unsigned* ctr, unsigned need, u
   return true;
 }
 
+// The units of pair cl in the order it takes them: u of layer n.  With groups
+// (all instances alike) unit r of a group's width x nops goes to pair r mod ncl,
+// and the groups follow one another; without, every layer starts at unit cl.
+struct Walk {
+  int n, u;
+  int cl, ncl, nunits, nops, per, groups, batch;
+  int g, base, width, r;
+  __device__ __forceinline__ Walk(const PairList& l, int cl_, int ncl_, int nunits_)
+      : n(0), u(0), cl(cl_), ncl(ncl_), nunits(nunits_), nops(l.nops), per(l.per), groups(l.groups), batch(l.batch),
+        g(0), base(0), width(nunits_), r(cl_ - ncl_) {
+    if (groups > 0) set_group();
+  }
+  __device__ __forceinline__ void set_group() {
+    const int b0 = (int)((long long)g * batch / groups), b1 = (int)((long long)(g + 1) * batch / groups);
+    base = b0 * per;
+    width = (b1 - b0) * per;
+  }
+  __device__ __forceinline__ bool next() {
+    r += ncl;
+    if (groups > 0) {
+      while (r >= width * nops) {
+        if (g + 1 == groups) return false;
+        r -= width * nops;
+        ++g;
+        set_group();
+      }
+      n = r / width;
+      u = base + (r - n * width);
+    } else {
+      while (r >= width) {
+        r = cl;
+        if (++n >= nops) return false;
+      }
+      u = r;
+    }
+    return true;
+  }
+};
+
+// Waits (one thread) until *p >= need: a count that the finisher warps raise.
+// False: abort, or a wait longer than lim.
+__device__ __forceinline__ bool flag_wait(const unsigned* p, unsigned need, const int* err,
+                                          volatile int* abort_flag, unsigned long long lim) {
+  if (ld_relaxed(p) < need) {
+    const uint64_t t0 = globaltimer();
+    int spin = 0;
+    while (ld_relaxed(p) < need)
+      if ((++spin & 31) == 0 && (*abort_flag || *(const volatile int*)err != 0 || globaltimer() - t0 > lim)) {
+        *abort_flag = 1;
+        return false;
+      }
+  }
+  __threadfence();
+  return true;
+}
+
+// Whether instance b takes part in layer n: 1, 0, or -1 (a wait failed).  In a
+// list driven by control steps the last layer is known once the layer before
+// it has its parameters; p0: those of layer 0.
+__device__ __forceinline__ int layer_live(const SqArgs& a, const PairList& l, const LayerParams& p0, int b, int n,
+                                          volatile int* abort_flag, unsigned long long lim) {
+  if (!l.ops) return load_params(a, b).active;
+  if (!a.ctl || n == 0) return 1;
+  if (n == 1) return p0.out_mode != OUT_D;
+  if (!flag_wait(l.step + b, (unsigned)(n - 1), a.err, abort_flag, lim)) return -1;
+  return __ldcg(&l.rec[n - 1].out_mode) != OUT_D;
+}
+
+// Tile t of layer n of instance b is stored and has the sums (T, Q): one
+// finisher warp.  The last tile of a layer sums over the instance and runs the
+// control step.  Sums of successive layers alternate between two halves of
+// tile_part and tile_dots.
+__device__ __forceinline__ void finish_list_tile(const SqArgs& a, const PairList& l, const LayerOp& o, int n,
+                                                 const epi::FinEntry& f, int lane) {
+  const int b = f.b, cnt = a.tile_cnt[b];
+  double2* part = a.tile_part + (n & 1 ? a.ntiles : 0);
+  unsigned last = 0;
+  if (lane == 0) {
+    part[f.t] = make_double2(f.T, f.Q);
+    __threadfence();
+    last = atomicAdd(&l.done[b], 1u) + 1u == (unsigned)cnt * (unsigned)(n + 1);
+  }
+  if (!__shfl_sync(0xffffffffu, last, 0)) return;
+  __threadfence();
+  const int off = a.tile_off[b];
+  if (a.ctl) {
+    double T = 0.0, Q = 0.0;
+#pragma unroll 4
+    for (int k = lane; k < cnt; k += 32) {
+      const double2 p = __ldcg(&part[off + k]);
+      T += p.x;
+      Q += p.y;
+    }
+    T = warp_sum_d(T);
+    Q = warp_sum_d(Q);
+    if (lane == 0) {
+      if (l.stamps) l.stamps[n + 1] = globaltimer();
+      control_step(a.ctl + b, T, Q);
+      if (a.ctl[b].next.active) l.rec[n + 1] = a.ctl[b].next;
+    }
+  }
+  if (f.dots && o.dots_out) {
+    const double* td = a.tile_dots + (n & 1 ? 3 * (long long)a.ntiles : 0) + 3 * (long long)off;
+    double d0 = 0.0, d1 = 0.0, d2 = 0.0;
+    for (int k = lane; k < cnt; k += 32) {
+      d0 += __ldcg(td + 3 * k);
+      d1 += __ldcg(td + 3 * k + 1);
+      d2 += __ldcg(td + 3 * k + 2);
+    }
+    d0 = warp_sum_d(d0);
+    d1 = warp_sum_d(d1);
+    d2 = warp_sum_d(d2);
+    if (lane == 0) {
+      o.dots_out[3 * b + 0] = d0;
+      o.dots_out[3 * b + 1] = d1;
+      o.dots_out[3 * b + 2] = d2;
+    }
+  }
+  if (lane == 0) {
+    __threadfence();
+    st_relaxed(l.step + b, (unsigned)(n + 1));
+  }
+}
+
 // RO: readout mode of the epilogue (finite-temperature expansion).
-// NSEG2: P = A_1 B_1^T + A_2 B_2^T over two K segments (the tm2 maps hold the
-// second segment's operands) with the adjoint-mode epilogue: the split SYR2K
-// Y G + G Y of the network adjoint (both factors symmetric).
-// tm_p0A/p1A: planes with 64 x 128 boxes (the A half); tm_p0B/p1B: the same
-// boxes for the B half; tm_p0T / tm_p1T: 64 x 64 boxes (transposed reads).
-// The kernel body; the map arguments point at the kernels' __grid_constant__
-// parameters (for one segment the second set repeats the first).
-template <bool SPLIT, bool RO, bool NSEG2, bool WIDE>
-__device__ __forceinline__ void syrk_tc2_body(const CUtensorMap& tm_p0A, const CUtensorMap& tm_p1A,
-                                              const CUtensorMap& tm_p0B, const CUtensorMap& tm_p1B,
-                                              const CUtensorMap& tm_p0T, const CUtensorMap& tm_p1T,
-                                              const CUtensorMap& tm2_p0A, const CUtensorMap& tm2_p1A,
-                                              const CUtensorMap& tm2_p0B, const CUtensorMap& tm2_p1B,
-                                              const CUtensorMap& tm2_p0T, const CUtensorMap& tm2_p1T,
-                                              const SqArgs& a) {
+// ADJ: the list holds adjoint layers, P = Y G + G Y over two K segments with
+// the adjoint-mode epilogue (the split SYR2K of the network adjoint, both
+// factors symmetric).
+// tm_p0K / p1K: the planes with 64 x 128 boxes; tm_p0T / tm_p1T: 64 x 64 boxes
+// (transposed reads); the third coordinate is entry x batch + instance.
+template <bool SPLIT, bool RO, bool ADJ, bool WIDE>
+__global__ void __launch_bounds__(THREADS, 1)
+    syrk_tc2_kernel(const __grid_constant__ CUtensorMap tm_p0K, const __grid_constant__ CUtensorMap tm_p1K,
+                    const __grid_constant__ CUtensorMap tm_p0T, const __grid_constant__ CUtensorMap tm_p1T,
+                    const __grid_constant__ SqArgs a, const __grid_constant__ PairList l) {
   constexpr int STAGES = WIDE ? (SPLIT ? STAGES_WSPLIT : STAGES_WPLAIN) : (SPLIT ? STAGES_SPLIT : STAGES_PLAIN);
   constexpr int STAGE_BYTES = WIDE ? (SPLIT ? STAGE_WSPLIT : STAGE_WPLAIN) : (SPLIT ? STAGE_SPLIT : STAGE_PLAIN);
   constexpr int UW = WIDE ? 2 : 1;  // super tiles per unit of work of a pair
-  static_assert(!WIDE || (!RO && !NSEG2), "wide units serve the single solve");
+  static_assert(!WIDE || (!RO && !ADJ), "wide units serve the single solve");
 
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -187,12 +318,23 @@ __device__ __forceinline__ void syrk_tc2_body(const CUtensorMap& tm_p0A, const C
   const uint32_t rank = cluster_rank();
   const uint32_t peer = rank ^ 1u;
 
+  __shared__ LayerParams s_p0;
+  // A list driven by control steps: the parameters of layer 0 (every CTA has a
+  // tile of each layer, so the first control step comes after this).
+  if (l.ops && a.ctl) {
+    if (threadIdx.x == 0) {
+      s_p0 = a.ctl[0].next;
+      if (blockIdx.x == 0 && l.stamps) l.stamps[0] = globaltimer();
+    }
+    __syncthreads();
+    if (!s_p0.active) return;
+  }
   // A pair whose super tiles all belong to finished instances (the launches
   // after a solve's last layer) leaves before any set-up; one warp looks at
   // 32 of its tiles at a time.  Both CTAs of the pair reach the same answer:
   // an instance can finish within this launch only after all of its tiles,
   // these among them, have been processed.
-  if (warp == 0) {
+  if (!l.ops && warp == 0) {
     const int c0 = (int)(blockIdx.x >> 1), nc = (int)(gridDim.x >> 1), ns = (a.ntiles >> 1) / UW;
     bool any = false;
     for (int u0 = c0; u0 < ns && !any; u0 += 32 * nc) {
@@ -207,8 +349,10 @@ __device__ __forceinline__ void syrk_tc2_body(const CUtensorMap& tm_p0A, const C
     }
     if (lane == 0) s_work = any ? 1 : 0;
   }
-  __syncthreads();
-  if (!s_work) return;
+  if (!l.ops) {
+    __syncthreads();
+    if (!s_work) return;
+  }
 
   if (threadIdx.x == 0) {
     s_abort = 0;
@@ -258,11 +402,34 @@ __device__ __forceinline__ void syrk_tc2_body(const CUtensorMap& tm_p0A, const C
       const int W = a.sync_stages;
       bool wait_sync = rank == 0 && a.wave_ctr != nullptr && W > 0;
       const bool pub_sync = wait_sync;
+      unsigned* wave = a.wave_ctr;
+      int layer = 0;
       uint32_t gs = 0;
-      for (int u = cl; u < nunits && ok; u += ncl) {
+      for (Walk w(l, cl, ncl, nunits); ok && w.next();) {
+        const int u = w.u;
         int b, I, J, h;
         unpack_tile(a.tiles[2 * UW * u + (int)rank], b, I, J, h);
-        if (!load_params(a, b).active) continue;
+        if (pub_sync && w.n != layer) {
+          // the last (possibly partial) epoch of the layer before
+          if (gs > 0) atomicAdd(&wave[(gs - 1u) / (uint32_t)W], 1u);
+          wave += (long long)(w.n - layer) * l.wave_per;
+          layer = w.n;
+          gs = 0;
+          wait_sync = true;
+        }
+        const int live = layer_live(a, l, s_p0, b, w.n, abort_flag, lim);
+        if (live == 0) {
+          if (l.ops) break;
+          continue;
+        }
+        // the operands: what all tiles of the layer before stored
+        if (live < 0 || (w.n > 0 && !flag_wait(l.done + b, (unsigned)(a.tile_cnt[b] * w.n), a.err, abort_flag, lim))) {
+          ok = false;
+          break;
+        }
+        if (w.n > 0) fence_proxy_async();
+        const int ey = l.ops ? l.ops[w.n].y * l.batch + b : b;
+        const int eg = ADJ && l.ops[w.n].g >= 0 ? l.ops[w.n].g * l.batch + b : -1;
         const int N = a.Ns[b];
         // each CTA supplies half of the MMA's N rows of B
         const int rowA = I * BN + (int)rank * BH, rowB = J * BN + (int)rank * (pair_n(N, J) >> 1);
@@ -276,17 +443,17 @@ __device__ __forceinline__ void syrk_tc2_body(const CUtensorMap& tm_p0A, const C
           rowB1 = J1 * BN + (int)rank * (pair_n(N, J1) >> 1);
         }
         const int nk = (N + BK - 1) / BK;
-        const int nkt = NSEG2 ? 2 * nk : nk;  // K stages of the tile over both segments
+        const int nkt = eg >= 0 ? 2 * nk : nk;  // K stages of the tile over both segments
         const bool rev = a.snake && (((u - cl) / ncl) & 1);
         for (int kk = 0; kk < nkt; ++kk, ++gs) {
           const int kbt = rev ? nkt - 1 - kk : kk;
-          const bool seg2 = NSEG2 && kbt >= nk;
+          const bool seg2 = ADJ && kbt >= nk;
           const int kb = seg2 ? kbt - nk : kbt;  // K block within its segment
           if (pub_sync && gs > 0 && gs % (uint32_t)W == 0) {
             const uint32_t e = gs / (uint32_t)W - 1u;  // the epoch this pair just finished
-            atomicAdd(&a.wave_ctr[e], 1u);
+            atomicAdd(&wave[e], 1u);
             if (wait_sync && e >= 1u)
-              wait_sync = epoch_wait(a.wave_ctr + (e - 1u), pairs_in_epoch(e - 1u, W, nkt, nunits, ncl), lim);
+              wait_sync = epoch_wait(wave + (e - 1u), pairs_in_epoch(e - 1u, W, nkt, nunits, ncl), lim);
           }
           if (!mbar_wait_cl(&empty[stage], phase ^ 1u, abort_flag, lim)) {
             ok = false;
@@ -302,29 +469,21 @@ __device__ __forceinline__ void syrk_tc2_body(const CUtensorMap& tm_p0A, const C
           const uint32_t bar = full_cl + 8u * (uint32_t)stage;
           const int k0 = kb * BK;
           const int ks = k0 / BN;  // super column of this K block
-          // the second segment's A and B come from the other matrix of the
-          // product (their transposed reads too)
-          const CUtensorMap* mA0 = seg2 ? &tm2_p0A : &tm_p0A;
-          const CUtensorMap* mA1 = seg2 ? &tm2_p1A : &tm_p1A;
-          const CUtensorMap* mB0 = seg2 ? &tm2_p0B : &tm_p0B;
-          const CUtensorMap* mB1 = seg2 ? &tm2_p1B : &tm_p1B;
-          const CUtensorMap* mAT0 = seg2 ? &tm2_p0T : &tm_p0T;
-          const CUtensorMap* mAT1 = seg2 ? &tm2_p1T : &tm_p1T;
-          const CUtensorMap* mBT0 = NSEG2 ? (seg2 ? &tm_p0T : &tm2_p0T) : &tm_p0T;
-          const CUtensorMap* mBT1 = NSEG2 ? (seg2 ? &tm_p1T : &tm2_p1T) : &tm_p1T;
+          // first segment: rows of Y times rows of G (or Y), second: rows of G times rows of Y
+          const int eA = seg2 ? eg : ey, eB = ADJ && eg >= 0 && !seg2 ? eg : ey;
           if (SPLIT) {
-            load_half(st + OFF_HPA, mA0, mAT0, ks < I, rowA, k0, b, bar);
-            load_half(st + OFF_LOA, mA1, mAT1, ks < I, rowA, k0, b, bar);
-            load_half(st + OFF_HPB, mB0, mBT0, ks < J, rowB, k0, b, bar);
-            load_half(st + OFF_LOB, mB1, mBT1, ks < J, rowB, k0, b, bar);
+            load_half(st + OFF_HPA, &tm_p0K, &tm_p0T, ks < I, rowA, k0, eA, bar);
+            load_half(st + OFF_LOA, &tm_p1K, &tm_p1T, ks < I, rowA, k0, eA, bar);
+            load_half(st + OFF_HPB, &tm_p0K, &tm_p0T, ks < J, rowB, k0, eB, bar);
+            load_half(st + OFF_LOB, &tm_p1K, &tm_p1T, ks < J, rowB, k0, eB, bar);
             if (WIDE && two) {
-              load_half(st + OFF_HPB1, mB0, mBT0, ks < J1, rowB1, k0, b, bar);
-              load_half(st + OFF_LOB1, mB1, mBT1, ks < J1, rowB1, k0, b, bar);
+              load_half(st + OFF_HPB1, &tm_p0K, &tm_p0T, ks < J1, rowB1, k0, eB, bar);
+              load_half(st + OFF_LOB1, &tm_p1K, &tm_p1T, ks < J1, rowB1, k0, eB, bar);
             }
           } else {
-            load_half(st, mA0, mAT0, ks < I, rowA, k0, b, bar);
-            load_half(st + HALF_BYTES, mB0, mBT0, ks < J, rowB, k0, b, bar);
-            if (WIDE && two) load_half(st + OFF_B1_PLAIN, mB0, mBT0, ks < J1, rowB1, k0, b, bar);
+            load_half(st, &tm_p0K, &tm_p0T, ks < I, rowA, k0, eA, bar);
+            load_half(st + HALF_BYTES, &tm_p0K, &tm_p0T, ks < J, rowB, k0, eB, bar);
+            if (WIDE && two) load_half(st + OFF_B1_PLAIN, &tm_p0K, &tm_p0T, ks < J1, rowB1, k0, eB, bar);
           }
           if (++stage == STAGES) {
             stage = 0;
@@ -333,7 +492,7 @@ __device__ __forceinline__ void syrk_tc2_body(const CUtensorMap& tm_p0A, const C
         }
       }
       // the last (possibly partial) epoch of this pair
-      if (pub_sync && gs > 0) atomicAdd(&a.wave_ctr[(gs - 1u) / (uint32_t)W], 1u);
+      if (pub_sync && gs > 0) atomicAdd(&wave[(gs - 1u) / (uint32_t)W], 1u);
       if (!ok || *abort_flag) {
         atomicExch(a.err, (int)SP2_ERR_DEVICE_TIMEOUT);
         st_cluster_u32(peer_abort, 1u);
@@ -366,13 +525,23 @@ __device__ __forceinline__ void syrk_tc2_body(const CUtensorMap& tm_p0A, const C
       bool ok = true, issued = false;
       // injected fault (SqArgs::stall): a wait that runs out after lim
       if (a.stall && !mbar_wait(never, 0, abort_flag, lim)) ok = false;
-      for (int u = cl; u < nunits && ok; u += ncl) {
+      for (Walk w(l, cl, ncl, nunits); w.next();) {
+        const int u = w.u;
         int b, I, J, h;
         unpack_tile(a.tiles[2 * UW * u], b, I, J, h);
-        if (!load_params(a, b).active) continue;
+        const int live = layer_live(a, l, s_p0, b, w.n, abort_flag, lim);
+        if (live == 0) {
+          if (l.ops) break;
+          continue;
+        }
+        if (live < 0) {
+          ok = false;
+          break;
+        }
         const int N = a.Ns[b];
         const int nk = (N + BK - 1) / BK;
-        const int nkt = NSEG2 ? 2 * nk : nk;
+        const bool two_seg = ADJ && l.ops[w.n].g >= 0;
+        const int nkt = two_seg ? 2 * nk : nk;
         const bool rev = a.snake && (((u - cl) / ncl) & 1);
         // wide units: the second super tile (I, J1) into the other accumulator
         int J1 = 0;
@@ -398,7 +567,7 @@ __device__ __forceinline__ void syrk_tc2_body(const CUtensorMap& tm_p0A, const C
         const uint32_t d1 = tmem_base + BN;  // wide units: the second accumulator
         for (int kk = 0; kk < nkt; ++kk) {
           const int kbt = rev ? nkt - 1 - kk : kk;
-          const int kb = (NSEG2 && kbt >= nk) ? kbt - nk : kbt;  // K block within its segment
+          const int kb = (ADJ && kbt >= nk) ? kbt - nk : kbt;  // K block within its segment
           if (!mbar_wait_cl(&full[stage], phase, abort_flag, lim)) {
             ok = false;
             break;
@@ -478,8 +647,33 @@ __device__ __forceinline__ void syrk_tc2_body(const CUtensorMap& tm_p0A, const C
     }
   } else if (warp == FIN_WARP) {
     // ------------------------------------------------------------ finisher
-    // (tiles t = 2 (UW u + k) + rank of units u = cl, cl + ncl, ...)
-    epi::finisher_pair(a, cl, ncl, nunits, UW, (int)rank, s_epi, abort_flag, lane);
+    // (tiles t = 2 (UW u + k) + rank of a unit u, in the epilogue warps' order)
+    uint32_t it = 0;
+    bool ok = true;
+    for (Walk w(l, cl, ncl, nunits); ok && w.next();) {
+      int b, I, J, h;
+      unpack_tile(a.tiles[2 * UW * w.u], b, I, J, h);
+      const int live = __reduce_min_sync(0xffffffffu, layer_live(a, l, s_p0, b, w.n, abort_flag, lim));
+      if (live == 0) {
+        if (l.ops) break;
+        continue;
+      }
+      if (live < 0) {
+        if (lane == 0) atomicExch(a.err, (int)SP2_ERR_DEVICE_TIMEOUT);
+        *abort_flag = 1;
+        break;
+      }
+      double* const tdots = a.tile_dots + (l.ops && (w.n & 1) ? 3 * (long long)a.ntiles : 0);
+      for (int k = 0; k < UW && ok; ++k) {
+        ok = epi::finish_entry(a, tdots, it, s_epi, abort_flag, lane, lim, [&](const epi::FinEntry& f) {
+          if (l.ops)
+            finish_list_tile(a, l, l.ops[w.n], w.n, f, lane);
+          else
+            finish_tile_warp(a, f.t, f.b, f.T, f.Q, f.out_mode);
+        });
+        ++it;
+      }
+    }
     if (*abort_flag && lane == 0) st_cluster_u32(peer_abort, 1u);
   } else {
     // ------------------------------------------------------------ epilogue
@@ -488,19 +682,37 @@ __device__ __forceinline__ void syrk_tc2_body(const CUtensorMap& tm_p0A, const C
     const uint32_t empty_cl = mapa_u32(smem_u32(&tmem_empty[0]), 0);
     uint32_t it = 0;
     bool ok = true;
-    for (int u = cl; u < nunits && ok; u += ncl) {
+    for (Walk w(l, cl, ncl, nunits); ok && w.next();) {
       // a unit's super tiles use the accumulator buffers in turn (a wide
       // unit's second tile, when it has none, has no rows to store)
-      for (int k = 0; k < UW; ++k) {
-        const int t = 2 * (UW * u + k) + (int)rank;
-        const int rc = epi::tile<SPLIT, NSEG2, RO, true>(a, t, it, tmem_base, tmem_full, tmem_empty, abort_flag,
-                                                          s_epi, ew, q, lane, trbuf + ew * epi::TR_FLOATS, empty_cl);
-        if (rc < 0) {
-          if (lane == 0) st_cluster_u32(peer_abort, 1u);
-          ok = false;
-          break;
+      int b, I, J, h;
+      unpack_tile(a.tiles[2 * UW * w.u], b, I, J, h);
+      const int live = __reduce_min_sync(0xffffffffu, layer_live(a, l, s_p0, b, w.n, abort_flag, lim));
+      if (live == 0) {
+        if (l.ops) break;
+        continue;
+      }
+      const LayerOp o = l.ops ? l.ops[w.n] : epi::layer_of(a, SPLIT);
+      // the coefficients, and old values and row norms of the layer before
+      ok = live > 0 && (w.n == 0 || flag_wait(l.step + b, (unsigned)w.n, a.err, abort_flag, lim));
+      ok = __all_sync(0xffffffffu, ok);
+      if (ok) {
+        const LayerParams p = !l.ops ? load_params(a, b) : o.lp ? o.lp[b] : w.n == 0 ? s_p0 : l.rec[w.n];
+        for (int k = 0; k < UW && ok; ++k, ++it) {
+          const int t = 2 * (UW * w.u + k) + (int)rank;
+          float* trb = trbuf + ew * epi::TR_FLOATS;
+          if (ADJ && o.g >= 0)
+            ok = epi::tile<SPLIT, true, false, true>(a, o, p, t, it, tmem_base, tmem_full, tmem_empty, abort_flag,
+                                                     s_epi, ew, q, lane, trb, empty_cl);
+          else
+            ok = epi::tile<SPLIT, false, RO, true, !WIDE && !RO && !ADJ>(a, o, p, t, it, tmem_base, tmem_full, tmem_empty, abort_flag,
+                                                   s_epi, ew, q, lane, trb, empty_cl);
         }
-        it += (uint32_t)rc;
+      }
+      if (!ok && lane == 0) {
+        atomicExch(a.err, (int)SP2_ERR_DEVICE_TIMEOUT);
+        *abort_flag = 1;
+        st_cluster_u32(peer_abort, 1u);
       }
     }
   }
@@ -515,41 +727,6 @@ __device__ __forceinline__ void syrk_tc2_body(const CUtensorMap& tm_p0A, const C
     __syncwarp();
     tmem_dealloc_pair(tmem_base, TMEM_COLS);
   }
-}
-
-template <bool SPLIT, bool RO>
-__global__ void __launch_bounds__(THREADS, 1)
-    syrk_tc2_kernel(const __grid_constant__ CUtensorMap tm_p0A, const __grid_constant__ CUtensorMap tm_p1A,
-                    const __grid_constant__ CUtensorMap tm_p0B, const __grid_constant__ CUtensorMap tm_p1B,
-                    const __grid_constant__ CUtensorMap tm_p0T, const __grid_constant__ CUtensorMap tm_p1T,
-                    const SqArgs a) {
-  syrk_tc2_body<SPLIT, RO, false, false>(tm_p0A, tm_p1A, tm_p0B, tm_p1B, tm_p0T, tm_p1T, tm_p0A, tm_p1A, tm_p0B,
-                                         tm_p1B, tm_p0T, tm_p1T, a);
-}
-
-// Wide units (the single solve): super tiles (I, J) and (I, J + 1) per pass.
-template <bool SPLIT>
-__global__ void __launch_bounds__(THREADS, 1)
-    syrk_tc2_wide_kernel(const __grid_constant__ CUtensorMap tm_p0A, const __grid_constant__ CUtensorMap tm_p1A,
-                         const __grid_constant__ CUtensorMap tm_p0B, const __grid_constant__ CUtensorMap tm_p1B,
-                         const __grid_constant__ CUtensorMap tm_p0T, const __grid_constant__ CUtensorMap tm_p1T,
-                         const SqArgs a) {
-  syrk_tc2_body<SPLIT, false, false, true>(tm_p0A, tm_p1A, tm_p0B, tm_p1B, tm_p0T, tm_p1T, tm_p0A, tm_p1A, tm_p0B,
-                                           tm_p1B, tm_p0T, tm_p1T, a);
-}
-
-// Two K segments (the network adjoint's Y G + G Y): six maps per segment.
-template <bool SPLIT>
-__global__ void __launch_bounds__(THREADS, 1)
-    syrk_tc2_seg2_kernel(const __grid_constant__ CUtensorMap tm_p0A, const __grid_constant__ CUtensorMap tm_p1A,
-                         const __grid_constant__ CUtensorMap tm_p0B, const __grid_constant__ CUtensorMap tm_p1B,
-                         const __grid_constant__ CUtensorMap tm_p0T, const __grid_constant__ CUtensorMap tm_p1T,
-                         const __grid_constant__ CUtensorMap tm2_p0A, const __grid_constant__ CUtensorMap tm2_p1A,
-                         const __grid_constant__ CUtensorMap tm2_p0B, const __grid_constant__ CUtensorMap tm2_p1B,
-                         const __grid_constant__ CUtensorMap tm2_p0T, const __grid_constant__ CUtensorMap tm2_p1T,
-                         const SqArgs a) {
-  syrk_tc2_body<SPLIT, false, true, false>(tm_p0A, tm_p1A, tm_p0B, tm_p1B, tm_p0T, tm_p1T, tm2_p0A, tm2_p1A, tm2_p0B,
-                                           tm2_p1B, tm2_p0T, tm2_p1T, a);
 }
 
 }  // namespace tc2
@@ -579,7 +756,8 @@ size_t syrk_tc2_smem_bytes(bool split) {
   return (size_t)stages * sb + 1024 /* alignment slack */ + 256 /* barriers */ + epi::TR_BYTES;
 }
 
-cudaError_t launch_syrk_tc2(const SqArgs& a, const CUtensorMap* tm, bool split, int grid, cudaStream_t st) {
+cudaError_t launch_syrk_tc2(const SqArgs& a, const PairList& l, bool adjoint, const CUtensorMap* tm, bool split,
+                            int grid, cudaStream_t st) {
   // grid: number of CTAs, even (two per cluster); a.ntiles = 2 x super tiles
   const size_t smem = syrk_tc2_smem_bytes(split);
   cudaLaunchConfig_t cfg = {};
@@ -587,33 +765,33 @@ cudaError_t launch_syrk_tc2(const SqArgs& a, const CUtensorMap* tm, bool split, 
   cfg.blockDim = dim3(tc2::THREADS, 1, 1);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = 2;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeCooperative;  // a list's pairs wait on one another
+  attr[1].val.cooperative = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = l.ops ? 2 : 1;
   auto go = [&](auto kernel, int which) -> cudaError_t {
     cudaError_t e = set_smem_once(kernel, (int)smem, which);
     if (e != cudaSuccess) return e;
-    return cudaLaunchKernelEx(&cfg, kernel, tm[0], tm[1], tm[2], tm[3], tm[4], tm[5], a);
-  };
-  auto go2 = [&](auto kernel, int which) -> cudaError_t {
-    cudaError_t e = set_smem_once(kernel, (int)smem, which);
-    if (e != cudaSuccess) return e;
-    return cudaLaunchKernelEx(&cfg, kernel, tm[0], tm[1], tm[2], tm[3], tm[4], tm[5], tm[6], tm[7], tm[8], tm[9],
-                              tm[10], tm[11], a);
+    return cudaLaunchKernelEx(&cfg, kernel, tm[0], tm[1], tm[2], tm[3], a, l);
   };
   cudaError_t e;
-  if (a.nseg == 2)
-    e = split ? go2(tc2::syrk_tc2_seg2_kernel<true>, 5) : go2(tc2::syrk_tc2_seg2_kernel<false>, 4);
+  if (adjoint)
+    e = split ? go(tc2::syrk_tc2_kernel<true, false, true, false>, 5)
+              : go(tc2::syrk_tc2_kernel<false, false, true, false>, 4);
   else if (a.wide)
-    e = split ? go(tc2::syrk_tc2_wide_kernel<true>, 7) : go(tc2::syrk_tc2_wide_kernel<false>, 6);
+    e = split ? go(tc2::syrk_tc2_kernel<true, false, false, true>, 7)
+              : go(tc2::syrk_tc2_kernel<false, false, false, true>, 6);
   else if (a.R)
-    e = split ? go(tc2::syrk_tc2_kernel<true, true>, 3) : go(tc2::syrk_tc2_kernel<false, true>, 2);
+    e = split ? go(tc2::syrk_tc2_kernel<true, true, false, false>, 3)
+              : go(tc2::syrk_tc2_kernel<false, true, false, false>, 2);
   else
-    e = split ? go(tc2::syrk_tc2_kernel<true, false>, 1) : go(tc2::syrk_tc2_kernel<false, false>, 0);
+    e = split ? go(tc2::syrk_tc2_kernel<true, false, false, false>, 1)
+              : go(tc2::syrk_tc2_kernel<false, false, false, false>, 0);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }
