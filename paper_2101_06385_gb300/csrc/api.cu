@@ -1195,8 +1195,13 @@ sp2_status density_matrix_impl(const float* H, int N, int N_occ, double tol, int
   cudaStream_t st = g.stream;
 
   // CTA pairs on wide units (two super tiles of a row per pass, a quarter
-  // fewer operand bytes) where that takes no more waves of 76 pairs, counted
-  // in super-tile times, than single super tiles (SP2_WIDE=0/1 forces it)
+  // fewer operand bytes) by the waves of 76 pairs, counted in super-tile times
+  // (SP2_WIDE=0/1 forces it).  Split products: at large N where it takes no more
+  // waves (power bound: N = 16384 358 -> 348 ms; its epilogue no longer overlaps
+  // the next unit: 4096 6.57 -> 6.74).  Plain FP16 products are bound by the
+  // operand bytes, and a wave of wide units takes 0.82 of two waves of single
+  // ones: N = 3000 3.03 -> 2.63 ms, 4096 3.74 -> 3.21, 6500 12.4 -> 12.0, 16384
+  // 157 -> 135, but 5000 (3 against 4 waves) 6.15 -> 6.62.
   bool wide = false;
   if (tc && g.pair_kernel && g.wide != 0) {
     const int T = (N + kTcBN - 1) / kTcBN, npairs = std::max(1, g.num_sms / 2);
@@ -1206,7 +1211,7 @@ sp2_status density_matrix_impl(const float* H, int N, int N_occ, double tol, int
     build_tiles(N, 1, kTcBN, 3, wl, per);
     const int nunits = per / 4;
     const int waves = (nsup + npairs - 1) / npairs, waves_w = 2 * ((nunits + npairs - 1) / npairs);
-    wide = g.wide == 1 || (N >= 8192 && waves_w <= waves);
+    wide = g.wide == 1 || (split ? N >= 8192 && waves_w <= waves : 0.82 * waves_w < waves);
   }
   int ntiles = 0;
   CKS(upload_tiles(N, 1, tc ? (g.pair_kernel ? (wide ? 3 : 2) : 1) : 0, &ntiles));
@@ -1359,13 +1364,16 @@ sp2_status density_matrix_impl(const float* H, int N, int N_occ, double tol, int
       const int grid = std::min(wide ? ntiles / 2 : ntiles, g.num_sms) & ~1;  // every pair has a unit
       // epoch counters of the soft pair synchronisation, one zeroed slice per
       // layer (per pair: super tiles, or wide units of two)
+      // where it pays: split products with operand planes beyond L2 (N = 12000 143.6
+      // -> 142.8 ms, 16384 361 -> 348; 5000 11.4 -> 11.7).  Plain FP16 stages are a
+      // third as long and lose more in step than they save: 8192 20.3 -> 23.9 ms.
       unsigned* wave = nullptr;
       size_t per = 0;
-      CKS(wave_counters(ntiles, grid, (N + 63) / 64, nlaunch, &wave, &per));
+      if (split && N >= 6144) CKS(wave_counters(ntiles, grid, (N + 63) / 64, nlaunch, &wave, &per));
       A.wave_ctr = wave;
       l.wave_per = (int)per;
       A.sync_stages = g.wave_sync;
-      A.snake = wave ? g.snake : 0;
+      A.snake = g.wave_sync > 0 ? g.snake : 0;
       CK(launch_syrk_tc2(A, l, false, pool.m, split, grid, st));
     } else {
       const int grid = std::min(ntiles, g.num_sms);

@@ -20,7 +20,7 @@ def _solve_input(N):
 
 # the smallest size of the path (odd rows), a last column of one, wide units
 # (a row's odd last tile without a partner)
-@pytest.mark.parametrize("N,wide", [(2817, "0"), (3073, "0"), (2900, "1"), (3400, "1")])
+@pytest.mark.parametrize("N,wide", [(2945, "0"), (3073, "0"), (2945, "1"), (3400, "1")])
 @pytest.mark.parametrize("mode", ["split", "fp16", "accelerated"])
 def test_solve_same_bits(sp2, N, wide, mode):  # noqa: F811
     H, n_occ = _solve_input(N)
@@ -40,7 +40,7 @@ def test_solve_same_bits(sp2, N, wide, mode):  # noqa: F811
 
 @pytest.mark.parametrize("max_iter", [1, 2, 3])
 def test_last_layers(sp2, max_iter):  # noqa: F811
-    H, n_occ = _solve_input(2817)
+    H, n_occ = _solve_input(2945)
     run = lambda m: m.density_matrix(H, n_occ, max_iter=max_iter)  # noqa: E731
     (D, st), (D1, s1) = run(sp2), _with_env("SP2_SQUARE_KERNEL", "single", run)
     assert torch.equal(D, D1) and (st.status, st.iterations) == (s1.status, s1.iterations)
@@ -93,7 +93,7 @@ def test_expansion(sp2, B, N):  # noqa: F811
 
 
 def test_wait_runs_out(sp2):  # noqa: F811
-    H, n_occ = _solve_input(2817)
+    H, n_occ = _solve_input(2945)
     try:
         sp2.set_fault("timeout,wait_ms=100")
         t0 = time.perf_counter()
