@@ -407,6 +407,24 @@ struct PairLists {
   }
 };
 
+// The input pass of a list of layers (csrc/resident_net.cu) into plane entry
+// `entry` of the pool; FP64 row norms as rownorm_kernel's of a matrix at `norm`.
+NetInput pair_input(const PlanePool& pool, int from, const float* in, int entry, int N, int B, const void* norm) {
+  NetInput x;
+  memset(&x, 0, sizeof(x));
+  x.N = N;
+  x.batch = B;
+  x.from = from;
+  x.in = in;
+  x.p0 = pool.p0_of(entry);
+  x.p1 = pool.p1_of(entry);
+  x.ld_h = pool.ld_h;
+  x.slot_h = pool.slot_h;
+  x.vec_norm = (N & 3) == 0 && ((uintptr_t)norm & 15) == 0;
+  x.lo_scale = std::ldexp(1.0f, g.lo_scale_exp);
+  return x;
+}
+
 // One layer, as SqArgs describes it.
 PairList one_layer(int B) {
   PairList l;
@@ -2432,14 +2450,9 @@ sp2_status sp2_network_forward(const float* H, int B, int N, int L, const float*
   if (tc) {
     ld_h = round_up(N, 64);
     slot_h = ld_h * N;
-    if (pairs) {
-      (split ? hp[0] : hi[0]) = pool.p0;
-      lo[0] = pool.p1;
-    } else {
-      for (int k = 0; k < 2; ++k) {
-        CKS(planes_for(split, k, (size_t)slot_h * B * 2, &hi[k], &lo[k], &hp[k]));
-        CKS(tmaps4_for(split ? hp[k] : hi[k], lo[k], N, B, ld_h, slot_h, m[k]));
-      }
+    for (int k = 0; k < 2 && !pairs; ++k) {
+      CKS(planes_for(split, k, (size_t)slot_h * B * 2, &hi[k], &lo[k], &hp[k]));
+      CKS(tmaps4_for(split ? hp[k] : hi[k], lo[k], N, B, ld_h, slot_h, m[k]));
     }
     A.ld_h = ld_h;
     A.slot_h = slot_h;
@@ -2449,17 +2462,18 @@ sp2_status sp2_network_forward(const float* H, int B, int N, int L, const float*
     CKS(ws(B_Y0, (size_t)slot * B * 4, &Y[0]));
     CKS(ws(B_Y1, (size_t)slot * B * 4, &Y[1]));
   }
-  // input layer X_0 (no control step)
-  CK(launch_input_layer((const float* const*)hs, (const int*)ns, N, (float*)Y[0], N, slot, (__half*)hi[0],
-                        (__half*)lo[0], (__half*)hp[0],
-                        ld_h, slot_h, N, (int)ld_h, A.lo_scale, (Ctl*)ctl, nullptr, (double2*)part, (unsigned*)tick,
-                        g.shift, 0, B, igrid, st));
-  if (ckpt)
-    CK(launch_materialize((float*)Y[0], N, slot, N, B, (const double*)alpha, ckpt_slot(0), N, slot, mgrid, st));
   if (pairs) {
-    // every layer in one launch (with one each, and the checkpoints copied by
-    // passes of their own, 64 x 2048 x 20 layers took 27 ms)
-    CK(launch_rownorm(X_out, N, slot, (const int*)ns, B, N, (double*)rn, N, nullptr, nullptr, nullptr, rgrid, st));
+    // X_0 (no control step) and its checkpoint, then every layer in one launch
+    // (with one each, and the checkpoints copied by passes of their own, 64 x
+    // 2048 x 20 layers took 27 ms)
+    NetInput x = pair_input(pool, NET_INPUT, H, 0, N, B, X_out);
+    x.shift = g.shift;
+    x.ctl = (const Ctl*)ctl;
+    x.rn = (double*)rn;
+    x.y = X_out;
+    x.x0 = ckpt;
+    x.alpha0 = (const double*)alpha;
+    CK(launch_net_input(x, B, st));
     A.tri_planes = 1;
     CK(launch_syrk_tc2(A, lists.list(0, false, true, ntiles / 2 / B), false, pool.m, split,
                        std::min(ntiles, g.num_sms) & ~1, st));
@@ -2467,6 +2481,13 @@ sp2_status sp2_network_forward(const float* H, int B, int N, int L, const float*
       CK(cudaMemcpyAsync(ckpt_slot(L / ckpt_every), X_out, (size_t)B * slot * 4, cudaMemcpyDeviceToDevice, st));
     return SP2_OK;
   }
+  // input layer X_0 (no control step)
+  CK(launch_input_layer((const float* const*)hs, (const int*)ns, N, (float*)Y[0], N, slot, (__half*)hi[0],
+                        (__half*)lo[0], (__half*)hp[0],
+                        ld_h, slot_h, N, (int)ld_h, A.lo_scale, (Ctl*)ctl, nullptr, (double2*)part, (unsigned*)tick,
+                        g.shift, 0, B, igrid, st));
+  if (ckpt)
+    CK(launch_materialize((float*)Y[0], N, slot, N, B, (const double*)alpha, ckpt_slot(0), N, slot, mgrid, st));
   for (int n = 0; n < L; ++n) {
     const int cur = n & 1;
     float* Yc = (float*)Y[tc ? 0 : cur];
@@ -2631,8 +2652,9 @@ sp2_status sp2_network_backward(const float* H, int B, int N, int L, const float
         o.g = ce + gp;
         // G is read on upper super tiles only, except after the last adjoint
         // layer (dL/dX_0 is returned whole)
-        o.tri_y = n == 0 ? 0 : 1;
-        o.Yin = o.Yout = (float*)G;
+        o.tri_y = n == 0 && G_in ? 0 : 1;
+        o.Yin = (float*)G;
+        o.Yout = n == 0 && G_in ? G_in : (float*)G;
         o.aux = segY(n - n0);
         o.p0_out = pool.p0_of(ce + (gp ^ 1));
         o.p1_out = pool.p1_of(ce + (gp ^ 1));
@@ -2689,9 +2711,15 @@ sp2_status sp2_network_backward(const float* H, int B, int N, int L, const float
   const int tgrid = std::min(ntiles, g.num_sms) & (pairs ? ~1 : ~0);
   const SqArgs& R0 = A;
 
-  CK(cudaMemcpyAsync(G, G_out, (size_t)B * slot * 4, cudaMemcpyDeviceToDevice, st));
-  CK(launch_split_pad((float*)G, N, slot, N, B, ls, split ? nullptr : g0(0), g1(0), split ? g0(0) : nullptr, ld_h,
-                      slot_h, sgrid, st));
+  if (pairs) {
+    NetInput x = pair_input(pool, NET_FULL, G_out, ce, N, B, nullptr);
+    x.y = (float*)G;
+    CK(launch_net_input(x, B, st));
+  } else {
+    CK(cudaMemcpyAsync(G, G_out, (size_t)B * slot * 4, cudaMemcpyDeviceToDevice, st));
+    CK(launch_split_pad((float*)G, N, slot, N, B, ls, split ? nullptr : g0(0), g1(0), split ? g0(0) : nullptr, ld_h,
+                        slot_h, sgrid, st));
+  }
   int cur = 0;
 
   for (int sgi = nseg_layers - 1; sgi >= 0; --sgi) {
@@ -2699,13 +2727,12 @@ sp2_status sp2_network_backward(const float* H, int B, int N, int L, const float
     // Y_{n0} = X_{n0} - alpha_{n0} I from the checkpoint and its planes, then
     // recompute to Y_{n1-1}: each launch also writes the planes of its
     // output and carries the row norms to the next (as in the forward pass)
-    CK(launch_materialize(ckpt + (size_t)sgi * B * slot, N, slot, N, B, (const double*)nal + (size_t)n0 * B,
-                          segY(0), N, slot, mgrid, st));
-    CK(launch_split_pad(segY(0), N, slot, N, B, ls, split ? nullptr : segp0(0), segp1(0), split ? segp0(0) : nullptr,
-                        ld_h, slot_h, sgrid, st));
-    if (n1 - n0 > 1)
-      CK(launch_rownorm(segY(0), N, slot, (const int*)ns, B, N, (double*)rn, N, nullptr, nullptr, nullptr, rgrid, st));
     if (pairs) {
+      NetInput x = pair_input(pool, NET_X, ckpt + (size_t)sgi * B * slot, 0, N, B, segY(0));
+      x.add = (const double*)nal + (size_t)n0 * B;
+      x.y = segY(0);
+      x.rn = n1 - n0 > 1 ? (double*)rn : nullptr;
+      CK(launch_net_input(x, B, st));
       // the segment's recomputation and adjoint layers in one launch
       SqArgs P = A;
       P.tri_planes = 1;
@@ -2716,6 +2743,12 @@ sp2_status sp2_network_backward(const float* H, int B, int N, int L, const float
                          st));
       continue;
     }
+    CK(launch_materialize(ckpt + (size_t)sgi * B * slot, N, slot, N, B, (const double*)nal + (size_t)n0 * B,
+                          segY(0), N, slot, mgrid, st));
+    CK(launch_split_pad(segY(0), N, slot, N, B, ls, split ? nullptr : segp0(0), segp1(0), split ? segp0(0) : nullptr,
+                        ld_h, slot_h, sgrid, st));
+    if (n1 - n0 > 1)
+      CK(launch_rownorm(segY(0), N, slot, (const int*)ns, B, N, (double*)rn, N, nullptr, nullptr, nullptr, rgrid, st));
     for (int n = n0; n + 1 < n1; ++n) {
       const int k = n - n0;
       SqArgs F = R0;
@@ -2760,7 +2793,7 @@ sp2_status sp2_network_backward(const float* H, int B, int N, int L, const float
       cur ^= 1;
     }
   }
-  if (G_in) CK(cudaMemcpyAsync(G_in, G, (size_t)B * slot * 4, cudaMemcpyDeviceToDevice, st));
+  if (G_in && !pairs) CK(cudaMemcpyAsync(G_in, G, (size_t)B * slot * 4, cudaMemcpyDeviceToDevice, st));
   void* hd;
   CKS(staging((size_t)L * B * 3 * sizeof(double) + 16, &hd));
   CK(cudaMemcpyAsync(hd, dots, (size_t)L * B * 3 * sizeof(double), cudaMemcpyDeviceToHost, st));
@@ -2846,7 +2879,6 @@ sp2_status sp2_fermi_expansion(const float* H, int B, int N, int L, const double
   CKS(ws(B_DPTR, B * sizeof(float*), &dptr));
   const int ggrid = (int)std::min<long long>((N + 7) / 8, std::max((N + 63) / 64, 2 * g.num_sms / B + 1));
   const int igrid = (int)std::min<long long>(N, std::max(1, 8 * g.num_sms / B + 1));
-  const int rgrid = (int)std::min<long long>((N + 7) / 8, std::max(1, 2 * g.num_sms / B + 1));
   void *part, *tick, *err;
   CKS(ws(B_PART, (size_t)B * std::max(ggrid, igrid) * sizeof(double2), &part));
   CKS(ws(B_TICKET, std::max(64, B) * sizeof(unsigned), &tick, true));
@@ -3000,11 +3032,15 @@ sp2_status sp2_fermi_expansion(const float* H, int B, int N, int L, const double
   A.tri_planes = 1;  // upper super tiles only
 
   // S_0 (shifted form) into D_out and its planes, R_0 = c_0 X_0, row norms of Y_0
-  CK(launch_input_layer((const float* const*)hs, (const int*)ns, N, D_out, N, slot, split ? nullptr : pool.p0,
-                        pool.p1, split ? pool.p0 : nullptr, ld_h, slot_h, N, (int)ld_h, A.lo_scale, (Ctl*)ctl,
-                        nullptr, (double2*)part, (unsigned*)tick, 1, 0, B, igrid, st));
-  CK(launch_readout_init(D_out, N, slot, N, B, (float)(-c[0]), (const double*)dd, (float*)R, igrid, st));
-  CK(launch_rownorm(D_out, N, slot, (const int*)ns, B, N, (double*)rn, N, nullptr, nullptr, nullptr, rgrid, st));
+  NetInput x = pair_input(pool, NET_INPUT, H, 0, N, B, D_out);
+  x.shift = 1;
+  x.ctl = (const Ctl*)ctl;
+  x.rn = (double*)rn;
+  x.y = D_out;
+  x.r = (float*)R;
+  x.r_scale = (float)(-c[0]);
+  x.r_add = (const double*)dd;
+  CK(launch_net_input(x, B, st));
   CK(launch_syrk_tc2(A, lists.list(0, false, true, ntiles / 2 / B), false, pool.m, split,
                      std::min(ntiles, g.num_sms) & ~1, st));
   return SP2_OK;

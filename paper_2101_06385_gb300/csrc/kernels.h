@@ -150,9 +150,6 @@ cudaError_t launch_split(const float* X, long long n, float lo_scale, __half* hi
 cudaError_t launch_split_pad(const float* X, long long ld_x, long long slot_x, int N, int B, float lo_scale,
                              __half* hi, __half* lo, __half* hp, long long ld_h, long long slot_h, int grid,
                              cudaStream_t st);
-// R[b] = s Y[b] + d[b] I (diagonal in FP64): the readout of the input layer.
-cudaError_t launch_readout_init(const float* Y, long long ld_y, long long slot_y, int N, int B, float s,
-                                const double* d, float* R, int grid_x, cudaStream_t st);
 cudaError_t launch_materialize(const float* Y, long long ld_y, long long slot_y, int N, int B, const double* alpha,
                                float* out, long long ld_o, long long slot_o, int grid_x, cudaStream_t st);
 cudaError_t launch_observable(const float* D, const float* A, long long n, double* block_out, int grid,
@@ -291,6 +288,10 @@ struct NetInput {
   double* rn;              // [count][N], or nullptr
   float* x0;               // [count][N][N] Y_0 + alpha0 I, or nullptr
   const double* alpha0;
+  float* y;                // [count][N][N] Y_0 from the row's super tile on, or nullptr
+  float* r;                // [count][N][N] r_scale Y_0 + r_add[b] I, likewise, or nullptr
+  float r_scale;
+  const double* r_add;
   float lo_scale;
 };
 // The layers' coefficients and FP64 shifts from the bounds in ctl, on the device.

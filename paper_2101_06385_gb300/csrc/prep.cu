@@ -563,44 +563,6 @@ __global__ void split_pad_kernel(const float* __restrict__ X, long long ld_x, lo
   }
 }
 
-// ---------------------------------------------------------------- readout
-// R[b] = s Y[b] + d[b] I over the N x N block of each slot (diagonal in
-// FP64): the input layer's term c_0 X_0 of the finite-temperature readout.
-// R must not alias Y (the diagonal is read back after the rows are written).
-__global__ void readout_init_kernel(const float* __restrict__ Y, long long ld_y, long long slot_y, int N, float s,
-                                    const double* __restrict__ d, float* __restrict__ R) {
-  const int b = blockIdx.y;
-  const float* Yb = Y + (long long)b * slot_y;
-  float* Rb = R + (long long)b * slot_y;
-  const bool vec = ((ld_y | slot_y | N) & 3) == 0 && ((((uintptr_t)Y) | ((uintptr_t)R)) & 15) == 0;
-  for (int r = blockIdx.x; r < N; r += gridDim.x) {
-    const float* yr = Yb + (long long)r * ld_y;
-    float* rr = Rb + (long long)r * ld_y;
-    if (vec) {
-      for (int c4 = threadIdx.x; c4 < (N >> 2); c4 += blockDim.x) {
-        const float4 v = reinterpret_cast<const float4*>(yr)[c4];
-        reinterpret_cast<float4*>(rr)[c4] = make_float4(s * v.x, s * v.y, s * v.z, s * v.w);
-      }
-    } else {
-      for (int c = threadIdx.x; c < N; c += blockDim.x) rr[c] = s * yr[c];
-    }
-  }
-  // the diagonal of this block's rows in FP64, after the row writes above
-  __syncthreads();
-  for (long long k = threadIdx.x;; k += blockDim.x) {
-    const long long r = blockIdx.x + k * gridDim.x;
-    if (r >= N) break;
-    Rb[r * ld_y + r] = (float)((double)s * (double)Yb[r * ld_y + r] + d[b]);
-  }
-}
-
-cudaError_t launch_readout_init(const float* Y, long long ld_y, long long slot_y, int N, int B, float s,
-                                const double* d, float* R, int grid_x, cudaStream_t st) {
-  dim3 grid(grid_x, B);
-  readout_init_kernel<<<grid, 256, 0, st>>>(Y, ld_y, slot_y, N, s, d, R);
-  return cudaGetLastError();
-}
-
 // ---------------------------------------------------------------- materialise
 // out[b] = Y[b] + alpha[b] I (FP64 add on the diagonal, one rounding): the
 // full iterate X = alpha I + Y, e.g. for a network checkpoint.  Each block
