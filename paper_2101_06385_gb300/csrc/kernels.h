@@ -187,7 +187,7 @@ size_t syrk_tc2_smem_bytes(bool split);
 // instances' order is the same in every slot's list.
 constexpr int kResTile = 128;
 constexpr int kResStamps = kMaxL + 2;
-constexpr int kMeetRows = 96;  // words of a gang's meeting rows
+constexpr int kMeetRows = 102;  // words of a gang's meeting rows
 struct ResMaps {
   CUtensorMap m[2][4];  // per plane parity: {p0, p1} with 64 x 128 boxes, {p0, p1} with 64 x 64 boxes
 };

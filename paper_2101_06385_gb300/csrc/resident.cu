@@ -47,13 +47,18 @@ struct Slot {
   int b, I, J, N;        // instance, tile row and column (128 units), size
   int par, first;        // parity of the operand planes; first layer
   int closed;            // no more work in this slot
-  int pad;
+  int layer;             // its number
+  int cnt, me;           // the gang, and this tile's place in it
+  int direct;            // the producer itself watches the gang's arrivals
+  int stored;            // epilogue warps that have stored their part of the planes
+  long long* rows;       // the gang's meeting rows
   SolveState st;
 };
 
 struct Shared {
   uint64_t full[STAGES_PLAIN], empty[STAGES_PLAIN];
-  uint64_t ready[2];     // control warp -> producer: operands complete, products may start (or slot closed)
+  uint64_t ready[2];     // control warp -> producer: an instance's first operands, the next ones unless the
+                         //   producer watches the gang's arrivals, or the slot's end
   uint64_t coef[2];      // control warp -> epilogue: the layer's coefficients are set
   uint64_t acc_full[2];  // MMA issuer -> epilogue
   uint64_t epi_done[2];  // epilogue warps -> control warp
@@ -107,6 +112,31 @@ __device__ __forceinline__ double row_norm(const ResArgs& a, const Slot& s, int 
 #pragma unroll
   for (int u = 0; u < 16; ++u) acc += fix_sq(v[u]);
   return (double)acc * Q_LO_UNIT;
+}
+
+// The warp has stored its part of the layer's planes and row norms and read its
+// accumulator; the last of the tile counts it in its gang (Slot::direct: N =
+// 1000 718 -> 683 us, single FP16 2048 787 -> 761).  A lone tile's next products
+// are let go by the control warp, whose sums take no longer than the fence (N =
+// 128 261 against 268 us), and so are those of two slots: a producer that polls
+// for one gang sees the other slot late (512 matrices 26.4 against 26.6 ms).
+__device__ __forceinline__ void stored(Shared& sh, int c, int lane) {
+  Slot& s = sh.slot[c];
+  if (!s.direct) return;
+  tc_fence_before();
+  __syncwarp();
+  if (lane == 0) {
+    __threadfence_block();
+    if (atomicAdd(&s.stored, 1) == EPI_WARPS - 1) {
+      __threadfence_block();
+      s.stored = 0;
+      s.par ^= 1;
+      s.first = 0;
+      const int k = s.layer;
+      s.layer = k + 1;
+      arrive(s.rows, k, s.me);
+    }
+  }
 }
 
 // One layer of the warp's 32 x 32 chunk of a slot's tile (the lane layouts and
@@ -256,6 +286,7 @@ __device__ __forceinline__ bool epilogue(const ResArgs& a, Shared& sh, int c, ui
         const int cm = c0 + 4 * c4 + r4;
         if (cm < N) rnp[(long long)(R0 >> 5) * a.ld_rnp + cm] = csum;
       }
+      stored(sh, c, lane);
       uint32_t w[32];
 #pragma unroll
       for (int k = 0; k < 32; ++k) w[k] = __float_as_uint(y[k]);
@@ -264,7 +295,7 @@ __device__ __forceinline__ bool epilogue(const ResArgs& a, Shared& sh, int c, ui
     }
     sq = warp_sum_ll(fix_sq(sql));
     if (nan || big || sq > SQ_LIMIT) sq = nan ? WARP_NAN : WARP_BIG;
-    if (!outD) fence_proxy_async();  // the planes are read by the TMA units next
+    if (!outD && !s.direct) fence_proxy_async();  // the planes are read by the TMA unit next
     if (outD) {
       if (dchunk) {
 #pragma unroll
@@ -312,6 +343,8 @@ __device__ __forceinline__ bool epilogue(const ResArgs& a, Shared& sh, int c, ui
         }
       }
     }
+  } else if (!outD) {
+    stored(sh, c, lane);
   }
   tmem_st_wait();
   tc_fence_before();
@@ -354,6 +387,12 @@ __device__ __forceinline__ void control(const ResArgs& a, Shared& sh, int c, int
       s.par = 0;
       s.first = 1;
       s.closed = 0;
+      s.layer = 0;
+      s.cnt = cnt;
+      s.direct = cnt > 1 && !a.two_slots;
+      s.me = t - off;
+      s.stored = 0;
+      s.rows = rows;
       if (act) {
         mbar_arrive(&sh.ready[c]);
         mbar_arrive(&sh.coef[c]);
@@ -367,10 +406,10 @@ __device__ __forceinline__ void control(const ResArgs& a, Shared& sh, int c, int
         break;
       }
       done_phase ^= 1u;
-      // after the launch that writes D the solve is over; any other layer has
-      // a next one, whose products need this one's planes but not its sums
+      // after the layer that writes D the solve is over; any other has a next one
       const bool outD = hot->next.out_mode == OUT_D;
-      if (lane == 0 && !outD) {
+      const bool direct = cnt > 1 && !a.two_slots;
+      if (lane == 0 && !outD && !direct) {
         s.par ^= 1;
         s.first = 0;
         if (cnt == 1) mbar_arrive(&sh.ready[c]);
@@ -393,7 +432,7 @@ __device__ __forceinline__ void control(const ResArgs& a, Shared& sh, int c, int
           ok = false;
           break;
         }
-        if (lane == 0 && !outD) mbar_arrive(&sh.ready[c]);
+        if (lane == 0 && !outD && !direct) mbar_arrive(&sh.ready[c]);
         G = meet_sums(rows, k, lane);
         if (leader) meet_empty(rows, k, lane);
         if (outD && leader) {
@@ -480,6 +519,9 @@ __global__ void __launch_bounds__(THREADS, 1) resident_kernel(const __grid_const
     // ------------------------------------------------------------ producer
     if (lane == 0) {
       uint32_t rphase = 0;  // bit c: phase of ready[c]
+      // slot 0's gang and the layer whose planes it waits for (Slot::direct), or none
+      long long* rows = nullptr;
+      int cnt = 0, layer = 0;
       bool open0 = true, open1 = a.two_slots != 0, ok = true;
       int last = 1, stage = 0;
       uint32_t phase = 0, seq = 0;
@@ -491,28 +533,43 @@ __global__ void __launch_bounds__(THREADS, 1) resident_kernel(const __grid_const
       while (ok && (open0 || open1)) {
         int c = -1;
         const uint64_t w0 = globaltimer();
+        bool gang = false;  // slot 0 is ready through its gang's arrivals
         for (int spin = 0; c < 0; ++spin) {
           const int o = last ^ 1;
           if ((o ? open1 : open0) && mbar_test(&sh.ready[o], (rphase >> o) & 1u))
             c = o;
           else if ((last ? open1 : open0) && mbar_test(&sh.ready[last], (rphase >> last) & 1u))
             c = last;
-          else if ((spin & 63) == 63 && (*abort_flag || globaltimer() - w0 > idle))
+          else if (rows && arrived(rows, layer) >= cnt) {
+            __threadfence();  // what the gang stored before it arrived
+            gang = true;
+            c = 0;
+          } else if ((spin & 63) == 63 && (*abort_flag || globaltimer() - w0 > idle))
             break;
         }
         if (c < 0) {
           ok = false;
           break;
         }
-        rphase ^= 1u << c;
+        if (!gang) rphase ^= 1u << c;
         last = c;
         const volatile Slot& s = sh.slot[c];
-        if (s.closed) {
+        if (!gang && s.closed) {
           (c ? open1 : open0) = false;
+          if (c == 0) rows = nullptr;
           continue;
         }
         const int b = s.b, I = s.I, J = s.J, N = s.N, par = s.par;
-        // (the planes' writers have fenced them against the async proxy)
+        // after this layer's products: its gang's planes, or (the last layer) the
+        // control warp
+        if (c == 0) {
+          rows = s.direct ? s.rows : nullptr;
+          cnt = s.cnt;
+          layer = s.layer;
+        }
+        // a gang's planes come from generic stores and are read by the TMA unit (a
+        // proxy fence by each of the storing threads took 0.8 us)
+        if (gang) fence_proxy_async();
         sh.wq[seq % WQ] = c;
         mbar_arrive(&sh.wq_full[seq % WQ]);
         ++seq;

@@ -187,7 +187,7 @@ __device__ __forceinline__ void to_double(const GangSums& s, double& trY, double
 // the last read; so met, a solve takes, by calls of the public entry: N = 2048
 // single FP16 873 -> 795 us, N = 1000 748 -> 712 us, FP32 N = 512 622 -> 480 us.
 constexpr int MEET_GROUPS = 8, MEET_WORDS = 4;  // a sector: t, q_hi, count and q_lo, unused
-static_assert(3 * MEET_GROUPS * MEET_WORDS == kMeetRows, "three rows");
+static_assert(3 * (MEET_GROUPS * MEET_WORDS + 2) == kMeetRows, "three rows, of sums and of arrivals");
 constexpr int MEET_SHIFT = 40;                  // the count above q_lo (304 x 2^28 < 2^37)
 
 __device__ __forceinline__ long long* meet_row(long long* rows, int k) {
@@ -246,9 +246,32 @@ __device__ __forceinline__ GangSums meet_sums(long long* rows, int k, int lane) 
   return s;
 }
 
+// Arrivals: what the next layer's products need of a layer are its planes, not
+// its sums.  A member's last epilogue warp counts it in one of four words as
+// soon as the member's planes are stored, and each producer polls the four
+// itself: a control warp that woke, added up the sums and then polled for both
+// let the products start 1.5 us later.
+__device__ __forceinline__ unsigned* arrival_row(long long* rows, int k) {
+  return reinterpret_cast<unsigned*>(rows + 3 * MEET_GROUPS * MEET_WORDS) + 4 * (k % 3);
+}
+__device__ __forceinline__ void arrive(long long* rows, int k, int me) {
+  __threadfence();
+  asm volatile("red.relaxed.gpu.global.add.u32 [%0], 1;" ::"l"(arrival_row(rows, k) + (me & 3)) : "memory");
+}
+// How many have; before anything they stored is read: a fence.
+__device__ __forceinline__ int arrived(long long* rows, int k) {
+  unsigned a, b, c, d;
+  asm volatile("ld.relaxed.gpu.global.v4.u32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(a), "=r"(b), "=r"(c), "=r"(d)
+               : "l"(arrival_row(rows, k))
+               : "memory");
+  return (int)(a + b + c + d);
+}
+
 // After the meeting of layer k, by the leader's warp.
 __device__ __forceinline__ void meet_empty(long long* rows, int k, int lane) {
   __stcg(meet_row(rows, k + 2) + lane, 0ll);
+  if (lane < 4) __stcg(arrival_row(rows, k + 2) + lane, 0u);
   __syncwarp();
 }
 static_assert(MEET_GROUPS * MEET_WORDS == 32, "one word a lane");
