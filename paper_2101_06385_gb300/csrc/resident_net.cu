@@ -475,7 +475,9 @@ __device__ __forceinline__ bool epilogue(const NetArgs& a, Shared& sh, int c, ui
     double none;
     if (dchunk) lanes_sum(dtr, 0.f, s0, none);
   }
-  if (live && o.out >= 0) fence_proxy_async();  // the planes are read by the TMA units next
+  // the planes are read by the TMA units next: a lone tile's by its own (a gang's
+  // cross behind the meeting's fence and one proxy fence by each producer)
+  if (live && o.out >= 0 && a.per == 1) fence_proxy_async();
   tmem_st_wait();
   tc_fence_before();
   __syncwarp();
@@ -655,7 +657,7 @@ __global__ void __launch_bounds__(THREADS, 1) resident_net_kernel(const __grid_c
         const int b = s.b, I = s.I, J = s.J;
         const bool adj = s.op.kind != 0;
         const int by = s.op.y * a.batch + b, bg = s.op.g * a.batch + b;
-        // (the planes' writers have fenced them against the async proxy)
+        if (a.per > 1) fence_proxy_async();  // the gang's planes, acquired through ready
         sh.wq[seq % WQ] = c;
         mbar_arrive(&sh.wq_full[seq % WQ]);
         ++seq;
