@@ -1973,19 +1973,23 @@ sp2_status network_prologue(const float* H, int B, int N, int L, const float* co
 
 namespace {
 
-// The resident network kernel takes matrices up to n_many in any number and
-// larger ones while the batch's tiles fit the slots.  The launches' CTA pairs
-// cannot fill the chip with few matrices and pay for the padding of small ones
-// (forward, 8 layers: two of N = 2048 502 against 641 us, 300 of 256 1.02
-// against 1.22 ms; backward 1.27 against 1.48 and 2.3 against 2.9 ms); on many
-// large ones their 256 x 256 tiles are faster (32 of 2048: 6.3 against 5.9 and
-// 17.2 against 14.4 ms).  n_many: 1024 forward (30 of them 1.23 against 1.32
-// ms), 512 backward (30 of 1024 3.1 against 2.9 ms).
+// The resident network kernel takes matrices up to n_many in any number, and
+// larger ones while each gang has a window of CTAs and a slot of its own, or a
+// single one its tiles.  The CTA pairs cannot fill the chip with few matrices
+// (backward, 8 layers: 6 of N = 900 719 against 962 us, 4 of 1280 869 against
+// 1079, 2 of 2048 1229 against 1322) and pay for the padding of small ones (64 of
+// 512 1.40 against 1.65 ms, 48 of 896 3.34 against 3.51); many large ones are
+// faster on their 256 x 256 tiles (5 of 1280 1288 against 1127 us, 3 of 1536 1429
+// against 1157, 32 of 1024 3.40 against 2.58 ms).  One matrix from N = 2049 to 2816
+// is within 8 % on either.  n_many: 896 (24 of 960: forward 945 against 919 us,
+// backward 2.35 against 1.99 ms), 1152 for the expansion, whose epilogue reads and
+// writes more on the pairs (20 of 1100 1.29 against 1.65 ms; 12 of 1200 1.07
+// against 1.08).
 bool net_fits(int B, int N, int n_many) {
   if (!resident_fits(N)) return false;
   int n = 0;
   resident_tiles(N, 0, nullptr, &n);
-  return N <= n_many || (long long)n * B <= 2 * g.num_sms;
+  return N <= n_many || B <= 2 * (g.num_sms / n) || (B == 1 && n <= 2 * g.num_sms);
 }
 
 // A run of the resident network kernel (csrc/resident_net.cu) over B matrices
@@ -2349,7 +2353,7 @@ sp2_status sp2_network_forward(const float* H, int B, int N, int L, const float*
       set_err("sp2_network_forward: non-finite coefficient");
       return SP2_ERR_INVALID_ARG;
     }
-  if (net_fits(B, N, 1024)) return net_forward_resident(H, B, N, L, coef, ckpt_every, X_out, ckpt, bounds);
+  if (net_fits(B, N, 896)) return net_forward_resident(H, B, N, L, coef, ckpt_every, X_out, ckpt, bounds);
   const bool tc = tc_precision(g.precision);
   const bool split = g.precision == SP2_PREC_SPLIT_FP16;
   cudaStream_t st = g.stream;
@@ -2544,7 +2548,7 @@ sp2_status sp2_network_backward(const float* H, int B, int N, int L, const float
   const long long slot = (long long)N * N;
   const int ce = ckpt_every;
   // (the planes of all segments' first iterates, as large as the checkpoints, within 32 GiB)
-  if (net_fits(B, N, 512) && (double)((L + ce - 1) / ce + ce + 1) * B * round_up(N, 64) * N * 4.0 < 0x1p35)
+  if (net_fits(B, N, 896) && (double)((L + ce - 1) / ce + ce + 1) * B * round_up(N, 64) * N * 4.0 < 0x1p35)
     return net_backward_resident(H, B, N, L, coef, ce, ckpt, G_out, dcoef, G_in);
   void* G;
   CKS(ws(B_G, (size_t)B * slot * 4, &G));
@@ -2835,7 +2839,7 @@ sp2_status sp2_fermi_expansion(const float* H, int B, int N, int L, const double
   cudaStream_t st = g.stream;
   const long long slot = (long long)N * N;
 
-  if (net_fits(B, N, 1024)) {
+  if (net_fits(B, N, 1152)) {
     NetRun run;
     void *rn, *R;
     CKS(ws(B_RN, (size_t)B * N * sizeof(double), &rn));

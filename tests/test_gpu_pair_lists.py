@@ -48,7 +48,7 @@ def test_last_layers(sp2, max_iter):  # noqa: F811
 
 # several uneven groups of matrices, one group, a matrix larger than a group;
 # segments of one layer, of several, and as long as the network
-@pytest.mark.parametrize("B,N,L,ce", [(20, 1100, 5, 2), (13, 700, 4, 1), (7, 1793, 6, 4), (2, 3000, 3, 3)])
+@pytest.mark.parametrize("B,N,L,ce", [(20, 1100, 5, 2), (13, 1000, 4, 1), (7, 1793, 6, 4), (2, 3000, 3, 3)])
 @pytest.mark.parametrize("precision", ["split", "fp16"])
 def test_network_same_bits(sp2, B, N, L, ce, precision):  # noqa: F811
     g = torch.Generator(device="cuda").manual_seed(N + B)
@@ -74,7 +74,7 @@ def test_network_same_bits(sp2, B, N, L, ce, precision):  # noqa: F811
 
 # the expansion has no single-CTA path: against its layers in FP64 on the GPU's
 # matrix product, each split layer adding at most 2^-20 of the operands' norm
-@pytest.mark.parametrize("B,N", [(20, 1100), (7, 1793), (2, 3000)])
+@pytest.mark.parametrize("B,N", [(14, 1300), (7, 1793), (2, 3000)])
 def test_expansion(sp2, B, N):  # noqa: F811
     g = torch.Generator(device="cuda").manual_seed(N + B)
     H = torch.randn(B, N, N, generator=g, device="cuda")
