@@ -99,16 +99,20 @@ typedef struct {
   double flops_alg;               /* algorithmic FLOPs: layers x 3N^3 (split), N^3 (fp16/fp32) */
   double prologue_ms;             /* device time of the bounds, input layer and first row-norm
                                      kernels */
-  int launches;                   /* squaring launches enqueued (max_iter + 2; max_iter for the
-                                     accelerated solves); launches past the last layer find the
-                                     solve finished and return at once */
+  int launches;                   /* layer slots enqueued (max_iter + 2; max_iter for the accelerated
+                                     solves).  The resident kernels (up to N = 2944, FP32 up to 2048)
+                                     and the CTA pairs of a single solve run all of them in one
+                                     launch that ends with the last layer; elsewhere each is a launch,
+                                     and those past the last layer return at once */
   int8_t sigma[SP2_MAX_LAYERS];   /* sigma[k] = sigma_{k+1} in {+1,-1}; 0 past the end */
   double iderr[SP2_MAX_LAYERS];   /* iderr[k] = IdErr_{k+1} */
   float layer_ms[SP2_MAX_LAYERS]; /* device time of layer k (k < launches): the loop layers, then
-                                     the two refinement layers of Eq. 15 (one squaring launch per
-                                     layer on the tensor-core path; launch plus row-norm pass on
-                                     the FFMA path) */
-  float square_ms[SP2_MAX_LAYERS];/* device time of squaring launch k alone */
+                                     the two refinement layers of Eq. 15.  Where one launch runs all
+                                     layers: from the end of the layer before to its own, of this
+                                     instance, 0 past the last layer.  Else the launch (with the
+                                     row-norm pass on the FFMA path) */
+  float square_ms[SP2_MAX_LAYERS];/* device time of squaring launch k alone; equal to layer_ms where
+                                     one launch runs all layers */
   double energy;                  /* Tr[D H] (Alg. 1, last line), accumulated by the launch that
                                      writes D (tensor-core path; 0 on the FFMA path) */
 } sp2_stats;
@@ -117,14 +121,18 @@ typedef struct {
  * SPLIT_FP16, s = 11, shift on, eps 0}.  Calling again re-applies a config
  * (the workspace is kept).  Errors: INVALID_ARG (bad field), CUDA.
  * Schedule switches read here from the environment (none changes a result
- * except where stated): SP2_SQUARE_KERNEL=single (single CTAs instead of CTA
- * pairs), SP2_BATCHED_KERNEL=single|pairs (fix the batched schedule instead
+ * except where stated): SP2_SQUARE_KERNEL=single (single CTAs, a launch a
+ * layer, instead of the resident kernels and CTA pairs),
+ * SP2_BATCHED_KERNEL=single|pairs (a launch a layer on this schedule instead of
+ * the resident kernel; where that does not apply, a matrix above 2944, instead
  * of timing both on the first call of a batch signature), SP2_GRAPHS=0
  * (enqueue the batched launches directly instead of replaying a CUDA graph),
  * SP2_WAVE_SYNC=<K stages> (epoch of the pairs' soft synchronisation in the
- * single solve, 16; 0 off), SP2_TILE_GROUP=<n> (side of the square tile
- * groups, 8), SP2_WIDE=0|1 (two super tiles of a row per pair pass in the
- * single solve; default: where it takes no more waves, i.e. N = 16384),
+ * single split solve from N = 6144 on, 16; 0 off), SP2_TILE_GROUP=<n> (side of
+ * the square tile groups, 8), SP2_WIDE=0|1 (two super tiles of a row per pair
+ * pass in the single solve, 1 also instead of the resident kernel; default: by
+ * the waves of pairs it takes, i.e. at N = 16384, and plain FP16 at most sizes
+ * above 2944),
  * SP2_SNAKE=1 (alternate waves walk K backwards: changes the accumulation
  * order), SP2_FAULT=<spec> (test-only fault injection, sp2_set_fault). */
 sp2_status sp2_init(const sp2_config* cfg);

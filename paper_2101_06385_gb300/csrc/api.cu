@@ -837,7 +837,7 @@ void resident_tiles(int N, int b, std::vector<uint32_t>* out, int* count) {
 }
 
 // The resident kernel takes a solve whose largest instance has no more tiles
-// than the chip has slots (two per SM; N <= 2816 on 152 SMs): below that the
+// than the chip has slots (two per SM; N <= 2944 on 152 SMs): below that the
 // CTA pairs' 256 x 256 tiles cannot fill the chip (at N = 2048 there are 36
 // for 76 pairs) and every layer pays a launch.
 bool resident_fits(int Nmax) {
