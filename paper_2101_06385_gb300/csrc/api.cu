@@ -1037,6 +1037,7 @@ sp2_status resident_solve(const float* const* H, const int* N, const int* N_occ,
   A.err = (int*)(dp + P.err);
   A.wait_ns = g.wait_ns;
   A.two_slots = nt > grid ? 1 : 0;
+  A.local = Nmax <= kResTile ? 1 : 0;
   A.stall = (single && g.fault_stall) ? 1 : 0;
   if (single) g.fault_stall = false;
   ResMaps maps;

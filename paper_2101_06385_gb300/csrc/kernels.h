@@ -217,6 +217,7 @@ struct ResArgs {
   unsigned* stamps;        // [batch][kResStamps] ns from an instance's start to the end of its k-th layer
   float lo_scale, lo_unscale;
   int shift, two_slots;
+  int local;               // every instance is one tile: its planes stay in shared memory
   int stall;               // as SqArgs
   int* err;
   unsigned long long wait_ns;

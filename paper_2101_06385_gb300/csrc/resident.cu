@@ -120,9 +120,11 @@ __device__ __forceinline__ double row_norm(const ResArgs& a, const Slot& s, int 
 // are let go by the control warp, whose sums take no longer than the fence (N =
 // 128 261 against 268 us), and so are those of two slots: a producer that polls
 // for one gang sees the other slot late (512 matrices 26.4 against 26.6 ms).
+template <bool LOCAL>
 __device__ __forceinline__ void stored(Shared& sh, int c, int lane) {
   Slot& s = sh.slot[c];
   if (!s.direct) return;
+  if (LOCAL) fence_proxy_async_shared();  // the MMAs read the planes next
   tc_fence_before();
   __syncwarp();
   if (lane == 0) {
@@ -134,16 +136,19 @@ __device__ __forceinline__ void stored(Shared& sh, int c, int lane) {
       s.first = 0;
       const int k = s.layer;
       s.layer = k + 1;
-      arrive(s.rows, k, s.me);
+      if (LOCAL)
+        mbar_arrive(&sh.ready[c]);
+      else
+        arrive(s.rows, k, s.me);
     }
   }
 }
 
 // One layer of the warp's 32 x 32 chunk of a slot's tile (the lane layouts and
 // arithmetic of epi::tile).  False: the accumulator wait failed.
-template <bool SPLIT>
-__device__ __forceinline__ bool epilogue(const ResArgs& a, Shared& sh, int c, uint32_t acc_phase, uint32_t tmem_base,
-                                         int ew, int q, int lane, float* trb, unsigned long long lim) {
+template <bool SPLIT, bool LOCAL>
+__device__ __forceinline__ bool epilogue(const ResArgs& a, Shared& sh, int c, uint8_t* area, uint32_t acc_phase,
+                                         uint32_t tmem_base, int ew, int q, int lane, float* trb, unsigned long long lim) {
   const Slot& s = sh.slot[c];
   const Ctl* ct = s.st.ctl();
   const int b = s.b, N = s.N, first = s.first;
@@ -232,6 +237,16 @@ __device__ __forceinline__ bool epilogue(const ResArgs& a, Shared& sh, int c, ui
   tc_fence_after();
 
   double dtr = 0.0;
+  // the warp's sums to the control warp
+  auto report = [&]() {
+    __syncwarp();
+    if (lane == 0) {
+      sh.red_t[c][ew] = tr;
+      sh.red_q[c][ew] = sq;
+      if (outD) sh.red_e[c][ew] = dtr;
+      mbar_arrive(&sh.epi_done[c]);
+    }
+  };
   if (live) {
     const bool full = nrows == 32 && c0 + 32 <= N;
     {
@@ -273,10 +288,24 @@ __device__ __forceinline__ bool epilogue(const ResArgs& a, Shared& sh, int c, ui
     }
     const float sql = ((rs[0] + rs[1]) + (rs[2] + rs[3])) + ((rs[4] + rs[5]) + (rs[6] + rs[7]));
     const bool nan = __any_sync(0xffffffffu, isnan(sql)), big = __any_sync(0xffffffffu, !(sql < 16.f));
+    auto sum_squares = [&]() {
+      sq = warp_sum_ll(fix_sq(sql));
+      if (nan || big || sq > SQ_LIMIT) sq = nan ? WARP_NAN : WARP_BIG;
+    };
     if (!outD) {
-      // operand planes of Y' (Eq. 12) first: they are what the gang waits for
-      const long long po = (long long)b * a.slot_h + (long long)(R0 + r4) * a.ld_h + ce;
-      store_planes<SPLIT>(y, a.p0[s.par ^ 1] + po, SPLIT ? a.p1[s.par ^ 1] + po : nullptr, a.ld_h, nrows - r4, lo_scale);
+      if (LOCAL) {
+        // a lone tile's control step bounds its layer: the sums first, then the
+        // planes, which go no further than the operand tiles
+        sum_squares();
+        report();
+        store_planes_shared<SPLIT>(y, area + (hc >> 1) * (SPLIT ? 2 : 1) * HALF_BYTES, q * 32 + r4,
+                                   (hc & 1) * 32 + 4 * c4, nrows - r4, lo_scale);
+      } else {
+        // operand planes of Y' (Eq. 12) first: they are what the gang waits for
+        const long long po = (long long)b * a.slot_h + (long long)(R0 + r4) * a.ld_h + ce;
+        store_planes<SPLIT>(y, a.p0[s.par ^ 1] + po, SPLIT ? a.p1[s.par ^ 1] + po : nullptr, a.ld_h, nrows - r4,
+                            lo_scale);
+      }
       // row norms of the next layer
       float* rnp = a.rnp[s.par] + (long long)b * a.slot_rnp;
       const float rsum = epi::lane_sums<8, 0>(rs);
@@ -286,15 +315,14 @@ __device__ __forceinline__ bool epilogue(const ResArgs& a, Shared& sh, int c, ui
         const int cm = c0 + 4 * c4 + r4;
         if (cm < N) rnp[(long long)(R0 >> 5) * a.ld_rnp + cm] = csum;
       }
-      stored(sh, c, lane);
+      stored<LOCAL>(sh, c, lane);
       uint32_t w[32];
 #pragma unroll
       for (int k = 0; k < 32; ++k) w[k] = __float_as_uint(y[k]);
       __syncwarp();
       tmem_st32(ty, w);
     }
-    sq = warp_sum_ll(fix_sq(sql));
-    if (nan || big || sq > SQ_LIMIT) sq = nan ? WARP_NAN : WARP_BIG;
+    if (outD || !LOCAL) sum_squares();
     if (!outD && !s.direct) fence_proxy_async();  // the planes are read by the TMA unit next
     if (outD) {
       if (dchunk) {
@@ -344,21 +372,17 @@ __device__ __forceinline__ bool epilogue(const ResArgs& a, Shared& sh, int c, ui
       }
     }
   } else if (!outD) {
-    stored(sh, c, lane);
+    if (LOCAL) report();
+    stored<LOCAL>(sh, c, lane);
   }
   tmem_st_wait();
   tc_fence_before();
-  __syncwarp();
-  if (lane == 0) {
-    sh.red_t[c][ew] = tr;
-    sh.red_q[c][ew] = sq;
-    if (outD) sh.red_e[c][ew] = dtr;
-    mbar_arrive(&sh.epi_done[c]);
-  }
+  if (outD || !LOCAL) report();
   return true;
 }
 
 // Control of one slot: takes the tiles of its list and drives their layers.
+template <bool LOCAL>
 __device__ __forceinline__ void control(const ResArgs& a, Shared& sh, int c, int lane, unsigned long long idle) {
   Slot& s = sh.slot[c];
   Ctl* hot = s.st.ctl();
@@ -389,7 +413,7 @@ __device__ __forceinline__ void control(const ResArgs& a, Shared& sh, int c, int
       s.closed = 0;
       s.layer = 0;
       s.cnt = cnt;
-      s.direct = cnt > 1 && !a.two_slots;
+      s.direct = LOCAL || (cnt > 1 && !a.two_slots);
       s.me = t - off;
       s.stored = 0;
       s.rows = rows;
@@ -408,7 +432,7 @@ __device__ __forceinline__ void control(const ResArgs& a, Shared& sh, int c, int
       done_phase ^= 1u;
       // after the layer that writes D the solve is over; any other has a next one
       const bool outD = hot->next.out_mode == OUT_D;
-      const bool direct = cnt > 1 && !a.two_slots;
+      const bool direct = LOCAL || (cnt > 1 && !a.two_slots);
       if (lane == 0 && !outD && !direct) {
         s.par ^= 1;
         s.first = 0;
@@ -469,7 +493,9 @@ __device__ __forceinline__ void control(const ResArgs& a, Shared& sh, int c, int
   }
 }
 
-template <bool SPLIT>
+// LOCAL: every instance is one tile, whose planes stay in the operand tiles of its
+// slot (N = 128: a layer 5.4 -> 4.6 us, N = 64: 3.7).
+template <bool SPLIT, bool LOCAL>
 __global__ void __launch_bounds__(THREADS, 1) resident_kernel(const __grid_constant__ ResMaps maps, const ResArgs a) {
   constexpr int STAGES = SPLIT ? STAGES_SPLIT : STAGES_PLAIN;
   constexpr int STAGE_BYTES = SPLIT ? STAGE_SPLIT : STAGE_PLAIN;
@@ -559,11 +585,11 @@ __global__ void __launch_bounds__(THREADS, 1) resident_kernel(const __grid_const
           if (c == 0) rows = nullptr;
           continue;
         }
-        const int b = s.b, I = s.I, J = s.J, N = s.N, par = s.par;
+        const int b = s.b, I = s.I, J = s.J, N = s.N, par = s.par, first = s.first;
         // after this layer's products: its gang's planes, or (the last layer) the
         // control warp
         if (c == 0) {
-          rows = s.direct ? s.rows : nullptr;
+          rows = s.direct && !LOCAL ? s.rows : nullptr;
           cnt = s.cnt;
           layer = s.layer;
         }
@@ -581,9 +607,19 @@ __global__ void __launch_bounds__(THREADS, 1) resident_kernel(const __grid_const
             ok = false;
             break;
           }
-          uint8_t* dst = smem + stage * STAGE_BYTES;
-          mbar_expect_tx(&sh.full[stage], (same ? 1 : 2) * PLANES * HALF_BYTES);
+          // (a lone tile's operands have a place of their own; after the first layer
+          // its epilogue has left them there)
+          uint8_t* dst = smem + (LOCAL ? (2 * c + kb) * PLANES * HALF_BYTES : stage * STAGE_BYTES);
           ++armed[stage];
+          if (LOCAL && !first) {
+            mbar_arrive(&sh.full[stage]);
+            if (++stage == STAGES) {
+              stage = 0;
+              phase ^= 1u;
+            }
+            continue;
+          }
+          mbar_expect_tx(&sh.full[stage], (same ? 1 : 2) * PLANES * HALF_BYTES);
           const int k0 = kb * BK, ks = k0 / BN;  // super column of this K block
           const bool ta = ks < (I >> 1), tb = ks < (J >> 1);
           load_half(dst, &m[0], &m[2], ta, rowA, k0, b, &sh.full[stage]);
@@ -636,7 +672,8 @@ __global__ void __launch_bounds__(THREADS, 1) resident_kernel(const __grid_const
             break;
           }
           tc_fence_after();
-          const uint32_t st = smem_u32(smem + stage * STAGE_BYTES);
+          const uint32_t st =
+              smem_u32(smem + (LOCAL ? (2 * c + kb) * PLANES * HALF_BYTES : stage * STAGE_BYTES));
           const uint32_t sb = same ? st : st + PLANES * HALF_BYTES;
           const int ks = kb * BK / BN;
           const bool ta = ks < (I >> 1), tb = ks < (J >> 1);
@@ -677,7 +714,7 @@ __global__ void __launch_bounds__(THREADS, 1) resident_kernel(const __grid_const
     }
   } else if (warp >= CTL_WARP) {
     const int c = warp - CTL_WARP;
-    if (c == 0 || a.two_slots) control(a, sh, c, lane, idle);
+    if (c == 0 || a.two_slots) control<LOCAL>(a, sh, c, lane, idle);
   } else {
     // ------------------------------------------------------------ epilogue
     const int ew = warp - 2, q = warp & 3;
@@ -686,7 +723,8 @@ __global__ void __launch_bounds__(THREADS, 1) resident_kernel(const __grid_const
       if (!__all_sync(0xffffffffu, mbar_wait(&sh.wq_full[seq % WQ], (seq / WQ) & 1u, abort_flag, idle))) break;
       const int c = *(volatile int*)&sh.wq[seq % WQ];
       if (c == WQ_END) break;
-      if (!epilogue<SPLIT>(a, sh, c, (aphase >> c) & 1u, tmem_base, ew, q, lane, trbuf + ew * (16 * 32), lim)) {
+      uint8_t* area = smem + 2 * c * PLANES * HALF_BYTES;
+      if (!epilogue<SPLIT, LOCAL>(a, sh, c, area, (aphase >> c) & 1u, tmem_base, ew, q, lane, trbuf + ew * (16 * 32), lim)) {
         if (lane == 0) atomicExch(a.err, (int)SP2_ERR_DEVICE_TIMEOUT);
         *abort_flag = 1;
         break;
@@ -787,9 +825,6 @@ cudaError_t launch_resident_input(const ResArgs& a, int vec_norm, int Nmax, int 
 cudaError_t launch_resident(const ResArgs& a, const ResMaps& maps, bool split, int grid, cudaStream_t st) {
   constexpr int smem = res::OPERAND_BYTES + res::TR_BYTES + (int)sizeof(res::Shared);
   static_assert(smem <= 227 * 1024, "shared memory");
-  cudaError_t e = split ? cudaFuncSetAttribute(res::resident_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)
-                        : cudaFuncSetAttribute(res::resident_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid, 1, 1);
   cfg.blockDim = dim3(res::THREADS, 1, 1);
@@ -800,8 +835,12 @@ cudaError_t launch_resident(const ResArgs& a, const ResMaps& maps, bool split, i
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return split ? cudaLaunchKernelEx(&cfg, res::resident_kernel<true>, maps, a)
-               : cudaLaunchKernelEx(&cfg, res::resident_kernel<false>, maps, a);
+  auto go = [&](auto kernel) -> cudaError_t {
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    return e == cudaSuccess ? cudaLaunchKernelEx(&cfg, kernel, maps, a) : e;
+  };
+  if (a.local) return split ? go(res::resident_kernel<true, true>) : go(res::resident_kernel<false, true>);
+  return split ? go(res::resident_kernel<true, false>) : go(res::resident_kernel<false, false>);
 }
 
 }  // namespace sp2

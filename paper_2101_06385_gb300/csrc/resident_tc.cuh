@@ -102,13 +102,12 @@ __device__ __forceinline__ void turn_tmem(float* trb, uint32_t taddr, int lane, 
 // fp16(2^s x - hp), both differences exact; plain FP16 keeps hi alone), four
 // halves per plane and row; p0, p1 at the lane's first row and column, rows
 // 4 i < rows_left.
-template <bool SPLIT>
-__device__ __forceinline__ void store_planes(const float (&y)[32], __half* p0, __half* p1, long long ld_h,
-                                             int rows_left, float lo_scale) {
+template <bool SPLIT, class Put>
+__device__ __forceinline__ void split_chunk(const float (&y)[32], float lo_scale, Put put) {
   const __half2 s2 = __float2half2_rn(lo_scale);
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
-    uint32_t pa[2], pl[2];
+    uint32_t pa[2], pl[2] = {0u, 0u};
 #pragma unroll
     for (int e2 = 0; e2 < 2; ++e2) {
       const float x0 = y[4 * i + 2 * e2], x1 = y[4 * i + 2 * e2 + 1];
@@ -121,13 +120,38 @@ __device__ __forceinline__ void store_planes(const float (&y)[32], __half* p0, _
       }
       pa[e2] = *reinterpret_cast<const uint32_t*>(&p2);
     }
+    put(i, make_uint2(pa[0], pa[1]), make_uint2(pl[0], pl[1]));
+  }
+}
+
+template <bool SPLIT>
+__device__ __forceinline__ void store_planes(const float (&y)[32], __half* p0, __half* p1, long long ld_h,
+                                             int rows_left, float lo_scale) {
+  split_chunk<SPLIT>(y, lo_scale, [&](int i, uint2 a, uint2 l) {
     if (4 * i < rows_left) {
-      *reinterpret_cast<uint2*>(p0) = make_uint2(pa[0], pa[1]);
-      if (SPLIT) *reinterpret_cast<uint2*>(p1) = make_uint2(pl[0], pl[1]);
+      *reinterpret_cast<uint2*>(p0) = a;
+      if (SPLIT) *reinterpret_cast<uint2*>(p1) = l;
     }
     p0 += 4 * ld_h;
     if (SPLIT) p1 += 4 * ld_h;
-  }
+  });
+}
+
+// The same into operand tiles in shared memory (128 rows of 128 bytes, 16-byte
+// groups XOR-swizzled by row as a TMA load leaves them): t0 the tile of the
+// chunk's K block, the second plane's HALF_BYTES after it; row, col: the lane's
+// first row and column in the tile.
+template <bool SPLIT>
+__device__ __forceinline__ void store_planes_shared(const float (&y)[32], uint8_t* t0, int row, int col, int rows_left,
+                                                    float lo_scale) {
+  split_chunk<SPLIT>(y, lo_scale, [&](int i, uint2 a, uint2 l) {
+    if (4 * i < rows_left) {
+      const int r = row + 4 * i;
+      uint8_t* p = t0 + r * 128 + ((((col >> 3) ^ r) & 7) << 4) + ((col & 4) << 1);
+      *reinterpret_cast<uint2*>(p) = a;
+      if (SPLIT) *reinterpret_cast<uint2*>(p + HALF_BYTES) = l;
+    }
+  });
 }
 
 // One row of an input matrix by one warp: y = y0(value, column) for each
