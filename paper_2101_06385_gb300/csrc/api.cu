@@ -318,10 +318,10 @@ void rnp_step(SqArgs& A, void** rnp, int k) {
   A.rnp_in = k > 0 ? (const float*)rnp[(k - 1) & 1] : nullptr;
 }
 
-// Epoch counters of the CTA pairs' soft synchronisation for nlaunch launches
+// Epoch counters of the CTA pairs' soft synchronisation for nlaunch layers
 // over a tile list of ntiles entries (two per super tile, every tile active)
 // whose tiles have nkt K stages: one zeroed slice of *per counters per
-// launch, or none when the synchronisation is off (SP2_WAVE_SYNC=0).
+// layer, or none when the synchronisation is off (SP2_WAVE_SYNC=0).
 sp2_status wave_counters(int ntiles, int grid, int nkt, int nlaunch, unsigned** wave, size_t* per) {
   *wave = nullptr;
   *per = 0;

@@ -77,10 +77,11 @@ struct SqArgs {
   // Soft synchronisation of the CTA pairs' K progress (CTA-pair kernel, one
   // instance): every sync_stages K stages a pair publishes the epoch it
   // finished in wave_ctr[epoch] and, before loading further, waits (bounded;
-  // it stops waiting for the rest of the launch after one time-out) until
+  // it stops waiting for the rest of the layer after one time-out) until
   // every pair has finished the epoch before that one.  Pairs that share an
   // operand panel then read it within a short time of each other, while it
-  // is still in L2.  wave_ctr: zeroed counters of this launch; nullptr = off.
+  // is still in L2.  wave_ctr: zeroed counters, PairList::wave_per of each layer;
+  // nullptr = off.
   unsigned* wave_ctr;
   int sync_stages;
   int wide;                // CTA-pair kernel: 1 = units of two super tiles (I, J), (I, J + 1) of a

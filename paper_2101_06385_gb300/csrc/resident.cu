@@ -3,9 +3,10 @@
 // A CTA owns one or two 128 x 128 tiles of the upper super tiles and keeps
 // each for all layers of its solve: the FP32 iterate of the tile stays in
 // tensor memory next to its accumulator, and only the FP16 operand planes go
-// through L2.  The CTAs of one instance (its gang) meet after every layer at
-// their sums in global memory and each runs the control step of Alg. 1 on the
-// same sums, so a solve costs no launch per layer and stops at its last one.
+// through L2 (with instances of one tile not even those).  The CTAs of one
+// instance (its gang) meet after every layer: the next products start when all
+// its planes are stored, and each CTA runs the control step of Alg. 1 on the same
+// sums meanwhile, so a solve costs no launch per layer and stops at its last one.
 //
 // What bounds it: for small N the chain of one layer (operand loads, K / 64
 // stages of twelve dependent MMAs at 0.47 us each, epilogue, gang meeting);

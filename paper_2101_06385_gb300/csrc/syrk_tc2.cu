@@ -145,7 +145,7 @@ __device__ __forceinline__ unsigned pairs_in_epoch(uint32_t e, int W, int nk, in
   return 0u;
 }
 
-// Waits until *ctr >= need; false (stop waiting for the rest of the launch)
+// Waits until *ctr >= need; false (stop waiting for the rest of the layer)
 // once the wait has taken longer than a small fraction of the wait bound.
 __device__ __forceinline__ bool epoch_wait(const unsigned* ctr, unsigned need, unsigned long long lim) {
   const volatile unsigned* c = ctr;
