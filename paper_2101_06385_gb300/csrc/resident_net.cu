@@ -38,8 +38,9 @@ struct Slot {
   int b, I, J, t;  // matrix, tile row and column (128 units), tile index
   int closed;      // no more work in this slot
   int pad;
-  NetOp op;        // operation in progress and its coefficients (a layer's first
-  LayerParams p;   // touch of them in global memory would stand in its chain)
+  NetOp op[2];       // operations in progress, by the parity of their number in the slot, and
+  LayerParams p[2];  // their coefficients (a layer's first touch of them in global memory would
+                     // stand in its chain)
 };
 static_assert(sizeof(NetOp) % 8 == 0 && sizeof(LayerParams) % 8 == 0, "copied in 8-byte words");
 
@@ -47,13 +48,15 @@ struct Shared {
   uint64_t full[STAGES_PLAIN], empty[STAGES_PLAIN];
   uint64_t ready[2];     // control warp -> producer: operands complete (or slot closed)
   uint64_t acc_full[2];  // MMA issuer -> epilogue
-  uint64_t epi_done[2];  // epilogue warps -> control warp
+  uint64_t stored[2];    // epilogue warps -> control warp: planes and row norms stored, accumulator read (one slot)
+  uint64_t epi_done[2][2];  // [slot][parity] the same: operation finished (a warp without rows may be an
+                            //   operation ahead of the others: it must not stand in for them)
   uint64_t wq_full[WQ];  // producer -> MMA issuer and epilogue: next slot
   uint64_t drain;
   int wq[WQ];
   uint32_t tmem;
   int abort;
-  double red[2][EPI_WARPS][3];  // dot products per warp: tr Yin, <Yin, aux>, <P, aux>
+  double red[2][2][EPI_WARPS][3];  // [parity] dot products per warp: tr Yin, <Yin, aux>, <P, aux>
   Slot slot[2];
 };
 
@@ -161,12 +164,13 @@ __device__ __forceinline__ void sum3(double& a, double& b, double& c) {
 
 // One operation on the warp's 32 x 32 chunk of a slot's tile (lane layouts of
 // epi::tile).  False: the accumulator wait failed.
-template <bool SPLIT>
+template <bool SPLIT, bool EARLY>
 __device__ __forceinline__ bool epilogue(const NetArgs& a, Shared& sh, int c, uint32_t acc_phase, uint32_t tmem_base,
                                          int ew, int q, int lane, float* trb, unsigned long long lim) {
   const Slot& s = sh.slot[c];
-  const NetOp& o = s.op;
-  const LayerParams& p = s.p;  // (in shared memory: registers hold the chunk)
+  const uint32_t cur = EARLY ? acc_phase : 0u;  // (both count the slot's operations)
+  const NetOp& o = s.op[cur];
+  const LayerParams& p = s.p[cur];  // (in shared memory: registers hold the chunk)
   const int b = s.b, N = a.N, I = s.I, J = s.J;
   const bool adj = o.kind != 0;
   const int hc = ew >> 2, R0 = I * TB + q * 32, c0 = J * TB + hc * 32;
@@ -184,6 +188,16 @@ __device__ __forceinline__ bool epilogue(const NetArgs& a, Shared& sh, int c, ui
   // the tile's private store of an iterate: 8 float4 per lane, lanes side by side
   const long long priv = ((long long)s.t * EPI_WARPS + ew) * 1024 + lane * 4;
 
+  // The warp has read its accumulator and stored its part of the planes and row
+  // norms.  (The planes are read by the TMA units next: a lone tile's by its own;
+  // a gang's cross behind the meeting's fence and one proxy fence by each producer.)
+  auto stored = [&]() {
+    if (!EARLY) return;
+    if (live && o.out >= 0 && a.per == 1) fence_proxy_async();
+    tc_fence_before();
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&sh.stored[c]);
+  };
   // kind 1: Y's four columns of row 4 i + r4
   auto aux4 = [&](int i) {
     if (o.aux) return *reinterpret_cast<const float4*>(o.aux + priv + i * 128);
@@ -361,6 +375,7 @@ __device__ __forceinline__ bool epilogue(const NetArgs& a, Shared& sh, int c, ui
         if (cm < N) rnp[(long long)(R0 >> 5) * a.ld_rnp + cm] = csum;
       }
     }
+    stored();
     if (o.tmem) {
       uint32_t w[32];
 #pragma unroll
@@ -466,6 +481,7 @@ __device__ __forceinline__ bool epilogue(const NetArgs& a, Shared& sh, int c, ui
       }
     }
   }
+  if (!live) stored();
   double s0 = 0.0, s1 = 0.0, s2 = 0.0;
   if (adj) {
     const double twice = mirror ? 2.0 : 1.0;
@@ -475,28 +491,28 @@ __device__ __forceinline__ bool epilogue(const NetArgs& a, Shared& sh, int c, ui
     double none;
     if (dchunk) lanes_sum(dtr, 0.f, s0, none);
   }
-  // the planes are read by the TMA units next: a lone tile's by its own (a gang's
-  // cross behind the meeting's fence and one proxy fence by each producer)
-  if (live && o.out >= 0 && a.per == 1) fence_proxy_async();
+  if (!EARLY && live && o.out >= 0 && a.per == 1) fence_proxy_async();
   tmem_st_wait();
   tc_fence_before();
   __syncwarp();
   if (lane == 0) {
     if (adj) {
-      sh.red[c][ew][0] = s0;
-      sh.red[c][ew][1] = s1;
-      sh.red[c][ew][2] = s2;
+      sh.red[cur][c][ew][0] = s0;
+      sh.red[cur][c][ew][1] = s1;
+      sh.red[cur][c][ew][2] = s2;
     }
-    mbar_arrive(&sh.epi_done[c]);
+    mbar_arrive(&sh.epi_done[c][cur]);
   }
   return true;
 }
 
 // Control of one slot: takes the tiles of its list through their operations.
+template <bool EARLY>
 __device__ __forceinline__ void control(const NetArgs& a, Shared& sh, int c, int lane, unsigned long long idle) {
   Slot& s = sh.slot[c];
   const int sl = c * (int)gridDim.x + (int)blockIdx.x;
-  uint32_t done_phase = 0;
+  uint32_t done_phase = 0, next = 0;  // parities of the operation to finish, to begin
+  uint32_t done_round = 0;            // phase of epi_done[c][done_phase]
   bool ok = true;
   for (int li = a.list_off[sl]; ok && li < a.list_off[sl + 1]; ++li) {
     const int t = a.list[li], cnt = a.per;
@@ -514,8 +530,9 @@ __device__ __forceinline__ void control(const NetArgs& a, Shared& sh, int c, int
       if (lane < PW) wp = reinterpret_cast<const long long*>(a.lp + (long long)layer * a.batch + b)[lane];
     };
     auto begin = [&]() {
-      if (lane < OW) reinterpret_cast<long long*>(&s.op)[lane] = wo;
-      if (lane < PW) reinterpret_cast<long long*>(&s.p)[lane] = wp;
+      if (lane < OW) reinterpret_cast<long long*>(&s.op[next])[lane] = wo;
+      if (lane < PW) reinterpret_cast<long long*>(&s.p[next])[lane] = wp;
+      if (EARLY) next ^= 1u;
       __syncwarp();
       if (lane == 0) mbar_arrive(&sh.ready[c]);
     };
@@ -531,19 +548,17 @@ __device__ __forceinline__ void control(const NetArgs& a, Shared& sh, int c, int
     for (int k = 0; k < a.nops; ++k) {
       const int kind = __shfl_sync(0xffffffffu, (int)wo, 0);
       if (k + 1 < a.nops) fetch(k + 1);
-      if (!__all_sync(0xffffffffu, mbar_wait(&sh.epi_done[c], done_phase, &sh.abort, idle))) {
+      // The next operation's products need the gang's planes; the rest of this one's
+      // epilogue (readout, whole matrices, dot products) runs beside them: expansion
+      // of 8 x 512 220 -> 201 us, network step of 6 x 300 667 -> 634.
+      const uint32_t cur = EARLY ? done_phase : 0u;
+      auto finished = [&]() {
+        return mbar_wait(&sh.epi_done[c][cur], EARLY ? done_round : done_phase, &sh.abort, idle);
+      };
+      if (!__all_sync(0xffffffffu, EARLY ? mbar_wait(&sh.stored[c], done_phase, &sh.abort, idle) : finished())) {
         ok = false;
         break;
       }
-      done_phase ^= 1u;
-      const int dot = s.op.dot;
-      double d0 = 0.0, d1 = 0.0, d2 = 0.0;
-      if (kind != 0 && lane < EPI_WARPS) {
-        d0 = sh.red[c][lane][0];
-        d1 = sh.red[c][lane][1];
-        d2 = sh.red[c][lane][2];
-      }
-      __syncwarp();
       if (k + 1 < a.nops && cnt > 1) {
         if (lane == 0) meet_join(rows, k, t - off, GangSums{0, 0, 0}, false);
         if (!meet_wait(rows, k, cnt, lane, a.err, &sh.abort, idle)) {
@@ -552,7 +567,21 @@ __device__ __forceinline__ void control(const NetArgs& a, Shared& sh, int c, int
         }
         if (t == off) meet_empty(rows, k, lane);
       }
+      const int dot = s.op[cur].dot;
       if (k + 1 < a.nops) begin();
+      if (EARLY && !__all_sync(0xffffffffu, finished())) {
+        ok = false;
+        break;
+      }
+      double d0 = 0.0, d1 = 0.0, d2 = 0.0;
+      if (kind != 0 && lane < EPI_WARPS) {
+        d0 = sh.red[cur][c][lane][0];
+        d1 = sh.red[cur][c][lane][1];
+        d2 = sh.red[cur][c][lane][2];
+      }
+      done_round ^= done_phase;
+      done_phase ^= 1u;
+      __syncwarp();
       if (kind != 0) {  // under the next operation's products
         sum3(d0, d1, d2);
         if (lane == 0) {
@@ -575,7 +604,10 @@ __device__ __forceinline__ void control(const NetArgs& a, Shared& sh, int c, int
   }
 }
 
-template <bool SPLIT>
+// EARLY: one slot; the next operation begins when this one's planes are stored
+// (with two, where the other slot's products fill the time, its second set of
+// operands cost 2 to 4 %).
+template <bool SPLIT, bool EARLY>
 __global__ void __launch_bounds__(THREADS, 1) resident_net_kernel(const __grid_constant__ NetMaps maps, const NetArgs a) {
   constexpr int STAGES = SPLIT ? STAGES_SPLIT : STAGES_PLAIN;
   constexpr int STAGE_BYTES = SPLIT ? STAGE_SPLIT : STAGE_PLAIN;
@@ -598,7 +630,9 @@ __global__ void __launch_bounds__(THREADS, 1) resident_net_kernel(const __grid_c
     for (int k = 0; k < 2; ++k) {
       mbar_init(&sh.ready[k], 1);
       mbar_init(&sh.acc_full[k], 1);
-      mbar_init(&sh.epi_done[k], EPI_WARPS);
+      mbar_init(&sh.stored[k], EPI_WARPS);
+      mbar_init(&sh.epi_done[k][0], EPI_WARPS);
+      mbar_init(&sh.epi_done[k][1], EPI_WARPS);
     }
     for (int k = 0; k < WQ; ++k) mbar_init(&sh.wq_full[k], 1);
     mbar_init(&sh.drain, 1);
@@ -655,8 +689,9 @@ __global__ void __launch_bounds__(THREADS, 1) resident_net_kernel(const __grid_c
           continue;
         }
         const int b = s.b, I = s.I, J = s.J;
-        const bool adj = s.op.kind != 0;
-        const int by = s.op.y * a.batch + b, bg = s.op.g * a.batch + b;
+        const uint32_t cur = EARLY ? ((rphase >> c) & 1u) ^ 1u : 0u;  // (toggled above)
+        const bool adj = s.op[cur].kind != 0;
+        const int by = s.op[cur].y * a.batch + b, bg = s.op[cur].g * a.batch + b;
         if (a.per > 1) fence_proxy_async();  // the gang's planes, acquired through ready
         sh.wq[seq % WQ] = c;
         mbar_arrive(&sh.wq_full[seq % WQ]);
@@ -705,6 +740,7 @@ __global__ void __launch_bounds__(THREADS, 1) resident_net_kernel(const __grid_c
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
     if (lane == 0) {
+      uint32_t ophase = 0;  // bit c: parity of slot c's operation
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true, issued = false;
@@ -717,7 +753,8 @@ __global__ void __launch_bounds__(THREADS, 1) resident_net_kernel(const __grid_c
         if (c == WQ_END) break;
         const volatile Slot& s = sh.slot[c];
         const int I = s.I, J = s.J;
-        const bool adj = s.op.kind != 0, same = I == J && !adj;
+        const bool adj = s.op[EARLY ? (ophase >> c) & 1u : 0u].kind != 0, same = I == J && !adj;
+        ophase ^= 1u << c;
         const int nkt = adj ? 2 * nk : nk;
         tc_fence_after();
         const uint32_t d = tmem_base + c * SLOT_COLS;
@@ -768,7 +805,7 @@ __global__ void __launch_bounds__(THREADS, 1) resident_net_kernel(const __grid_c
     }
   } else if (warp >= CTL_WARP) {
     const int c = warp - CTL_WARP;
-    if (c == 0 || a.two_slots) control(a, sh, c, lane, idle);
+    if (c == 0 || a.two_slots) control<EARLY>(a, sh, c, lane, idle);
   } else {
     // ------------------------------------------------------------ epilogue
     const int ew = warp - 2, q = warp & 3;
@@ -777,7 +814,7 @@ __global__ void __launch_bounds__(THREADS, 1) resident_net_kernel(const __grid_c
       if (!__all_sync(0xffffffffu, mbar_wait(&sh.wq_full[seq % WQ], (seq / WQ) & 1u, abort_flag, idle))) break;
       const int c = *(volatile int*)&sh.wq[seq % WQ];
       if (c == WQ_END) break;
-      if (!epilogue<SPLIT>(a, sh, c, (aphase >> c) & 1u, tmem_base, ew, q, lane, trbuf + ew * (16 * 32), lim)) {
+      if (!epilogue<SPLIT, EARLY>(a, sh, c, (aphase >> c) & 1u, tmem_base, ew, q, lane, trbuf + ew * (16 * 32), lim)) {
         if (lane == 0) atomicExch(a.err, (int)SP2_ERR_DEVICE_TIMEOUT);
         *abort_flag = 1;
         break;
@@ -968,7 +1005,8 @@ cudaError_t launch_resident_net(const NetArgs& a, const NetMaps& maps, bool spli
     const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     return e == cudaSuccess ? cudaLaunchKernelEx(&cfg, kernel, maps, a) : e;
   };
-  return split ? go(net::resident_net_kernel<true>) : go(net::resident_net_kernel<false>);
+  if (a.two_slots) return split ? go(net::resident_net_kernel<true, false>) : go(net::resident_net_kernel<false, false>);
+  return split ? go(net::resident_net_kernel<true, true>) : go(net::resident_net_kernel<false, true>);
 }
 
 }  // namespace sp2

@@ -136,7 +136,7 @@ def test_input_that_is_not_symmetric_stops_alike(sp2):
 # one matrix a CTA, gangs, more matrices than slots; segments of one layer, of
 # several, longer than the network; sizes off every boundary
 @pytest.mark.parametrize("B,N,L,ce", [(8, 128, 7, 3), (1, 1, 3, 1), (3, 257, 5, 2), (5, 100, 6, 1), (2, 1000, 4, 4),
-                                      (400, 40, 3, 2), (1, 2053, 3, 2), (20, 700, 3, 2)])
+                                      (400, 40, 3, 2), (1, 2053, 3, 2), (20, 700, 3, 2), (100, 40, 3, 2)])
 @pytest.mark.parametrize("precision", ["split", "fp16"])
 def test_network_same_bits(sp2, B, N, L, ce, precision):
     g = torch.Generator(device="cuda").manual_seed(N + B)
