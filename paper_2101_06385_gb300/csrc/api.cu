@@ -63,7 +63,7 @@ enum BufId {
   B_HI0, B_LO0, B_HI1, B_LO1, B_Y0, B_Y1, B_CTL, B_TILES, B_TOFF, B_TCNT, B_TPART, B_IDONE,
   B_PART, B_TICKET, B_ERR, B_DPTR, B_NS, B_HS, B_TRACES, B_PARAMS, B_BOUNDS, B_RN, B_PART2,
   B_G, B_SEG, B_GH0, B_GL0, B_GH1, B_GL1, B_DOTS, B_TDOTS, B_PARAMS2, B_NALPHA, B_HP0, B_HP1, B_RNP0, B_RNP1,
-  B_READOUT, B_RDIAG, B_SEGP, B_WAVE, B_PACK, B_PLANES0, B_PLANES1, B_OPS, B_COUNT
+  B_READOUT, B_RDIAG, B_SEGP, B_WAVE, B_PACK, B_PLANES0, B_PLANES1, B_OPS, B_TSUMS, B_COUNT
 };
 
 struct Buf {
@@ -963,11 +963,12 @@ sp2_status resident_solve(const float* const* H, const int* N, const int* N_occ,
                                                       std::max((Nmax + 63) / 64, 2 * g.num_sms / B + 1));
   const int grid = std::min(nt, g.num_sms);
   const ResPack P(B, nt, grid);
-  void *pack, *part, *sums, *rn, *tdots;
+  void *pack, *part, *sums, *rn, *tdots, *tsums;
   CKS(ws(B_PACK, P.all, &pack));
   CKS(ws(B_PART, (size_t)B * std::max(iblocks, ggrid) * sizeof(double2), &part));
   CKS(ws(B_TPART, (size_t)B * kMeetRows * sizeof(long long), &sums));
   CKS(ws(B_TDOTS, (size_t)nt * sizeof(double), &tdots));
+  CKS(ws(B_TSUMS, (size_t)nt * 8 * sizeof(long long), &tsums));
   const long long ld_h = round_up(Nmax, 64), slot_h = ld_h * Nmax;
   void *hi[2], *lo[2], *hp[2];
   CKS(planes_for(split, 0, (size_t)slot_h * B * 2, &hi[0], &lo[0], &hp[0]));
@@ -1031,6 +1032,7 @@ sp2_status resident_solve(const float* const* H, const int* N, const int* N_occ,
   A.ld_rnp = carry.ld_rnp;
   A.slot_rnp = carry.slot_rnp;
   A.part = (double2*)part;
+  A.tile_sums = (long long*)tsums;
   A.tile_dots = (double*)tdots;
   A.dots_out = (double*)(dp + P.dots);
   A.sums = (long long*)sums;

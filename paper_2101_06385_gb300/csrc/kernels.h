@@ -210,6 +210,7 @@ struct ResArgs {
   long long ld_rnp, slot_rnp;
   double2* part;           // [batch][blocks] block sums of the input layer
   long long* sums;         // [batch][kMeetRows] meeting rows (csrc/resident.cuh), zero
+  long long* tile_sums;    // [2][ntiles][4] a tile's sums by the layer's parity (csrc/resident.cuh)
   double* tile_dots;       // [ntiles] Tr[D H] per tile
   double* dots_out;        // [batch][3], entry 0: Tr[D H]
   unsigned* tickets;       // [batch] zero: finished blocks of the input layer

@@ -69,6 +69,7 @@ struct Shared {
   uint32_t tmem;
   int abort;
   long long red_t[2][EPI_WARPS], red_q[2][EPI_WARPS];  // a layer's sums per warp (fixed point)
+  double2 red_d[2][EPI_WARPS];                         // the same in FP64, where a sum is marked out of range
   double red_e[2][EPI_WARPS];                          // Tr[D H] (last layer)
   Slot slot[2];
 };
@@ -76,12 +77,16 @@ struct Shared {
 // A layer's sums tr Y' and ||Y'||_F^2 in 64-bit fixed point, exact in any
 // order: FP64 adds (64 cycles each, 19 of them a warp on the SM's one pipe)
 // would cost a layer's epilogue a microsecond, integer ones half of one
-// shuffle.  Y' has spectral norm <= 1, so a lane's FP32 sum of 32 squares is
-// at most 4 and a tile's at most 128: units of 2^-53 and 2^-50 (trace) lose
-// less than the FP64 sums did.  Anything outside (an H that is not symmetric)
-// or not a number is marked and becomes infinity or NaN in the control step.
+// shuffle.  With a shift alpha in [0, 1] Y' = S' - alpha I has spectral norm <=
+// 1, so a lane's FP32 sum of 32 squares is at most 4, a tile's at most 128 and a
+// diagonal element at most 1: units of 2^-53 and 2^-50 (trace) lose less than the
+// FP64 sums did.  A spectrum of H that lies on one side of zero starts with alpha
+// outside [0, 1] and squares it until a branch brings it back, so any magnitude
+// can occur: a warp whose sum leaves the range, or is not a number, marks it and
+// hands it over in FP64.
 constexpr long long SQ_LIMIT = (1ll << 58) + (1ll << 50);  // a 32 x 32 block's 32, with rounding
-constexpr long long WARP_NAN = -1, WARP_BIG = -2;          // marks of a warp's sum that is no number, or out of range
+constexpr float T_LIMIT = 2.f;                             // a diagonal element (2^13 in units of 2^-50 fill 63 bits)
+constexpr long long T_OUT = 1ll << 62, SQ_OUT = -1;        // marks of a warp's sum that is in Shared::red_d
 
 __device__ __forceinline__ long long fix_sq(float v) {
   // v = hi 2^-25 + lo 2^-53, both steps exact or rounded once
@@ -91,27 +96,47 @@ __device__ __forceinline__ long long fix_sq(float v) {
 }
 
 // Row norm (Y^2)_rr of the layer's input: FP64 ones of the input layer, or the
-// sum of the previous layer's segment sums (at most 1 together; 2^-53 of fixed
-// point is what an FP64 sum near 1 resolves).  The segments were written by
-// other SMs during this launch: read through L2.
+// sum of the previous layer's segment sums (at most 1 together with a shift in
+// [0, 1]; 2^-53 of fixed point is what an FP64 sum near 1 resolves), in FP64 where
+// one is above 4 or no number.  The segments were written by other SMs during this
+// launch: read through L2.
 __device__ __forceinline__ double row_norm(const ResArgs& a, const Slot& s, int r) {
   if (s.first) return a.rn[(long long)s.b * a.ld_rn + r];
   const float* p = a.rnp[s.par ^ 1] + (long long)s.b * a.slot_rnp + r;
   const int nseg = (s.N + 31) >> 5;
   long long acc = 0;
+  unsigned top = 0;  // the largest as its bits (no sum of squares is negative; NaN is above every number)
   int g = 0;
   for (; g + 16 <= nseg; g += 16) {
     float v[16];
 #pragma unroll
     for (int u = 0; u < 16; ++u) v[u] = __ldcg(p + (long long)(g + u) * a.ld_rnp);
 #pragma unroll
-    for (int u = 0; u < 16; ++u) acc += fix_sq(v[u]);
+    for (int u = 0; u < 16; ++u) {
+      acc += fix_sq(v[u]);
+      top = max(top, __float_as_uint(v[u]));
+    }
   }
   float v[16];
 #pragma unroll
   for (int u = 0; u < 16; ++u) v[u] = g + u < nseg ? __ldcg(p + (long long)(g + u) * a.ld_rnp) : 0.f;
 #pragma unroll
-  for (int u = 0; u < 16; ++u) acc += fix_sq(v[u]);
+  for (int u = 0; u < 16; ++u) {
+    acc += fix_sq(v[u]);
+    top = max(top, __float_as_uint(v[u]));
+  }
+  if (top > 0x40800000u) {
+    auto every8 = [&](int first) {  // epi::row_norm's order
+      double sum = 0.0;
+#pragma unroll 1
+      for (int k = first; k < nseg; k += 8) sum += (double)__ldcg(p + (long long)k * a.ld_rnp);
+      return sum;
+    };
+    double sum = 0.0;
+#pragma unroll 1
+    for (int h = 0; h < 8; h += 4) sum += (every8(h) + every8(h + 1)) + (every8(h + 2) + every8(h + 3));
+    return sum;
+  }
   return (double)acc * Q_LO_UNIT;
 }
 
@@ -226,13 +251,20 @@ __device__ __forceinline__ bool epilogue(const ResArgs& a, Shared& sh, int c, ui
 #pragma unroll
     for (int k = 0; k < 32; ++k)
       if (k == id) yold_d = y[k];
+    double yd = 0.0;
     if (dlane) {
-      const double yd = p.ca_d * (double)yold_d + p.cb_d * rn_l + p.cc_d;
+      yd = p.ca_d * (double)yold_d + p.cb_d * rn_l + p.cc_d;
       tr = __double2ll_rn(yd * 0x1p50);
       ydf = (float)yd;
       ydo = outD ? (float)(yd + p.alpha_out) : ydf;
     }
-    tr = warp_sum_ll(tr);
+    if (__any_sync(0xffffffffu, !(fabsf(ydf) < T_LIMIT))) {
+      const double T = warp_sum_d(yd);
+      if (lane == 0) sh.red_d[c][ew].x = T;
+      tr = T_OUT;
+    } else {
+      tr = warp_sum_ll(tr);
+    }
   }
   if (!__all_sync(0xffffffffu, mbar_wait(&sh.acc_full[c], acc_phase, &sh.abort, lim))) return false;
   tc_fence_after();
@@ -288,10 +320,14 @@ __device__ __forceinline__ bool epilogue(const ResArgs& a, Shared& sh, int c, ui
       }
     }
     const float sql = ((rs[0] + rs[1]) + (rs[2] + rs[3])) + ((rs[4] + rs[5]) + (rs[6] + rs[7]));
-    const bool nan = __any_sync(0xffffffffu, isnan(sql)), big = __any_sync(0xffffffffu, !(sql < 16.f));
+    const bool wild = __any_sync(0xffffffffu, !(sql < 16.f));
     auto sum_squares = [&]() {
       sq = warp_sum_ll(fix_sq(sql));
-      if (nan || big || sq > SQ_LIMIT) sq = nan ? WARP_NAN : WARP_BIG;
+      if (wild || sq > SQ_LIMIT) {
+        const double Q = warp_sum_d((double)sql);
+        if (lane == 0) sh.red_d[c][ew].y = Q;
+        sq = SQ_OUT;
+      }
     };
     if (!outD) {
       if (LOCAL) {
@@ -439,18 +475,26 @@ __device__ __forceinline__ void control(const ResArgs& a, Shared& sh, int c, int
         s.first = 0;
         if (cnt == 1) mbar_arrive(&sh.ready[c]);
       }
-      // the tile's sums: squares that are no number, or out of range, are marked
-      long long rq = lane < EPI_WARPS ? sh.red_q[c][lane] : 0;
-      const long long mark = __any_sync(0xffffffffu, rq == WARP_NAN) ? SQ_NAN
-                             : __any_sync(0xffffffffu, rq == WARP_BIG) ? SQ_BIG : 0;
-      rq = warp_sum_ll(rq) << (twice ? 1 : 0);
-      GangSums G{warp_sum_ll(lane < EPI_WARPS ? sh.red_t[c][lane] : 0), mark ? mark : rq >> 28,
-                 mark ? 0 : rq & ((1ll << 28) - 1)};
+      // the tile's sums; with one out of range all of them in FP64
+      long long rq = lane < EPI_WARPS ? sh.red_q[c][lane] : 0, rt = lane < EPI_WARPS ? sh.red_t[c][lane] : 0;
+      const int mul = twice ? 1 : 0;
+      double trY = 0.0, sqY = 0.0;
+      const bool out = __any_sync(0xffffffffu, rq == SQ_OUT || rt == T_OUT);
+      GangSums G{0, SQ_BIG, 0};
+      if (!out) {
+        rq = warp_sum_ll(rq);  // at most 2^62 + 2^54: the doubling does not fit into the word
+        G = GangSums{warp_sum_ll(rt), rq >> (28 - mul), (rq << mul) & ((1ll << 28) - 1)};
+      } else {
+        const double2 d = lane < EPI_WARPS ? sh.red_d[c][lane] : make_double2(0.0, 0.0);
+        trY = warp_sum_d(rt == T_OUT ? d.x : (double)rt * T_UNIT);
+        sqY = warp_sum_d(rq == SQ_OUT ? d.y : (double)rq * Q_LO_UNIT) * (twice ? 2.0 : 1.0);
+      }
       double E = 0.0;
       if (outD) E = warp_sum_d(lane < EPI_WARPS ? sh.red_e[c][lane] : 0.0);
       if (cnt > 1) {
         if (lane == 0) {
           if (outD) a.tile_dots[t] = E;
+          put_sums(a.tile_sums + 4 * ((long long)(k & 1) * a.ntiles + t), G, out, trY, sqY);
           meet_join(rows, k, t - off, G);
         }
         if (!meet_wait(rows, k, cnt, lane, a.err, &sh.abort, idle)) {
@@ -460,6 +504,7 @@ __device__ __forceinline__ void control(const ResArgs& a, Shared& sh, int c, int
         if (lane == 0 && !outD && !direct) mbar_arrive(&sh.ready[c]);
         G = meet_sums(rows, k, lane);
         if (leader) meet_empty(rows, k, lane);
+        if (out_of_range(G)) sum_slots(a.tile_sums + 4 * ((long long)(k & 1) * a.ntiles + off), cnt, lane, trY, sqY);
         if (outD && leader) {
           E = 0.0;
           for (int i = lane; i < cnt; i += 32) E += __ldcg(&a.tile_dots[off + i]);
@@ -467,8 +512,7 @@ __device__ __forceinline__ void control(const ResArgs& a, Shared& sh, int c, int
         }
       }
       if (lane == 0) {
-        double trY, sqY;
-        to_double(G, trY, sqY);
+        if (!out_of_range(G)) to_double(G, trY, sqY);
         resident_step(s.st, trY, sqY, leader ? a.ctl + b : nullptr);
         if (!outD) mbar_arrive(&sh.coef[c]);
         if (leader) {

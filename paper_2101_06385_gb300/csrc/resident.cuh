@@ -163,8 +163,9 @@ __device__ __forceinline__ long long warp_sum_ll(long long v) {
 
 // A layer's sums over a gang in 64-bit fixed point, exact in any order: tr Y' in
 // units of 2^-50, ||Y'||_F^2 as q_hi 2^-25 + q_lo 2^-53 (q_lo of each member in
-// [0, 2^28)).  A member whose squares are no number, or out of range, adds
-// SQ_NAN or SQ_BIG to q_hi, far above any sum (N 2^25) and each other.
+// [0, 2^28)).  A member with a sum out of range, or no number, adds SQ_BIG to
+// q_hi, far above any sum in range (N 2^25): every member then adds up the
+// members' slots (put_sums) in FP64.
 struct GangSums {
   long long t, q_hi, q_lo;
 };
@@ -176,6 +177,36 @@ __device__ __forceinline__ void to_double(const GangSums& s, double& trY, double
   const double off = __longlong_as_double(nan ? 0x7ff8000000000000ll : 0x7ff0000000000000ll);
   trY = nan ? off : (double)s.t * T_UNIT;
   sqY = big ? off : (double)s.q_hi * Q_HI_UNIT + (double)s.q_lo * Q_LO_UNIT;
+}
+
+__device__ __forceinline__ bool out_of_range(const GangSums& s) { return s.q_hi >= SQ_BIG / 2; }
+
+// A member's sums of one layer in its slot, four words: fixed point, or (out) FP64.
+// Two slots by the layer's parity: before a member writes the one of layer k + 2 the
+// meeting of layer k + 1 is over, which everyone joined after reading layer k's.
+__device__ __forceinline__ void put_sums(long long* slot, const GangSums& s, bool out, double t, double q) {
+  if (out)
+    __stcg(reinterpret_cast<longlong2*>(slot), make_longlong2(__double_as_longlong(t), __double_as_longlong(q)));
+  else
+    __stcg(reinterpret_cast<longlong2*>(slot), make_longlong2(s.t, s.q_hi));
+  __stcg(reinterpret_cast<longlong2*>(slot) + 1, make_longlong2(s.q_lo, out ? 1 : 0));
+}
+// The sums of cnt slots (one warp, in every lane).
+__device__ __forceinline__ void sum_slots(const long long* slots, int cnt, int lane, double& t, double& q) {
+  t = q = 0.0;
+  for (int i = lane; i < cnt; i += 32) {
+    const longlong2 a = __ldcg(reinterpret_cast<const longlong2*>(slots + 4 * i));
+    const longlong2 b = __ldcg(reinterpret_cast<const longlong2*>(slots + 4 * i) + 1);
+    if (b.y) {
+      t += __longlong_as_double(a.x);
+      q += __longlong_as_double(a.y);
+    } else {
+      t += (double)a.x * T_UNIT;
+      q += (double)a.y * Q_HI_UNIT + (double)b.x * Q_LO_UNIT;
+    }
+  }
+  t = warp_sum_d(t);
+  q = warp_sum_d(q);
 }
 
 // The meeting of a gang after a layer.  Members add their sums and then their
