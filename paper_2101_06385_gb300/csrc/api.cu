@@ -1136,8 +1136,9 @@ sp2_status fp32_solve(const float* H, int N, int N_occ, double tol, int max_iter
   const size_t o_st = sizeof(Ctl), o_err = o_st + (kResStamps + 2) / 2 * 8, o_ptr = o_err + 16,
                o_sums = o_ptr + 64, o_tiles = o_sums + 2 * kMeetRows * sizeof(long long), bytes = o_tiles + (size_t)nt * sizeof(uint32_t);
   static_assert(sizeof(Ctl) % 8 == 0, "the offsets after it keep 8-byte alignment");
-  void *pack, *part, *rn, *Y[2];
+  void *pack, *part, *rn, *slots, *Y[2];
   CKS(ws(B_PACK, bytes, &pack));
+  CKS(ws(B_TSUMS, (size_t)grid * 16 * sizeof(long long), &slots));
   CKS(ws(B_PART, std::max(std::max(ggrid, igrid), rgrid) * sizeof(double2), &part));
   CKS(ws(B_RN, (size_t)N * sizeof(double), &rn));
   const long long ld_y = round_up(N, 4), slot_y = ld_y * N;
@@ -1175,6 +1176,7 @@ sp2_status fp32_solve(const float* H, int N, int N_occ, double tol, int max_iter
   A.ctl = (Ctl*)dp;
   A.rn = (double*)rn;
   A.sums = (long long*)(dp + o_sums);
+  A.slots = (long long*)slots;
   A.stamps = (unsigned*)(dp + o_st);
   A.err = (int*)(dp + o_err);
   A.wait_ns = g.wait_ns;

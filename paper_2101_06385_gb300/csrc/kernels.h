@@ -327,6 +327,7 @@ struct Res32Args {
   Ctl* ctl;
   double* rn;              // [N] row norms of the layer's input
   long long* sums;         // [2][kMeetRows] meeting rows of the traces and of the square norms, zero
+  long long* slots;        // [2][2][grid][4] by the layer's parity: each CTA's trace, then its square norm
   unsigned* stamps;        // as ResArgs
   int* err;
   unsigned long long wait_ns;

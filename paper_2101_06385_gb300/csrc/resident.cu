@@ -85,8 +85,7 @@ struct Shared {
 // can occur: a warp whose sum leaves the range, or is not a number, marks it and
 // hands it over in FP64.
 constexpr long long SQ_LIMIT = (1ll << 58) + (1ll << 50);  // a 32 x 32 block's 32, with rounding
-constexpr float T_LIMIT = 2.f;                             // a diagonal element (2^13 in units of 2^-50 fill 63 bits)
-constexpr long long T_OUT = 1ll << 62, SQ_OUT = -1;        // marks of a warp's sum that is in Shared::red_d
+constexpr long long SQ_OUT = -1;                           // marks a warp's sum that is in Shared::red_d (as T_OUT)
 
 __device__ __forceinline__ long long fix_sq(float v) {
   // v = hi 2^-25 + lo 2^-53, both steps exact or rounded once

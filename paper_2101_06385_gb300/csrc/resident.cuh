@@ -169,14 +169,14 @@ __device__ __forceinline__ long long warp_sum_ll(long long v) {
 struct GangSums {
   long long t, q_hi, q_lo;
 };
-constexpr long long SQ_NAN = 1ll << 52, SQ_BIG = 1ll << 42;
+constexpr long long SQ_BIG = 1ll << 42;
+constexpr float T_LIMIT = 2.f;            // range of a diagonal element (N of them fill 2^13 / 2^-50 = 63 bits)
+constexpr long long T_OUT = 1ll << 62;    // marks a warp's trace that left it
 constexpr double T_UNIT = 0x1p-50, Q_HI_UNIT = 0x1p-25, Q_LO_UNIT = 0x1p-53;
 
 __device__ __forceinline__ void to_double(const GangSums& s, double& trY, double& sqY) {
-  const bool nan = s.q_hi >= SQ_NAN / 2, big = s.q_hi >= SQ_BIG / 2;
-  const double off = __longlong_as_double(nan ? 0x7ff8000000000000ll : 0x7ff0000000000000ll);
-  trY = nan ? off : (double)s.t * T_UNIT;
-  sqY = big ? off : (double)s.q_hi * Q_HI_UNIT + (double)s.q_lo * Q_LO_UNIT;
+  trY = (double)s.t * T_UNIT;
+  sqY = (double)s.q_hi * Q_HI_UNIT + (double)s.q_lo * Q_LO_UNIT;
 }
 
 __device__ __forceinline__ bool out_of_range(const GangSums& s) { return s.q_hi >= SQ_BIG / 2; }

@@ -58,6 +58,7 @@ struct Shared {
   uint64_t gate, coef, tiles_done, rn_done;
   int abort;
   long long red_t[4];
+  double red_d[4];  // the same in FP64, where red_t is marked out of range
   double red_q[RN_WARPS];
   SolveState st;
 };
@@ -102,10 +103,9 @@ __device__ __forceinline__ double row_norms(const float* Y, long long ld, int N,
   return blk;
 }
 
-// A CTA's sum of row norms for the meeting (they are at most 1 each).
+// A CTA's sum of row norms for the meeting (with a shift in [0, 1] they are at most
+// 1 each; q < 2^15).
 __device__ __forceinline__ GangSums to_fixed(double q) {
-  if (isnan(q)) return GangSums{0, SQ_NAN, 0};
-  if (!(q < 0x1p15)) return GangSums{0, SQ_BIG, 0};
   const long long hi = __double2ll_rd(q * 0x1p25);
   return GangSums{0, hi, min((1ll << 28) - 1, __double2ll_rn((q * 0x1p25 - (double)hi) * 0x1p28))};
 }
@@ -129,26 +129,47 @@ __device__ __forceinline__ bool control(const Res32Args& a, Shared<TS>& sh, int 
     const uint32_t ph = k & 1;
     if (!__all_sync(0xffffffffu, mbar_wait(&sh.tiles_done, ph, &sh.abort, lim))) return false;
     const bool outD = hot->next.out_mode == OUT_D;
-    const long long T = warp_sum_ll(lane < FW ? sh.red_t[lane] : 0);
-    if (lane == 0) meet_join(a.sums, k, me, GangSums{T, 0, 0});
+    // traces and square norms out of the fixed-point range, or no number, go through
+    // the members' slots in FP64, as in csrc/resident.cu
+    double trY = 0.0, sqY = 0.0;
+    const long long rt = lane < FW ? sh.red_t[lane] : 0;
+    const bool out_t = __any_sync(0xffffffffu, rt == T_OUT);
+    GangSums S{0, SQ_BIG, 0};
+    if (!out_t)
+      S = GangSums{warp_sum_ll(rt), 0, 0};
+    else
+      trY = warp_sum_d(rt == T_OUT ? sh.red_d[lane] : (double)rt * T_UNIT);
+    long long* slots = a.slots + (long long)(k & 1) * 8 * G;  // of the traces, then of the norms
+    if (lane == 0) {
+      put_sums(slots + 4 * me, S, out_t, trY, 0.0);
+      meet_join(a.sums, k, me, S);
+    }
     if (!meet_wait(a.sums, k, G, lane, a.err, ab, lim)) return false;
     if (lane == 0 && !outD) mbar_arrive(&sh.gate);
-    GangSums S = meet_sums(a.sums, k, lane);
+    S = meet_sums(a.sums, k, lane);
     if (me == 0) meet_empty(a.sums, k, lane);
+    const bool wide = out_of_range(S);
+    if (wide) sum_slots(slots, G, lane, trY, sqY);
     if (!outD) {
       if (!__all_sync(0xffffffffu, mbar_wait(&sh.rn_done, ph, &sh.abort, lim))) return false;
       const double Q = warp_sum_d(lane < RN_WARPS ? sh.red_q[lane] : 0.0);
       long long* norms = a.sums + kMeetRows;
-      if (lane == 0) meet_join(norms, k, me, to_fixed(Q));
+      slots += 4 * G;
+      if (lane == 0) {
+        const bool out_q = !(Q < 0x1p15);
+        const GangSums q = out_q ? GangSums{0, SQ_BIG, 0} : to_fixed(Q);
+        put_sums(slots + 4 * me, q, out_q, 0.0, Q);
+        meet_join(norms, k, me, q);
+      }
       if (!meet_wait(norms, k, G, lane, a.err, ab, lim)) return false;
       const GangSums q = meet_sums(norms, k, lane);
       if (me == 0) meet_empty(norms, k, lane);
-      S.q_hi = q.q_hi;
-      S.q_lo = q.q_lo;
+      double t;
+      if (out_of_range(q)) sum_slots(slots, G, lane, t, sqY);
+      else to_double(q, t, sqY);
     }
     if (lane == 0) {
-      double trY, sqY;
-      to_double(S, trY, sqY);
+      if (!wide) trY = (double)S.t * T_UNIT;
       resident_step(sh.st, trY, sqY, me == 0 ? a.ctl : nullptr);
       if (!outD) mbar_arrive(&sh.coef);
       if (me == 0 && k + 1 < kResStamps) a.stamps[k + 1] = (unsigned)(globaltimer() - t0);
@@ -230,7 +251,8 @@ __global__ void __launch_bounds__(Cfg<TS>::THREADS, 1) resident_fp32_kernel(cons
       const float* Y = a.Y[k & 1];
       float* Yn = a.Y[(k + 1) & 1];
       long long tr = 0;
-      bool outD = false;
+      double trd = 0.0;
+      bool outD = false, out_t = false;
       for (int t = blockIdx.x; t < a.ntiles && ok; t += G) {
         int b, I, J, h;
         unpack_tile(a.tiles[t], b, I, J, h);
@@ -322,12 +344,20 @@ __global__ void __launch_bounds__(Cfg<TS>::THREADS, 1) resident_fp32_kernel(cons
             const int r = r0 + e;
             const double yd = p.ca_d * (double)__ldcg(Y + (long long)r * ld + r) + p.cb_d * __ldcg(a.rn + r) + p.cc_d;
             tr += __double2ll_rn(yd * 0x1p50);
+            trd += yd;
+            out_t = out_t || !(fabsf((float)yd) < T_LIMIT);
             out[(long long)r * lo + r] = outD ? (float)(yd + p.alpha_out) : (float)yd;
           }
         }
       }
       if (!ok) break;
-      tr = warp_sum_ll(tr);
+      if (__any_sync(0xffffffffu, out_t)) {
+        trd = warp_sum_d(trd);
+        if (lane == 0) sh.red_d[warp] = trd;
+        tr = T_OUT;
+      } else {
+        tr = warp_sum_ll(tr);
+      }
       __syncwarp();
       if (lane == 0) {
         sh.red_t[warp] = tr;

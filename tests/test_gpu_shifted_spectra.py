@@ -68,6 +68,7 @@ def _same(got, want, exact, tol):
     assert not isinstance(got, int), got
     (D, st), (D1, s1) = got, want
     assert st.status == s1.status and st.converged_by == s1.converged_by and st.sigmas == s1.sigmas
+    assert np.isfinite(st.trace) == np.isfinite(s1.trace)
     err = float(np.abs(D1.cpu().numpy() - exact).max())
     if err <= tol:
         assert float(np.abs(D.cpu().numpy() - exact).max()) <= tol
@@ -120,3 +121,24 @@ def test_wild_input_stops_alike(sp2):
             assert np.isnan(st.trace) == np.isnan(s1.trace)
             acc = lambda m: m.density_matrix_accelerated(H, N // 2, -0.1, 0.1, precision=prec)
             assert _outcome(lambda: acc(sp2)) == _outcome(lambda: _launch_per_layer(acc))
+
+
+# FP32: tiles of 32, one a CTA and several, and of 64
+@pytest.mark.parametrize("N", [64, 200, 700, 1100])
+@pytest.mark.parametrize("accelerated", [False, True])
+def test_fp32_solve(sp2, N, accelerated):
+    right = 0
+    for lo in (0.2, 1.0, -3.0, 4.0):
+        for frac in (0.2, 0.5, 0.8) if N < 1000 else (0.5,):
+            n_occ = int(N * frac)
+            h, exact, mid = _tridiagonal(N, n_occ, lo, N + n_occ)
+            H = torch.from_numpy(h).cuda()
+
+            def solve(m):
+                if accelerated:
+                    return m.density_matrix_accelerated(H, n_occ, mid - 0.15, mid + 0.15, precision="fp32")
+                return m.density_matrix(H, n_occ, precision="fp32")
+
+            got, want = _outcome(lambda: solve(sp2)), _outcome(lambda: _launch_per_layer(solve))
+            right += bool(_same(got, want, exact, 5e-5))
+    assert right >= 1
