@@ -156,6 +156,8 @@ const char* sp2_last_error(void);
  *   alloc_fail  the library's next workspace request fails as if cudaMalloc
  *               had run out of memory: the call returns SP2_ERR_OOM before it
  *               enqueues any work (D_out untouched)
+ *   alloc_limit=<n>  workspace requests above n MiB, 1..1000000, fail that way
+ *               while in force (buffers that are large enough already are used)
  *   nan_input   the next sp2_density_matrix / _accelerated reads row 0 of H
  *               as holding a NaN: SP2_ERR_NONFINITE, no layer runs
  *   timeout     in the next single-matrix solve's first squaring launch the
@@ -267,7 +269,11 @@ sp2_status sp2_network_forward(const float* H, int B, int N, int L, const float*
  * Workspace: the ckpt_every iterates of one checkpoint segment are
  * recomputed and kept in FP32 together with their FP16 operand planes
  * (about ckpt_every * B * N^2 * 8 bytes on the split path, * 6 on plain FP16),
- * plus the FP32 adjoint and its planes.  Errors: INVALID_ARG, UNSUPPORTED
+ * plus the FP32 adjoint and its planes.  The resident kernel (N <= 896, larger
+ * ones in small batches) also keeps the planes of every segment's first iterate,
+ * (L / ckpt_every) * B * N^2 * 4 bytes, and iterates in whole 128 x 128 tiles; it
+ * is used while that takes no more than 6 GiB, or twice the above, and its
+ * allocations succeed.  Errors: INVALID_ARG, UNSUPPORTED
  * (FP32 precision), CUDA / OOM, DEVICE_TIMEOUT.
  */
 sp2_status sp2_network_backward(const float* H, int B, int N, int L, const float* coef, int ckpt_every,

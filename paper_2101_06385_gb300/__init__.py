@@ -190,7 +190,7 @@ def init(device: int = 0, precision: str = "split", lo_scale_exp: int = 11, shif
 
 
 def set_fault(spec: Optional[str]) -> None:
-    """Arms injected faults for tests of the error paths: "alloc_fail",
+    """Arms injected faults for tests of the error paths: "alloc_fail", "alloc_limit=<n>",
     "nan_input", "timeout", "wait_ms=<n>" (comma-separated; None or "none"
     clears).  See sp2_set_fault in include/sp2.h."""
     _check(_load().sp2_set_fault(None if spec is None else spec.encode()))

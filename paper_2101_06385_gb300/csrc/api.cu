@@ -105,6 +105,7 @@ struct State {
   std::vector<uint64_t> bgraph_key;
   // injected faults (sp2_set_fault / SP2_FAULT): each fires once
   bool fault_alloc = false, fault_nan = false, fault_stall = false;
+  size_t alloc_limit = 0;  // injected: larger workspace requests fail (0: none)
   // side of the square groups of the tile order (SP2_TILE_GROUP, default 8)
   int tile_group = 8;
   // K stages per epoch of the soft pair synchronisation (SP2_WAVE_SYNC, default
@@ -136,13 +137,28 @@ sp2_status ws(BufId id, size_t bytes, void** out, bool zero = false) {
       b.p = nullptr;
       b.bytes = 0;
     }
-    CK(cudaMalloc(&b.p, bytes));
+    const cudaError_t e = g.alloc_limit && bytes > g.alloc_limit ? cudaErrorMemoryAllocation : cudaMalloc(&b.p, bytes);
+    if (e != cudaSuccess) {
+      cudaGetLastError();  // the next launch's check must not find it
+      b.p = nullptr;
+      set_err("workspace request of %zu bytes failed: %s", bytes, cudaGetErrorString(e));
+      return e == cudaErrorMemoryAllocation ? SP2_ERR_OOM : SP2_ERR_CUDA;
+    }
     b.bytes = bytes;
     if (id == B_TILES || id == B_TOFF || id == B_TCNT) g.tiles_key_N = -1;
     zero = true;
   }
   if (zero) CK(cudaMemsetAsync(b.p, 0, b.bytes, g.stream));
   *out = b.p;
+  return SP2_OK;
+}
+
+sp2_status ws_free(BufId id) {
+  Buf& b = g.buf[id];
+  if (!b.p) return SP2_OK;
+  CK(cudaStreamSynchronize(g.stream));
+  CK(cudaFree(b.p));
+  b = Buf();
   return SP2_OK;
 }
 
@@ -504,6 +520,7 @@ sp2_status sp2_set_fault(const char* spec) {
   t_err.clear();
   bool alloc = false, nan = false, stall = false;
   unsigned long long wait_ns = 0;
+  size_t alloc_limit = 0;
   const std::string sp = spec ? spec : "";
   size_t pos = 0;
   while (pos <= sp.size()) {
@@ -517,6 +534,14 @@ sp2_status sp2_set_fault(const char* spec) {
       nan = true;
     } else if (item == "timeout") {
       stall = true;
+    } else if (item.compare(0, 12, "alloc_limit=") == 0) {
+      char* e = nullptr;
+      const long v = std::strtol(item.c_str() + 12, &e, 10);
+      if (!e || *e != '\0' || e == item.c_str() + 12 || v < 1 || v > 1000000) {
+        set_err("sp2_set_fault: alloc_limit must be an integer in [1, 1000000] MiB, got '%s'", item.c_str() + 12);
+        return SP2_ERR_INVALID_ARG;
+      }
+      alloc_limit = (size_t)v << 20;
     } else if (item.compare(0, 8, "wait_ms=") == 0) {
       char* e = nullptr;
       const long v = std::strtol(item.c_str() + 8, &e, 10);
@@ -526,12 +551,13 @@ sp2_status sp2_set_fault(const char* spec) {
       }
       wait_ns = (unsigned long long)v * 1000000ull;
     } else {
-      set_err("sp2_set_fault: unknown item '%s' (alloc_fail, nan_input, timeout, wait_ms=<n>, none)", item.c_str());
+      set_err("sp2_set_fault: unknown item '%s' (alloc_fail, alloc_limit=<n>, nan_input, timeout, wait_ms=<n>, none)", item.c_str());
       return SP2_ERR_INVALID_ARG;
     }
     pos = end + 1;
   }
   g.fault_alloc = alloc;
+  g.alloc_limit = alloc_limit;
   g.fault_nan = nan;
   g.fault_stall = stall;
   g.wait_ns = wait_ns;
@@ -2238,6 +2264,23 @@ sp2_status net_forward_resident(const float* H, int B, int N, int L, const float
 
 void coef_gradient(const double* dd, const double* alpha, int L, int B, double* dcoef);
 
+// Whether the adjoint's workspace on the resident kernel is in proportion.  It
+// keeps the planes of every segment's first iterate (one input pass makes them
+// all) and iterates in whole 128 x 128 tiles: up to 6 GiB, or twice what the CTA
+// pairs take, which keep one segment's planes and iterates.  More of it (64 of 896
+// take 4.6 GB with a segment a layer, 20 of them; 4096 of N = 1 with 256 layers in
+// one segment would take 69 GB, on the pairs 0.3) goes to the pairs.
+bool backward_fits(int B, int N, int L, int ce) {
+  const bool split = g.precision == SP2_PREC_SPLIT_FP16;
+  const double plane = (double)B * N * round_up(N, 64) * (split ? 4.0 : 2.0), mat = 4.0 * B * N * N;
+  const int nseg = (L + ce - 1) / ce, kept = std::min(ce, L);
+  int per = 0;
+  resident_tiles(N, 0, nullptr, &per);
+  const double resident = plane * (nseg + kept + 1) + 4.0 * B * per * kResTile * kResTile * std::max(1, kept - 1);
+  const double pairs = plane * (ce + 2) + mat * (ce + 1);
+  return resident <= std::max(6.0 * 0x1p30, 2.0 * pairs);
+}
+
 // The network's adjoint on the resident kernel: per checkpoint segment, from
 // the last one, the recomputation of its iterates and the adjoint layers.
 sp2_status net_backward_resident(const float* H, int B, int N, int L, const float* coef, int ce, const float* ckpt,
@@ -2561,9 +2604,14 @@ sp2_status sp2_network_backward(const float* H, int B, int N, int L, const float
   cudaStream_t st = g.stream;
   const long long slot = (long long)N * N;
   const int ce = ckpt_every;
-  // (the planes of all segments' first iterates, as large as the checkpoints, within 32 GiB)
-  if (net_fits(B, N, 896) && (double)((L + ce - 1) / ce + ce + 1) * B * round_up(N, 64) * N * 4.0 < 0x1p35)
-    return net_backward_resident(H, B, N, L, coef, ce, ckpt, G_out, dcoef, G_in);
+  if (net_fits(B, N, 896) && backward_fits(B, N, L, ce)) {
+    const bool injected = g.fault_alloc;
+    const sp2_status s = net_backward_resident(H, B, N, L, coef, ce, ckpt, G_out, dcoef, G_in);
+    if (s != SP2_ERR_OOM || injected) return s;
+    // the pairs need less; what the attempt holds goes back first
+    t_err.clear();
+    for (BufId id : {B_PLANES0, B_PLANES1, B_SEG}) CKS(ws_free(id));
+  }
   void* G;
   CKS(ws(B_G, (size_t)B * slot * 4, &G));
   bool ok = false;
