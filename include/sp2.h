@@ -28,7 +28,11 @@
  *   or a negative error.  On SP2_ERR_INVALID_ARG nothing is enqueued and the
  *   outputs are untouched.  Errors found on the device (non-finite or
  *   degenerate spectral bounds, device wait time-outs) are reported through
- *   the status of a synchronising call; outputs are then unspecified.
+ *   the status of a synchronising call; outputs are then unspecified.  A call
+ *   that returns before the end of its work (stats == NULL, the network's
+ *   forward pass, the expansion) cannot report a device wait that runs out: the
+ *   first later call that finds it returns SP2_ERR_DEVICE_TIMEOUT instead of
+ *   doing its work, sp2_network_backward also at its end.
  * - No C++ exception crosses this interface.  sp2_last_error() returns a
  *   thread-local description of the last failure.
  * - Not re-entrant: one thread at a time per process (the workspace is
@@ -160,11 +164,13 @@ const char* sp2_last_error(void);
  *               while in force (buffers that are large enough already are used)
  *   nan_input   the next sp2_density_matrix / _accelerated reads row 0 of H
  *               as holding a NaN: SP2_ERR_NONFINITE, no layer runs
- *   timeout     in the next single-matrix solve's first squaring launch the
- *               MMA issuer waits on a barrier that nothing arrives on; the
- *               wait runs out, every CTA stops issuing, drains its copies and
- *               MMAs, frees its tensor memory and returns; the call returns
- *               SP2_ERR_DEVICE_TIMEOUT (D_out holds no meaningful values)
+ *   timeout     in the first squaring launch of the next single-matrix solve,
+ *               forward pass or expansion the MMA issuer waits on a barrier
+ *               that nothing arrives on; the wait runs out, every CTA stops
+ *               issuing, drains its copies and MMAs, frees its tensor memory and
+ *               returns; the call (the next one, where it does not wait for its
+ *               end) returns SP2_ERR_DEVICE_TIMEOUT (the outputs hold no
+ *               meaningful values)
  *   wait_ms=<n> bound of every device wait of the tensor-core squaring
  *               kernels, 1..60000 ms (default 4000); stays in force
  * alloc_fail, nan_input and timeout each fire once.  The environment variable

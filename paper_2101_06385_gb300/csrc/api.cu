@@ -82,6 +82,9 @@ struct State {
   int num_sms = 148;
   PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
   Buf buf[B_COUNT];
+  // word in mapped host memory that a kernel sets when a wait of it ran out, for
+  // calls that return before their end (its device address too)
+  int *late = nullptr, *late_dev = nullptr;
   // pinned staging for small host<->device transfers
   void* stage = nullptr;
   size_t stage_bytes = 0;
@@ -221,6 +224,13 @@ void build_tiles(int N, int B, int tile, int halves, std::vector<uint32_t>& out,
   out.reserve((size_t)per_instance * B);
   for (int b = 0; b < B; ++b)
     for (uint32_t t : one) out.push_back(t | ((uint32_t)b << 20));
+}
+
+// The injected stall, once.
+int take_stall() {
+  const int s = g.fault_stall ? 1 : 0;
+  g.fault_stall = false;
+  return s;
 }
 
 bool tc_precision(int p) { return p == SP2_PREC_SPLIT_FP16 || p == SP2_PREC_FP16; }
@@ -484,11 +494,23 @@ void fill_stats(const Ctl& c, sp2_stats* s, double ms, int precision) {
   }
 }
 
+// A time-out found in the call's own error word.
+sp2_status timed_out() {
+  if (g.late) *(volatile int*)g.late = 0;
+  set_err("a bounded device wait timed out");
+  return SP2_ERR_DEVICE_TIMEOUT;
+}
+
+// One left behind by an earlier call that did not wait for its end: reported once.
+sp2_status late_error() {
+  if (!g.late || *(volatile int*)g.late == 0) return SP2_OK;
+  *(volatile int*)g.late = 0;
+  set_err("a bounded device wait timed out in an earlier call, whose outputs are not valid");
+  return SP2_ERR_DEVICE_TIMEOUT;
+}
+
 sp2_status status_of(const Ctl& c, int dev_err) {
-  if (dev_err != 0) {
-    set_err("a bounded device wait timed out");
-    return SP2_ERR_DEVICE_TIMEOUT;
-  }
+  if (dev_err != 0) return timed_out();
   if (c.status < 0) {
     set_err(c.status == SP2_ERR_NONFINITE      ? "non-finite spectral bounds (NaN or Inf in H)"
             : c.status == SP2_ERR_INVALID_ARG  ? "HOMO/LUMO estimates leave no gap inside the spectral bounds"
@@ -606,6 +628,11 @@ sp2_status sp2_init(const sp2_config* cfg) {
     }
     g.encode = (PFN_cuTensorMapEncodeTiled_v12000)fn;
   }
+  if (!g.late) {
+    CK(cudaHostAlloc(&g.late, sizeof(int), cudaHostAllocMapped));
+    *(volatile int*)g.late = 0;
+    CK(cudaHostGetDevicePointer(&g.late_dev, g.late, 0));
+  }
   if (!g.stage_done) {
     CK(cudaEventCreateWithFlags(&g.stage_done, cudaEventDisableTiming));
     CK(cudaEventCreate(&g.ev0));
@@ -649,6 +676,8 @@ sp2_status sp2_finalize(void) {
     if (g.buf[i].p) cudaFree(g.buf[i].p);
     g.buf[i] = Buf();
   }
+  if (g.late) cudaFreeHost(g.late);
+  g.late = g.late_dev = nullptr;
   if (g.stage) cudaFreeHost(g.stage);
   g.stage = nullptr;
   g.stage_bytes = 0;
@@ -752,6 +781,7 @@ sp2_status sp2_layer(const float* X, int B, int N, float a, float b, float c, fl
     set_err("sp2_layer: invalid argument");
     return SP2_ERR_INVALID_ARG;
   }
+  CKS(late_error());
   const bool tc = tc_precision(g.precision);
   const bool split = g.precision == SP2_PREC_SPLIT_FP16;
   int ntiles = 0;
@@ -802,6 +832,7 @@ sp2_status sp2_layer(const float* X, int B, int N, float a, float b, float c, fl
   A.lo_scale = std::ldexp(1.0f, g.lo_scale_exp);
   A.lo_unscale = std::ldexp(1.0f, -g.lo_scale_exp);
   A.err = (int*)err;
+  A.late = g.late_dev;
   void* rn;
   CKS(ws(B_RN, (size_t)B * N * sizeof(double), &rn));
   const int rgrid = (int)std::min<long long>((N + 7) / 8, std::max(1, 2 * g.num_sms / B));
@@ -834,11 +865,7 @@ sp2_status sp2_layer(const float* X, int B, int N, float a, float b, float c, fl
     CK(cudaMemcpyAsync((char*)hb + 2 * B * sizeof(double), err, sizeof(int), cudaMemcpyDeviceToHost, g.stream));
     CK(cudaStreamSynchronize(g.stream));
     memcpy(traces_out, hb, 2 * B * sizeof(double));
-    int e = *(int*)((char*)hb + 2 * B * sizeof(double));
-    if (e) {
-      set_err("a bounded device wait timed out");
-      return SP2_ERR_DEVICE_TIMEOUT;
-    }
+    if (*(int*)((char*)hb + 2 * B * sizeof(double))) return timed_out();
   }
   return SP2_OK;
 }
@@ -1071,11 +1098,11 @@ sp2_status resident_solve(const float* const* H, const int* N, const int* N_occ,
   A.lo_unscale = std::ldexp(1.0f, -g.lo_scale_exp);
   A.shift = g.shift;
   A.err = (int*)(dp + P.err);
+  A.late = g.late_dev;
   A.wait_ns = g.wait_ns;
   A.two_slots = nt > grid ? 1 : 0;
   A.local = Nmax <= kResTile ? 1 : 0;
-  A.stall = (single && g.fault_stall) ? 1 : 0;
-  if (single) g.fault_stall = false;
+  A.stall = single ? take_stall() : 0;
   ResMaps maps;
   for (int k = 0; k < 2; ++k) {
     CKS(tmaps4_for(A.p0[k], A.p1[k], Nmax, B, ld_h, slot_h, maps.m[k], kTransBox));
@@ -1205,6 +1232,7 @@ sp2_status fp32_solve(const float* H, int N, int N_occ, double tol, int max_iter
   A.slots = (long long*)slots;
   A.stamps = (unsigned*)(dp + o_st);
   A.err = (int*)(dp + o_err);
+  A.late = g.late_dev;
   A.wait_ns = g.wait_ns;
   const float* const* hp = (const float* const*)(dp + o_ptr);
   const int* np = (const int*)(dp + o_ptr + 8);
@@ -1364,6 +1392,7 @@ sp2_status density_matrix_impl(const float* H, int N, int N_occ, double tol, int
   A.lo_scale = std::ldexp(1.0f, g.lo_scale_exp);
   A.lo_unscale = std::ldexp(1.0f, -g.lo_scale_exp);
   A.err = (int*)err;
+  A.late = g.late_dev;
   A.rn = (const double*)rn;
   A.ld_rn = N;
   if (tc) {
@@ -1417,8 +1446,7 @@ sp2_status density_matrix_impl(const float* H, int N, int N_occ, double tol, int
       PairList l = lists.list(0, true, false, 0);
       A.tri_planes = 1;
       A.wide = wide ? 1 : 0;
-      A.stall = g.fault_stall ? 1 : 0;
-      g.fault_stall = false;
+      A.stall = take_stall();
       const int grid = std::min(wide ? ntiles / 2 : ntiles, g.num_sms) & ~1;  // every pair has a unit
       // epoch counters of the soft pair synchronisation, one zeroed slice per
       // layer (per pair: super tiles, or wide units of two)
@@ -1441,8 +1469,7 @@ sp2_status density_matrix_impl(const float* H, int N, int N_occ, double tol, int
         A.lo_out = (__half*)lo[cur ^ 1];
         A.hp_out = (__half*)hp[cur ^ 1];
         rnp_step(A, rnp, k);
-        A.stall = (k == 0 && g.fault_stall) ? 1 : 0;
-        g.fault_stall = false;
+        A.stall = take_stall();
         CK(launch_syrk_tc1(A, m[cur], split, grid, st));
         CK(cudaEventRecord(g.lsq[k], st));
         CK(cudaEventRecord(g.lev[k + 1], st));
@@ -1521,6 +1548,7 @@ sp2_status sp2_density_matrix(const float* H, int N, int N_occ, double tol, int 
     set_err("sp2_density_matrix: invalid argument");
     return SP2_ERR_INVALID_ARG;
   }
+  CKS(late_error());
   return density_matrix_impl(H, N, N_occ, tol, max_iter, D_out, stats, false, 0.0, 0.0);
 }
 
@@ -1534,6 +1562,7 @@ sp2_status sp2_density_matrix_accelerated(const float* H, int N, int N_occ, doub
     set_err("sp2_density_matrix_accelerated: invalid argument");
     return SP2_ERR_INVALID_ARG;
   }
+  CKS(late_error());
   return density_matrix_impl(H, N, N_occ, tol, max_iter, D_out, stats, true, homo, lumo);
 }
 
@@ -1652,6 +1681,7 @@ sp2_status batched_once(const float* const* H, const int* N, const int* N_occ, i
   A.lo_scale = std::ldexp(1.0f, g.lo_scale_exp);
   A.lo_unscale = std::ldexp(1.0f, -g.lo_scale_exp);
   A.err = (int*)err;
+  A.late = g.late_dev;
   if (tc) {
     // Tr[D H] per instance from the launch that writes D
     A.Hobs = (const float* const*)hs;
@@ -1821,6 +1851,7 @@ sp2_status batched_impl(const float* const* H, const int* N, const int* N_occ, i
     }
     Nmax = std::max(Nmax, N[i]);
   }
+  CKS(late_error());
   const int prec = g.precision;
   const bool tc = tc_precision(prec);
   cudaStream_t st = g.stream;
@@ -2118,6 +2149,7 @@ struct NetRun {
     A.shift = g.shift;
     A.two_slots = nt > grid ? 1 : 0;
     A.err = (int*)(pack + o_err);
+    A.late = g.late_dev;
     A.wait_ns = g.wait_ns;
     plan.batch = B;
     plan.L = L;
@@ -2258,6 +2290,7 @@ sp2_status net_forward_resident(const float* H, int B, int N, int L, const float
   x.x0 = ckpt;
   x.alpha0 = R.dev(0);
   CK(launch_net_input(x, B, g.stream));
+  R.A.stall = take_stall();
   CK(launch_resident_net(R.A, R.maps, split, R.grid, g.stream));
   return R.wait_and_check(back);
 }
@@ -2367,10 +2400,8 @@ sp2_status net_backward_resident(const float* H, int B, int N, int L, const floa
   CK(cudaMemcpyAsync(hp + db + ab + sb, R.A.err, sizeof(int), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
   CKS(R.check((const int*)(hp + db + ab)));
-  if (*(const int*)(hp + db + ab + sb)) {
-    set_err("a bounded device wait timed out");
-    return SP2_ERR_DEVICE_TIMEOUT;
-  }
+  if (*(const int*)(hp + db + ab + sb)) return timed_out();
+  CKS(late_error());  // of the forward pass whose checkpoints were read
   coef_gradient((const double*)hp, (const double*)(hp + db), L, B, dcoef);
   return SP2_OK;
 }
@@ -2410,6 +2441,7 @@ sp2_status sp2_network_forward(const float* H, int B, int N, int L, const float*
       set_err("sp2_network_forward: non-finite coefficient");
       return SP2_ERR_INVALID_ARG;
     }
+  CKS(late_error());
   if (net_fits(B, N, 896)) return net_forward_resident(H, B, N, L, coef, ckpt_every, X_out, ckpt, bounds);
   const bool tc = tc_precision(g.precision);
   const bool split = g.precision == SP2_PREC_SPLIT_FP16;
@@ -2499,6 +2531,7 @@ sp2_status sp2_network_forward(const float* H, int B, int N, int L, const float*
   A.lo_scale = std::ldexp(1.0f, g.lo_scale_exp);
   A.lo_unscale = std::ldexp(1.0f, -g.lo_scale_exp);
   A.err = (int*)err;
+  A.late = g.late_dev;
   A.ld_y = N;
   A.slot_y = slot;
   const int mgrid = (int)std::min<long long>(N, std::max(1, 4 * g.num_sms / B + 1));
@@ -2536,6 +2569,7 @@ sp2_status sp2_network_forward(const float* H, int B, int N, int L, const float*
     x.alpha0 = (const double*)alpha;
     CK(launch_net_input(x, B, st));
     A.tri_planes = 1;
+    A.stall = take_stall();
     CK(launch_syrk_tc2(A, lists.list(0, false, true, ntiles / 2 / B), false, pool.m, split,
                        std::min(ntiles, g.num_sms) & ~1, st));
     if (ckpt && L % ckpt_every == 0)
@@ -2567,6 +2601,7 @@ sp2_status sp2_network_forward(const float* H, int B, int N, int L, const float*
       A.lo_out = (__half*)lo[cur ^ 1];
       A.hp_out = (__half*)hp[cur ^ 1];
       rnp_step(A, rnp, n);
+      A.stall = take_stall();
       CK(launch_syrk_tc1(A, m[cur], split, std::min(ntiles, g.num_sms), st));
     } else {
       A.Yin = Yc;
@@ -2600,6 +2635,7 @@ sp2_status sp2_network_backward(const float* H, int B, int N, int L, const float
     set_err("sp2_network_backward: the adjoint runs on the tensor-core paths (split or fp16)");
     return SP2_ERR_UNSUPPORTED;
   }
+  CKS(late_error());
   const bool split = g.precision == SP2_PREC_SPLIT_FP16;
   cudaStream_t st = g.stream;
   const long long slot = (long long)N * N;
@@ -2767,6 +2803,7 @@ sp2_status sp2_network_backward(const float* H, int B, int N, int L, const float
   A.lo_scale = ls;
   A.lo_unscale = std::ldexp(1.0f, -g.lo_scale_exp);
   A.err = (int*)err;
+  A.late = g.late_dev;
   A.ld_y = N;
   A.slot_y = slot;
   A.ld_h = ld_h;
@@ -2866,10 +2903,8 @@ sp2_status sp2_network_backward(const float* H, int B, int N, int L, const float
   CK(cudaMemcpyAsync((char*)hd + (size_t)L * B * 3 * sizeof(double), err, sizeof(int), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
   const double* dd = (const double*)hd;
-  if (*(const int*)((char*)hd + (size_t)L * B * 3 * sizeof(double))) {
-    set_err("a bounded device wait timed out");
-    return SP2_ERR_DEVICE_TIMEOUT;
-  }
+  if (*(const int*)((char*)hd + (size_t)L * B * 3 * sizeof(double))) return timed_out();
+  CKS(late_error());  // of the forward pass whose checkpoints were read
   coef_gradient(dd, plan.alpha.data(), L, B, dcoef);
   return SP2_OK;
 }
@@ -2897,6 +2932,7 @@ sp2_status sp2_fermi_expansion(const float* H, int B, int N, int L, const double
     set_err("sp2_fermi_expansion: needs a tensor-core precision (split or fp16)");
     return SP2_ERR_UNSUPPORTED;
   }
+  CKS(late_error());
   const bool split = g.precision == SP2_PREC_SPLIT_FP16;
   cudaStream_t st = g.stream;
   const long long slot = (long long)N * N;
@@ -2933,6 +2969,7 @@ sp2_status sp2_fermi_expansion(const float* H, int B, int N, int L, const double
     x.vec_norm = (N & 3) == 0 && ((uintptr_t)D_out & 15) == 0;
     x.rn = (double*)rn;
     CK(launch_net_input(x, B, st));
+    run.A.stall = take_stall();
     CK(launch_resident_net(run.A, run.maps, split, run.grid, st));
     return fixed ? SP2_OK : run.wait_and_check(back);
   }
@@ -3088,6 +3125,7 @@ sp2_status sp2_fermi_expansion(const float* H, int B, int N, int L, const double
   A.lo_scale = std::ldexp(1.0f, g.lo_scale_exp);
   A.lo_unscale = std::ldexp(1.0f, -g.lo_scale_exp);
   A.err = (int*)err;
+  A.late = g.late_dev;
   A.Yin = D_out;
   A.Yout = D_out;
   A.ld_y = N;
@@ -3107,6 +3145,7 @@ sp2_status sp2_fermi_expansion(const float* H, int B, int N, int L, const double
   x.r_scale = (float)(-c[0]);
   x.r_add = (const double*)dd;
   CK(launch_net_input(x, B, st));
+  A.stall = take_stall();
   CK(launch_syrk_tc2(A, lists.list(0, false, true, ntiles / 2 / B), false, pool.m, split,
                      std::min(ntiles, g.num_sms) & ~1, st));
   return SP2_OK;

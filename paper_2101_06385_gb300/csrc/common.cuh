@@ -139,6 +139,17 @@ __device__ __forceinline__ float input_diag(float h, const InputScale& s) {
   return (float)(-(double)h * s.inv + s.diag_add);
 }
 
+// A bounded wait of a launch ran out (or the launch cannot run): the call's error
+// word, and the host's one (mapped memory), which outlives the call.
+template <class Args>
+__device__ __forceinline__ void give_up(const Args& a, int code = SP2_ERR_DEVICE_TIMEOUT) {
+  atomicExch(a.err, code);
+  if (a.late) {
+    *(volatile int*)a.late = code;
+    __threadfence_system();
+  }
+}
+
 __device__ __forceinline__ double warp_sum_d(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);

@@ -243,7 +243,7 @@ __device__ __forceinline__ bool tile(const SqArgs& a, const LayerOp& o, const La
   const bool got = __all_sync(0xffffffffu, PAIR ? mbar_wait_cl(&tmem_full[buf], (it >> 1) & 1u, abort_flag, lim)
                                                 : mbar_wait(&tmem_full[buf], (it >> 1) & 1u, abort_flag, lim));
   if (!got) {
-    if (lane == 0) atomicExch(a.err, (int)SP2_ERR_DEVICE_TIMEOUT);
+    if (lane == 0) give_up(a);
     *abort_flag = 1;
     return false;
   }
@@ -630,7 +630,7 @@ __device__ __forceinline__ bool tile(const SqArgs& a, const LayerOp& o, const La
       f.d2 = d2;
       mbar_arrive(&sh.fin_full[e]);
     } else {
-      atomicExch(a.err, (int)SP2_ERR_DEVICE_TIMEOUT);
+      give_up(a);
     }
   }
   return true;
@@ -646,7 +646,7 @@ __device__ __forceinline__ bool finish_entry(const SqArgs& a, double* tile_dots,
   using namespace sp2::tc;
   const uint32_t e = it % FQ;
   if (!__all_sync(0xffffffffu, mbar_wait(&sh.fin_full[e], (it / FQ) & 1u, abort_flag, lim))) {
-    if (lane == 0) atomicExch(a.err, (int)SP2_ERR_DEVICE_TIMEOUT);
+    if (lane == 0) give_up(a);
     *abort_flag = 1;
     return false;
   }

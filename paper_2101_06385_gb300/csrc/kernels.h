@@ -71,6 +71,7 @@ struct SqArgs {
   float lo_scale;          // 2^s
   float lo_unscale;        // 2^-s
   int* err;                // device error word (SP2_ERR_DEVICE_TIMEOUT on a timed-out wait)
+  int* late;               // the host's word for calls that return before their end, or nullptr
   unsigned long long wait_ns;  // bound of every mbarrier wait of the tcgen05 kernels (0: 4 s)
   int stall;               // fault injection: the MMA issuer first waits on a barrier that
                            // nothing arrives on, so that wait runs out after wait_ns
@@ -222,6 +223,7 @@ struct ResArgs {
   int local;               // every instance is one tile: its planes stay in shared memory
   int stall;               // as SqArgs
   int* err;
+  int* late;               // as SqArgs
   unsigned long long wait_ns;
 };
 cudaError_t launch_resident_input(const ResArgs& a, int vec_norm, int Nmax, int batch, cudaStream_t st);
@@ -276,7 +278,9 @@ struct NetArgs {
   long long* sums;         // [batch][kMeetRows] meeting rows, zero
   float lo_scale, lo_unscale;
   int shift, two_slots;
+  int stall;               // as SqArgs
   int* err;
+  int* late;               // as SqArgs
   unsigned long long wait_ns;
 };
 struct NetInput {
@@ -330,6 +334,7 @@ struct Res32Args {
   long long* slots;        // [2][2][grid][4] by the layer's parity: each CTA's trace, then its square norm
   unsigned* stamps;        // as ResArgs
   int* err;
+  int* late;               // as SqArgs
   unsigned long long wait_ns;
 };
 cudaError_t launch_resident_fp32(const Res32Args& a, int tile, int grid, cudaStream_t st);

@@ -528,7 +528,7 @@ __device__ __forceinline__ void control(const ResArgs& a, Shared& sh, int c, int
     __syncwarp();
   }
   if (!ok && lane == 0) {
-    atomicExch(a.err, (int)SP2_ERR_DEVICE_TIMEOUT);
+    give_up(a);
     *(volatile int*)&sh.abort = 1;
   }
   if (lane == 0) {
@@ -550,7 +550,7 @@ __global__ void __launch_bounds__(THREADS, 1) resident_kernel(const __grid_const
   Shared& sh = *reinterpret_cast<Shared*>(smem + OPERAND_BYTES + TR_BYTES);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (smem_u32(smem_raw) & 1023u) {  // the swizzled operand tiles need it; the same for every CTA
-    if (threadIdx.x == 0) atomicExch(a.err, (int)SP2_ERR_UNSUPPORTED);
+    if (threadIdx.x == 0) give_up(a, SP2_ERR_UNSUPPORTED);
     return;
   }
 
@@ -681,7 +681,7 @@ __global__ void __launch_bounds__(THREADS, 1) resident_kernel(const __grid_const
       sh.wq[seq % WQ] = WQ_END;
       mbar_arrive(&sh.wq_full[seq % WQ]);
       if (!ok || *abort_flag) {
-        atomicExch(a.err, (int)SP2_ERR_DEVICE_TIMEOUT);
+        give_up(a);
         *abort_flag = 1;
         for (int k = 0; k < STAGES; ++k) {  // copies in flight land before the CTA leaves
           if (armed[k] == 0) continue;
@@ -746,7 +746,7 @@ __global__ void __launch_bounds__(THREADS, 1) resident_kernel(const __grid_const
         if (ok) mma_commit(&sh.acc_full[c]);
       }
       if (!ok || *abort_flag) {
-        atomicExch(a.err, (int)SP2_ERR_DEVICE_TIMEOUT);
+        give_up(a);
         *abort_flag = 1;
       }
       if (issued) {
@@ -769,7 +769,7 @@ __global__ void __launch_bounds__(THREADS, 1) resident_kernel(const __grid_const
       if (c == WQ_END) break;
       uint8_t* area = smem + 2 * c * PLANES * HALF_BYTES;
       if (!epilogue<SPLIT, LOCAL>(a, sh, c, area, (aphase >> c) & 1u, tmem_base, ew, q, lane, trbuf + ew * (16 * 32), lim)) {
-        if (lane == 0) atomicExch(a.err, (int)SP2_ERR_DEVICE_TIMEOUT);
+        if (lane == 0) give_up(a);
         *abort_flag = 1;
         break;
       }

@@ -367,7 +367,7 @@ __global__ void __launch_bounds__(Cfg<TS>::THREADS, 1) resident_fp32_kernel(cons
     }
   }
   if (!ok) {
-    if (lane == 0) atomicExch(a.err, (int)SP2_ERR_DEVICE_TIMEOUT);
+    if (lane == 0) give_up(a);
     *ab = 1;
   }
 }

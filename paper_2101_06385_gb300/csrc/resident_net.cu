@@ -52,7 +52,7 @@ struct Shared {
   uint64_t epi_done[2][2];  // [slot][parity] the same: operation finished (a warp without rows may be an
                             //   operation ahead of the others: it must not stand in for them)
   uint64_t wq_full[WQ];  // producer -> MMA issuer and epilogue: next slot
-  uint64_t drain;
+  uint64_t drain, never;
   int wq[WQ];
   uint32_t tmem;
   int abort;
@@ -595,7 +595,7 @@ __device__ __forceinline__ void control(const NetArgs& a, Shared& sh, int c, int
     __syncwarp();
   }
   if (!ok && lane == 0) {
-    atomicExch(a.err, (int)SP2_ERR_DEVICE_TIMEOUT);
+    give_up(a);
     *(volatile int*)&sh.abort = 1;
   }
   if (lane == 0) {
@@ -618,7 +618,7 @@ __global__ void __launch_bounds__(THREADS, 1) resident_net_kernel(const __grid_c
   Shared& sh = *reinterpret_cast<Shared*>(smem + OPERAND_BYTES + TR_BYTES);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (smem_u32(smem_raw) & 1023u) {  // the swizzled operand tiles need it; the same for every CTA
-    if (threadIdx.x == 0) atomicExch(a.err, (int)SP2_ERR_UNSUPPORTED);
+    if (threadIdx.x == 0) give_up(a, SP2_ERR_UNSUPPORTED);
     return;
   }
   if (threadIdx.x == 0) {
@@ -636,6 +636,7 @@ __global__ void __launch_bounds__(THREADS, 1) resident_net_kernel(const __grid_c
     }
     for (int k = 0; k < WQ; ++k) mbar_init(&sh.wq_full[k], 1);
     mbar_init(&sh.drain, 1);
+    mbar_init(&sh.never, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
@@ -727,7 +728,7 @@ __global__ void __launch_bounds__(THREADS, 1) resident_net_kernel(const __grid_c
       sh.wq[seq % WQ] = WQ_END;
       mbar_arrive(&sh.wq_full[seq % WQ]);
       if (!ok || *abort_flag) {
-        atomicExch(a.err, (int)SP2_ERR_DEVICE_TIMEOUT);
+        give_up(a);
         *abort_flag = 1;
         for (int k = 0; k < STAGES; ++k) {  // copies in flight land before the CTA leaves
           if (armed[k] == 0) continue;
@@ -744,6 +745,7 @@ __global__ void __launch_bounds__(THREADS, 1) resident_net_kernel(const __grid_c
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true, issued = false;
+      if (a.stall && !mbar_wait(&sh.never, 0, abort_flag, lim)) ok = false;
       for (uint32_t seq = 0; ok; ++seq) {
         if (!mbar_wait(&sh.wq_full[seq % WQ], (seq / WQ) & 1u, abort_flag, idle)) {
           ok = false;
@@ -793,7 +795,7 @@ __global__ void __launch_bounds__(THREADS, 1) resident_net_kernel(const __grid_c
         if (ok) mma_commit(&sh.acc_full[c]);
       }
       if (!ok || *abort_flag) {
-        atomicExch(a.err, (int)SP2_ERR_DEVICE_TIMEOUT);
+        give_up(a);
         *abort_flag = 1;
       }
       if (issued) {
@@ -815,7 +817,7 @@ __global__ void __launch_bounds__(THREADS, 1) resident_net_kernel(const __grid_c
       const int c = *(volatile int*)&sh.wq[seq % WQ];
       if (c == WQ_END) break;
       if (!epilogue<SPLIT, EARLY>(a, sh, c, (aphase >> c) & 1u, tmem_base, ew, q, lane, trbuf + ew * (16 * 32), lim)) {
-        if (lane == 0) atomicExch(a.err, (int)SP2_ERR_DEVICE_TIMEOUT);
+        if (lane == 0) give_up(a);
         *abort_flag = 1;
         break;
       }

@@ -136,7 +136,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         }
       }
       if (!ok || *abort_flag) {
-        atomicExch(a.err, (int)SP2_ERR_DEVICE_TIMEOUT);
+        give_up(a);
         // Drain: the copies this thread issued land before the CTA exits
         // (the k-th arming of a stage completes the phase of parity (k-1)&1).
         for (int s = 0; s < STAGES; ++s) {
@@ -202,7 +202,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         if (!ok) break;
         mma_commit(tmem_full);
       }
-      if (!ok) atomicExch(a.err, (int)SP2_ERR_DEVICE_TIMEOUT);
+      if (!ok) give_up(a);
       if (issued) {
         // all MMAs of this CTA have completed once this commit lands
         mma_commit(drain);
@@ -235,7 +235,7 @@ __global__ void __launch_bounds__(THREADS, 1)
       if (lane == 0) s_got[q] = got ? 1 : 0;
       asm volatile("bar.sync 1, 128;" ::: "memory");
       if (!(s_got[0] & s_got[1] & s_got[2] & s_got[3])) {
-        if (!got && lane == 0) atomicExch(a.err, (int)SP2_ERR_DEVICE_TIMEOUT);
+        if (!got && lane == 0) give_up(a);
         break;
       }
       acc_phase ^= 1u;

@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         }
       }
       if (!ok || *abort_flag) {
-        atomicExch(a.err, (int)SP2_ERR_DEVICE_TIMEOUT);
+        give_up(a);
         for (int s = 0; s < STAGES; ++s) {
           if (armed[s] == 0) continue;
           const uint64_t t0 = globaltimer();
@@ -211,7 +211,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         mma_commit(&tmem_full[buf]);
         ++it;
       }
-      if (!ok) atomicExch(a.err, (int)SP2_ERR_DEVICE_TIMEOUT);
+      if (!ok) give_up(a);
       if (issued) {
         mma_commit(drain);
         const uint64_t t0 = globaltimer();

@@ -494,7 +494,7 @@ __global__ void __launch_bounds__(THREADS, 1)
       // the last (possibly partial) epoch of this pair
       if (pub_sync && gs > 0) atomicAdd(&wave[(gs - 1u) / (uint32_t)W], 1u);
       if (!ok || *abort_flag) {
-        atomicExch(a.err, (int)SP2_ERR_DEVICE_TIMEOUT);
+        give_up(a);
         st_cluster_u32(peer_abort, 1u);
         if (rank == 0) {
           // the armed phases complete once both CTAs' bytes have landed
@@ -635,7 +635,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         it += UW;
       }
       if (!ok || *abort_flag) {
-        atomicExch(a.err, (int)SP2_ERR_DEVICE_TIMEOUT);
+        give_up(a);
         st_cluster_u32(peer_abort, 1u);
       }
       if (issued) {
@@ -659,7 +659,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         continue;
       }
       if (live < 0) {
-        if (lane == 0) atomicExch(a.err, (int)SP2_ERR_DEVICE_TIMEOUT);
+        if (lane == 0) give_up(a);
         *abort_flag = 1;
         break;
       }
@@ -710,7 +710,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         }
       }
       if (!ok && lane == 0) {
-        atomicExch(a.err, (int)SP2_ERR_DEVICE_TIMEOUT);
+        give_up(a);
         *abort_flag = 1;
         st_cluster_u32(peer_abort, 1u);
       }
