@@ -171,6 +171,9 @@ const char* sp2_last_error(void);
  *               returns; the call (the next one, where it does not wait for its
  *               end) returns SP2_ERR_DEVICE_TIMEOUT (the outputs hold no
  *               meaningful values)
+ *   no_cooperative  cooperative launches are refused while in force, as for a
+ *               process or stream that has too few SMs to hold them: the calls
+ *               then run with a launch a layer
  *   wait_ms=<n> bound of every device wait of the tensor-core squaring
  *               kernels, 1..60000 ms (default 4000); stays in force
  * alloc_fail, nan_input and timeout each fire once.  The environment variable

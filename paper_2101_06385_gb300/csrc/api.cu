@@ -79,8 +79,12 @@ struct State {
   int lo_scale_exp = 11;
   int shift = 1;
   double eps = 0.0;
-  int num_sms = 148;
+  int device_sms = 148;
+  int num_sms = 148;  // that the library stream can use (stream_sms)
+  int max_pairs = 0;  // CTA pairs that the device can run at the same time (0: not known)
   PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
+  PFN_cuStreamGetGreenCtx_v12040 stream_green = nullptr;
+  PFN_cuGreenCtxGetDevResource_v12040 green_resource = nullptr;
   Buf buf[B_COUNT];
   // word in mapped host memory that a kernel sets when a wait of it ran out, for
   // calls that return before their end (its device address too)
@@ -109,6 +113,7 @@ struct State {
   // injected faults (sp2_set_fault / SP2_FAULT): each fires once
   bool fault_alloc = false, fault_nan = false, fault_stall = false;
   size_t alloc_limit = 0;  // injected: larger workspace requests fail (0: none)
+  bool fault_no_coop = false;  // injected: cooperative launches are refused
   // side of the square groups of the tile order (SP2_TILE_GROUP, default 8)
   int tile_group = 8;
   // K stages per epoch of the soft pair synchronisation (SP2_WAVE_SYNC, default
@@ -382,6 +387,62 @@ struct PlanePool {
   __half* p1_of(int k) const { return p1 ? p1 + entry * k : nullptr; }
 };
 
+// The SMs that the library stream can use: a stream of a green context has its
+// context's alone.  The kernels whose CTAs wait on one another need all of them
+// running at once, so their grids (and which sizes they take) go by this.
+void stream_sms() {
+  g.num_sms = g.device_sms;
+  if (!g.stream_green || !g.green_resource || (uintptr_t)g.stream <= 2) return;  // 0 to 2: the default streams
+  CUgreenCtx gc = nullptr;
+  CUdevResource r;
+  if (g.stream_green((CUstream)g.stream, &gc) == CUDA_SUCCESS && gc &&
+      g.green_resource(gc, &r, CU_DEV_RESOURCE_TYPE_SM) == CUDA_SUCCESS && r.sm.smCount > 0)
+    g.num_sms = std::min(g.device_sms, (int)r.sm.smCount);
+}
+
+// CTAs of a launch of the pair kernel over ntiles half super tiles (or units).
+int pair_grid(int ntiles) {
+  int n = std::min(ntiles, g.num_sms);
+  if (g.max_pairs > 0) n = std::min(n, 2 * g.max_pairs);
+  return std::max(2, n & ~1);
+}
+
+// A cooperative launch.  What the device (or the share of it that a service gives
+// the process) cannot hold at once is refused with an error that leaves the context
+// usable; the caller then takes the launch-per-layer way.
+constexpr sp2_status kRefused = (sp2_status)2;  // never returned to the user
+template <class F>
+cudaError_t coop_launch(F f) {
+  return g.fault_no_coop ? cudaErrorCooperativeLaunchTooLarge : f();
+}
+bool refused(cudaError_t e) {
+  if (e != cudaErrorCooperativeLaunchTooLarge) return false;
+  cudaGetLastError();
+  return true;
+}
+
+// A list of layers on the CTA pairs: one cooperative launch, or one launch a layer.
+cudaError_t launch_pairs(const SqArgs& a, const PairList& l, bool adjoint, const CUtensorMap* m, bool split, int grid) {
+  const cudaError_t e = coop_launch([&] { return launch_syrk_tc2(a, l, adjoint, m, split, grid, g.stream); });
+  if (!refused(e)) return e;
+  SqArgs b = a;
+  b.wave_ctr = nullptr;  // pairs that do not run together do not keep in step
+  for (int n = 0; n < l.nops; ++n) {
+    PairList one = l;
+    one.ops = l.ops + n;
+    one.nops = 1;
+    one.groups = 0;
+    one.cooperative = 0;
+    if (l.rec) one.rec = l.rec + n;
+    if (l.stamps) one.stamps = l.stamps + n;
+    cudaError_t s = cudaMemsetAsync(l.done, 0, sizeof(unsigned) * 2 * l.batch, g.stream);
+    if (s == cudaSuccess) s = launch_syrk_tc2(b, one, adjoint, m, split, grid, g.stream);
+    if (s != cudaSuccess) return s;
+    b.stall = 0;
+  }
+  return cudaSuccess;
+}
+
 // Lists of layers for the CTA-pair kernel (one launch each), their flags and
 // records in one device buffer, uploaded with one copy.
 struct PairLists {
@@ -419,6 +480,7 @@ struct PairLists {
     l.nops = (i + 1 < (int)first.size() ? first[i + 1] : (int)ops.size()) - first[i];
     l.batch = B;
     l.per = per;
+    l.cooperative = 1;
     if (grouped) {
       const int need = (int)std::ceil(1.9 * (g.num_sms / 2) / per);
       l.groups = std::max(1, B / std::max(1, need));
@@ -543,6 +605,7 @@ sp2_status sp2_set_fault(const char* spec) {
   bool alloc = false, nan = false, stall = false;
   unsigned long long wait_ns = 0;
   size_t alloc_limit = 0;
+  bool no_coop = false;
   const std::string sp = spec ? spec : "";
   size_t pos = 0;
   while (pos <= sp.size()) {
@@ -556,6 +619,8 @@ sp2_status sp2_set_fault(const char* spec) {
       nan = true;
     } else if (item == "timeout") {
       stall = true;
+    } else if (item == "no_cooperative") {
+      no_coop = true;
     } else if (item.compare(0, 12, "alloc_limit=") == 0) {
       char* e = nullptr;
       const long v = std::strtol(item.c_str() + 12, &e, 10);
@@ -573,13 +638,16 @@ sp2_status sp2_set_fault(const char* spec) {
       }
       wait_ns = (unsigned long long)v * 1000000ull;
     } else {
-      set_err("sp2_set_fault: unknown item '%s' (alloc_fail, alloc_limit=<n>, nan_input, timeout, wait_ms=<n>, none)", item.c_str());
+      set_err("sp2_set_fault: unknown item '%s' (alloc_fail, alloc_limit=<n>, nan_input, timeout, no_cooperative, "
+              "wait_ms=<n>, none)",
+              item.c_str());
       return SP2_ERR_INVALID_ARG;
     }
     pos = end + 1;
   }
   g.fault_alloc = alloc;
   g.alloc_limit = alloc_limit;
+  g.fault_no_coop = no_coop;
   g.fault_nan = nan;
   g.fault_stall = stall;
   g.wait_ns = wait_ns;
@@ -617,7 +685,7 @@ sp2_status sp2_init(const sp2_config* cfg) {
     set_err("libsp2 is built for sm_103a (compute capability 10.x); device has %d.%d", major, minor);
     return SP2_ERR_UNSUPPORTED;
   }
-  CK(cudaDeviceGetAttribute(&g.num_sms, cudaDevAttrMultiProcessorCount, c.device));
+  CK(cudaDeviceGetAttribute(&g.device_sms, cudaDevAttrMultiProcessorCount, c.device));
   if (!g.encode) {
     void* fn = nullptr;
     cudaDriverEntryPointQueryResult q;
@@ -627,7 +695,18 @@ sp2_status sp2_init(const sp2_config* cfg) {
       return SP2_ERR_UNSUPPORTED;
     }
     g.encode = (PFN_cuTensorMapEncodeTiled_v12000)fn;
+    // (absent from older drivers, which have no green contexts)
+    auto optional = [&](const char* name) -> void* {
+      void* p = nullptr;
+      const bool ok = cudaGetDriverEntryPointByVersion(name, &p, 12040, cudaEnableDefault, &q) == cudaSuccess &&
+                      q == cudaDriverEntryPointSuccess;
+      if (!ok) cudaGetLastError();
+      return ok ? p : nullptr;
+    };
+    g.stream_green = (PFN_cuStreamGetGreenCtx_v12040)optional("cuStreamGetGreenCtx");
+    g.green_resource = (PFN_cuGreenCtxGetDevResource_v12040)optional("cuGreenCtxGetDevResource");
   }
+  if (g.max_pairs == 0 || !g.init) g.max_pairs = syrk_tc2_max_pairs();
   if (!g.late) {
     CK(cudaHostAlloc(&g.late, sizeof(int), cudaHostAllocMapped));
     *(volatile int*)g.late = 0;
@@ -660,6 +739,7 @@ sp2_status sp2_init(const sp2_config* cfg) {
   }
   g.device = c.device;
   g.stream = (cudaStream_t)c.stream;
+  stream_sms();
   g.precision = c.precision;
   g.lo_scale_exp = c.lo_scale_exp;
   g.shift = c.shift_identity ? 1 : 0;
@@ -704,6 +784,7 @@ sp2_status sp2_finalize(void) {
 sp2_status sp2_set_stream(void* stream) {
   CKS(require_init());
   g.stream = (cudaStream_t)stream;
+  stream_sms();
   return SP2_OK;
 }
 
@@ -1126,7 +1207,9 @@ sp2_status resident_solve(const float* const* H, const int* N, const int* N_occ,
   }
   CK(cudaEventRecord(g.stage_done, st));
   CK(cudaEventRecord(g.lev[0], st));
-  CK(launch_resident(A, maps, split, grid, st));
+  const cudaError_t le = coop_launch([&] { return launch_resident(A, maps, split, grid, st); });
+  if (refused(le)) return kRefused;
+  CK(le);
   CK(cudaEventRecord(g.ev1, st));
 
   if (!stats) return SP2_OK;
@@ -1245,7 +1328,9 @@ sp2_status fp32_solve(const float* H, int N, int N_occ, double tol, int max_iter
                         (double2*)part, tick, g.shift, 1, 1, igrid, st));
   CK(launch_rownorm(A.Y[0], ld_y, slot_y, np, 1, N, A.rn, N, A.ctl, (double2*)part, tick, rgrid, st));
   CK(cudaEventRecord(g.lev[0], st));
-  CK(launch_resident_fp32(A, tile, grid, st));
+  const cudaError_t le = coop_launch([&] { return launch_resident_fp32(A, tile, grid, st); });
+  if (refused(le)) return kRefused;
+  CK(le);
   CK(cudaEventRecord(g.ev1, st));
   if (!stats) return SP2_OK;
   void* back;
@@ -1270,11 +1355,13 @@ sp2_status fp32_solve(const float* H, int N, int N_occ, double tol, int max_iter
 // the HOMO/LUMO estimates) instead of the trace rule with refinement.
 sp2_status density_matrix_impl(const float* H, int N, int N_occ, double tol, int max_iter, float* D_out,
                                sp2_stats* stats, bool accel, double homo, double lumo) {
+  sp2_status res = kRefused;
   if (resident_fits(N))
-    return resident_solve(&H, &N, &N_occ, 1, N, tol, max_iter, &D_out, stats, accel ? &homo : nullptr,
-                          accel ? &lumo : nullptr, true);
-  if (const int tile = fp32_tile(N))
-    return fp32_solve(H, N, N_occ, tol, max_iter, D_out, stats, accel, homo, lumo, tile);
+    res = resident_solve(&H, &N, &N_occ, 1, N, tol, max_iter, &D_out, stats, accel ? &homo : nullptr,
+                         accel ? &lumo : nullptr, true);
+  else if (const int tile = fp32_tile(N))
+    res = fp32_solve(H, N, N_occ, tol, max_iter, D_out, stats, accel, homo, lumo, tile);
+  if (res != kRefused) return res;
   const int prec = g.precision;
   const bool tc = tc_precision(prec);
   const bool split = prec == SP2_PREC_SPLIT_FP16;
@@ -1447,7 +1534,7 @@ sp2_status density_matrix_impl(const float* H, int N, int N_occ, double tol, int
       A.tri_planes = 1;
       A.wide = wide ? 1 : 0;
       A.stall = take_stall();
-      const int grid = std::min(wide ? ntiles / 2 : ntiles, g.num_sms) & ~1;  // every pair has a unit
+      const int grid = pair_grid(wide ? ntiles / 2 : ntiles);  // every pair has a unit
       // epoch counters of the soft pair synchronisation, one zeroed slice per
       // layer (per pair: super tiles, or wide units of two)
       // where it pays: split products with operand planes beyond L2 (N = 12000 143.6
@@ -1460,7 +1547,7 @@ sp2_status density_matrix_impl(const float* H, int N, int N_occ, double tol, int
       l.wave_per = (int)per;
       A.sync_stages = g.wave_sync;
       A.snake = g.wave_sync > 0 ? g.snake : 0;
-      CK(launch_syrk_tc2(A, l, false, pool.m, split, grid, st));
+      CK(launch_pairs(A, l, false, pool.m, split, grid));
     } else {
       const int grid = std::min(ntiles, g.num_sms);
       for (int k = 0; k < nlaunch; ++k) {
@@ -1737,7 +1824,7 @@ sp2_status batched_once(const float* const* H, const int* N, const int* N_occ, i
                             nullptr, (double2*)part, (unsigned*)tick, g.shift, 1, B, igrid, st));
       CK(launch_rownorm((float*)Y[0], ld_y, slot_y, (const int*)ns, B, Nmax, (double*)rn, Nmax, (Ctl*)ctl,
                         (double2*)part, (unsigned*)tick, rgrid, st));
-      const int grid = std::min(nt, g.num_sms) & (pairs ? ~1 : ~0);
+      const int grid = pairs ? pair_grid(nt) : std::min(nt, g.num_sms);
       CK(cudaEventRecordWithFlags(g.lev[0], st, evf));
       for (int k = 0; k < nlaunch; ++k) {
         const int cur = k & 1;
@@ -1857,8 +1944,10 @@ sp2_status batched_impl(const float* const* H, const int* N, const int* N_occ, i
   cudaStream_t st = g.stream;
   const int B = batch;
 
-  if (g.batched_sched == 0 && resident_fits(Nmax))
-    return resident_solve(H, N, N_occ, B, Nmax, tol, max_iter, D_out, stats, homo, lumo, false);
+  if (g.batched_sched == 0 && resident_fits(Nmax)) {
+    const sp2_status s = resident_solve(H, N, N_occ, B, Nmax, tol, max_iter, D_out, stats, homo, lumo, false);
+    if (s != kRefused) return s;
+  }
 
   // schedule: fixed (SP2_BATCHED_KERNEL=single|pairs) or tuned once per batch
   // signature by timing each candidate on the call itself (every candidate
@@ -2291,7 +2380,9 @@ sp2_status net_forward_resident(const float* H, int B, int N, int L, const float
   x.alpha0 = R.dev(0);
   CK(launch_net_input(x, B, g.stream));
   R.A.stall = take_stall();
-  CK(launch_resident_net(R.A, R.maps, split, R.grid, g.stream));
+  const cudaError_t le = coop_launch([&] { return launch_resident_net(R.A, R.maps, split, R.grid, g.stream); });
+  if (refused(le)) return kRefused;
+  CK(le);
   return R.wait_and_check(back);
 }
 
@@ -2387,7 +2478,9 @@ sp2_status net_backward_resident(const float* H, int B, int N, int L, const floa
   x.rn = (double*)rn;
   CK(launch_net_input(x, nseg * B, st));
   CK(launch_net_input(R.input(NET_FULL, G_out, p_g), B, st));
-  CK(launch_resident_net(R.A, R.maps, split, R.grid, st));
+  const cudaError_t le = coop_launch([&] { return launch_resident_net(R.A, R.maps, split, R.grid, st); });
+  if (refused(le)) return kRefused;
+  CK(le);
   CK(launch_net_dots((const double*)tdots, R.nt, R.per, L, B, (double*)dots, st));
   // dot products, shifts, statuses, error word
   const size_t db = (size_t)L * B * 3 * sizeof(double), ab = nalpha * sizeof(double), sb = (size_t)B * sizeof(int);
@@ -2442,7 +2535,10 @@ sp2_status sp2_network_forward(const float* H, int B, int N, int L, const float*
       return SP2_ERR_INVALID_ARG;
     }
   CKS(late_error());
-  if (net_fits(B, N, 896)) return net_forward_resident(H, B, N, L, coef, ckpt_every, X_out, ckpt, bounds);
+  if (net_fits(B, N, 896)) {
+    const sp2_status s = net_forward_resident(H, B, N, L, coef, ckpt_every, X_out, ckpt, bounds);
+    if (s != kRefused) return s;
+  }
   const bool tc = tc_precision(g.precision);
   const bool split = g.precision == SP2_PREC_SPLIT_FP16;
   cudaStream_t st = g.stream;
@@ -2570,8 +2666,7 @@ sp2_status sp2_network_forward(const float* H, int B, int N, int L, const float*
     CK(launch_net_input(x, B, st));
     A.tri_planes = 1;
     A.stall = take_stall();
-    CK(launch_syrk_tc2(A, lists.list(0, false, true, ntiles / 2 / B), false, pool.m, split,
-                       std::min(ntiles, g.num_sms) & ~1, st));
+    CK(launch_pairs(A, lists.list(0, false, true, ntiles / 2 / B), false, pool.m, split, pair_grid(ntiles)));
     if (ckpt && L % ckpt_every == 0)
       CK(cudaMemcpyAsync(ckpt_slot(L / ckpt_every), X_out, (size_t)B * slot * 4, cudaMemcpyDeviceToDevice, st));
     return SP2_OK;
@@ -2643,10 +2738,11 @@ sp2_status sp2_network_backward(const float* H, int B, int N, int L, const float
   if (net_fits(B, N, 896) && backward_fits(B, N, L, ce)) {
     const bool injected = g.fault_alloc;
     const sp2_status s = net_backward_resident(H, B, N, L, coef, ce, ckpt, G_out, dcoef, G_in);
-    if (s != SP2_ERR_OOM || injected) return s;
+    if (s != kRefused && (s != SP2_ERR_OOM || injected)) return s;
     // the pairs need less; what the attempt holds goes back first
     t_err.clear();
-    for (BufId id : {B_PLANES0, B_PLANES1, B_SEG}) CKS(ws_free(id));
+    if (s == SP2_ERR_OOM)
+      for (BufId id : {B_PLANES0, B_PLANES1, B_SEG}) CKS(ws_free(id));
   }
   void* G;
   CKS(ws(B_G, (size_t)B * slot * 4, &G));
@@ -2811,7 +2907,7 @@ sp2_status sp2_network_backward(const float* H, int B, int N, int L, const float
   const int sgrid = (int)std::min<long long>((long long)N * B, 8LL * g.num_sms);
   const int mgrid = (int)std::min<long long>(N, std::max(1, 4 * g.num_sms / B + 1));
   const int rgrid = (int)std::min<long long>((N + 7) / 8, std::max(1, 2 * g.num_sms / B + 1));
-  const int tgrid = std::min(ntiles, g.num_sms) & (pairs ? ~1 : ~0);
+  const int tgrid = pairs ? pair_grid(ntiles) : std::min(ntiles, g.num_sms);
   const SqArgs& R0 = A;
 
   if (pairs) {
@@ -2842,8 +2938,7 @@ sp2_status sp2_network_backward(const float* H, int B, int N, int L, const float
       P.tile_dots = (double*)tdots;
       P.rn = (const double*)rn;
       P.ld_rn = N;
-      CK(launch_syrk_tc2(P, lists.list(nseg_layers - 1 - sgi, false, true, ntiles / 2 / B), true, pool.m, split, tgrid,
-                         st));
+      CK(launch_pairs(P, lists.list(nseg_layers - 1 - sgi, false, true, ntiles / 2 / B), true, pool.m, split, tgrid));
       continue;
     }
     CK(launch_materialize(ckpt + (size_t)sgi * B * slot, N, slot, N, B, (const double*)nal + (size_t)n0 * B,
@@ -2970,8 +3065,11 @@ sp2_status sp2_fermi_expansion(const float* H, int B, int N, int L, const double
     x.rn = (double*)rn;
     CK(launch_net_input(x, B, st));
     run.A.stall = take_stall();
-    CK(launch_resident_net(run.A, run.maps, split, run.grid, st));
-    return fixed ? SP2_OK : run.wait_and_check(back);
+    const cudaError_t le = coop_launch([&] { return launch_resident_net(run.A, run.maps, split, run.grid, st); });
+    if (!refused(le)) {
+      CK(le);
+      return fixed ? SP2_OK : run.wait_and_check(back);
+    }
   }
 
   // per-instance records; fixed bounds go straight into the control blocks
@@ -3146,8 +3244,7 @@ sp2_status sp2_fermi_expansion(const float* H, int B, int N, int L, const double
   x.r_add = (const double*)dd;
   CK(launch_net_input(x, B, st));
   A.stall = take_stall();
-  CK(launch_syrk_tc2(A, lists.list(0, false, true, ntiles / 2 / B), false, pool.m, split,
-                     std::min(ntiles, g.num_sms) & ~1, st));
+  CK(launch_pairs(A, lists.list(0, false, true, ntiles / 2 / B), false, pool.m, split, pair_grid(ntiles)));
   return SP2_OK;
 }
 

@@ -129,6 +129,7 @@ struct PairList {
   LayerParams* rec;        // [nops + 1] parameters chosen by the control steps (ctl set: one instance)
   unsigned long long* stamps;  // [nops + 1] ns at the start and after each layer (ctl set), or nullptr
   int wave_per;            // SqArgs::wave_ctr entries of a layer (groups = 0)
+  int cooperative;         // more than one layer: the pairs wait on one another
 };
 
 // tensor-core tile geometry
@@ -177,11 +178,12 @@ size_t syrk_tc1_smem_bytes(bool split);
 // come in (h = 0, h = 1) pairs of one super tile, a.ntiles = 2 x super tiles.
 // tmaps: {p0, p1} with 64 x 128 boxes and {p0, p1} with 64 x 64 boxes, through
 // which the K blocks left of the diagonal are read transposed from the upper
-// tiles.  A list of layers (l.ops) is one cooperative launch; adjoint: it holds
-// adjoint layers.
+// tiles.  A list of several layers is a cooperative launch, of at most
+// syrk_tc2_max_pairs() pairs; adjoint: it holds adjoint layers.
 cudaError_t launch_syrk_tc2(const SqArgs& a, const PairList& l, bool adjoint, const CUtensorMap* tmaps, bool split,
                             int grid, cudaStream_t st);
 size_t syrk_tc2_smem_bytes(bool split);
+int syrk_tc2_max_pairs();  // pairs of the device that can run at the same time (0: not known)
 
 // Resident solve (csrc/resident.cu): all layers of a batch of instances in one
 // cooperative launch on 128 x 128 tiles; the tiles of one instance are

@@ -324,7 +324,7 @@ __global__ void __launch_bounds__(THREADS, 1)
   if (l.ops && a.ctl) {
     if (threadIdx.x == 0) {
       s_p0 = a.ctl[0].next;
-      if (blockIdx.x == 0 && l.stamps) l.stamps[0] = globaltimer();
+      if (blockIdx.x == 0 && l.stamps && s_p0.active) l.stamps[0] = globaltimer();
     }
     __syncthreads();
     if (!s_p0.active) return;
@@ -756,6 +756,28 @@ size_t syrk_tc2_smem_bytes(bool split) {
   return (size_t)stages * sb + 1024 /* alignment slack */ + 256 /* barriers */ + epi::TR_BYTES;
 }
 
+int syrk_tc2_max_pairs() {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(2, 1, 1);
+  cfg.blockDim = dim3(tc2::THREADS, 1, 1);
+  cfg.dynamicSmemBytes = syrk_tc2_smem_bytes(true);
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 2;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  auto kernel = tc2::syrk_tc2_kernel<true, false, false, false>;
+  int n = 0;
+  if (set_smem_once(kernel, (int)cfg.dynamicSmemBytes, 1) != cudaSuccess ||
+      cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return n;
+}
+
 cudaError_t launch_syrk_tc2(const SqArgs& a, const PairList& l, bool adjoint, const CUtensorMap* tm, bool split,
                             int grid, cudaStream_t st) {
   // grid: number of CTAs, even (two per cluster); a.ntiles = 2 x super tiles
@@ -773,7 +795,7 @@ cudaError_t launch_syrk_tc2(const SqArgs& a, const PairList& l, bool adjoint, co
   attr[1].id = cudaLaunchAttributeCooperative;  // a list's pairs wait on one another
   attr[1].val.cooperative = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = l.ops ? 2 : 1;
+  cfg.numAttrs = l.cooperative ? 2 : 1;
   auto go = [&](auto kernel, int which) -> cudaError_t {
     cudaError_t e = set_smem_once(kernel, (int)smem, which);
     if (e != cudaSuccess) return e;
