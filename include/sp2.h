@@ -164,9 +164,9 @@ const char* sp2_last_error(void);
  *               while in force (buffers that are large enough already are used)
  *   nan_input   the next sp2_density_matrix / _accelerated reads row 0 of H
  *               as holding a NaN: SP2_ERR_NONFINITE, no layer runs
- *   timeout     in the first squaring launch of the next single-matrix solve,
- *               forward pass or expansion the MMA issuer waits on a barrier
- *               that nothing arrives on; the wait runs out, every CTA stops
+ *   timeout     in the first squaring launch of the next tensor-core solve (one
+ *               matrix or a batch), forward pass or expansion the MMA issuer
+ *               waits on a barrier that nothing arrives on; the wait runs out, every CTA stops
  *               issuing, drains its copies and MMAs, frees its tensor memory and
  *               returns; the call (the next one, where it does not wait for its
  *               end) returns SP2_ERR_DEVICE_TIMEOUT (the outputs hold no

@@ -1183,7 +1183,7 @@ sp2_status resident_solve(const float* const* H, const int* N, const int* N_occ,
   A.wait_ns = g.wait_ns;
   A.two_slots = nt > grid ? 1 : 0;
   A.local = Nmax <= kResTile ? 1 : 0;
-  A.stall = single ? take_stall() : 0;
+  A.stall = take_stall();
   ResMaps maps;
   for (int k = 0; k < 2; ++k) {
     CKS(tmaps4_for(A.p0[k], A.p1[k], Nmax, B, ld_h, slot_h, maps.m[k], kTransBox));
@@ -1804,6 +1804,7 @@ sp2_status batched_once(const float* const* H, const int* N, const int* N_occ, i
   A.ld_y = ld_y;
   A.slot_y = slot_y;
 
+  const int stall = take_stall();
   // event records become graph nodes only with the external flag, which is
   // valid during capture alone
   auto enqueue = [&](cudaStream_t st, bool capturing) -> sp2_status {
@@ -1832,6 +1833,7 @@ sp2_status batched_once(const float* const* H, const int* N, const int* N_occ, i
         A.lo_out = (__half*)lo[cur ^ 1];
         A.hp_out = (__half*)hp[cur ^ 1];
         rnp_step(A, rnp, k);
+        A.stall = k == 0 ? stall : 0;
         if (pairs)
           CK(launch_syrk_tc2(A, one_layer(B), false, m[cur], split, grid, st));
         else
@@ -1862,12 +1864,12 @@ sp2_status batched_once(const float* const* H, const int* N, const int* N_occ, i
   };
 
   // The whole sequence replays as one CUDA graph while everything baked into
-  // it (sizes, grids, workspace addresses, stream) is unchanged; the per-call
+  // it (sizes, grids, wait bound, workspace addresses, stream) is unchanged; the per-call
   // records (control blocks, pointers, tile list) were uploaded above.
   if (g.use_graphs) {
     const uint64_t key[] = {(uint64_t)B, (uint64_t)Nmax, (uint64_t)nt, (uint64_t)nlaunch, (uint64_t)prec, (uint64_t)pairs,
                             (uint64_t)g.shift, (uint64_t)g.lo_scale_exp, (uint64_t)igrid, (uint64_t)rgrid,
-                            (uint64_t)ggrid, (uint64_t)g.num_sms, (uint64_t)(uintptr_t)st,
+                            (uint64_t)ggrid, (uint64_t)g.num_sms, (uint64_t)g.wait_ns, (uint64_t)stall, (uint64_t)(uintptr_t)st,
                             (uint64_t)(uintptr_t)hs, (uint64_t)(uintptr_t)ns, (uint64_t)(uintptr_t)ctl,
                             (uint64_t)(uintptr_t)dt, (uint64_t)(uintptr_t)doff, (uint64_t)(uintptr_t)dcnt,
                             (uint64_t)(uintptr_t)dpart, (uint64_t)(uintptr_t)ddone, (uint64_t)(uintptr_t)err,
