@@ -174,8 +174,11 @@ const char* sp2_last_error(void);
  *   no_cooperative  cooperative launches are refused while in force, as for a
  *               process or stream that has too few SMs to hold them: the calls
  *               then run with a launch a layer
- *   wait_ms=<n> bound of every device wait of the tensor-core squaring
- *               kernels, 1..60000 ms (default 4000); stays in force
+ *   wait_ms=<n> bound of the device waits of the tensor-core squaring kernels,
+ *               1..60000 ms (default 4000); stays in force.  Waits that last as
+ *               long as other solves of the same launch do (the resident kernels'
+ *               for work and for the tiles of their matrix, all of the resident
+ *               FP32 kernel's) are bounded by the larger of n and 4000 ms
  * alloc_fail, nan_input and timeout each fire once.  The environment variable
  * SP2_FAULT, when set, is applied by sp2_init.  Needs neither a GPU nor
  * sp2_init.  Returns SP2_ERR_INVALID_ARG (and changes nothing) for an unknown
