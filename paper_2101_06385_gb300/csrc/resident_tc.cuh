@@ -99,7 +99,7 @@ __device__ __forceinline__ void turn_tmem(float* trb, uint32_t taddr, int lane, 
 }
 
 // Stores the operand planes of the chunk (Eq. 12: hp = 2^s fp16(x) and lo' =
-// fp16(2^s x - hp), both differences exact; plain FP16 keeps hi alone), four
+// fp16(2^s (x - fp16(x))), finite where hp is not; plain FP16 keeps hi alone), four
 // halves per plane and row; p0, p1 at the lane's first row and column, rows
 // 4 i < rows_left.
 template <bool SPLIT, class Put>
@@ -113,10 +113,10 @@ __device__ __forceinline__ void split_chunk(const float (&y)[32], float lo_scale
       const float x0 = y[4 * i + 2 * e2], x1 = y[4 * i + 2 * e2 + 1];
       __half2 p2 = __floats2half2_rn(x0, x1);
       if (SPLIT) {
-        p2 = __hmul2(p2, s2);
-        const float2 pf = __half22float2(p2);
-        const __half2 l2 = __floats2half2_rn(fmaf(x0, lo_scale, -pf.x), fmaf(x1, lo_scale, -pf.y));
+        const float2 hf = __half22float2(p2);
+        const __half2 l2 = __floats2half2_rn((x0 - hf.x) * lo_scale, (x1 - hf.y) * lo_scale);
         pl[e2] = *reinterpret_cast<const uint32_t*>(&l2);
+        p2 = __hmul2(p2, s2);
       }
       pa[e2] = *reinterpret_cast<const uint32_t*>(&p2);
     }
