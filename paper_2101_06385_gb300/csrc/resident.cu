@@ -52,6 +52,7 @@ struct Slot {
   int cnt, me;           // the gang, and this tile's place in it
   int direct;            // the producer itself watches the gang's arrivals
   int stored;            // epilogue warps that have stored their part of the planes
+  int exact;             // every sum in FP64 (fp64_sums)
   long long* rows;       // the gang's meeting rows
   SolveState st;
 };
@@ -83,7 +84,7 @@ struct Shared {
 // FP64 sums did.  A spectrum of H that lies on one side of zero starts with alpha
 // outside [0, 1] and squares it until a branch brings it back, so any magnitude
 // can occur: a warp whose sum leaves the range, or is not a number, marks it and
-// hands it over in FP64.
+// hands it over in FP64 (so do all of a solve where fp64_sums says so).
 constexpr long long SQ_LIMIT = (1ll << 58) + (1ll << 50);  // a 32 x 32 block's 32, with rounding
 constexpr long long SQ_OUT = -1;                           // marks a warp's sum that is in Shared::red_d (as T_OUT)
 
@@ -124,7 +125,7 @@ __device__ __forceinline__ double row_norm(const ResArgs& a, const Slot& s, int 
     acc += fix_sq(v[u]);
     top = max(top, __float_as_uint(v[u]));
   }
-  if (top > 0x40800000u) {
+  if (top > 0x40800000u || s.exact) {
     auto every8 = [&](int first) {  // epi::row_norm's order
       double sum = 0.0;
 #pragma unroll 1
@@ -257,7 +258,7 @@ __device__ __forceinline__ bool epilogue(const ResArgs& a, Shared& sh, int c, ui
       ydf = (float)yd;
       ydo = outD ? (float)(yd + p.alpha_out) : ydf;
     }
-    if (__any_sync(0xffffffffu, !(fabsf(ydf) < T_LIMIT))) {
+    if (__any_sync(0xffffffffu, !(fabsf(ydf) < T_LIMIT) || s.exact)) {
       const double T = warp_sum_d(yd);
       if (lane == 0) sh.red_d[c][ew].x = T;
       tr = T_OUT;
@@ -319,7 +320,7 @@ __device__ __forceinline__ bool epilogue(const ResArgs& a, Shared& sh, int c, ui
       }
     }
     const float sql = ((rs[0] + rs[1]) + (rs[2] + rs[3])) + ((rs[4] + rs[5]) + (rs[6] + rs[7]));
-    const bool wild = __any_sync(0xffffffffu, !(sql < 16.f));
+    const bool wild = __any_sync(0xffffffffu, !(sql < 16.f) || s.exact);
     auto sum_squares = [&]() {
       sq = warp_sum_ll(fix_sq(sql));
       if (wild || sq > SQ_LIMIT) {
@@ -452,6 +453,7 @@ __device__ __forceinline__ void control(const ResArgs& a, Shared& sh, int c, int
       s.direct = LOCAL || (cnt > 1 && !a.two_slots);
       s.me = t - off;
       s.stored = 0;
+      s.exact = fp64_sums(hot) ? 1 : 0;
       s.rows = rows;
       if (act) {
         mbar_arrive(&sh.ready[c]);

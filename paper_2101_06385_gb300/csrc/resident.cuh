@@ -45,6 +45,10 @@ struct PreparedCoef {
 
 // A solve's control block without its history, the history's last four layers
 // and the prepared step, in shared memory.
+// With no state or every state occupied S goes to 0 or I and the sums of Y below any
+// fixed unit: those solves keep all of them in FP64 (fp64_sums).
+__device__ __forceinline__ bool fp64_sums(const Ctl* c) { return c->n_occ == 0 || c->n_occ == c->N; }
+
 struct SolveState {
   int sg[4];
   double ie[4];

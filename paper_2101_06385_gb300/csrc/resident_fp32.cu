@@ -119,6 +119,7 @@ __device__ __forceinline__ bool control(const Res32Args& a, Shared<TS>& sh, int 
   const volatile int* ab = &sh.abort;
   sh.st.load(a.ctl, lane);
   if (!hot->next.active) return true;
+  const bool exact = fp64_sums(hot);
   const uint64_t t0 = globaltimer();
   if (lane == 0) {
     mbar_arrive(&sh.gate);
@@ -156,7 +157,7 @@ __device__ __forceinline__ bool control(const Res32Args& a, Shared<TS>& sh, int 
       long long* norms = a.sums + kMeetRows;
       slots += 4 * G;
       if (lane == 0) {
-        const bool out_q = !(Q < 0x1p15);
+        const bool out_q = !(Q < 0x1p15) || exact;
         const GangSums q = out_q ? GangSums{0, SQ_BIG, 0} : to_fixed(Q);
         put_sums(slots + 4 * me, q, out_q, 0.0, Q);
         meet_join(norms, k, me, q);
@@ -252,7 +253,7 @@ __global__ void __launch_bounds__(Cfg<TS>::THREADS, 1) resident_fp32_kernel(cons
       float* Yn = a.Y[(k + 1) & 1];
       long long tr = 0;
       double trd = 0.0;
-      bool outD = false, out_t = false;
+      bool outD = false, out_t = fp64_sums(sh.st.ctl());
       for (int t = blockIdx.x; t < a.ntiles && ok; t += G) {
         int b, I, J, h;
         unpack_tile(a.tiles[t], b, I, J, h);

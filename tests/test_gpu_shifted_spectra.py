@@ -142,3 +142,32 @@ def test_fp32_solve(sp2, N, accelerated):
             got, want = _outcome(lambda: solve(sp2)), _outcome(lambda: _launch_per_layer(solve))
             right += bool(_same(got, want, exact, 5e-5))
     assert right >= 1
+
+
+@pytest.mark.parametrize("N", [1, 24, 308, 1100])
+@pytest.mark.parametrize("precision", ["split", "fp16", "fp32"])
+def test_no_state_or_every_state_occupied(sp2, N, precision):
+    """S goes to 0 or I, the sums of Y below the fixed-point units: as many layers all the same."""
+    import paper_2101_06385_gb300 as m
+
+    h = _tridiagonal(N, N // 2, -1.0, N)[0] if N > 1 else np.array([[0.3]], dtype=np.float32)
+    H = torch.from_numpy(h).cuda()
+    for shift in (True, False):
+        for n_occ in (0, N):
+
+            def solve(single):
+                if single:
+                    os.environ["SP2_SQUARE_KERNEL"] = "single"
+                try:
+                    m.finalize()
+                    m.init(0, shift_identity=shift)
+                    return m.density_matrix(H, n_occ, precision=precision)
+                finally:
+                    os.environ.pop("SP2_SQUARE_KERNEL", None)
+
+            (D, st), (D1, s1) = solve(False), solve(True)
+            assert (st.status, st.converged_by, st.iterations) == (s1.status, s1.converged_by, s1.iterations)
+            assert float((D - D1).abs().max()) <= 1e-6
+            assert abs(st.trace - n_occ) <= 1e-6 * max(1, n_occ)
+    m.finalize()
+    m.init(0)
