@@ -1100,9 +1100,9 @@ sp2_status resident_solve(const float* const* H, const int* N, const int* N_occ,
   void *pack, *part, *sums, *rn, *tdots, *tsums;
   CKS(ws(B_PACK, P.all, &pack));
   CKS(ws(B_PART, (size_t)B * std::max(iblocks, ggrid) * sizeof(double2), &part));
-  CKS(ws(B_TPART, (size_t)B * kMeetRows * sizeof(long long), &sums));
+  CKS(ws(B_TPART, (size_t)B * 2 * kMeetRows * sizeof(long long), &sums));
   CKS(ws(B_TDOTS, (size_t)nt * sizeof(double), &tdots));
-  CKS(ws(B_TSUMS, (size_t)nt * 8 * sizeof(long long), &tsums));
+  CKS(ws(B_TSUMS, (size_t)nt * sizeof(double2), &tsums));
   const long long ld_h = round_up(Nmax, 64), slot_h = ld_h * Nmax;
   void *hi[2], *lo[2], *hp[2];
   CKS(planes_for(split, 0, (size_t)slot_h * B * 2, &hi[0], &lo[0], &hp[0]));
@@ -1166,7 +1166,7 @@ sp2_status resident_solve(const float* const* H, const int* N, const int* N_occ,
   A.ld_rnp = carry.ld_rnp;
   A.slot_rnp = carry.slot_rnp;
   A.part = (double2*)part;
-  A.tile_sums = (long long*)tsums;
+  A.tile_sums = (double2*)tsums;
   A.tile_dots = (double*)tdots;
   A.dots_out = (double*)(dp + P.dots);
   A.sums = (long long*)sums;
@@ -1270,11 +1270,11 @@ sp2_status fp32_solve(const float* H, int N, int N_occ, double tol, int max_iter
   // one upload: control block, stamps, error word (read back), then pointers,
   // size, tickets, the meeting rows and the tiles
   const size_t o_st = sizeof(Ctl), o_err = o_st + (kResStamps + 2) / 2 * 8, o_ptr = o_err + 16,
-               o_sums = o_ptr + 64, o_tiles = o_sums + 2 * kMeetRows * sizeof(long long), bytes = o_tiles + (size_t)nt * sizeof(uint32_t);
+               o_sums = o_ptr + 64, o_tiles = o_sums + 3 * kMeetRows * sizeof(long long), bytes = o_tiles + (size_t)nt * sizeof(uint32_t);
   static_assert(sizeof(Ctl) % 8 == 0, "the offsets after it keep 8-byte alignment");
   void *pack, *part, *rn, *slots, *Y[2];
   CKS(ws(B_PACK, bytes, &pack));
-  CKS(ws(B_TSUMS, (size_t)grid * 16 * sizeof(long long), &slots));
+  CKS(ws(B_TSUMS, (size_t)grid * sizeof(double2), &slots));
   CKS(ws(B_PART, std::max(std::max(ggrid, igrid), rgrid) * sizeof(double2), &part));
   CKS(ws(B_RN, (size_t)N * sizeof(double), &rn));
   const long long ld_y = round_up(N, 4), slot_y = ld_y * N;
@@ -1312,7 +1312,7 @@ sp2_status fp32_solve(const float* H, int N, int N_occ, double tol, int max_iter
   A.ctl = (Ctl*)dp;
   A.rn = (double*)rn;
   A.sums = (long long*)(dp + o_sums);
-  A.slots = (long long*)slots;
+  A.slots = (double2*)slots;
   A.stamps = (unsigned*)(dp + o_st);
   A.err = (int*)(dp + o_err);
   A.late = g.late_dev;

@@ -212,8 +212,8 @@ struct ResArgs {
   float* rnp[2];           // row-norm segment sums, as SqArgs::rnp_out
   long long ld_rnp, slot_rnp;
   double2* part;           // [batch][blocks] block sums of the input layer
-  long long* sums;         // [batch][kMeetRows] meeting rows (csrc/resident.cuh), zero
-  long long* tile_sums;    // [2][ntiles][4] a tile's sums by the layer's parity (csrc/resident.cuh)
+  long long* sums;         // [batch][2][kMeetRows] meeting rows (csrc/resident.cuh), zero: of the layers, of FP64 sums
+  double2* tile_sums;      // [ntiles] a tile's sums in FP64 (csrc/resident.cuh, meet_fp64)
   double* tile_dots;       // [ntiles] Tr[D H] per tile
   double* dots_out;        // [batch][3], entry 0: Tr[D H]
   unsigned* tickets;       // [batch] zero: finished blocks of the input layer
@@ -332,8 +332,8 @@ struct Res32Args {
   int ntiles;
   Ctl* ctl;
   double* rn;              // [N] row norms of the layer's input
-  long long* sums;         // [2][kMeetRows] meeting rows of the traces and of the square norms, zero
-  long long* slots;        // [2][2][grid][4] by the layer's parity: each CTA's trace, then its square norm
+  long long* sums;         // [3][kMeetRows] meeting rows of the traces, of the square norms, of FP64 sums, zero
+  double2* slots;          // [grid] each CTA's sum in FP64 (meet_fp64)
   unsigned* stamps;        // as ResArgs
   int* err;
   int* late;               // as SqArgs

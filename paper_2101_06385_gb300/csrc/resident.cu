@@ -52,7 +52,8 @@ struct Slot {
   int cnt, me;           // the gang, and this tile's place in it
   int direct;            // the producer itself watches the gang's arrivals
   int stored;            // epilogue warps that have stored their part of the planes
-  int exact;             // every sum in FP64 (fp64_sums)
+  float t_limit, sq_limit;  // ranges of a diagonal element and a lane's squares in fixed point; 0: all
+  unsigned rn_limit;        //   sums in FP64 (fp64_sums); of a row norm's segment (its bits)
   long long* rows;       // the gang's meeting rows
   SolveState st;
 };
@@ -86,6 +87,8 @@ struct Shared {
 // can occur: a warp whose sum leaves the range, or is not a number, marks it and
 // hands it over in FP64 (so do all of a solve where fp64_sums says so).
 constexpr long long SQ_LIMIT = (1ll << 58) + (1ll << 50);  // a 32 x 32 block's 32, with rounding
+constexpr float SQ_LANE = 4.f;                             // a lane's sum of 32 squares: elements below T_LIMIT
+constexpr unsigned RN_LIMIT = 0x40800000u;                 // a row norm's segment: 4.0
 constexpr long long SQ_OUT = -1;                           // marks a warp's sum that is in Shared::red_d (as T_OUT)
 
 __device__ __forceinline__ long long fix_sq(float v) {
@@ -125,7 +128,7 @@ __device__ __forceinline__ double row_norm(const ResArgs& a, const Slot& s, int 
     acc += fix_sq(v[u]);
     top = max(top, __float_as_uint(v[u]));
   }
-  if (top > 0x40800000u || s.exact) {
+  if (top > s.rn_limit) {
     auto every8 = [&](int first) {  // epi::row_norm's order
       double sum = 0.0;
 #pragma unroll 1
@@ -245,20 +248,21 @@ __device__ __forceinline__ bool epilogue(const ResArgs& a, Shared& sh, int c, ui
   const bool outD = (p.out_mode == OUT_D);
   // the diagonal needs no product: its square comes from the row norms
   long long tr = 0, sq = 0;
+  double yd = 0.0;
   float ydf = 0.f, ydo = 0.f;
   if (dchunk) {
     float yold_d = 0.f;
 #pragma unroll
     for (int k = 0; k < 32; ++k)
       if (k == id) yold_d = y[k];
-    double yd = 0.0;
     if (dlane) {
       yd = p.ca_d * (double)yold_d + p.cb_d * rn_l + p.cc_d;
       tr = __double2ll_rn(yd * 0x1p50);
       ydf = (float)yd;
       ydo = outD ? (float)(yd + p.alpha_out) : ydf;
     }
-    if (__any_sync(0xffffffffu, !(fabsf(ydf) < T_LIMIT) || s.exact)) {
+    // (a lone tile's chain runs through here: it looks at the range with its squares)
+    if (!LOCAL && __any_sync(0xffffffffu, dlane && !(fabsf(ydf) < s.t_limit))) {
       const double T = warp_sum_d(yd);
       if (lane == 0) sh.red_d[c][ew].x = T;
       tr = T_OUT;
@@ -320,13 +324,18 @@ __device__ __forceinline__ bool epilogue(const ResArgs& a, Shared& sh, int c, ui
       }
     }
     const float sql = ((rs[0] + rs[1]) + (rs[2] + rs[3])) + ((rs[4] + rs[5]) + (rs[6] + rs[7]));
-    const bool wild = __any_sync(0xffffffffu, !(sql < 16.f) || s.exact);
+    const bool wild = __any_sync(0xffffffffu, !(sql < s.sq_limit));
     auto sum_squares = [&]() {
       sq = warp_sum_ll(fix_sq(sql));
       if (wild || sq > SQ_LIMIT) {
         const double Q = warp_sum_d((double)sql);
         if (lane == 0) sh.red_d[c][ew].y = Q;
         sq = SQ_OUT;
+        if (LOCAL) {
+          const double T = warp_sum_d(yd);
+          if (lane == 0) sh.red_d[c][ew].x = T;
+          tr = T_OUT;
+        }
       }
     };
     if (!outD) {
@@ -434,7 +443,8 @@ __device__ __forceinline__ void control(const ResArgs& a, Shared& sh, int c, int
     s.st.load(gc, lane);  // as the input layer's control step left it
     const int cnt = a.tile_cnt[b], off = a.tile_off[b];
     const bool leader = t == off;
-    long long* rows = a.sums + (long long)b * kMeetRows;
+    long long* rows = a.sums + (long long)b * 2 * kMeetRows;
+    int wide = 0;  // layers whose sums met in FP64
     const bool twice = (I >> 1) != (J >> 1);  // the mirror's squares
     bool act = hot->next.active != 0;
     unsigned* st = a.stamps + (long long)b * kResStamps;
@@ -453,7 +463,10 @@ __device__ __forceinline__ void control(const ResArgs& a, Shared& sh, int c, int
       s.direct = LOCAL || (cnt > 1 && !a.two_slots);
       s.me = t - off;
       s.stored = 0;
-      s.exact = fp64_sums(hot) ? 1 : 0;
+      const bool fp64 = fp64_sums(hot);
+      s.t_limit = fp64 ? 0.f : T_LIMIT;
+      s.sq_limit = fp64 ? 0.f : SQ_LANE;
+      s.rn_limit = fp64 ? 0u : RN_LIMIT;
       s.rows = rows;
       if (act) {
         mbar_arrive(&sh.ready[c]);
@@ -478,7 +491,7 @@ __device__ __forceinline__ void control(const ResArgs& a, Shared& sh, int c, int
       }
       // the tile's sums; with one out of range all of them in FP64
       long long rq = lane < EPI_WARPS ? sh.red_q[c][lane] : 0, rt = lane < EPI_WARPS ? sh.red_t[c][lane] : 0;
-      const int mul = twice ? 1 : 0;
+      const int mul = !LOCAL && twice ? 1 : 0;
       double trY = 0.0, sqY = 0.0;
       const bool out = __any_sync(0xffffffffu, rq == SQ_OUT || rt == T_OUT);
       GangSums G{0, SQ_BIG, 0};
@@ -495,7 +508,6 @@ __device__ __forceinline__ void control(const ResArgs& a, Shared& sh, int c, int
       if (cnt > 1) {
         if (lane == 0) {
           if (outD) a.tile_dots[t] = E;
-          put_sums(a.tile_sums + 4 * ((long long)(k & 1) * a.ntiles + t), G, out, trY, sqY);
           meet_join(rows, k, t - off, G);
         }
         if (!meet_wait(rows, k, cnt, lane, a.err, &sh.abort, idle)) {
@@ -503,9 +515,17 @@ __device__ __forceinline__ void control(const ResArgs& a, Shared& sh, int c, int
           break;
         }
         if (lane == 0 && !outD && !direct) mbar_arrive(&sh.ready[c]);
+        const GangSums mine = G;
         G = meet_sums(rows, k, lane);
         if (leader) meet_empty(rows, k, lane);
-        if (out_of_range(G)) sum_slots(a.tile_sums + 4 * ((long long)(k & 1) * a.ntiles + off), cnt, lane, trY, sqY);
+        if (out_of_range(G)) {
+          if (!out) to_double(mine, trY, sqY);
+          if (!meet_fp64(rows + kMeetRows, wide, a.tile_sums + off, t - off, cnt, lane, trY, sqY, a.err, &sh.abort,
+                         idle)) {
+            ok = false;
+            break;
+          }
+        }
         if (outD && leader) {
           E = 0.0;
           for (int i = lane; i < cnt; i += 32) E += __ldcg(&a.tile_dots[off + i]);
@@ -834,7 +854,7 @@ __global__ void __launch_bounds__(256) resident_input_kernel(const ResArgs a, in
   }
   __syncthreads();
   // the gang's meeting rows of the resident launch
-  if (blockIdx.x == 0 && threadIdx.x < kMeetRows) a.sums[(long long)b * kMeetRows + threadIdx.x] = 0;
+  if (blockIdx.x == 0 && threadIdx.x < 2 * kMeetRows) a.sums[(long long)b * 2 * kMeetRows + threadIdx.x] = 0;
   double2* part = a.part + (long long)b * gridDim.x;
   if (threadIdx.x == 0) {
     double q = 0.0, t = 0.0;

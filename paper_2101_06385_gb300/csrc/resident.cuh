@@ -168,8 +168,8 @@ __device__ __forceinline__ long long warp_sum_ll(long long v) {
 // A layer's sums over a gang in 64-bit fixed point, exact in any order: tr Y' in
 // units of 2^-50, ||Y'||_F^2 as q_hi 2^-25 + q_lo 2^-53 (q_lo of each member in
 // [0, 2^28)).  A member with a sum out of range, or no number, adds SQ_BIG to
-// q_hi, far above any sum in range (N 2^25): every member then adds up the
-// members' slots (put_sums) in FP64.
+// q_hi, far above any sum in range (N 2^25): all members then meet once more, with
+// their sums in FP64 (meet_fp64).
 struct GangSums {
   long long t, q_hi, q_lo;
 };
@@ -184,34 +184,6 @@ __device__ __forceinline__ void to_double(const GangSums& s, double& trY, double
 }
 
 __device__ __forceinline__ bool out_of_range(const GangSums& s) { return s.q_hi >= SQ_BIG / 2; }
-
-// A member's sums of one layer in its slot, four words: fixed point, or (out) FP64.
-// Two slots by the layer's parity: before a member writes the one of layer k + 2 the
-// meeting of layer k + 1 is over, which everyone joined after reading layer k's.
-__device__ __forceinline__ void put_sums(long long* slot, const GangSums& s, bool out, double t, double q) {
-  if (out)
-    __stcg(reinterpret_cast<longlong2*>(slot), make_longlong2(__double_as_longlong(t), __double_as_longlong(q)));
-  else
-    __stcg(reinterpret_cast<longlong2*>(slot), make_longlong2(s.t, s.q_hi));
-  __stcg(reinterpret_cast<longlong2*>(slot) + 1, make_longlong2(s.q_lo, out ? 1 : 0));
-}
-// The sums of cnt slots (one warp, in every lane).
-__device__ __forceinline__ void sum_slots(const long long* slots, int cnt, int lane, double& t, double& q) {
-  t = q = 0.0;
-  for (int i = lane; i < cnt; i += 32) {
-    const longlong2 a = __ldcg(reinterpret_cast<const longlong2*>(slots + 4 * i));
-    const longlong2 b = __ldcg(reinterpret_cast<const longlong2*>(slots + 4 * i) + 1);
-    if (b.y) {
-      t += __longlong_as_double(a.x);
-      q += __longlong_as_double(a.y);
-    } else {
-      t += (double)a.x * T_UNIT;
-      q += (double)a.y * Q_HI_UNIT + (double)b.x * Q_LO_UNIT;
-    }
-  }
-  t = warp_sum_d(t);
-  q = warp_sum_d(q);
-}
 
 // The meeting of a gang after a layer.  Members add their sums and then their
 // count into one of eight sectors of the layer's row; a member waits until the
@@ -310,6 +282,31 @@ __device__ __forceinline__ void meet_empty(long long* rows, int k, int lane) {
   __syncwarp();
 }
 static_assert(MEET_GROUPS * MEET_WORDS == 32, "one word a lane");
+
+// The gang's sums in FP64 (one warp, in every lane): the members, who all know that a
+// sum was out of range, leave theirs in slots and meet on rows of their own, j-th
+// time.  The slots are read before the next layer's meeting is joined, so they are
+// free when that one says the same again.  False: abort or time-out.
+__device__ __forceinline__ bool meet_fp64(long long* rows, int& j, double2* slots, int me, int cnt, int lane,
+                                          double& t, double& q, const int* err, const volatile int* abort_flag,
+                                          unsigned long long limit) {
+  if (lane == 0) {
+    __stcg(slots + me, make_double2(t, q));
+    meet_join(rows, j, me, GangSums{0, 0, 0}, false);
+  }
+  if (!meet_wait(rows, j, cnt, lane, err, abort_flag, limit)) return false;
+  t = q = 0.0;
+  for (int i = lane; i < cnt; i += 32) {
+    const double2 v = __ldcg(slots + i);
+    t += v.x;
+    q += v.y;
+  }
+  t = warp_sum_d(t);
+  q = warp_sum_d(q);
+  if (me == 0) meet_empty(rows, j, lane);
+  ++j;
+  return true;
+}
 
 }  // namespace res
 }  // namespace sp2

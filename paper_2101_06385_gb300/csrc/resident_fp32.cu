@@ -120,6 +120,8 @@ __device__ __forceinline__ bool control(const Res32Args& a, Shared<TS>& sh, int 
   sh.st.load(a.ctl, lane);
   if (!hot->next.active) return true;
   const bool exact = fp64_sums(hot);
+  long long* fp64_rows = a.sums + 2 * kMeetRows;
+  int wide = 0;  // meetings of sums in FP64
   const uint64_t t0 = globaltimer();
   if (lane == 0) {
     mbar_arrive(&sh.gate);
@@ -130,8 +132,8 @@ __device__ __forceinline__ bool control(const Res32Args& a, Shared<TS>& sh, int 
     const uint32_t ph = k & 1;
     if (!__all_sync(0xffffffffu, mbar_wait(&sh.tiles_done, ph, &sh.abort, lim))) return false;
     const bool outD = hot->next.out_mode == OUT_D;
-    // traces and square norms out of the fixed-point range, or no number, go through
-    // the members' slots in FP64, as in csrc/resident.cu
+    // traces and square norms out of the fixed-point range, or no number, meet once
+    // more in FP64, as in csrc/resident.cu
     double trY = 0.0, sqY = 0.0;
     const long long rt = lane < FW ? sh.red_t[lane] : 0;
     const bool out_t = __any_sync(0xffffffffu, rt == T_OUT);
@@ -140,37 +142,35 @@ __device__ __forceinline__ bool control(const Res32Args& a, Shared<TS>& sh, int 
       S = GangSums{warp_sum_ll(rt), 0, 0};
     else
       trY = warp_sum_d(rt == T_OUT ? sh.red_d[lane] : (double)rt * T_UNIT);
-    long long* slots = a.slots + (long long)(k & 1) * 8 * G;  // of the traces, then of the norms
-    if (lane == 0) {
-      put_sums(slots + 4 * me, S, out_t, trY, 0.0);
-      meet_join(a.sums, k, me, S);
-    }
+    if (lane == 0) meet_join(a.sums, k, me, S);
     if (!meet_wait(a.sums, k, G, lane, a.err, ab, lim)) return false;
     if (lane == 0 && !outD) mbar_arrive(&sh.gate);
+    const long long own = S.t;
     S = meet_sums(a.sums, k, lane);
     if (me == 0) meet_empty(a.sums, k, lane);
-    const bool wide = out_of_range(S);
-    if (wide) sum_slots(slots, G, lane, trY, sqY);
+    if (!out_of_range(S)) {
+      trY = (double)S.t * T_UNIT;
+    } else {
+      if (!out_t) trY = (double)own * T_UNIT;
+      if (!meet_fp64(fp64_rows, wide, a.slots, me, G, lane, trY, sqY, a.err, ab, lim)) return false;
+    }
     if (!outD) {
       if (!__all_sync(0xffffffffu, mbar_wait(&sh.rn_done, ph, &sh.abort, lim))) return false;
       const double Q = warp_sum_d(lane < RN_WARPS ? sh.red_q[lane] : 0.0);
       long long* norms = a.sums + kMeetRows;
-      slots += 4 * G;
-      if (lane == 0) {
-        const bool out_q = !(Q < 0x1p15) || exact;
-        const GangSums q = out_q ? GangSums{0, SQ_BIG, 0} : to_fixed(Q);
-        put_sums(slots + 4 * me, q, out_q, 0.0, Q);
-        meet_join(norms, k, me, q);
-      }
+      if (lane == 0) meet_join(norms, k, me, !(Q < 0x1p15) || exact ? GangSums{0, SQ_BIG, 0} : to_fixed(Q));
       if (!meet_wait(norms, k, G, lane, a.err, ab, lim)) return false;
       const GangSums q = meet_sums(norms, k, lane);
       if (me == 0) meet_empty(norms, k, lane);
-      double t;
-      if (out_of_range(q)) sum_slots(slots, G, lane, t, sqY);
-      else to_double(q, t, sqY);
+      double t = 0.0;
+      if (!out_of_range(q)) {
+        to_double(q, t, sqY);
+      } else {
+        sqY = Q;
+        if (!meet_fp64(fp64_rows, wide, a.slots, me, G, lane, t, sqY, a.err, ab, lim)) return false;
+      }
     }
     if (lane == 0) {
-      if (!wide) trY = (double)S.t * T_UNIT;
       resident_step(sh.st, trY, sqY, me == 0 ? a.ctl : nullptr);
       if (!outD) mbar_arrive(&sh.coef);
       if (me == 0 && k + 1 < kResStamps) a.stamps[k + 1] = (unsigned)(globaltimer() - t0);
@@ -252,7 +252,6 @@ __global__ void __launch_bounds__(Cfg<TS>::THREADS, 1) resident_fp32_kernel(cons
       const float* Y = a.Y[k & 1];
       float* Yn = a.Y[(k + 1) & 1];
       long long tr = 0;
-      double trd = 0.0;
       bool outD = false, out_t = fp64_sums(sh.st.ctl());
       for (int t = blockIdx.x; t < a.ntiles && ok; t += G) {
         int b, I, J, h;
@@ -345,7 +344,6 @@ __global__ void __launch_bounds__(Cfg<TS>::THREADS, 1) resident_fp32_kernel(cons
             const int r = r0 + e;
             const double yd = p.ca_d * (double)__ldcg(Y + (long long)r * ld + r) + p.cb_d * __ldcg(a.rn + r) + p.cc_d;
             tr += __double2ll_rn(yd * 0x1p50);
-            trd += yd;
             out_t = out_t || !(fabsf((float)yd) < T_LIMIT);
             out[(long long)r * lo + r] = outD ? (float)(yd + p.alpha_out) : (float)yd;
           }
@@ -353,6 +351,16 @@ __global__ void __launch_bounds__(Cfg<TS>::THREADS, 1) resident_fp32_kernel(cons
       }
       if (!ok) break;
       if (__any_sync(0xffffffffu, out_t)) {
+        // the same elements once more, in FP64
+        const LayerParams p = sh.st.ctl()->next;
+        double trd = 0.0;
+#pragma unroll 1
+        for (int t = blockIdx.x; t < a.ntiles; t += G) {
+          int b, I, J, h;
+          unpack_tile(a.tiles[t], b, I, J, h);
+          for (int r = I * TS + tid; I == J && r < min(N, (I + 1) * TS); r += C::FT)
+            trd += p.ca_d * (double)__ldcg(Y + (long long)r * ld + r) + p.cb_d * __ldcg(a.rn + r) + p.cc_d;
+        }
         trd = warp_sum_d(trd);
         if (lane == 0) sh.red_d[warp] = trd;
         tr = T_OUT;

@@ -98,6 +98,21 @@ __device__ __forceinline__ void turn_tmem(float* trb, uint32_t taddr, int lane, 
   }
 }
 
+// (a - b) s by components, as two packed operations.
+__device__ __forceinline__ float2 scaled_difference(float2 a, float2 b, float s) {
+  float2 r;
+  asm("{\n\t.reg .b64 x, y, z;\n\t"
+      "mov.b64 x, {%2, %3};\n\t"
+      "mov.b64 y, {%4, %5};\n\t"
+      "mov.b64 z, {%6, %6};\n\t"
+      "sub.rn.f32x2 x, x, y;\n\t"
+      "mul.rn.f32x2 x, x, z;\n\t"
+      "mov.b64 {%0, %1}, x;\n\t}\n"
+      : "=f"(r.x), "=f"(r.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(s));
+  return r;
+}
+
 // Stores the operand planes of the chunk (Eq. 12: hp = 2^s fp16(x) and lo' =
 // fp16(2^s (x - fp16(x))), finite where hp is not; plain FP16 keeps hi alone), four
 // halves per plane and row; p0, p1 at the lane's first row and column, rows
@@ -114,7 +129,8 @@ __device__ __forceinline__ void split_chunk(const float (&y)[32], float lo_scale
       __half2 p2 = __floats2half2_rn(x0, x1);
       if (SPLIT) {
         const float2 hf = __half22float2(p2);
-        const __half2 l2 = __floats2half2_rn((x0 - hf.x) * lo_scale, (x1 - hf.y) * lo_scale);
+        const float2 lf = scaled_difference(make_float2(x0, x1), hf, lo_scale);
+        const __half2 l2 = __floats2half2_rn(lf.x, lf.y);
         pl[e2] = *reinterpret_cast<const uint32_t*>(&l2);
         p2 = __hmul2(p2, s2);
       }
