@@ -1,14 +1,17 @@
 // C ABI of libsp2.so: argument checks, workspace, launch sequences.
 //
 // A call of sp2_density_matrix enqueues, on the library stream:
-//   K1 Gershgorin bounds -> K2 input layer + split -> FP64 row norms of Y_0
-//   and the first control step -> (max_iter + 2) squaring launches.  Each
-//   squaring launch reads the layer coefficients that the previous launch's
-//   control step left on the device, leaves the row norms of its output for
-//   the next one, runs the control step in its last tile, and does nothing
-//   once the solve has finished, so no host round trip is needed inside the
-//   loop.  The two launches after the loop's last layer are the refinement of
-//   Eq. 15; the last one writes D_out.
+//   K1 Gershgorin bounds -> K2 input layer + split, FP64 row norms of Y_0 and
+//   the first control step -> all layers in one cooperative launch, which ends
+//   with the solve's last one: the resident kernels (csrc/resident.cu, on the
+//   CUDA cores csrc/resident_fp32.cu) up to the sizes whose tiles the chip
+//   holds, above them a list of layers on the CTA pairs (csrc/syrk_tc2.cu).
+//   Control steps run on the device, so there is no host round trip inside the
+//   loop; the two layers after its last one are the refinement of Eq. 15, and
+//   the last of them writes D_out.
+// Networks and expansions go the same two ways (csrc/resident_net.cu, lists).
+// A launch a layer remains for batches with a larger matrix, large FP32 solves,
+// SP2_SQUARE_KERNEL=single, and where a cooperative launch is refused.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_runtime.h>

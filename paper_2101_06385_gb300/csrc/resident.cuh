@@ -191,8 +191,8 @@ __device__ __forceinline__ bool out_of_range(const GangSums& s) { return s.q_hi 
 // has met for layer k every member is done with the row of layer k - 1, so the
 // leader empties it then, for layer k + 2.  With a slot per member that everyone
 // polled, 144 readers (N = 2048) of 144 slots took 4 us from the last write to
-// the last read; so met, a solve takes, by calls of the public entry: N = 2048
-// single FP16 873 -> 795 us, N = 1000 748 -> 712 us, FP32 N = 512 622 -> 480 us.
+// the last read: calls of the public entry took 10 % longer at N = 2048 with single
+// FP16, 5 % at N = 1000 and 30 % in FP32 at N = 512.
 constexpr int MEET_GROUPS = 8, MEET_WORDS = 4;  // a sector: t, q_hi, count and q_lo, unused
 static_assert(3 * (MEET_GROUPS * MEET_WORDS + 2) == kMeetRows, "three rows, of sums and of arrivals");
 constexpr int MEET_SHIFT = 40;                  // the count above q_lo (304 x 2^28 < 2^37)

@@ -37,7 +37,6 @@ using namespace sp2::res;
 struct Slot {
   int b, I, J, t;  // matrix, tile row and column (128 units), tile index
   int closed;      // no more work in this slot
-  int pad;
   NetOp op[2];       // operations in progress, by the parity of their number in the slot, and
   LayerParams p[2];  // their coefficients (a layer's first touch of them in global memory would
                      // stand in its chain)

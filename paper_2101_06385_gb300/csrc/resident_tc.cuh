@@ -31,7 +31,10 @@ constexpr int THREADS = 32 * (CTL_WARP + 2);
 constexpr uint32_t TMEM_COLS = 512;  // two slots of an accumulator and an iterate
 constexpr uint32_t SLOT_COLS = 256, Y_COL = 128;
 constexpr uint32_t IDESC_T = (1u << 4) | ((uint32_t)(TB >> 3) << 17) | ((uint32_t)(TB >> 4) << 24);
-constexpr int WQ = 4;       // work queue entries (at most two outstanding)
+// Work queue entries.  A slot's next entry follows once all its epilogue warps have
+// read the one before (they have stored its planes), so a slot has at most one entry
+// that some warp has not read: two with both slots, a third in work, the end mark.
+constexpr int WQ = 4;
 constexpr int WQ_END = 255;
 
 // Loads one 128-row operand of K block k0: K-major, or the stored block left
